@@ -18,11 +18,14 @@
 // tile [0, N-1)), so a warp's loads for one r are contiguous.  The table is
 // computed in FP64 on the host (fft_twiddle_table) and rounded to T; the
 // inverse transform (sigma = +1) uses its conjugate.  No normalisation.
+// The FP64 group transforms (gfft) run in 64-bit block fixed point
+// (fft64.cuh) with a table of their own in the same order.
 #pragma once
 #include <cmath>
 #include <vector>
 
 #include "common.cuh"
+#include "fft64.cuh"
 
 namespace lm {
 
@@ -56,14 +59,6 @@ __device__ __forceinline__ void dft8(cplx<T>* v) {
   v[1] = cadd<T>(a1, b1); v[5] = csub<T>(a1, b1);
   v[2] = cadd<T>(a2, b2); v[6] = csub<T>(a2, b2);
   v[3] = cadd<T>(a3, b3); v[7] = csub<T>(a3, b3);
-}
-
-// Pass sequence shared by the kernels (block_fft, gfft) and the host
-// table builder: radix-8 passes, then one radix-4 or radix-2 pass for the
-// remaining bits.
-__host__ __device__ __forceinline__ int fft_num_passes(int log2N) { return (log2N + 2) / 3; }
-__host__ __device__ __forceinline__ int fft_pass_lr(int log2N, int p) {
-  return p < log2N / 3 ? 3 : log2N % 3;
 }
 
 // Twiddles w^{r k}, 1 <= r < R, w = exp(sigma 2 pi i / (Ns R)), of one
@@ -218,61 +213,65 @@ __device__ __forceinline__ void gsync(int grp) {
 
 // Twiddles w^{r k}, 1 <= r < R, of a butterfly of the pass with stride
 // Ns = 2^LNS (see butterfly_twiddles).
-template <typename T, int SIGN, int R, int LNS, bool TWC>
-__device__ __forceinline__ void twiddles_ct(cplx<T>* w, int k, const cplx<T>* __restrict__ tw) {
-  constexpr int LR = R == 8 ? 3 : (R == 4 ? 2 : 1);
-  const cplx<T>* t = tw + (k - 1);
-  if (sizeof(T) == 4) {
-    auto ev = [&](int r) {
-      cplx<T> c;
-      if (TWC) {
-        float sn, cs;
-        // 2 r k / (Ns R), exact in FP32 (a power-of-two scale)
-        sincospif((float)(r * k) * (2.0f / (float)(1 << (LNS + LR))), &sn, &cs);
-        c.x = (T)cs;
-        c.y = (T)(-sn);
-      } else {
-        c = __ldg(t + (r << LNS));
-      }
-      if (SIGN > 0) c.y = -c.y;
-      return c;
-    };
-    w[1] = ev(1);
-    if (R >= 4) {
-      w[2] = ev(2);
-      w[3] = cmul<T>(w[1], w[2]);
-    }
-    if (R == 8) {
-      w[4] = ev(4);
-      w[5] = cmul<T>(w[4], w[1]);
-      w[6] = cmul<T>(w[4], w[2]);
-      w[7] = cmul<T>(w[4], w[3]);
-    }
-  } else {
-#pragma unroll
-    for (int r = 1; r < R; ++r) {
-      w[r] = __ldg(t + (r << LNS));
-      if (SIGN > 0) w[r].y = -w[r].y;
-    }
+template <int SIGN, int R, int LNS>
+__device__ __forceinline__ void twiddles_ct(float2* w, int k, const float2* __restrict__ tw) {
+  const float2* t = tw + (k - 1);
+  auto ev = [&](int r) {
+    float2 c = __ldg(t + (r << LNS));
+    if (SIGN > 0) c.y = -c.y;
+    return c;
+  };
+  w[1] = ev(1);
+  if (R >= 4) {
+    w[2] = ev(2);
+    w[3] = cmul<float>(w[1], w[2]);
+  }
+  if (R == 8) {
+    w[4] = ev(4);
+    w[5] = cmul<float>(w[4], w[1]);
+    w[6] = cmul<float>(w[4], w[2]);
+    w[7] = cmul<float>(w[4], w[3]);
   }
 }
 
+// Arithmetic of the group transforms.  FP32: float2 values.  FP64: 64-bit
+// block fixed point (fft64.cuh), where pass P shifts its inputs right by sh.
+struct PassShift {
+  int sh, half;
+};
+template <int SIGN, int R, int LNS>
+__device__ __forceinline__ void twiddle_ct(float2* v, int k, const float2* __restrict__ tw, PassShift) {
+  float2 wr[8];
+  twiddles_ct<SIGN, R, LNS>(wr, k, tw);
+#pragma unroll
+  for (int r = 1; r < R; ++r) v[r] = cmul<float>(v[r], wr[r]);
+}
+template <int SIGN, int R, int LNS>
+__device__ __forceinline__ void twiddle_ct(cfx* v, int k, const TwFx* __restrict__ tw, PassShift s) {
+  const int4* t = reinterpret_cast<const int4*>(tw + (k - 1));
+  v[0] = fx_shift(v[0], s.sh, s.half);
+#pragma unroll
+  for (int r = 1; r < R; ++r) {
+    const int4 q = __ldg(t + (r << LNS));
+    v[r] = fx_twiddle<SIGN>(v[r], TwFx{q.x, q.y, q.z, q.w}, s.sh, s.half);
+  }
+}
+template <int SIGN, int R> __device__ __forceinline__ void butterfly(float2* v) { dft_r<float, SIGN, R>(v); }
+template <int SIGN, int R> __device__ __forceinline__ void butterfly(cfx* v) { fdft_r<SIGN, R>(v); }
+
 // Middle pass P (radix 8, stride Ns = 8^P) from `in` to `out`.
-template <typename T, int SIGN, int L, int P, bool TWC>
-__device__ __forceinline__ void gpass8(const cplx<T>* in, cplx<T>* out, int j, const cplx<T>* __restrict__ tw) {
+template <typename V, typename W, int SIGN, int L, int P>
+__device__ __forceinline__ void gpass8(const V* in, V* out, int j, const W* __restrict__ tw, PassShift s) {
   constexpr int G = 1 << (L - 3), LNS = 3 * P, NS = 1 << LNS;
   constexpr int RS = G + G / 8;    // shared-memory distance of G positions (G % 8 == 0)
   constexpr int WS = NS + NS / 8;  // of Ns positions
-  cplx<T> v[8];
+  V v[8];
   const int rb = j + (j >> 3);
 #pragma unroll
   for (int r = 0; r < 8; ++r) v[r] = in[rb + r * RS];
   const int k = j & (NS - 1);
-  cplx<T> wr[8];
-  twiddles_ct<T, SIGN, 8, LNS, TWC>(wr, k, tw);
-#pragma unroll
-  for (int r = 1; r < 8; ++r) v[r] = cmul<T>(v[r], wr[r]);
-  dft8<T, SIGN>(v);
+  twiddle_ct<SIGN, 8, LNS>(v, k, tw, s);
+  butterfly<SIGN, 8>(v);
   const int o = ((j - k) << 3) + k;
   const int ob = o + (o >> 3);
 #pragma unroll
@@ -280,13 +279,12 @@ __device__ __forceinline__ void gpass8(const cplx<T>* in, cplx<T>* out, int j, c
 }
 
 // Last pass (radix 8, 4 or 2) from `in` into the registers x.
-template <typename T, int SIGN, int L, bool TWC>
-__device__ __forceinline__ void gpass_last(cplx<T> (&x)[8], const cplx<T>* in, int j,
-                                           const cplx<T>* __restrict__ tw) {
+template <typename V, typename W, int SIGN, int L>
+__device__ __forceinline__ void gpass_last(V (&x)[8], const V* in, int j, const W* __restrict__ tw, PassShift s) {
   constexpr int G = 1 << (L - 3), NP = (L + 2) / 3, P = NP - 1;
   constexpr int LNS = 3 * P, NS = 1 << LNS, LR = L - LNS, R = 1 << LR, NB = 8 / R;
   constexpr int RS = (G * NB) + (G * NB) / 8;  // distance of N/R positions (a multiple of 8)
-  cplx<T> v[8];
+  V v[8];
 #pragma unroll
   for (int u = 0; u < NB; ++u) {
     const int jj = u * G + j;
@@ -294,49 +292,143 @@ __device__ __forceinline__ void gpass_last(cplx<T> (&x)[8], const cplx<T>* in, i
     const int rb = jj + (jj >> 3);
 #pragma unroll
     for (int r = 0; r < R; ++r) v[u * R + r] = in[rb + r * RS];
-    cplx<T> wr[8];
-    twiddles_ct<T, SIGN, R, LNS, TWC>(wr, k, tw);
-#pragma unroll
-    for (int r = 1; r < R; ++r) v[u * R + r] = cmul<T>(v[u * R + r], wr[r]);
+    twiddle_ct<SIGN, R, LNS>(v + u * R, k, tw, s);
   }
 #pragma unroll
   for (int u = 0; u < NB; ++u) {
-    dft_r<T, SIGN, R>(v + u * R);
+    butterfly<SIGN, R>(v + u * R);
 #pragma unroll
     for (int q = 0; q < R; ++q) x[u + q * NB] = v[u * R + q];
   }
 }
 
-template <typename T, int SIGN, int L, int P, int SYNC, bool TWC>
-__device__ __forceinline__ void gpass_mid(cplx<T>* buf0, cplx<T>* buf1, int& w, int j, int grp,
-                                          const cplx<T>* __restrict__ tw) {
+// Shift of pass P (P >= 1) when the sum bound allows Dn bits in all, and the
+// bits dropped by the passes up to P.
+template <int P> __device__ __forceinline__ int pass_drop(int Dn) { return Dn < 3 * P ? Dn : 3 * P; }
+template <int P> __device__ __forceinline__ PassShift pass_shift(int Dn) {
+  const int sh = pass_drop<P>(Dn) - pass_drop<P - 1>(Dn);
+  return PassShift{sh, (1 << sh) >> 1};
+}
+
+template <typename V, typename W, int SIGN, int L, int P, int SYNC>
+__device__ __forceinline__ void gpass_mid(V* buf0, V* buf1, int& w, int j, int grp, const W* __restrict__ tw,
+                                          int Dn) {
   constexpr int NP = (L + 2) / 3;
   if constexpr (P < NP - 1) {
-    gpass8<T, SIGN, L, P, TWC>(w ? buf1 : buf0, w ? buf0 : buf1, j, tw);
+    gpass8<V, W, SIGN, L, P>(w ? buf1 : buf0, w ? buf0 : buf1, j, tw, pass_shift<P>(Dn));
     gsync<SYNC, (1 << (L - 3))>(grp);
     w ^= 1;
-    gpass_mid<T, SIGN, L, P + 1, SYNC, TWC>(buf0, buf1, w, j, grp, tw);
+    gpass_mid<V, W, SIGN, L, P + 1, SYNC>(buf0, buf1, w, j, grp, tw, Dn);
   }
 }
 
-// The transform of x (positions j + m G in, positions j + m G out); w selects
-// the exchange buffer that is free to write and is left pointing at the
-// buffer not read last.
-template <typename T, int SIGN, int L, int SYNC, bool TWC>
-__device__ __forceinline__ void gfft(cplx<T> (&x)[8], cplx<T>* buf0, cplx<T>* buf1, int& w, int j, int grp,
-                                     const cplx<T>* __restrict__ tw) {
-  static_assert(L >= 4 && L <= 11, "transform length 16..2048");
-  constexpr int G = 1 << (L - 3);
-  dft8<T, SIGN>(x);
-  {
-    cplx<T>* out = w ? buf1 : buf0;
-    const int b = 9 * j;  // sidx(8 j + q) = 9 j + q
+// First pass (radix 8, no twiddles) of x into the free exchange buffer.
+template <typename V, int SIGN> __device__ __forceinline__ void gpass_first(V (&x)[8], V* out, int j) {
+  butterfly<SIGN, 8>(x);
+  const int b = 9 * j;  // sidx(8 j + q) = 9 j + q
 #pragma unroll
-    for (int q = 0; q < 8; ++q) out[b + q] = x[q];
+  for (int q = 0; q < 8; ++q) out[b + q] = x[q];
+}
+
+// Reduction scratch of a block's transforms (FP64 only): the groups' warps
+// leave their maxima in the first half and their sums in the second.  lC:
+// log2 of the interleaved columns of a column tile (SYNC 2).
+constexpr int GRED_WORDS = 512;
+struct GRed {
+  unsigned* red;
+  int lC;
+};
+template <typename T> struct GRedWords { static constexpr int value = sizeof(T) == 8 ? GRED_WORDS : 1; };
+
+// Reduce v over a transform's threads: MAX or sum.  Within a warp by
+// shuffles; the warps' results go to `slots`, to be combined by gred_read
+// after a barrier of the group.
+template <bool MAX, int SYNC, int G>
+__device__ __forceinline__ unsigned gred_warp(unsigned v, unsigned* slots, int grp, int lC) {
+  const int lo = SYNC == 2 ? 1 << lC : 1;
+  const int hi = SYNC == 0 && G < 32 ? G / 2 : 16;
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) {
+    if (off <= hi && off >= lo) {
+      const unsigned o = __shfl_xor_sync(0xffffffffu, v, off);
+      v = MAX ? max(v, o) : v + o;
+    }
   }
-  gsync<SYNC, G>(grp);
-  gpass_mid<T, SIGN, L, 1, SYNC, TWC>(buf0, buf1, w, j, grp, tw);
-  gpass_last<T, SIGN, L, TWC>(x, w ? buf1 : buf0, j, tw);
+  if (SYNC == 1) {
+    if ((threadIdx.x & 31) == 0) slots[grp * 16 + ((threadIdx.x % G) >> 5)] = v;
+  } else if (SYNC == 2) {
+    if ((threadIdx.x & 31) < (1u << lC)) slots[((threadIdx.x >> 5) << lC) + (threadIdx.x & 31)] = v;
+  }
+  return v;
+}
+template <bool MAX, int SYNC, int G>
+__device__ __forceinline__ unsigned gred_read(unsigned v, const unsigned* slots, int grp, int lC) {
+  if (SYNC == 1) {
+    v = 0;
+#pragma unroll
+    for (int i = 0; i < G / 32; ++i) v = MAX ? max(v, slots[grp * 16 + i]) : v + slots[grp * 16 + i];
+  } else if (SYNC == 2) {
+    const int nw = blockDim.x >> 5, c = threadIdx.x & ((1 << lC) - 1);
+    v = 0;
+    for (int i = 0; i < nw; ++i) v = MAX ? max(v, slots[(i << lC) + c]) : v + slots[(i << lC) + c];
+  }
+  return v;
+}
+
+// The transform of x (positions j + m G in, positions j + m G out), times
+// 2^SC; w selects the exchange buffer that is free to write and is left
+// pointing at the buffer not read last.
+template <typename T, int SIGN, int L, int SYNC, int SC = 0>
+__device__ __forceinline__ void gfft(cplx<T> (&x)[8], cplx<T>* buf0, cplx<T>* buf1, int& w, int j, int grp,
+                                     const twid<T>* __restrict__ tw, GRed gr) {
+  static_assert(L >= 4 && L <= 11, "transform length 16..2048");
+  constexpr int G = 1 << (L - 3), NP = (L + 2) / 3;
+  if constexpr (sizeof(T) == 4) {
+    gpass_first<float2, SIGN>(x, w ? buf1 : buf0, j);
+    gsync<SYNC, G>(grp);
+    gpass_mid<float2, float2, SIGN, L, 1, SYNC>(buf0, buf1, w, j, grp, tw, 0);
+    gpass_last<float2, float2, SIGN, L>(x, w ? buf1 : buf0, j, tw, PassShift{0, 0});
+    if constexpr (SC != 0) {
+      constexpr float f = SC < 0 ? 1.0f / (float)(1 << (SC < 0 ? -SC : 0)) : (float)(1 << (SC < 0 ? 0 : SC));
+#pragma unroll
+      for (int m = 0; m < 8; ++m) x[m] = cscale<float>(x[m], f);
+    }
+  } else {
+    cfx* b0 = reinterpret_cast<cfx*>(buf0);
+    cfx* b1 = reinterpret_cast<cfx*>(buf1);
+    unsigned mx = 0;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) mx = max(mx, max(fx_abs_hi(x[m].x), fx_abs_hi(x[m].y)));
+    mx = gred_warp<true, SYNC, G>(mx, gr.red, grp, gr.lC);
+    if (SYNC != 0) gsync<SYNC, G>(grp);
+    mx = gred_read<true, SYNC, G>(mx, gr.red, grp, gr.lC);
+    const int emax = max((int)(mx >> 20), FX_EMIN);
+    cfx v[8];
+    unsigned ms = 0;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+      v[m].x = fx_from_double(x[m].x, emax, ms);
+      v[m].y = fx_from_double(x[m].y, emax, ms);
+    }
+    unsigned sum = gred_warp<false, SYNC, G>(fx_sum_units(ms), gr.red + GRED_WORDS / 2, grp, gr.lC);
+    gpass_first<cfx, SIGN>(v, w ? b1 : b0, j);
+    gsync<SYNC, G>(grp);
+    sum = gred_read<false, SYNC, G>(sum, gr.red + GRED_WORDS / 2, grp, gr.lC);
+    const int Dn = fx_sum_shift(sum);
+    gpass_mid<cfx, TwFx, SIGN, L, 1, SYNC>(b0, b1, w, j, grp, tw, Dn);
+    gpass_last<cfx, TwFx, SIGN, L>(v, w ? b1 : b0, j, tw, pass_shift<NP - 1>(Dn));
+    // exponents near the top of the range: 2^512 below, then a product that
+    // overflows as FP64 does (NaN for a transform with non-finite inputs)
+    const bool top = emax > 1980;
+    const int e = emax + pass_drop<NP - 1>(Dn) + SC - (top ? 512 : 0);
+#pragma unroll
+    for (int m = 0; m < 8; ++m) x[m] = mk<double>(fx_to_double(v[m].x, e), fx_to_double(v[m].y, e));
+    if (top) {
+      const double f = emax >= 2047 ? __longlong_as_double(0x7ff8000000000000LL) : 1.3407807929942597e154;
+#pragma unroll
+      for (int m = 0; m < 8; ++m) x[m] = cscale<double>(x[m], f);
+    }
+  }
   w ^= 1;
 }
 

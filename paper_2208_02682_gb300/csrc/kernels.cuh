@@ -222,8 +222,8 @@ __device__ __forceinline__ void load_pair_spectrum_ct(cplx<T> (&x)[8], const cpl
   }
 }
 
-// Spectrum Z of p + i q held at the thread's positions -> kx in [0, KXP)
-// halves of p and q, scaled by 1/N, into row `rowoff` of mixed fields da and
+// Spectrum Z of p + i q, times 1/(2 N), held at the thread's positions -> kx
+// in [0, KXP) halves of p and q (times 1/N) into row `rowoff` of mixed fields da and
 // db (db null: p only).  One exchange through the free buffer.
 template <typename T, int L, int SYNC>
 __device__ __forceinline__ void store_pair_spectrum_ct(const cplx<T> (&x)[8], cplx<T>* buf0, cplx<T>* buf1, int& w,
@@ -240,7 +240,6 @@ __device__ __forceinline__ void store_pair_spectrum_ct(const cplx<T> (&x)[8], cp
     for (int m = 0; m < 8; ++m) b[sidx<T>(j + m * G)] = x[m];
   }
   gsync<SYNC, G>(grp);
-  const T h = (T)0.5 / (T)N;
   cplx<T>* ra = da + rowoff;
   cplx<T>* rb = db ? db + rowoff : nullptr;
   for (int k = j; k < KXP; k += G) {
@@ -249,9 +248,9 @@ __device__ __forceinline__ void store_pair_spectrum_ct(const cplx<T> (&x)[8], cp
       const cplx<T> z1 = b[k + (k >> 3)];
       const int k2 = (N - k) & (N - 1);
       const cplx<T> z2 = b[k2 + (k2 >> 3)];
-      // P = (Z(k) + conj Z(N-k))/2, Q = (Z(k) - conj Z(N-k))/(2i)
-      P = mk<T>((z1.x + z2.x) * h, (z1.y - z2.y) * h);
-      Q = mk<T>((z1.y + z2.y) * h, (z2.x - z1.x) * h);
+      // P = Z(k) + conj Z(N-k), Q = (Z(k) - conj Z(N-k))/i
+      P = mk<T>(z1.x + z2.x, z1.y - z2.y);
+      Q = mk<T>(z1.y + z2.y, z2.x - z1.x);
     }
     ra[k] = P;
     if (rb) rb[k] = Q;

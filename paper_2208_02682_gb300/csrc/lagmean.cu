@@ -361,7 +361,7 @@ static void fill_desc(sw_handle* h, RunDesc<T>& d, int ppb) {
   d.pmix = (cplx<T>*)h->pmix;
   d.phys = (T*)h->phys;
   d.ef = (const T*)h->ef;
-  d.tw = (const cplx<T>*)h->tw;
+  d.tw = (const twid<T>*)h->tw;
   d.ctr = h->ctr;
   d.ticket = h->ticket;
   d.lC = h->lC;
@@ -834,7 +834,7 @@ extern "C" int64_t sw_state_bytes(const sw_params* p) {
 template <typename T>
 static void host_tables(const sw_params& p, const Geom& g, void* ef_host, void* tw_host, double2* tw64_host) {
   T* ef = (T*)ef_host;
-  cplx<T>* tw = (cplx<T>*)tw_host;
+  static_assert(sizeof(twid<T>) == sizeof(cplx<T>), "twiddle table size");
   for (int kyi = 0; kyi < g.NY; ++kyi)
     for (int kx = 0; kx < g.KXP; ++kx) {
       const double ky = kyi - g.K;
@@ -861,8 +861,9 @@ static void host_tables(const sw_params& p, const Geom& g, void* ef_host, void* 
   fft_twiddle_table(g.log2N, re.data(), im.data());
   for (int t = 0; t < g.N; ++t) {
     tw64_host[t] = make_double2(re[t], im[t]);
-    tw[t] = mk<T>((T)re[t], (T)im[t]);
+    if (sizeof(T) == 4) ((float2*)tw_host)[t] = make_float2((float)re[t], (float)im[t]);
   }
+  if (sizeof(T) == 8) fft_twiddle_table_fx(g.log2N, (TwFx*)tw_host);
 }
 
 extern "C" int sw_create(const sw_params* p, const double* ic_uvh, int ic_on_device, void* stream,

@@ -32,7 +32,7 @@ struct RunDesc {
   cplx<T>* pmix;  // row-pass products (mixed)
   T* phys;        // Strategy-2 gather buffer
   const T* ef;    // integrating-factor tables
-  const cplx<T>* tw;
+  const twid<T>* tw;
   long long* ctr;
   unsigned* ticket;
   int lC;         // column tile: C = 2^lC columns
@@ -94,6 +94,7 @@ template <typename T>
 __global__ void __launch_bounds__(col_max_threads<T>()) k_stage_col_inv(const RunDesc<T>* __restrict__ runs,
                                                        const int* __restrict__ start, int nruns, int stage) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ unsigned red[GRedWords<T>::value];  // FP64 transforms
   const int r = find_run(start, nruns, blockIdx.x);
   const RunDesc<T>& d = runs[r];
   pdl_wait();  // state written by the previous kernels: only after this
@@ -139,7 +140,7 @@ __global__ void __launch_bounds__(col_max_threads<T>()) k_stage_col_inv(const Ru
     }
     cplx<T>* b0 = reinterpret_cast<cplx<T>*>(smem_raw) + (size_t)c * col_buf_stride<T>(N, C);
     int w = 0;
-    gfft<T, +1, L, 2, false>(x, b0, b0 + row_stride<T>(N), w, j, 0, d.tw);
+    gfft<T, +1, L, 2>(x, b0, b0 + row_stride<T>(N), w, j, 0, d.tw, GRed{red, lC});
     cplx<T>* dst = d.mix + (long long)o * d.g.mi + kx;
 #pragma unroll
     for (int m = 0; m < 8; ++m) dst[(j + m * G) * KXP] = x[m];
@@ -154,6 +155,7 @@ template <typename T>
 __global__ void __launch_bounds__(col_max_threads<T>()) k_stage_col_fwd(const RunDesc<T>* __restrict__ runs,
                                                        const int* __restrict__ start, int nruns) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ unsigned red[GRedWords<T>::value];  // FP64 transforms
   const int r = find_run(start, nruns, blockIdx.x);
   const RunDesc<T>& d = runs[r];
   pdl_wait();  // state written by the previous kernels: only after this
@@ -172,15 +174,14 @@ __global__ void __launch_bounds__(col_max_threads<T>()) k_stage_col_fwd(const Ru
     for (int m = 0; m < 8; ++m) x[m] = src[(j + m * G) * KXP];
     cplx<T>* b0 = reinterpret_cast<cplx<T>*>(smem_raw) + (size_t)c * col_buf_stride<T>(N, C);
     int w = 0;
-    gfft<T, -1, L, 2, false>(x, b0, b0 + row_stride<T>(N), w, j, 0, d.tw);
-    const T inv = (T)1 / (T)N;
+    gfft<T, -1, L, 2, -L>(x, b0, b0 + row_stride<T>(N), w, j, 0, d.tw, GRed{red, lC});
     cplx<T>* dst = d.ps + (long long)p * d.g.ms + kx;
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
       const int k = j + m * G;
       if (k <= K || k >= N - K) {
         const int ky = k <= K ? k : k - N;
-        dst[(ky + K) * KXP] = kx <= K ? cscale<T>(x[m], inv) : mk<T>(0, 0);
+        dst[(ky + K) * KXP] = kx <= K ? x[m] : mk<T>(0, 0);
       }
     }
   });
@@ -259,15 +260,14 @@ __global__ void __launch_bounds__(1024, 1) k_stage_col_fwd_pipe(const RunDesc<fl
     __syncthreads();  // every thread has read the staged tile
     if (item + gridDim.x < total) pipe_stage(st, runs, start, nruns, item + gridDim.x);
     cp_async_commit();
-    gfft<float, -1, L, 2, false>(x, b0, b0 + row_stride<float>(N), w, j, 0, d.tw);
-    const float inv = 1.0f / (float)N;
+    gfft<float, -1, L, 2, -L>(x, b0, b0 + row_stride<float>(N), w, j, 0, d.tw, GRed{nullptr, 2});
     float2* dst = d.ps + (long long)p * d.g.ms + kx;
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
       const int k = j + m * G;
       if (k <= K || k >= N - K) {
         const int ky = k <= K ? k : k - N;
-        dst[(ky + K) * KXP] = kx <= K ? cscale<float>(x[m], inv) : mk<float>(0, 0);
+        dst[(ky + K) * KXP] = kx <= K ? x[m] : mk<float>(0, 0);
       }
     }
   }
@@ -286,6 +286,7 @@ template <typename T, bool WARP>
 __global__ void __launch_bounds__(256) k_stage_row_inv(const RunDesc<T>* __restrict__ runs,
                                                        const int* __restrict__ start, int nruns) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ unsigned red[GRedWords<T>::value];  // FP64 transforms
   const int r = find_run(start, nruns, blockIdx.x);
   const RunDesc<T>& d = runs[r];
   pdl_wait();  // state written by the previous kernels: only after this
@@ -311,7 +312,7 @@ __global__ void __launch_bounds__(256) k_stage_row_inv(const RunDesc<T>* __restr
     int w = 0;
     load_pair_spectrum_ct<T, L>(x, d.mix + (long long)ia * g.mi, d.mix + (long long)ib * g.mi, (long long)y * g.KXP,
                                 j, g.K);
-    gfft<T, +1, L, SYNC, false>(x, buf0, buf1, w, j, grp, d.tw);
+    gfft<T, +1, L, SYNC>(x, buf0, buf1, w, j, grp, d.tw, GRed{red, 0});
     T* pa = d.phys + (long long)oa * g.np + (long long)y * N + j;
     T* pb = d.phys + (long long)ob * g.np + (long long)y * N + j;
 #pragma unroll
@@ -379,6 +380,7 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), 2) k_stage_row_prod
                                                                                 const int* __restrict__ start,
                                                                                 int nruns, int stage) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ unsigned red[GRedWords<T>::value];  // FP64 transforms
   const int r = find_run(start, nruns, blockIdx.x);
   LM_STAGE_DESC(T);  // field and product lookups from shared memory
   pdl_wait();  // state written by the previous kernels: only after this
@@ -568,14 +570,14 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), 2) k_stage_row_prod
       gather(pa, S0);
       if (h2) gather(pa + 1, S1);
     }
-    if (product_heavy(L.pk[pa])) gfft<T, +1, L_, SYNC, false>(x, buf0, buf1, w, j, gi, d.tw);
+    if (product_heavy(L.pk[pa])) gfft<T, +1, L_, SYNC>(x, buf0, buf1, w, j, gi, d.tw, GRed{red, 0});
     form(pa, 0, S0);
     if (h2) {
       // the second product needs its own transform: park the first
 #pragma unroll
       for (int m = 0; m < 8; ++m) P0[m * G + j] = x[m].x;
       load_grad(pa + 1);
-      gfft<T, +1, L_, SYNC, false>(x, buf0, buf1, w, j, gi, d.tw);
+      gfft<T, +1, L_, SYNC>(x, buf0, buf1, w, j, gi, d.tw, GRed{red, 0});
       form(pa + 1, 1, S1);
 #pragma unroll
       for (int m = 0; m < 8; ++m) x[m].x = P0[m * G + j];
@@ -585,7 +587,7 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), 2) k_stage_row_prod
 #pragma unroll
       for (int m = 0; m < 8; ++m) x[m].y = (T)0;
     }
-    gfft<T, -1, L_, SYNC, false>(x, buf0, buf1, w, j, gi, d.tw);
+    gfft<T, -1, L_, SYNC, -L_ - 1>(x, buf0, buf1, w, j, gi, d.tw, GRed{red, 0});
     store_pair_spectrum_ct<T, L_, SYNC>(x, buf0, buf1, w, d.pmix + (long long)pa * g.mi,
                                         npq == 2 ? d.pmix + (long long)(pa + 1) * g.mi : nullptr, rowoff, j, gi,
                                         g.K, g.KXP);
