@@ -31,7 +31,7 @@ EXPORTS = ("sw_create", "sw_destroy", "sw_step", "lmean_begin", "lmean_step", "l
            "sw_server_create", "sw_server_submit", "sw_server_poll", "sw_server_stats_get",
            "sw_server_clock", "sw_server_destroy", "sw_state_bytes", "lmean_remap", "lmean_lift",
            "sw_spectrum", "sw_sl_create", "sw_sl_step", "sw_sl_end", "sw_sl_destroy", "sw_fma_peak")
-SW_K_NAMES = ("col_inv", "row_inv", "row_prod", "col_fwd", "update", "phys_q")
+SW_K_NAMES = ("col_inv", "row_inv", "row_prod", "col_fwd", "update", "phys_q", "col_stage")
 SW_K_COUNT = 8
 
 

@@ -2,15 +2,19 @@
 // GB300 kernels of the Lagrangian-mean shallow-water library.
 //
 // Data layout in HBM (all complex arrays interleaved re/im):
-//   spectral field  : [ky_idx][kx], ky_idx = ky + K in [0, 2K], kx in [0, KXP)
-//                     (K = floor((N-1)/3) is the 2/3-rule cutoff; KXP is K+1
-//                     rounded up to a multiple of 4; columns kx > K are zero)
+//   spectral field  : tiles of CT = 4 (FP32) or 2 (FP64) consecutive kx, each
+//                     [ky_idx][kx mod CT], ky_idx = ky + K in [0, 2K], kx in
+//                     [0, KXP) (K = floor((N-1)/3) is the 2/3-rule cutoff; KXP
+//                     is K+1 rounded up to a multiple of 4; columns kx > K are
+//                     zero): a column tile is one contiguous run
 //   column-transformed intermediate ("mixed" field, physical y, spectral kx):
-//                     [y][kx], y in [0, N), kx in [0, KXP)
+//                     [y/2][kx][y mod 2], kx in [0, KXP)
 //   physical field  : [y][x] real, row-major.
-// The mixed layout is written by the column pass with 4-wide kx tiles and read
-// by the row pass row by row, so both sides access 32-byte (FP32) or 64-byte
-// (FP64) contiguous runs.
+// The mixed layout interleaves pairs of rows: the row pass, which transforms
+// two rows as one complex sequence, reads and writes both with one 16- or
+// 32-byte access per lane, and the column pass moves runs of 2 rows x C
+// columns.  (The FP64 transforms around the stepping use plain rows [ky][kx]
+// and [y][kx] in buffers of their own.)
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -47,6 +51,30 @@ template <typename T>
 __host__ __device__ __forceinline__ int sidx(int n) {
   return n + (n >> 3);
 }
+// Spectral layout of the state: columns per tile, and the element of (ky_idx, kx).
+template <typename T> __host__ __device__ constexpr int spec_tile() { return sizeof(T) == 4 ? 4 : 2; }
+template <typename T> __host__ __device__ __forceinline__ int spec_index(int kyi, int kx, int NY) {
+  constexpr int S = sizeof(T) == 4 ? 4 : 2;
+  return (kx / S) * (NY * S) + kyi * S + kx % S;
+}
+// The two rows of a pair at one kx of a mixed field.
+__device__ __forceinline__ void ld_pair(const float2* p, float2& a, float2& b) {
+  const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+  a = make_float2(v.x, v.y);
+  b = make_float2(v.z, v.w);
+}
+__device__ __forceinline__ void ld_pair(const double2* p, double2& a, double2& b) {
+  a = __ldg(p);
+  b = __ldg(p + 1);
+}
+__device__ __forceinline__ void st_pair(float2* p, float2 a, float2 b) {
+  *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ void st_pair(double2* p, double2 a, double2 b) {
+  p[0] = a;
+  p[1] = b;
+}
+
 // Distance between the transforms of a block (rows, or the columns of a
 // column tile).
 template <typename T>
@@ -95,6 +123,28 @@ enum {
 };
 // integrating-factor classes
 enum { IF_DYN = 0, IF_LM = 1, IF_NONE = 2 };
+// tasks of the column-stage kernel (see k_stage_col)
+enum { CT_UV = 0, CT_E2 = 1, CT_KIN = 2, CT_H = 3, CT_G = 4, CT_P = 5, MAXCT = 10 };
+// A task's steps, in order: with op < 0 the forward transform of product
+// `prod` (-1: none, the values are there), whose result is kept (CA_KEEP),
+// parked (CA_PARK) or updates field `fld` (CA_U and CA_V: u and v of CT_UV;
+// CA_UPD; CA_UPD_PARK: the new value is parked too); with op = OP_* the inverse
+// transform of op(value) into mixed field `prod`, the value being what the
+// update before left (CA_X), the parked one (CA_PARKED) or that of field `fld`
+// in memory (CA_MEM).  half: which half of the block takes the step when the
+// block is split; bar: a block barrier comes before it then.
+enum {
+  CA_PARK = 0, CA_U = 1, CA_V = 2, CA_UPD = 3, CA_UPD_PARK = 4, CA_X = 5, CA_PARKED = 6, CA_MEM = 7, CA_KEEP = 8,
+  MAXCS = 8
+};
+// (Bytes: the descriptor is part of the column stage's static shared memory,
+// which at 2048^2 in FP32 has to stay below 196 KB with the buffers: above it
+// the SM's L1 shrinks from 60 to 28 KB, 245 -> 283 us.)
+struct ColTask {
+  signed char kind, slot;  // CT_*; mean-field slot or component
+  signed char n;
+  signed char prod[MAXCS], act[MAXCS], op[MAXCS], fld[MAXCS], half[MAXCS], bar[MAXCS];
+};
 // role of an evolved field in the right-hand side
 enum { R_U = 0, R_V = 1, R_H = 2, R_G = 3, R_P = 4, R_E = 5 };
 
@@ -127,11 +177,9 @@ struct Layout {
   int p_zv, p_zu, p_ke, p_hu, p_hv, p_q;
   int p_g[NLMF];
   int p_p[2];
-  // some pair (2q, 2q+1) of the row pass has a second product that needs a
-  // transform or gather of its own (only when the products are not all
-  // paired heavy-with-light, e.g. the kinematic model)
-  int heavy2;
-  int pad_;
+  // tasks of the column-stage kernel
+  int nct;
+  ColTask ct[MAXCT];
 };
 
 // discretisation of the mean equations (the C ABI's LM_SCHEME_* values)
@@ -143,13 +191,36 @@ struct StepConsts {
   int pad;
 };
 
+// Global store and load of a complex value that the compiler keeps in order
+// with one another but does not treat as touching other memory: after a plain
+// store through a pointer it would reload every run-descriptor field it uses
+// (kept in shared memory), a chain of waits per store.
+__device__ __forceinline__ void gst(float2* p, float2 v) {
+  asm volatile("st.global.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(v.x), "f"(v.y));
+}
+__device__ __forceinline__ void gst(double2* p, double2 v) {
+  asm volatile("st.global.v2.f64 [%0], {%1, %2};" ::"l"(p), "d"(v.x), "d"(v.y));
+}
+__device__ __forceinline__ float2 gld(const float2* p) {
+  float2 v;
+  asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double2 gld(const double2* p) {
+  double2 v;
+  asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+  return v;
+}
+
 // Programmatic dependent launch (PTX griddepcontrol).  The stage kernels of
 // a step are launched with programmatic stream serialisation, so a kernel's
 // blocks may start while the previous kernel of the stream finishes.
 // pdl_wait: before its first access to memory that earlier kernels write,
 // a stage kernel waits until they have completed and their writes are
-// visible (without the launch attribute it returns at once).  pdl_release:
-// after its last store, the kernel lets the next one be scheduled.
+// visible (without the launch attribute it returns at once).  pdl_release,
+// right after it: once every block of this kernel has started, the next
+// kernel's blocks may take what is free on the SMs, read their run
+// descriptors (which no kernel writes) and wait in turn.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

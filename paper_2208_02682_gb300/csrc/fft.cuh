@@ -199,7 +199,8 @@ __device__ __forceinline__ void dft_r(cplx<T>* v) {
 // table holds w^0 = 1 there; the product is exact).
 // SYNC: 0 the warp (G <= 32: several groups per warp execute the same
 // instructions), 1 named barrier grp + 1 over the group's G threads, 2 the
-// block (groups whose threads interleave, column tiles).  A named barrier
+// block (groups whose threads interleave, column tiles), 3 half grp of the
+// block (the same, two sets of them).  A named barrier
 // with a run-time id reserves all 16 of a block's barriers, which limits the
 // blocks resident on an SM, so kernels whose groups all fit in a warp are
 // compiled without it.
@@ -207,7 +208,10 @@ __device__ __forceinline__ void dft_r(cplx<T>* v) {
 template <int SYNC, int G>
 __device__ __forceinline__ void gsync(int grp) {
   if (SYNC == 2) __syncthreads();
-  else if (SYNC == 1) asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(G) : "memory");
+  else if (SYNC == 3) {
+    if (grp == 0) asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x >> 1) : "memory");
+    else asm volatile("bar.sync 2, %0;" ::"r"(blockDim.x >> 1) : "memory");
+  } else if (SYNC == 1) asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(G) : "memory");
   else __syncwarp();
 }
 
@@ -331,12 +335,13 @@ template <typename V, int SIGN> __device__ __forceinline__ void gpass_first(V (&
 }
 
 // Reduction scratch of a block's transforms (FP64 only): the groups' warps
-// leave their maxima in the first half and their sums in the second.  lC:
-// log2 of the interleaved columns of a column tile (SYNC 2).
+// leave their maxima in the first half and their sums in the second.  For
+// column tiles (SYNC 2 and 3) lC: log2 of the interleaved columns, tid and n:
+// the thread's index in and the threads of its set of transforms.
 constexpr int GRED_WORDS = 512;
 struct GRed {
   unsigned* red;
-  int lC;
+  int lC, tid, n;
 };
 template <typename T> struct GRedWords { static constexpr int value = sizeof(T) == 8 ? GRED_WORDS : 1; };
 
@@ -344,8 +349,9 @@ template <typename T> struct GRedWords { static constexpr int value = sizeof(T) 
 // shuffles; the warps' results go to `slots`, to be combined by gred_read
 // after a barrier of the group.
 template <bool MAX, int SYNC, int G>
-__device__ __forceinline__ unsigned gred_warp(unsigned v, unsigned* slots, int grp, int lC) {
-  const int lo = SYNC == 2 ? 1 << lC : 1;
+__device__ __forceinline__ unsigned gred_warp(unsigned v, unsigned* slots, int grp, const GRed& g) {
+  const int lC = g.lC;
+  const int lo = SYNC >= 2 ? 1 << lC : 1;
   const int hi = SYNC == 0 && G < 32 ? G / 2 : 16;
 #pragma unroll
   for (int off = 16; off >= 1; off >>= 1) {
@@ -356,31 +362,31 @@ __device__ __forceinline__ unsigned gred_warp(unsigned v, unsigned* slots, int g
   }
   if (SYNC == 1) {
     if ((threadIdx.x & 31) == 0) slots[grp * 16 + ((threadIdx.x % G) >> 5)] = v;
-  } else if (SYNC == 2) {
-    if ((threadIdx.x & 31) < (1u << lC)) slots[((threadIdx.x >> 5) << lC) + (threadIdx.x & 31)] = v;
+  } else if (SYNC >= 2) {
+    if ((g.tid & 31) < (1 << lC)) slots[((g.tid >> 5) << lC) + (g.tid & 31)] = v;
   }
   return v;
 }
 template <bool MAX, int SYNC, int G>
-__device__ __forceinline__ unsigned gred_read(unsigned v, const unsigned* slots, int grp, int lC) {
+__device__ __forceinline__ unsigned gred_read(unsigned v, const unsigned* slots, int grp, const GRed& g) {
   if (SYNC == 1) {
     v = 0;
 #pragma unroll
     for (int i = 0; i < G / 32; ++i) v = MAX ? max(v, slots[grp * 16 + i]) : v + slots[grp * 16 + i];
-  } else if (SYNC == 2) {
-    const int nw = blockDim.x >> 5, c = threadIdx.x & ((1 << lC) - 1);
+  } else if (SYNC >= 2) {
+    const int nw = g.n >> 5, c = g.tid & ((1 << g.lC) - 1);
     v = 0;
-    for (int i = 0; i < nw; ++i) v = MAX ? max(v, slots[(i << lC) + c]) : v + slots[(i << lC) + c];
+    for (int i = 0; i < nw; ++i) v = MAX ? max(v, slots[(i << g.lC) + c]) : v + slots[(i << g.lC) + c];
   }
   return v;
 }
 
 // The transform of x (positions j + m G in, positions j + m G out), times
-// 2^SC; w selects the exchange buffer that is free to write and is left
+// 2^sc; w selects the exchange buffer that is free to write and is left
 // pointing at the buffer not read last.
-template <typename T, int SIGN, int L, int SYNC, int SC = 0>
+template <typename T, int SIGN, int L, int SYNC>
 __device__ __forceinline__ void gfft(cplx<T> (&x)[8], cplx<T>* buf0, cplx<T>* buf1, int& w, int j, int grp,
-                                     const twid<T>* __restrict__ tw, GRed gr) {
+                                     const twid<T>* __restrict__ tw, GRed gr, int sc = 0) {
   static_assert(L >= 4 && L <= 11, "transform length 16..2048");
   constexpr int G = 1 << (L - 3), NP = (L + 2) / 3;
   if constexpr (sizeof(T) == 4) {
@@ -388,8 +394,8 @@ __device__ __forceinline__ void gfft(cplx<T> (&x)[8], cplx<T>* buf0, cplx<T>* bu
     gsync<SYNC, G>(grp);
     gpass_mid<float2, float2, SIGN, L, 1, SYNC>(buf0, buf1, w, j, grp, tw, 0);
     gpass_last<float2, float2, SIGN, L>(x, w ? buf1 : buf0, j, tw, PassShift{0, 0});
-    if constexpr (SC != 0) {
-      constexpr float f = SC < 0 ? 1.0f / (float)(1 << (SC < 0 ? -SC : 0)) : (float)(1 << (SC < 0 ? 0 : SC));
+    if (sc != 0) {
+      const float f = __int_as_float((127 + sc) << 23);
 #pragma unroll
       for (int m = 0; m < 8; ++m) x[m] = cscale<float>(x[m], f);
     }
@@ -399,9 +405,9 @@ __device__ __forceinline__ void gfft(cplx<T> (&x)[8], cplx<T>* buf0, cplx<T>* bu
     unsigned mx = 0;
 #pragma unroll
     for (int m = 0; m < 8; ++m) mx = max(mx, max(fx_abs_hi(x[m].x), fx_abs_hi(x[m].y)));
-    mx = gred_warp<true, SYNC, G>(mx, gr.red, grp, gr.lC);
+    mx = gred_warp<true, SYNC, G>(mx, gr.red, grp, gr);
     if (SYNC != 0) gsync<SYNC, G>(grp);
-    mx = gred_read<true, SYNC, G>(mx, gr.red, grp, gr.lC);
+    mx = gred_read<true, SYNC, G>(mx, gr.red, grp, gr);
     const int emax = max((int)(mx >> 20), FX_EMIN);
     cfx v[8];
     unsigned ms = 0;
@@ -410,17 +416,17 @@ __device__ __forceinline__ void gfft(cplx<T> (&x)[8], cplx<T>* buf0, cplx<T>* bu
       v[m].x = fx_from_double(x[m].x, emax, ms);
       v[m].y = fx_from_double(x[m].y, emax, ms);
     }
-    unsigned sum = gred_warp<false, SYNC, G>(fx_sum_units(ms), gr.red + GRED_WORDS / 2, grp, gr.lC);
+    unsigned sum = gred_warp<false, SYNC, G>(fx_sum_units(ms), gr.red + GRED_WORDS / 2, grp, gr);
     gpass_first<cfx, SIGN>(v, w ? b1 : b0, j);
     gsync<SYNC, G>(grp);
-    sum = gred_read<false, SYNC, G>(sum, gr.red + GRED_WORDS / 2, grp, gr.lC);
+    sum = gred_read<false, SYNC, G>(sum, gr.red + GRED_WORDS / 2, grp, gr);
     const int Dn = fx_sum_shift(sum);
     gpass_mid<cfx, TwFx, SIGN, L, 1, SYNC>(b0, b1, w, j, grp, tw, Dn);
     gpass_last<cfx, TwFx, SIGN, L>(v, w ? b1 : b0, j, tw, pass_shift<NP - 1>(Dn));
     // exponents near the top of the range: 2^512 below, then a product that
     // overflows as FP64 does (NaN for a transform with non-finite inputs)
     const bool top = emax > 1980;
-    const int e = emax + pass_drop<NP - 1>(Dn) + SC - (top ? 512 : 0);
+    const int e = emax + pass_drop<NP - 1>(Dn) + sc - (top ? 512 : 0);
 #pragma unroll
     for (int m = 0; m < 8; ++m) x[m] = mk<double>(fx_to_double(v[m].x, e), fx_to_double(v[m].y, e));
     if (top) {

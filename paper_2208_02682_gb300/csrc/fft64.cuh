@@ -36,7 +36,7 @@
 #include <cmath>
 #include <vector>
 
-#include "common.cuh"
+#include <cuda_runtime.h>
 
 #if defined(__CUDA_ARCH__)
 #define LM_HD __device__ __forceinline__
@@ -51,8 +51,7 @@ struct cfx {
 };
 
 // Twiddle c + i s with c = ch 2^-30 + cl 2^-62, s likewise; entries of the
-// pass-ordered table (see fft.cuh), w = exp(-i theta).  (|sl|, |cl| < 2^31:
-// c 2^30 is an integer or more than 2^-31 from a half-integer.)
+// pass-ordered table (see fft.cuh), w = exp(-i theta).
 struct __align__(16) TwFx {
   int ch, cl, sh, sl;
 };
@@ -228,25 +227,48 @@ __host__ __device__ __forceinline__ int fft_pass_lr(int log2N, int p) {
   return p < log2N / 3 ? 3 : log2N % 3;
 }
 
+// Host: cos and sin of (pi/4) i/E, 0 <= i <= E = 2^lE, as unsigned fractions of
+// 2^64 (1 as 2^64 - 1), by their Taylor series in 128-bit integer products: ten
+// terms of at most a unit's error each, so within 2^-60.  (Extended-precision
+// library calls are emulated, and slow, on some hosts.)
+inline void octant_fx(int i, int lE, unsigned long long& c, unsigned long long& s) {
+  typedef unsigned __int128 u128;
+  const unsigned long long pi4 = 0xC90FDAA22168C234ull;  // pi/4 2^64
+  const unsigned long long a = (unsigned long long)(((u128)pi4 * (unsigned)i) >> lE);
+  const unsigned long long a2 = (unsigned long long)(((u128)a * a) >> 64);
+  u128 one = (u128)1 << 64, cs = one, sn = a, tc = one, ts = a;
+  for (int n = 1; n <= 11; ++n) {
+    tc = ((tc * a2) >> 64) / (unsigned)((2 * n - 1) * (2 * n));
+    ts = ((ts * a2) >> 64) / (unsigned)((2 * n) * (2 * n + 1));
+    if (n & 1) {
+      cs -= tc;
+      sn -= ts;
+    } else {
+      cs += tc;
+      sn += ts;
+    }
+  }
+  c = cs >= one ? ~0ull : (unsigned long long)cs;
+  s = (unsigned long long)sn;
+}
+
 // Host: the same table in the fixed-point form of the FP64 group transforms
-// (N entries; the last is unused).  Angles are folded into the first octant,
-// whose N/8 + 1 cosines and sines are taken in long double (each well within
-// 2^-62; eight times fewer calls, which are slow where long double is
-// emulated).
+// (N entries; the last is unused).  Angles are folded into the first octant.
 inline void fft_twiddle_table_fx(int log2N, TwFx* tw) {
   const int N = 1 << log2N, E = N / 8;
   std::vector<TwFx> oct(E + 1);
-  auto split = [](long double v, int& h, int& l) {
-    const long long q = std::llrintl(v * 1073741824.0L);
-    long long r = std::llrintl((v * 1073741824.0L - (long double)q) * 4294967296.0L);
-    r = r > 2147483647LL ? 2147483647LL : (r < -2147483647LL ? -2147483647LL : r);
-    h = (int)q;
-    l = (int)r;
+  auto split = [](unsigned long long v, int& h, int& l) {
+    // v 2^-64 = h 2^-30 + l 2^-62
+    const unsigned long long u = (v >> 2) + ((v >> 1) & 1);
+    l = (int)(unsigned)u;
+    h = (int)((u >> 32) + ((unsigned)u >> 31));
+    if (l == -2147483647 - 1) l = -2147483647;  // negated in places
   };
   for (int i = 0; i <= E; ++i) {
-    const long double a = 6.283185307179586476925286766559005768L * i / N;
-    split(std::cos(a), oct[i].ch, oct[i].cl);
-    split(std::sin(a), oct[i].sh, oct[i].sl);
+    unsigned long long c, s;
+    octant_fx(i, log2N - 3, c, s);
+    split(c, oct[i].ch, oct[i].cl);
+    split(s, oct[i].sh, oct[i].sl);
   }
   // exp(-2 pi i n/N)
   auto entry = [&](int n) {

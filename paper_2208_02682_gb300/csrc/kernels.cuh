@@ -194,67 +194,70 @@ __device__ void row_pair_forward_store(cplx<T>* buf, cplx<T>* __restrict__ da,
 // Group-owned row transforms (one row per group of G = N/8 threads, N = 2^L
 // fixed at compile time; thread j holds positions j + m G, see gfft).
 
-// Hermitian-paired spectrum of one row of mixed fields a and b at the
-// thread's positions k = j + m G: Z(k) = A(k) + i B(k) for k <= K,
-// conj A(N-k) + i conj B(N-k) for k >= N-K, zero in between; the kx = 0
-// imaginary parts are dropped, as a real inverse transform does.
+// Hermitian-paired spectrum of the two real rows of a row pair (A, B: their kx
+// >= 0 halves, interleaved at r) at the thread's positions k = j + m G:
+// Z(k) = A(k) + i B(k) for k <= K, conj A(N-k) + i conj B(N-k) for k >= N-K,
+// zero in between; the kx = 0 imaginary parts are dropped, as a real inverse
+// transform does.  Parts are swapped: the inverse transform runs as a forward
+// one, and leaves row A in the imaginary and row B in the real part.
 template <typename T, int L>
-__device__ __forceinline__ void load_pair_spectrum_ct(cplx<T> (&x)[8], const cplx<T>* __restrict__ ma,
-                                                      const cplx<T>* __restrict__ mb, long long rowoff, int j,
-                                                      int K) {
+__device__ __forceinline__ void load_rows_ct(cplx<T> (&x)[8], const cplx<T>* __restrict__ r, int j, int K) {
   constexpr int N = 1 << L, G = N / 8;
-  const cplx<T>* ra = ma + rowoff;
-  const cplx<T>* rb = mb ? mb + rowoff : nullptr;
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
-    const int k = j + m * G;
-    cplx<T> z = mk<T>(0, 0);
-    if (k <= K) {
-      const cplx<T> A = ra[k];
-      const cplx<T> Bv = rb ? rb[k] : mk<T>(0, 0);
-      z = k == 0 ? mk<T>(A.x, Bv.x) : mk<T>(A.x - Bv.y, A.y + Bv.x);
-    } else if (k >= N - K) {
-      const cplx<T> A = ra[N - k];
-      const cplx<T> Bv = rb ? rb[N - k] : mk<T>(0, 0);
-      z = mk<T>(A.x + Bv.y, -A.y + Bv.x);
+    if (m == 3 || m == 4) {  // N/4 <= K < 3N/8: never in the box
+      x[m] = mk<T>(0, 0);
+      continue;
     }
-    x[m] = z;
+    const int k = j + m * G;
+    const int kk = m < 4 ? k : N - k;
+    const bool in = kk <= K;
+    cplx<T> A, Bv;
+    ld_pair(r + 2 * (in ? kk : 0), A, Bv);
+    cplx<T> z;
+    if (m < 4) z = mk<T>(A.y + Bv.x, A.x - Bv.y);
+    else z = mk<T>(Bv.x - A.y, A.x + Bv.y);
+    if (m == 0 && j == 0) z = mk<T>(Bv.x, A.x);
+    x[m] = in ? z : mk<T>(0, 0);
   }
 }
 
-// Spectrum Z of p + i q, times 1/(2 N), held at the thread's positions -> kx
-// in [0, KXP) halves of p and q (times 1/N) into row `rowoff` of mixed fields da and
-// db (db null: p only).  One exchange through the free buffer.
+// Spectrum Z of p + i q (the two rows), times 1/(2 N), held at the thread's
+// positions -> kx in [0, KXP) halves of p and q (times 1/N), interleaved at r.
+// One exchange through the free buffer.
 template <typename T, int L, int SYNC>
-__device__ __forceinline__ void store_pair_spectrum_ct(const cplx<T> (&x)[8], cplx<T>* buf0, cplx<T>* buf1, int& w,
-                                                       cplx<T>* __restrict__ da, cplx<T>* __restrict__ db,
-                                                       long long rowoff, int j, int grp, int K, int KXP) {
+__device__ __forceinline__ void store_rows_ct(const cplx<T> (&x)[8], cplx<T>* buf0, cplx<T>* buf1, int& w,
+                                              cplx<T>* __restrict__ r, int j, int grp, int K, int KXP) {
   constexpr int N = 1 << L, G = N / 8;
   cplx<T>* b = w ? buf1 : buf0;
   if constexpr (G % 8 == 0) {
     const int sb = j + (j >> 3);
 #pragma unroll
-    for (int m = 0; m < 8; ++m) b[sb + m * (G + G / 8)] = x[m];  // sidx(j + m G)
+    for (int m = 0; m < 8; ++m)
+      if (m != 3 && m != 4) b[sb + m * (G + G / 8)] = x[m];  // sidx(j + m G)
   } else {
 #pragma unroll
     for (int m = 0; m < 8; ++m) b[sidx<T>(j + m * G)] = x[m];
   }
   gsync<SYNC, G>(grp);
-  cplx<T>* ra = da + rowoff;
-  cplx<T>* rb = db ? db + rowoff : nullptr;
-  for (int k = j; k < KXP; k += G) {
-    cplx<T> P = mk<T>(0, 0), Q = mk<T>(0, 0);
-    if (k <= K) {
-      const cplx<T> z1 = b[k + (k >> 3)];
-      const int k2 = (N - k) & (N - 1);
-      const cplx<T> z2 = b[k2 + (k2 >> 3)];
-      // P = Z(k) + conj Z(N-k), Q = (Z(k) - conj Z(N-k))/i
-      P = mk<T>(z1.x + z2.x, z1.y - z2.y);
-      Q = mk<T>(z1.y + z2.y, z2.x - z1.x);
+  // KXP <= 3 G: K + 1 <= N/3, rounded up to a multiple of the column tile
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const int k = j + i * G;
+    if (k < KXP) {
+      cplx<T> P = mk<T>(0, 0), Q = mk<T>(0, 0);
+      if (k <= K) {
+        const cplx<T> z1 = b[k + (k >> 3)];
+        const int k2 = (N - k) & (N - 1);
+        const cplx<T> z2 = b[k2 + (k2 >> 3)];
+        // P = Z(k) + conj Z(N-k), Q = (Z(k) - conj Z(N-k))/i
+        P = mk<T>(z1.x + z2.x, z1.y - z2.y);
+        Q = mk<T>(z1.y + z2.y, z2.x - z1.x);
+      }
+      st_pair(r + 2 * k, P, Q);
     }
-    ra[k] = P;
-    if (rb) rb[k] = Q;
   }
+  for (int k = j + 3 * G; k < KXP; k += G) st_pair(r + 2 * k, mk<T>(0, 0), mk<T>(0, 0));
   w ^= 1;
 }
 
@@ -363,31 +366,56 @@ __global__ void __launch_bounds__(256) k_row_fwd(const __grid_constant__ RowFwdA
 // The 64-bit step count is converted through its two 31-bit halves (exact
 // in FP64 below 2^53 steps, and in FP32 below 2^24).
 template <typename T>
-__device__ __forceinline__ T stage_time(const long long* ctr, int stage, T dt, int stepper) {
-  const long long n = *ctr;
+__device__ __forceinline__ T stage_time(long long n, int stage, T dt, int stepper) {
   const T steps = (T)(int)(n >> 31) * (T)2147483648.0 + (T)(int)(n & 0x7fffffffLL);
   const T c = stage == 0 ? (T)0 : (stepper != 0 || stage == 3 ? (T)1 : (T)0.5);
   return (steps + c) * dt;
 }
 
-// Bilinear interpolation of the periodic grid field f at (x_i + xi_x, y_j + xi_y)
-// (Sec. 4.2.1).  The displacement in cells d = xi/dx gives the cell index
-// i + floor(d) and the weight d - floor(d).  Indices wrap with & (N-1), so any
-// displacement (even a non-finite one) reads inside the field.
+// Bilinear interpolation of the periodic grid fields at (x_i + xi_x, y_j + xi_y)
+// (Sec. 4.2.1): corner offsets and weights.  The displacement in cells d =
+// xi/dx gives the cell index i + floor(d) and the weight d - floor(d).  Indices
+// wrap with & (N-1), so any displacement (even a non-finite one) reads inside
+// the field.
+template <typename T> struct Bilin {
+  unsigned o00, o01, o10, o11;
+  T w00, w01, w10, w11;
+  __device__ __forceinline__ Bilin(int i, int j, T xi_x, T xi_y, T inv_dx, int N) {
+    const T dxc = xi_x * inv_dx, dyc = xi_y * inv_dx;
+    const T fx = floor(dxc), fy = floor(dyc);
+    const T ax = dxc - fx, ay = dyc - fy;
+    const unsigned msk = (unsigned)N - 1u;
+    const unsigned i0 = ((unsigned)i + (unsigned)(int)fx) & msk;
+    const unsigned j0 = ((unsigned)j + (unsigned)(int)fy) & msk;
+    const unsigned i1 = (i0 + 1u) & msk, j1 = (j0 + 1u) & msk;
+    o00 = j0 * N + i0;
+    o01 = j0 * N + i1;
+    o10 = j1 * N + i0;
+    o11 = j1 * N + i1;
+    w00 = ((T)1 - ax) * ((T)1 - ay);
+    w01 = ax * ((T)1 - ay);
+    w10 = ((T)1 - ax) * ay;
+    w11 = ax * ay;
+  }
+};
 template <typename T>
-__device__ __forceinline__ T bilinear(const T* __restrict__ f, int i, int j, T xi_x, T xi_y,
-                                      T inv_dx, int N) {
-  const T dxc = xi_x * inv_dx, dyc = xi_y * inv_dx;
-  const T fx = floor(dxc), fy = floor(dyc);
-  const T ax = dxc - fx, ay = dyc - fy;
-  const unsigned msk = (unsigned)N - 1u;
-  const unsigned i0 = ((unsigned)i + (unsigned)(int)fx) & msk;
-  const unsigned j0 = ((unsigned)j + (unsigned)(int)fy) & msk;
-  const unsigned i1 = (i0 + 1u) & msk, j1 = (j0 + 1u) & msk;
-  const T f00 = __ldg(f + j0 * N + i0), f01 = __ldg(f + j0 * N + i1);
-  const T f10 = __ldg(f + j1 * N + i0), f11 = __ldg(f + j1 * N + i1);
-  return ((T)1 - ax) * ((T)1 - ay) * f00 + ax * ((T)1 - ay) * f01 +
-         ((T)1 - ax) * ay * f10 + ax * ay * f11;
+__device__ __forceinline__ T bilinear(const T* __restrict__ f, int i, int j, T xi_x, T xi_y, T inv_dx, int N) {
+  const Bilin<T> b(i, j, xi_x, xi_y, inv_dx, N);
+  return b.w00 * __ldg(f + b.o00) + b.w01 * __ldg(f + b.o01) + b.w10 * __ldg(f + b.o10) + b.w11 * __ldg(f + b.o11);
+}
+__device__ __forceinline__ void ld_quad(const float* p, float* v) {
+  const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+  v[0] = q.x;
+  v[1] = q.y;
+  v[2] = q.z;
+  v[3] = q.w;
+}
+__device__ __forceinline__ void ld_quad(const double* p, double* v) {
+  const double2 a = __ldg(reinterpret_cast<const double2*>(p)), b = __ldg(reinterpret_cast<const double2*>(p) + 1);
+  v[0] = a.x;
+  v[1] = a.y;
+  v[2] = b.x;
+  v[3] = b.y;
 }
 
 // ---------------------------------------------------------------------------
@@ -401,28 +429,31 @@ __global__ void k_velocity_from_vorticity(cplx<T>* __restrict__ y, Geom g, int f
   const int mi = (int)m;
   const int kyi = mi / g.KXP, kx = mi - kyi * g.KXP;
   const T kxf = (T)kx, kyf = (T)(kyi - g.K);
-  const cplx<T> z = y[(long long)fh * g.ms + m];
+  const int o = spec_index<T>(kyi, kx, g.NY);
+  const cplx<T> z = y[(long long)fh * g.ms + o];
   const T k2 = kxf * kxf + kyf * kyf;
   const T inv = k2 > (T)0 ? (T)1 / k2 : (T)0;
-  y[(long long)fu * g.ms + m] = mk<T>(-kyf * z.y * inv, kyf * z.x * inv);
-  y[(long long)fv * g.ms + m] = mk<T>(kxf * z.y * inv, -kxf * z.x * inv);
+  y[(long long)fu * g.ms + o] = mk<T>(-kyf * z.y * inv, kyf * z.x * inv);
+  y[(long long)fv * g.ms + o] = mk<T>(kxf * z.y * inv, -kxf * z.x * inv);
 }
 
 // ---------------------------------------------------------------------------
 // Spectral FP64 copy of selected fields, value = (y - comp) * scale.
 template <typename T>
 __global__ void k_spec_to_f64(const cplx<T>* __restrict__ y, const cplx<T>* __restrict__ comp,
-                              double2* __restrict__ out, long long ms, int f0_idx, int f1_idx, double scale) {
+                              double2* __restrict__ out, long long ms, int NY, int KXP, int f0_idx, int f1_idx,
+                              double scale) {
   const long long m = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= ms) return;
+  const int o = spec_index<T>((int)m / KXP, (int)m % KXP, NY);
   const int idx[2] = {f0_idx, f1_idx};
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
     if (idx[q] < 0) continue;
-    const cplx<T> v = y[idx[q] * ms + m];
+    const cplx<T> v = y[idx[q] * ms + o];
     double re = (double)v.x, im = (double)v.y;
     if (comp) {
-      const cplx<T> c = comp[idx[q] * ms + m];
+      const cplx<T> c = comp[idx[q] * ms + o];
       re -= (double)c.x;
       im -= (double)c.y;
     }
@@ -435,9 +466,24 @@ __global__ void k_add_real(double2* p, double delta);
 
 // FP64 spectral -> T spectral (initial condition).
 template <typename T>
-__global__ void k_spec_from_f64(const double2* __restrict__ in, cplx<T>* __restrict__ y, long long n) {
-  const long long m = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (m < n) y[m] = mk<T>((T)in[m].x, (T)in[m].y);
+__global__ void k_spec_from_f64(const double2* __restrict__ in, cplx<T>* __restrict__ y, Geom g, int nfields) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= g.ms * nfields) return;
+  const int f = (int)(i / g.ms), m = (int)(i - f * g.ms);
+  y[f * g.ms + spec_index<T>(m / g.KXP, m % g.KXP, g.NY)] = mk<T>((T)in[i].x, (T)in[i].y);
+}
+
+// Copy of nf spectral fields between the tile-blocked layout and rows
+// [ky + K][kx] (checkpoint blobs); to_rows: out gets rows.
+template <typename T>
+__global__ void k_spec_rows(const cplx<T>* __restrict__ in, cplx<T>* __restrict__ out, Geom g, int nfields,
+                            int to_rows) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= g.ms * nfields) return;
+  const int f = (int)(i / g.ms), m = (int)(i - f * g.ms);
+  const long long o = f * g.ms + spec_index<T>(m / g.KXP, m % g.KXP, g.NY);
+  if (to_rows) out[i] = in[o];
+  else out[o] = in[i];
 }
 
 // ---------------------------------------------------------------------------

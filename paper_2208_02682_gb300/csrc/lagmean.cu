@@ -3,6 +3,7 @@
 // around it (initial condition, end-of-interval means, diagnostics).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -40,7 +41,7 @@ struct sw_handle {
   // device memory
   void* arena = nullptr;
   size_t arena_bytes = 0;
-  void *y = nullptr, *ys = nullptr, *ys2 = nullptr, *acc = nullptr, *comp = nullptr, *ps = nullptr;
+  void *y = nullptr, *ys = nullptr, *ys2 = nullptr, *acc = nullptr, *comp = nullptr;
   void *mix = nullptr, *pmix = nullptr, *phys = nullptr, *ef = nullptr, *tw = nullptr;
   double2 *tw64 = nullptr, *spec64 = nullptr, *mix64 = nullptr;
   double *out64 = nullptr, *part = nullptr, *dres = nullptr;
@@ -53,10 +54,10 @@ struct sw_handle {
   int64_t done = 0;
   int64_t steps_total = 0;
   Layout L{};
-  // launch shapes: column tile 2^lC columns; row_prod Bp rows and ppb
-  // product pairs per block (0: automatic, see batch_build_t)
-  // product pairs per block; row_inv Bi rows per block
-  int lC = 2, Bp = 1, ppb = 1, Bi = 1;
+  // launch shapes: column tiles of at most 2^lC columns; row_prod `points`
+  // per block (row pairs x N) and ppb products per block (0: automatic, see
+  // batch_build_t); the FP64 row transforms take Bi rows per block
+  int lC = 2, points = 256, ppb = 0, Bi = 1;
   uint64_t version = 1;  // bumped whenever L or the launch shapes change
   BatchExec* self = nullptr;  // batch of one used by sw_step / lmean_step
   int64_t launches = 0;  // kernels launched since creation
@@ -180,37 +181,21 @@ static Layout build_layout(const sw_params& p, int strategy, int fields, int eul
       L.p_g[j] = addp(PK_GBAR, gx, gy, ph_of[L.lmf[j]]);
     }
   }
-  // The row pass transforms products in pairs (2q, 2q + 1), one pair per
-  // group: pair each product that needs a transform of its own (advection or
-  // Strategy-2 gather) with one that needs none, so that the groups of a row
-  // carry similar work (the heavy one first: its spectrum is loaded before
-  // the row's base fields are ready).
+  // Products that need transforms of their own (advection, Strategy 2) first:
+  // the row pass's groups take products in this order.
   {
     auto heavy = [](int k) { return k == PK_ADV || k == PK_XI || k == PK_GBAR; };
-    int hv[MAXP], lt[MAXP], nh = 0, nl = 0;
-    for (int q = 0; q < np; ++q) {
-      if (heavy(L.pk[q])) hv[nh++] = q;
-      else lt[nl++] = q;
-    }
-    int order[MAXP], pos[MAXP], no = 0, ih = 0, il = 0;
-    while (ih < nh || il < nl) {
-      if (ih < nh) order[no++] = hv[ih++];
-      if (il < nl) order[no++] = lt[il++];
-    }
-    int pk[MAXP], pa[MAXP], pb[MAXP], pc[MAXP];
-    for (int q = 0; q < np; ++q) {
-      pos[order[q]] = q;
-      pk[q] = L.pk[order[q]];
-      pa[q] = L.pa[order[q]];
-      pb[q] = L.pb[order[q]];
-      pc[q] = L.pc[order[q]];
-    }
-    for (int q = 0; q < np; ++q) {
-      L.pk[q] = pk[q];
-      L.pa[q] = pa[q];
-      L.pb[q] = pb[q];
-      L.pc[q] = pc[q];
-    }
+    int pos[MAXP], no = 0;
+    const Layout Q = L;
+    for (int pass = 0; pass < 2; ++pass)
+      for (int q = 0; q < np; ++q)
+        if (heavy(Q.pk[q]) == (pass == 0)) {
+          pos[q] = no;
+          L.pk[no] = Q.pk[q];
+          L.pa[no] = Q.pa[q];
+          L.pb[no] = Q.pb[q];
+          L.pc[no++] = Q.pc[q];
+        }
     auto remap = [&](int& idx) {
       if (idx >= 0) idx = pos[idx];
     };
@@ -223,13 +208,93 @@ static Layout build_layout(const sw_params& p, int strategy, int fields, int eul
     for (int j = 0; j < NLMF; ++j) remap(L.p_g[j]);
     remap(L.p_p[0]);
     remap(L.p_p[1]);
-    L.heavy2 = 0;
-    for (int q = 1; q < np; q += 2)
-      if (heavy(L.pk[q])) L.heavy2 = 1;
   }
   L.ni = ni;
   L.np = np;
   return L;
+}
+
+// Tasks of the column-stage kernel (the longest first) for whole blocks or
+// for blocks split in two halves.
+static void build_tasks(Layout& L, bool dual) {
+  std::memset(L.ct, 0, sizeof(L.ct));
+  L.nct = 0;
+  ColTask* t = nullptr;
+  auto task = [&](int kind, int slot) {
+    t = &L.ct[L.nct++];
+    t->kind = (signed char)kind;
+    t->slot = (signed char)slot;
+  };
+  auto step = [&](int prod, int act, int op, int fld, int half = 0, int bar = 0) {
+    const int i = t->n++;
+    t->prod[i] = (signed char)prod;
+    t->act[i] = (signed char)act;
+    t->op[i] = (signed char)op;
+    t->fld[i] = (signed char)fld;
+    t->half[i] = (signed char)half;
+    t->bar[i] = (signed char)bar;
+  };
+  if (L.model == SW_MODEL_SW) {
+    task(CT_UV, 0);
+    step(L.p_ke, CA_PARK, -1, -1);
+    if (dual) {
+      step(L.p_zu, CA_KEEP, -1, -1, 1);
+      step(L.p_zv, CA_U, -1, L.f_u, 0, 1);
+      step(-1, CA_V, -1, L.f_v, 1);
+      step(L.i_v, CA_X, OP_ID, L.f_v, 1);
+      step(L.i_u, CA_X, OP_ID, L.f_u, 0, 1);
+      step(L.i_z, CA_MEM, OP_CURL, L.f_u, 1);
+    } else {
+      step(L.p_zv, CA_U, -1, L.f_u);
+      step(L.i_u, CA_X, OP_ID, L.f_u);
+      step(L.p_zu, CA_V, -1, L.f_v);
+      step(L.i_v, CA_X, OP_ID, L.f_v);
+      step(L.i_z, CA_MEM, OP_CURL, L.f_u);
+    }
+  } else if (L.model == SW_MODEL_EULER2D) {
+    task(CT_E2, 0);
+    step(L.p_zu, CA_PARK, -1, -1);
+    if (dual) step(L.p_zv, CA_KEEP, -1, -1, 1);
+    step(dual ? -1 : L.p_zv, CA_UPD, -1, L.f_h, 1, 1);
+    step(L.i_h, CA_X, OP_ID, L.f_h, 1, 1);
+    step(L.i_u, CA_MEM, OP_ID, L.f_u);
+    step(L.i_v, CA_MEM, OP_ID, L.f_v);
+  } else {
+    task(CT_KIN, 0);
+    for (int f = 0; f < 3; ++f) step(-1, CA_UPD, -1, f);
+    step(L.i_h, CA_MEM, OP_ID, L.f_h, 0, 1);
+    step(L.i_z, CA_MEM, OP_CURL, L.f_u, 0);
+    step(L.i_u, CA_MEM, OP_ID, L.f_u, 1);
+    step(L.i_v, CA_MEM, OP_ID, L.f_v, 1);
+  }
+  if (L.has_pos)
+    for (int c = 0; c < 2; ++c) {
+      const int q = L.p_p[c];
+      task(CT_P, c);
+      step(q, CA_UPD_PARK, -1, L.f_p[c]);
+      if (L.strategy == 2) {
+        step(L.i_xi[c], CA_X, OP_ID, L.f_p[c], 0, 1);
+        step(L.pa[q], CA_PARKED, OP_DX, L.f_p[c], 0);
+      } else {
+        step(L.pa[q], CA_X, OP_DX, L.f_p[c], 0, 1);
+      }
+      step(L.pb[q], CA_PARKED, OP_DY, L.f_p[c], 1);
+    }
+  for (int j = 0; j < L.nlm; ++j) {
+    const int q = L.p_g[j];
+    task(CT_G, j);
+    if (L.lmf[j] == LMF_Q) step(L.p_q, CA_PARK, -1, -1);
+    step(q, CA_UPD_PARK, -1, L.f_g[j]);
+    step(L.pa[q], CA_X, OP_DX, L.f_g[j], 0, 1);
+    step(L.pb[q], CA_PARKED, OP_DY, L.f_g[j], 1);
+  }
+  if (L.model == SW_MODEL_SW) {
+    task(CT_H, 0);
+    step(L.p_hu, CA_PARK, -1, -1);
+    if (dual) step(L.p_hv, CA_KEEP, -1, -1, 1);
+    step(dual ? -1 : L.p_hv, CA_UPD, -1, L.f_h, 1, 1);
+    step(L.i_h, CA_X, OP_ID, L.f_h, 1);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -238,7 +303,7 @@ static Layout build_layout(const sw_params& p, int strategy, int fields, int eul
 // (box modes NY*KX, mixed rows N*KX, physical N*N), not counting L2 hits or
 // padding.
 struct KBytes {
-  double col_inv, row_inv, phys_q, row_prod, col_fwd, update[4];
+  double col_inv, row_inv, row_prod, col_stage[4];
 };
 
 static KBytes kernel_bytes(const sw_handle* h, const Layout& L) {
@@ -253,13 +318,14 @@ static KBytes kernel_bytes(const sw_handle* h, const Layout& L) {
     if (L.i_src2[i] >= 0 && !seen[L.i_src2[i]]) { seen[L.i_src2[i]] = true; ++nsrc; }
   }
   b.col_inv = nsrc * MB * cs + L.ni * MI * cs;
-  // row inverse pass: u, v, h, zeta (and xi) rows to physical planes
-  const int nbase = L.strategy == 2 ? 6 : 4;
-  b.row_inv = nbase * MI * cs + nbase * NP * ts;
-  b.phys_q = 3 * NP * ts;
-  // row pass: base planes and gradient rows in, products out; Strategy 2
-  // also gathers q (the other gathered planes are base planes)
-  double rp = L.np * MI * cs + (L.ni - nbase) * MI * cs + nbase * NP * ts;
+  // row inverse pass: u, v, h, zeta (and xi, q) rows to physical planes, for
+  // the runs whose row pass does not form them itself
+  const int base = L.strategy == 2 ? 6 : 4;
+  const bool fused = h->fp32 ? row_prod_fused<float>(g.N, L) : row_prod_fused<double>(g.N, L);
+  b.row_inv = fused ? 0.0 : base * MI * cs + (base + (L.strategy == 2 && L.has_q)) * NP * ts;
+  // row pass: mixed rows (or gradients, and the base planes) in, products
+  // out; Strategy 2 also gathers q (the other gathered planes are base planes)
+  double rp = L.np * MI * cs + (fused ? L.ni * MI * cs : (L.ni - base) * MI * cs + base * NP * ts);
   if (L.strategy == 2) {
     bool gq = false;
     for (int p = 0; p < L.np; ++p)
@@ -267,16 +333,24 @@ static KBytes kernel_bytes(const sw_handle* h, const Layout& L) {
     if (gq) rp += NP * ts;
   }
   b.row_prod = rp;
-  b.col_fwd = L.np * (MI + MB) * cs;
-  int nk = 0;
-  for (int f = 0; f < L.nf; ++f) nk += L.fkahan[f];
-  const double nf = L.nf, np = L.np;
-  // integrating-factor tables: E per class at every stage; the stage that
-  // commits y_{n+1} also reads E^2 as hi + lo
-  b.update[0] = (nf + np + 2 * nf) * MB * cs + 2 * MB * ts;
-  b.update[1] = b.update[2] = (3 * nf + np + 2 * nf) * MB * cs + 2 * MB * ts;
-  b.update[3] = (3 * nf + np + nf + (h->fp32 ? 2 * nk : 0)) * MB * cs + 6 * MB * ts;
-  if (h->p.stepper != SW_STEP_RK4) b.update[1] += 4 * MB * ts;
+  int nk = 0, ne = 0;
+  for (int f = 0; f < L.nf; ++f) {
+    nk += L.fkahan[f];
+    ne += L.frole[f] == R_E;
+  }
+  const double nf = L.nf, mixed = (L.np + (L.np > 0 ? L.ni : 0)) * MI * cs;
+  // column stage: mixed products in, mixed fields out; y_n (not of the
+  // Eulerian accumulators before the commit), the accumulator, the stage
+  // inputs and outputs of u, v, h; integrating factors per class: E at every
+  // stage, E^2 as hi + lo at the commit
+  const bool rk4 = h->p.stepper == SW_STEP_RK4;
+  const int last = stage_count(h->p.stepper) - 1;
+  for (int st = 0; st < 4; ++st) {
+    if (st >= last)
+      b.col_stage[st] = mixed + (2 * nf + nf + 3 + (h->fp32 ? 2 * nk : 0)) * MB * cs + 4 * MB * ts;
+    else
+      b.col_stage[st] = mixed + ((nf - ne) + nf * (rk4 && st > 0 ? 2 : 1) + (st > 0 ? 3 : 0) + 3) * MB * cs + 2 * MB * ts;
+  }
   return b;
 }
 
@@ -293,8 +367,11 @@ struct Prof {
 // Batch executor: the device table of run descriptors, per-kernel block
 // prefix sums and the captured step graphs for a set of handles.
 static const int GRAPH_STEPS = 8;
-static const int SW_K_OF_KT[KT_COUNT] = {SW_K_COL_INV, SW_K_ROW_INV, SW_K_PHYS_Q, SW_K_ROW_PROD, SW_K_COL_FWD,
-                                         SW_K_UPDATE};
+// warps in the row pass below which its products are split over blocks
+static const long long ROW_WARPS = 1216;
+// column-stage blocks up to which blocks are split in two halves
+static const long long DUAL_BLOCKS = 456;
+static const int SW_K_OF_KT[KT_COUNT] = {SW_K_ROW_INV, SW_K_ROW_PROD, SW_K_COL_STAGE};
 
 struct BatchExec {
   std::vector<sw_handle*> members;
@@ -310,25 +387,24 @@ struct BatchExec {
   int threads[KT_COUNT] = {};
   size_t smem[KT_COUNT] = {};
   double bytes[KT_COUNT][4] = {};
-  cudaGraphExec_t g1 = nullptr, gm = nullptr;
+  double start_bytes = 0.0;  // of the transform-only launch (0: not needed)
+  cudaGraphExec_t g1 = nullptr, gm = nullptr, gf = nullptr;  // 1 step, GRAPH_STEPS steps, the final step
   int64_t kernels_per_step = 0;
   int64_t launches = 0;
+  int64_t replayed = 0;  // kernels of the last replay
   bool built = false;
   int nstages = 4;  // stage passes per step of the members' (common) stepper
   int stepper = SW_STEP_RK4;
+  bool dual = false;  // split column-stage blocks
   bool warp = false;  // every member's N <= 256: row kernels without named barriers
-  // pipelined column forward pass (FP32 members all of one size N >= 1024):
-  // log2 N, persistent blocks and shared memory; 0: one tile per block
-  int pipeL = 0;
-  int pipe_grid = 0;
-  size_t pipe_smem = 0;
   std::string err;
 };
 
 static void batch_drop_graphs(BatchExec* b) {
   if (b->g1) cudaGraphExecDestroy(b->g1);
   if (b->gm) cudaGraphExecDestroy(b->gm);
-  b->g1 = b->gm = nullptr;
+  if (b->gf) cudaGraphExecDestroy(b->gf);
+  b->g1 = b->gm = b->gf = nullptr;
 }
 
 static void batch_free(BatchExec* b) {
@@ -340,11 +416,12 @@ static void batch_free(BatchExec* b) {
 }
 
 template <typename T>
-static void fill_desc(sw_handle* h, RunDesc<T>& d, int ppb) {
+static void fill_desc(sw_handle* h, RunDesc<T>& d, int points, int ppb, int lC, bool dual) {
   std::memset(&d, 0, sizeof(d));
   const Geom& g = h->g;
   d.g = g;
   d.L = h->L;
+  build_tasks(d.L, dual);
   d.c = StepConsts{h->p.dt, h->p.f0, h->p.c2, h->p.adv_x, h->p.adv_y, h->p.stepper, 0};
   d.cdt = (T)h->p.dt;
   d.cf0 = (T)h->p.f0;
@@ -356,7 +433,6 @@ static void fill_desc(sw_handle* h, RunDesc<T>& d, int ppb) {
   d.ysb = (cplx<T>*)h->ys2;
   d.acc = (cplx<T>*)h->acc;
   d.comp = h->fp32 ? (cplx<T>*)h->comp : nullptr;
-  d.ps = (cplx<T>*)h->ps;
   d.mix = (cplx<T>*)h->mix;
   d.pmix = (cplx<T>*)h->pmix;
   d.phys = (T*)h->phys;
@@ -364,20 +440,25 @@ static void fill_desc(sw_handle* h, RunDesc<T>& d, int ppb) {
   d.tw = (const twid<T>*)h->tw;
   d.ctr = h->ctr;
   d.ticket = h->ticket;
-  d.lC = h->lC;
-  d.Bp = h->Bp;
-  d.ppb = ppb;
-  d.Wp = 1;
-  d.Bi = h->Bi;
+  d.lC = lC;
   const Layout& L = h->L;
-  const int ntile = g.KXP >> h->lC;
-  const int npairs = (L.np + 1) / 2;
-  d.nb[KT_COL_INV] = L.np > 0 ? ntile * L.ni : 0;
-  d.nb[KT_ROW_INV] = L.np > 0 ? (L.strategy == 2 ? 3 : 2) * (g.N / h->Bi) : 0;
-  d.nb[KT_PHYS_Q] = (L.np > 0 && L.strategy == 2 && L.has_q) ? (int)((g.np + 255) / 256) : 0;
-  d.nb[KT_ROW_PROD] = L.np > 0 ? (g.N / h->Bp) * ((npairs + ppb - 1) / ppb) : 0;
-  d.nb[KT_COL_FWD] = L.np > 0 ? ntile * L.np : 0;
-  d.nb[KT_UPDATE] = (int)((g.ms + update_modes(g.N) - 1) / update_modes(g.N)) * L.nf;
+  d.Bp = row_block_pairs(g.N, points);
+  d.ppb = ppb < L.np || L.np == 0 ? ppb : L.np;
+  d.Wp = 1;
+  d.Bi = row_block_pairs(g.N, points > 512 ? points : 512);
+  const int ntile = g.KXP >> lC;
+  const int chunks = L.np > 0 ? (L.np + d.ppb - 1) / d.ppb : 0;
+  for (int q = 0; q < L.np; ++q) {
+    // base fields product q is formed from
+    const int k = L.pk[q], u = 1 << PH_U, v = 1 << PH_V, e = 1 << PH_H, z = 1 << PH_Z;
+    d.umask[q / d.ppb] |= k == PK_ZV ? z | v : k == PK_ZU ? z | u : k == PK_KE ? u | v : k == PK_HU ? e | u
+                        : k == PK_HV ? e | v : k == PK_Q ? z | e : (k == PK_ADV && L.model != 1) ? u | v : 0;
+  }
+  d.fused = row_prod_fused<T>(g.N, L) ? 1 : 0;
+  d.gath = row_prod_gath<T>(g.N, L) ? 1 : 0;
+  d.nb[KT_ROW_INV] = L.np > 0 && !d.fused ? (L.strategy == 2 ? 5 : 3) * row_blocks(g.N, d.Bi) : 0;
+  d.nb[KT_ROW_PROD] = row_blocks(g.N, d.Bp) * chunks;
+  d.nb[KT_COL_STAGE] = L.np > 0 ? ntile * d.L.nct : (int)((g.ms + KIN_MODES - 1) / KIN_MODES);
 }
 
 // Build (or rebuild) the descriptor table of a batch from its members.
@@ -390,6 +471,7 @@ static int batch_build_t(BatchExec* b) {
     b->smem[k] = 0;
     for (int st = 0; st < 4; ++st) b->bytes[k][st] = 0.0;
   }
+  b->start_bytes = 0.0;
   b->start.assign((size_t)KT_COUNT * (n + 1), 0);
   const size_t cs = sizeof(cplx<T>);
   for (int r = 1; r < n; ++r)
@@ -399,69 +481,110 @@ static int batch_build_t(BatchExec* b) {
     }
   b->stepper = n > 0 ? b->members[0]->p.stepper : SW_STEP_RK4;
   b->nstages = stage_count(b->stepper);
+  // members with transforms need one grid size, or sizes from 64 to 512 (equal
+  // block shapes); members without (kinematic dynamics) have no such need
+  {
+    int lo = 0, hi = 0;
+    for (int r = 0; r < n; ++r) {
+      const int N = b->members[r]->g.N;
+      if (b->members[r]->L.np == 0) continue;
+      lo = lo ? std::min(lo, N) : N;
+      hi = std::max(hi, N);
+    }
+    if (lo != hi && (lo < 64 || hi > 512)) {
+      b->err = "batch members need equal block shapes (grid sizes 64..512, or one grid size)";
+      return SW_EINVAL;
+    }
+  }
   b->warp = true;
-  for (int r = 0; r < n; ++r) b->warp = b->warp && b->members[r]->g.N <= 256;
-  // row-pass groups per row: the largest number every member allows (the
-  // batch's row-pass blocks all have Bp * Wp * N/8 threads)
+  for (int r = 0; r < n; ++r) b->warp = b->warp && (b->members[r]->g.N <= 256 || b->members[r]->L.np == 0);
+  // row pass: products per block (automatic: all of them, unless that leaves
+  // the GPU short of warps, see below) and groups per row pair, the largest
+  // number every member allows (the batch's row-pass blocks all have
+  // Bp * Wp * N/8 threads)
+  int points = 0;
+  for (int r = 0; r < n; ++r)
+    if (b->members[r]->L.np > 0) points = std::max(points, std::max(b->members[r]->points, b->members[r]->g.N));
+  // (fewer row pairs where a block's arrays would not fit)
+  auto fits = [&](int pts) {
+    for (int r = 0; r < n; ++r) {
+      const sw_handle* h = b->members[r];
+      if (h->L.np > 0 && row_prod_smem<T>(h->g.N, row_block_pairs(h->g.N, pts), 1, h->L) > (size_t)200 * 1024) {
+        if (pts > 256) return false;
+      }
+    }
+    return true;
+  };
+  while (!fits(points)) {
+    bool half = true;
+    for (int r = 0; r < n; ++r) half = half && (b->members[r]->L.np == 0 || points / 2 >= b->members[r]->g.N);
+    if (!half) break;
+    points /= 2;
+  }
+  auto groups = [&](const sw_handle* h, int npb) {
+    return row_prod_groups<T>(h->g.N, row_block_pairs(h->g.N, points), npb < h->L.np ? npb : h->L.np, h->L);
+  };
   int W = 1 << 20;
+  long long warps = 0;
   for (int r = 0; r < n; ++r) {
     const sw_handle* h = b->members[r];
-    const int npairs = (h->L.np + 1) / 2;
-    const int npb = (h->ppb == 0 || h->ppb > npairs) ? npairs : h->ppb;
-    const int w = row_prod_groups<T>(h->g.N, h->Bp, npb, h->L);
-    W = w < W ? w : W;
+    if (h->L.np > 0) W = std::min(W, groups(h, h->ppb > 0 ? h->ppb : MAXP));
   }
-  if (n == 0) W = 1;
+  if (W > MAXP) W = 1;
+  for (int r = 0; r < n; ++r) {
+    const sw_handle* h = b->members[r];
+    if (h->L.np > 0) warps += std::max<long long>(1, (long long)W * (h->g.N / 2) * (h->g.N / 8) / 32);
+  }
+  // fewer warps than ROW_WARPS (about 8 per SM): the products are split over
+  // blocks, each transforming the base fields its products need
+  const int chunks = warps > 0 ? (int)std::min<long long>(MAXP, (ROW_WARPS + warps - 1) / warps) : 1;
+  // column tiles: the narrowest that still move whole 32-byte sectors (4 FP32
+  // or 2 FP64 columns of the largest grid, 1 at 2048^2 in FP64), at least a
+  // warp per block; the same points per block for every member.  Narrow tiles
+  // spread a grid over more SMs (column stage at 64^2 in FP64: 62 us with 2048
+  // points per block, 42 us so)
+  int P = 256;
+  for (int r = 0; r < n; ++r)
+    if (b->members[r]->L.np > 0) P = std::max(P, b->members[r]->g.N * (sizeof(T) == 4 ? 4 : 2));
+  if (sizeof(T) == 8) P = std::min(P, 2048);
+  // split column blocks (see ColShape) while they all fit on the GPU at once
+  long long col_blocks = 0;
+  for (int r = 0; r < n; ++r) {
+    const Layout& L = b->members[r]->L;
+    if (L.np > 0) col_blocks += (long long)b->members[r]->g.KXP * b->members[r]->g.N / P * (L.nlm + (L.has_pos ? 2 : 0) + 2);
+  }
+  b->dual = P / 4 <= DUAL_THREADS<T>() && col_blocks <= DUAL_BLOCKS;
   for (int r = 0; r < n; ++r) {
     sw_handle* h = b->members[r];
+    int lC = 0;
+    while ((h->g.N << lC) < P && lC < h->lC) ++lC;
     // automatic pairs per block: all of them when the row's groups share
     // them out or the grid has rows enough to fill the GPU (N >= 1024), else
     // one (the row's pairs spread over blocks)
-    fill_desc<T>(h, descs[r], h->ppb != 0 ? h->ppb : ((W > 1 || h->g.N >= 1024) ? MAXP : 1));
+    fill_desc<T>(h, descs[r], points, h->ppb != 0 ? h->ppb : std::max(1, (h->L.np + chunks - 1) / chunks), lC, b->dual);
     descs[r].Wp = W;
     const RunDesc<T>& d = descs[r];
     const int N = h->g.N;
-    const int thr[KT_COUNT] = {((1 << h->lC) * N) / 8, h->Bi * N / 8, 256, h->Bp * W * N / 8,
-                               ((1 << h->lC) * N) / 8, 256};
-    const size_t sm[KT_COUNT] = {(size_t)(1 << h->lC) * col_buf_stride<T>(N, 1 << h->lC) * cs,
-                                 (size_t)2 * h->Bi * row_stride<T>(N) * cs, 0,
-                                 row_prod_smem<T>(N, h->Bp, W, h->L),
-                                 (size_t)(1 << h->lC) * col_buf_stride<T>(N, 1 << h->lC) * cs, 0};
+    const int halves = b->dual ? 2 : 1;
+    const int cthr = (N << lC) / 8;
+    const size_t csm = ((size_t)col_buf_stride<T>(N, 1 << lC) << lC) * cs;
+    const int thr[KT_COUNT] = {d.Bi * N / 8, d.Bp * W * N / 8, halves * cthr};
+    const size_t sm[KT_COUNT] = {(size_t)2 * d.Bi * row_stride<T>(N) * cs,
+                                 row_prod_smem<T>(N, d.Bp, W, h->L), halves * csm + (size_t)6 * cthr * cs};
     const KBytes kb = kernel_bytes(h, h->L);
-    const double by[KT_COUNT] = {kb.col_inv, kb.row_inv, kb.phys_q, kb.row_prod, kb.col_fwd, 0.0};
+    if (h->L.np > 0) b->start_bytes += kb.col_inv;
+    const double by[KT_COUNT] = {kb.row_inv, kb.row_prod, 0.0};
     for (int k = 0; k < KT_COUNT; ++k) {
       b->start[(size_t)k * (n + 1) + r + 1] = b->start[(size_t)k * (n + 1) + r] + d.nb[k];
       if (d.nb[k] == 0) continue;
-      if (b->threads[k] && b->threads[k] != thr[k]) {
-        b->err = "batch members need equal block shapes (grid sizes 64..512, or one grid size)";
-        return SW_EINVAL;
+      if (h->L.np == 0) {
+        b->threads[k] = std::max(b->threads[k], 32);
+      } else {
+        b->threads[k] = thr[k];
       }
-      b->threads[k] = thr[k];
       if (sm[k] > b->smem[k]) b->smem[k] = sm[k];
-      for (int st = 0; st < 4; ++st) b->bytes[k][st] += (k == KT_UPDATE ? kb.update[st] : by[k]);
+      for (int st = 0; st < 4; ++st) b->bytes[k][st] += (k == KT_COL_STAGE ? kb.col_stage[st] : by[k]);
     }
-  }
-  // large FP32 grids of one size: a persistent column forward pass that
-  // stages the next tile while transforming the current one
-  b->pipeL = 0;
-  if (sizeof(T) == 4 && n > 0 && b->members[0]->g.N >= 1024) {
-    const int N0 = b->members[0]->g.N;
-    bool same = true;
-    for (int r = 0; r < n; ++r) same = same && b->members[r]->g.N == N0 && b->members[r]->lC == 2;
-    int dev = 0, nsm = 0;
-    const int total = b->start[(size_t)KT_COL_FWD * (n + 1) + n];
-    if (same && total > 0 && cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) {
-      const int L = b->members[0]->g.log2N;
-      const size_t sm = col_fwd_pipe_smem(N0);
-      const int occ = col_fwd_pipe_occupancy(L, b->threads[KT_COL_FWD], sm);
-      if (occ >= 1) {
-        b->pipeL = L;
-        b->pipe_grid = total < nsm * occ ? total : nsm * occ;
-        b->pipe_smem = sm;
-      }
-    }
-    cudaGetLastError();
   }
   const size_t desc_bytes = (sizeof(RunDesc<T>) * n + 255) & ~(size_t)255;
   const size_t need = desc_bytes + sizeof(int) * b->start.size();
@@ -516,39 +639,51 @@ static bool batch_stale(const BatchExec* b) {
     ++*nlaunch;                                                      \
   } while (0)
 
-// One RK4 step (4 stages) of every member of the batch.
+// One kernel kind over the batch (nothing if no member has blocks of it).
 template <typename T>
-static cudaError_t enqueue_batch_step(BatchExec* b, cudaStream_t s, Prof* pf, int64_t* nlaunch) {
-  const RunDesc<T>* runs = (const RunDesc<T>*)b->d_table;
+static cudaError_t enqueue_kernel(BatchExec* b, int k, int stage, bool fin, bool pdl, cudaStream_t s, Prof* pf,
+                                  int64_t* nlaunch) {
   const int n = b->nruns;
+  const int total = b->start[(size_t)k * (n + 1) + n];
   cudaError_t e;
-  static const int order[KT_COUNT] = {KT_COL_INV, KT_ROW_INV, KT_PHYS_Q, KT_ROW_PROD, KT_COL_FWD, KT_UPDATE};
+  if (total == 0) return cudaSuccess;
+  LAUNCH(stage < 0 ? SW_K_COL_INV : SW_K_OF_KT[k], stage < 0 ? b->start_bytes : b->bytes[k][stage],
+         launch_stage<T>(k, (const RunDesc<T>*)b->d_table, b->d_start + (size_t)k * (n + 1), n, total, b->threads[k],
+                         b->smem[k], fin ? stage | STAGE_FINAL : stage, b->warp, b->dual, pdl, s));
+  return cudaSuccess;
+}
+
+// Before the first step of a replay: the mixed fields of the state.  (The
+// state may have been set, and the layout changed, since the last one.)
+template <typename T>
+static cudaError_t enqueue_batch_start(BatchExec* b, cudaStream_t s, Prof* pf, int64_t* nlaunch) {
+  if (b->start_bytes == 0.0) return cudaSuccess;  // no products: nothing reads the mixed fields
+  return enqueue_kernel<T>(b, KT_COL_STAGE, -1, false, false, s, pf, nlaunch);
+}
+
+// One step of every member of the batch; leaves the mixed fields of the new
+// state for the next one (not after the final step of a replay).
+template <typename T>
+static cudaError_t enqueue_batch_step(BatchExec* b, bool final_step, cudaStream_t s, Prof* pf, int64_t* nlaunch) {
+  static const int order[] = {KT_ROW_INV, KT_ROW_PROD, KT_COL_STAGE};
   for (int stage = 0; stage < b->nstages; ++stage) {
-    // forward Euler's second pass is the update kernel alone
+    // forward Euler's second pass only commits
     const bool commit_only = b->stepper == SW_STEP_EULER && stage == 1;
-    for (int oi = 0; oi < KT_COUNT; ++oi) {
-      const int k = order[oi];
-      if (commit_only && k != KT_UPDATE) continue;
-      const int total = b->start[(size_t)k * (n + 1) + n];
-      if (total == 0) continue;
-      if (b->pipeL && k == KT_COL_FWD) {
-        LAUNCH(SW_K_OF_KT[k], b->bytes[k][stage],
-               launch_col_fwd_pipe(b->pipeL, (const RunDesc<float>*)b->d_table, b->d_start + (size_t)k * (n + 1), n,
-                                   b->pipe_grid, b->threads[k], b->pipe_smem, total, pf == nullptr, s));
-        continue;
-      }
-      LAUNCH(SW_K_OF_KT[k], b->bytes[k][stage],
-             launch_stage<T>(k, runs, b->d_start + (size_t)k * (n + 1), n, total, b->threads[k], b->smem[k], stage,
-                             b->warp, pf == nullptr, s));
+    for (int k : order) {
+      if (commit_only && k != KT_COL_STAGE) continue;
+      const bool fin = final_step && k == KT_COL_STAGE && stage == b->nstages - 1;
+      const cudaError_t e = enqueue_kernel<T>(b, k, stage, fin, pf == nullptr, s, pf, nlaunch);
+      if (e != cudaSuccess) return e;
     }
   }
   return cudaSuccess;
 }
 
-// Capture `steps` RK4 steps into an executable graph.  Capture runs on a
+// Capture `steps` steps into an executable graph (`final_step`: the last of
+// them ends a replay).  Capture runs on a
 // private stream (the caller's stream may be the legacy default stream, which
 // cannot be captured); the graphs are launched on the batch's stream.
-static int batch_capture(BatchExec* b, int steps, cudaGraphExec_t* out) {
+static int batch_capture(BatchExec* b, int steps, bool final_step, cudaGraphExec_t* out) {
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaSuccess;
   if (!b->cap && (e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking)) != cudaSuccess) {
@@ -561,7 +696,8 @@ static int batch_capture(BatchExec* b, int steps, cudaGraphExec_t* out) {
   }
   int64_t nl = 0;
   for (int i = 0; i < steps && e == cudaSuccess; ++i)
-    e = b->fp32 ? enqueue_batch_step<float>(b, b->cap, nullptr, &nl) : enqueue_batch_step<double>(b, b->cap, nullptr, &nl);
+    e = b->fp32 ? enqueue_batch_step<float>(b, final_step, b->cap, nullptr, &nl)
+                : enqueue_batch_step<double>(b, final_step, b->cap, nullptr, &nl);
   cudaError_t e2 = cudaStreamEndCapture(b->cap, &graph);
   if (e != cudaSuccess || e2 != cudaSuccess) {
     if (graph) cudaGraphDestroy(graph);
@@ -587,8 +723,9 @@ static int batch_ready(BatchExec* b) {
     if (rc) return rc;
   }
   if (!b->g1) {
-    int rc = batch_capture(b, 1, &b->g1);
-    if (rc == SW_OK) rc = batch_capture(b, GRAPH_STEPS, &b->gm);
+    int rc = batch_capture(b, 1, false, &b->g1);
+    if (rc == SW_OK) rc = batch_capture(b, 1, true, &b->gf);
+    if (rc == SW_OK) rc = batch_capture(b, GRAPH_STEPS, false, &b->gm);
     if (rc != SW_OK) {
       batch_drop_graphs(b);
       return rc;
@@ -601,15 +738,18 @@ static int batch_ready(BatchExec* b) {
 static int batch_replay(BatchExec* b, int64_t n) {
   int rc = batch_ready(b);
   if (rc) return rc;
-  cudaError_t e = cudaSuccess;
+  int64_t nl = 0;
+  cudaError_t e = b->fp32 ? enqueue_batch_start<float>(b, b->stream, nullptr, &nl)
+                          : enqueue_batch_start<double>(b, b->stream, nullptr, &nl);
   int64_t i = 0;
-  for (; e == cudaSuccess && i + GRAPH_STEPS <= n; i += GRAPH_STEPS) e = cudaGraphLaunch(b->gm, b->stream);
-  for (; e == cudaSuccess && i < n; ++i) e = cudaGraphLaunch(b->g1, b->stream);
+  for (; e == cudaSuccess && i + GRAPH_STEPS < n; i += GRAPH_STEPS) e = cudaGraphLaunch(b->gm, b->stream);
+  for (; e == cudaSuccess && i < n; ++i) e = cudaGraphLaunch(i + 1 < n ? b->g1 : b->gf, b->stream);
   if (e != cudaSuccess) {
     b->err = std::string("cudaGraphLaunch: ") + cudaGetErrorString(e);
     return SW_ECUDA;
   }
-  b->launches += n * b->kernels_per_step;
+  b->replayed = n * b->kernels_per_step + nl;
+  b->launches += b->replayed;
   return SW_OK;
 }
 
@@ -618,7 +758,7 @@ static int run_steps(sw_handle* h, int64_t n) {
   int rc = batch_replay(h->self, n);
   if (rc) return fail(h, rc, h->self->err);
   h->steps_total += n;
-  h->launches += n * h->self->kernels_per_step;
+  h->launches += h->self->replayed;
   return SW_OK;
 }
 
@@ -644,10 +784,10 @@ static int spectral_pair_to_phys(sw_handle* h, const OutSpec& a, const OutSpec* 
   cudaStream_t s = h->stream;
   // FP64 spectral copies (scale applied in the row pass epilogue)
   if (h->fp32)
-    CK(h, launch_spec_to_f64<float>((const cplx<float>*)h->y, (const cplx<float>*)h->comp, h->spec64, g.ms,
+    CK(h, launch_spec_to_f64<float>((const cplx<float>*)h->y, (const cplx<float>*)h->comp, h->spec64, g,
                                     a.field, b ? b->field : -1, 1.0, s));
   else
-    CK(h, launch_spec_to_f64<double>((const cplx<double>*)h->y, nullptr, h->spec64, g.ms, a.field,
+    CK(h, launch_spec_to_f64<double>((const cplx<double>*)h->y, nullptr, h->spec64, g, a.field,
                                      b ? b->field : -1, 1.0, s));
   ColInvArgs<double> ci;
   ci.src = h->spec64;
@@ -727,8 +867,8 @@ static int load_ic_from_out64(sw_handle* h) {
   // two-dimensional Euler model holds the vorticity there and derives u, v
   const bool e2 = h->p.model == SW_MODEL_EULER2D;
   if (!e2) CK(h, launch_add_real(h->spec64 + 2 * g.ms + (long long)g.K * g.KXP, -1.0, s));
-  if (h->fp32) CK(h, launch_spec_from_f64<float>(h->spec64, (cplx<float>*)h->y, 3 * g.ms, s));
-  else CK(h, launch_spec_from_f64<double>(h->spec64, (cplx<double>*)h->y, 3 * g.ms, s));
+  if (h->fp32) CK(h, launch_spec_from_f64<float>(h->spec64, (cplx<float>*)h->y, g, 3, s));
+  else CK(h, launch_spec_from_f64<double>(h->spec64, (cplx<double>*)h->y, g, 3, s));
   if (e2) {
     if (h->fp32) CK(h, launch_velocity_from_vorticity<float>((cplx<float>*)h->y, g, h->L.f_u, h->L.f_v, h->L.f_h, s));
     else CK(h, launch_velocity_from_vorticity<double>((cplx<double>*)h->y, g, h->L.f_u, h->L.f_v, h->L.f_h, s));
@@ -796,16 +936,16 @@ static void plan_geometry(int N, size_t tsz, Geom& g, int& lC) {
 
 // Offsets of the handle's device arena (256-byte aligned slices).
 struct ArenaPlan {
-  size_t o[19];
+  size_t o[18];
   size_t total;
 };
 
 static ArenaPlan plan_arena(const Geom& g, size_t tsz) {
   ArenaPlan A;
   const size_t cs = 2 * tsz;
-  const size_t sizes[19] = {
-      MAXF * g.ms * cs, MAXF * g.ms * cs, MAXF * g.ms * cs, MAXF * g.ms * cs,  // y, ys, ys2, acc
-      MAXF * g.ms * cs, MAXP * g.ms * cs,                                      // comp, ps
+  const size_t sizes[18] = {
+      MAXF * g.ms * cs, 3 * g.ms * cs, 3 * g.ms * cs, MAXF * g.ms * cs,        // y, ys, ys2, acc
+      MAXF * g.ms * cs,                                                        // comp
       MAXI * g.mi * cs, MAXP * g.mi * cs,                                      // mix, pmix
       NPH * g.np * tsz, 6 * g.ms * tsz, g.N * cs,                              // phys, ef, tw
       g.N * sizeof(double2), 4 * g.ms * sizeof(double2),                       // tw64, spec64
@@ -813,7 +953,7 @@ static ArenaPlan plan_arena(const Geom& g, size_t tsz) {
       2 * DIAG_BLOCKS * sizeof(double), 4 * sizeof(double),                    // part, dres
       sizeof(long long), sizeof(unsigned)};                                    // ctr, ticket
   size_t off = 0;
-  for (int i = 0; i < 19; ++i) {
+  for (int i = 0; i < 18; ++i) {
     A.o[i] = off;
     off += align256(sizes[i]);
   }
@@ -835,28 +975,32 @@ template <typename T>
 static void host_tables(const sw_params& p, const Geom& g, void* ef_host, void* tw_host, double2* tw64_host) {
   T* ef = (T*)ef_host;
   static_assert(sizeof(twid<T>) == sizeof(cplx<T>), "twiddle table size");
-  for (int kyi = 0; kyi < g.NY; ++kyi)
-    for (int kx = 0; kx < g.KXP; ++kx) {
-      const double ky = kyi - g.K;
-      const double k2 = (double)kx * kx + ky * ky;
-      const double k8 = p.visc == SW_VISC_LAPLACE ? k2 : k2 * k2 * k2 * k2;  // |k|^2p
-      const long long m = (long long)kyi * g.KXP + kx;
-      // per class (dynamics, mean fields): E = exp(-nu |k|^2p dt/2) for the
-      // stage values, and E^2 as an unevaluated sum hi + lo for the commit
-      // of y_{n+1} = E^2 y_n + ...: rounded to T alone, E^2 would move every
-      // damped mode by up to half an ulp of T per step, an error that grows
-      // linearly with the steps of an interval (in FP32 about 4e-5 after
-      // 1219 steps at 64^2); hi + lo carries it to about twice T's digits.
-      const double nus[2] = {p.nu8, p.lm_nu8};
-      for (int c = 0; c < 2; ++c) {
-        const double E = std::exp(-nus[c] * k8 * p.dt * 0.5);
-        const double E2 = E * E;
-        const T hi = (T)E2;
-        ef[(3 * c) * g.ms + m] = (T)E;
-        ef[(3 * c + 1) * g.ms + m] = hi;
-        ef[(3 * c + 2) * g.ms + m] = (T)(E2 - (double)hi);
-      }
-    }
+  // per class (dynamics, mean fields): E = exp(-nu |k|^2p dt/2) for the
+  // stage values, and E^2 as an unevaluated sum hi + lo for the commit
+  // of y_{n+1} = E^2 y_n + ...: rounded to T alone, E^2 would move every
+  // damped mode by up to half an ulp of T per step, an error that grows
+  // linearly with the steps of an interval (in FP32 about 4e-5 after
+  // 1219 steps at 64^2); hi + lo carries it to about twice T's digits.
+  // In the order of the spectral layout; ky and -ky share their values.
+  const double nus[2] = {p.nu8, p.lm_nu8};
+  const int classes = p.nu8 == p.lm_nu8 ? 1 : 2;
+  for (int c = 0; c < classes; ++c)
+    for (int kx0 = 0; kx0 < g.KXP; kx0 += spec_tile<T>())
+      for (int ky = 0; ky <= g.K; ++ky)
+        for (int kx = kx0; kx < kx0 + spec_tile<T>(); ++kx) {
+          const double k2 = (double)kx * kx + (double)ky * ky;
+          const double k8 = p.visc == SW_VISC_LAPLACE ? k2 : k2 * k2 * k2 * k2;  // |k|^2p
+          const double E = std::exp(-nus[c] * k8 * p.dt * 0.5);
+          const double E2 = E * E;
+          const T hi = (T)E2, lo = (T)(E2 - (double)hi);
+          for (int sg = 0; sg < 2; ++sg) {
+            const long long m = spec_index<T>(g.K + (sg ? -ky : ky), kx, g.NY);
+            ef[(3 * c) * g.ms + m] = (T)E;
+            ef[(3 * c + 1) * g.ms + m] = hi;
+            ef[(3 * c + 2) * g.ms + m] = lo;
+          }
+        }
+  if (classes == 1) std::memcpy(ef + 3 * g.ms, ef, 3 * g.ms * sizeof(T));
   std::vector<double> re(g.N, 1.0), im(g.N, 0.0);
   fft_twiddle_table(g.log2N, re.data(), im.data());
   for (int t = 0; t < g.N; ++t) {
@@ -892,15 +1036,13 @@ extern "C" int sw_create(const sw_params* p, const double* ic_uvh, int ic_on_dev
   plan_geometry(p->N, h->tsz, g, h->lC);
   const size_t cs = 2 * h->tsz;  // complex T
   h->diag_blocks = DIAG_BLOCKS;
-  h->Bp = row_block_rows(g.N);
   h->Bi = row_block_rows(g.N);
-  // all product pairs per block: the row's groups share them out
   h->ppb = 0;  // automatic (batch_build_t)
   const ArenaPlan A = plan_arena(g, h->tsz);
-  const size_t o_y = A.o[0], o_ys = A.o[1], o_ys2 = A.o[2], o_acc = A.o[3], o_comp = A.o[4], o_ps = A.o[5];
-  const size_t o_mix = A.o[6], o_pmix = A.o[7], o_phys = A.o[8], o_ef = A.o[9], o_tw = A.o[10];
-  const size_t o_tw64 = A.o[11], o_spec64 = A.o[12], o_mix64 = A.o[13], o_out64 = A.o[14];
-  const size_t o_part = A.o[15], o_dres = A.o[16], o_ctr = A.o[17], o_ticket = A.o[18];
+  const size_t o_y = A.o[0], o_ys = A.o[1], o_ys2 = A.o[2], o_acc = A.o[3], o_comp = A.o[4];
+  const size_t o_mix = A.o[5], o_pmix = A.o[6], o_phys = A.o[7], o_ef = A.o[8], o_tw = A.o[9];
+  const size_t o_tw64 = A.o[10], o_spec64 = A.o[11], o_mix64 = A.o[12], o_out64 = A.o[13];
+  const size_t o_part = A.o[14], o_dres = A.o[15], o_ctr = A.o[16], o_ticket = A.o[17];
   const size_t off = A.total;
   h->arena_bytes = off;
   cudaError_t e = cudaMalloc(&h->arena, h->arena_bytes);
@@ -910,7 +1052,7 @@ extern "C" int sw_create(const sw_params* p, const double* ic_uvh, int ic_on_dev
     return fail(nullptr, SW_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   }
   char* base = (char*)h->arena;
-  h->y = base + o_y; h->ys = base + o_ys; h->ys2 = base + o_ys2; h->acc = base + o_acc; h->comp = base + o_comp; h->ps = base + o_ps;
+  h->y = base + o_y; h->ys = base + o_ys; h->ys2 = base + o_ys2; h->acc = base + o_acc; h->comp = base + o_comp;
   h->mix = base + o_mix; h->pmix = base + o_pmix; h->phys = base + o_phys; h->ef = base + o_ef;
   h->tw = base + o_tw; h->tw64 = (double2*)(base + o_tw64); h->spec64 = (double2*)(base + o_spec64);
   h->mix64 = (double2*)(base + o_mix64); h->out64 = (double*)(base + o_out64);
@@ -1138,10 +1280,10 @@ static int phys_uvhz(sw_handle* h) {
   // zeta = i kx v - i ky u from FP64 copies of u, v
   const Geom& g = h->g;
   if (h->fp32)
-    CK(h, launch_spec_to_f64<float>((const cplx<float>*)h->y, nullptr, h->spec64, g.ms, h->L.f_u, h->L.f_v, 1.0,
+    CK(h, launch_spec_to_f64<float>((const cplx<float>*)h->y, nullptr, h->spec64, g, h->L.f_u, h->L.f_v, 1.0,
                                     h->stream));
   else
-    CK(h, launch_spec_to_f64<double>((const cplx<double>*)h->y, nullptr, h->spec64, g.ms, h->L.f_u, h->L.f_v, 1.0,
+    CK(h, launch_spec_to_f64<double>((const cplx<double>*)h->y, nullptr, h->spec64, g, h->L.f_u, h->L.f_v, 1.0,
                                      h->stream));
   ColInvArgs<double> ci;
   ci.src = h->spec64;
@@ -1212,7 +1354,9 @@ extern "C" int sw_diag(sw_handle* h, double out[3]) {
   // mass: the k = 0 coefficient of h (row ky = 0, column kx = 0)
   const size_t cs = 2 * h->tsz;
   unsigned char m0[16];
-  CK(h, cudaMemcpyAsync(m0, (char*)h->y + ((size_t)h->L.f_h * g.ms + (size_t)g.K * g.KXP) * cs, cs,
+  CK(h, cudaMemcpyAsync(m0, (char*)h->y +
+                            ((size_t)h->L.f_h * g.ms + (h->fp32 ? spec_index<float>(g.K, 0, g.NY)
+                                                                : spec_index<double>(g.K, 0, g.NY))) * cs, cs,
                         cudaMemcpyDeviceToHost, h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
   // the state holds eta = h - 1
@@ -1265,8 +1409,14 @@ extern "C" int sw_get_state(sw_handle* h, void* blob, size_t* size) {
   std::memcpy(blob, &hd, sizeof(hd));
   const size_t fb = (size_t)nf * h->g.ms * 2 * h->tsz;
   char* dst = (char*)blob + sizeof(hd);
-  CK(h, cudaMemcpyAsync(dst, h->y, fb, cudaMemcpyDeviceToHost, h->stream));
-  CK(h, cudaMemcpyAsync(dst + fb, h->comp, fb, cudaMemcpyDeviceToHost, h->stream));
+  // blobs hold rows [ky + K][kx] (through the mixed fields' buffer, which the
+  // next replay fills anew)
+  for (int k = 0; k < 2; ++k) {
+    const void* src = k == 0 ? h->y : h->comp;
+    if (h->fp32) CK(h, launch_spec_rows<float>((const float2*)src, (float2*)h->mix, h->g, nf, true, h->stream));
+    else CK(h, launch_spec_rows<double>((const double2*)src, (double2*)h->mix, h->g, nf, true, h->stream));
+    CK(h, cudaMemcpyAsync(dst + k * fb, h->mix, fb, cudaMemcpyDeviceToHost, h->stream));
+  }
   CK(h, cudaStreamSynchronize(h->stream));
   *size = need;
   return SW_OK;
@@ -1288,8 +1438,12 @@ extern "C" int sw_set_state(sw_handle* h, const void* blob, size_t size) {
   if (L.nf != hd.nf || size < blob_size(h, hd.nf)) return fail(h, SW_EINVAL, "blob size mismatch");
   const size_t fb = (size_t)hd.nf * h->g.ms * 2 * h->tsz;
   const char* src = (const char*)blob + sizeof(hd);
-  CK(h, cudaMemcpyAsync(h->y, src, fb, cudaMemcpyHostToDevice, h->stream));
-  CK(h, cudaMemcpyAsync(h->comp, src + fb, fb, cudaMemcpyHostToDevice, h->stream));
+  for (int k = 0; k < 2; ++k) {
+    void* dst = k == 0 ? h->y : h->comp;
+    CK(h, cudaMemcpyAsync(h->mix, src + k * fb, fb, cudaMemcpyHostToDevice, h->stream));
+    if (h->fp32) CK(h, launch_spec_rows<float>((const float2*)h->mix, (float2*)dst, h->g, hd.nf, false, h->stream));
+    else CK(h, launch_spec_rows<double>((const double2*)h->mix, (double2*)dst, h->g, hd.nf, false, h->stream));
+  }
   long long ctr = hd.done;
   CK(h, cudaMemcpyAsync(h->ctr, &ctr, sizeof(ctr), cudaMemcpyHostToDevice, h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
@@ -1371,7 +1525,16 @@ extern "C" int sw_kernel_times(sw_handle* h, int64_t nsteps, double ms[SW_K_COUN
   for (int64_t it = 0; rc == SW_OK && it < nsteps; ++it) {
     pf.n = 0;
     int64_t nl = 0;
-    e = h->fp32 ? enqueue_batch_step<float>(b, h->stream, &pf, &nl) : enqueue_batch_step<double>(b, h->stream, &pf, &nl);
+    if (it == 0) {
+      e = h->fp32 ? enqueue_batch_start<float>(b, h->stream, &pf, &nl) : enqueue_batch_start<double>(b, h->stream, &pf, &nl);
+      if (e != cudaSuccess) {
+        rc = fail_cuda(h, "sw_kernel_times start", e);
+        break;
+      }
+    }
+    const bool fin = it == nsteps - 1;
+    e = h->fp32 ? enqueue_batch_step<float>(b, fin, h->stream, &pf, &nl)
+                : enqueue_batch_step<double>(b, fin, h->stream, &pf, &nl);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) {
       rc = fail_cuda(h, "sw_kernel_times step", e);
@@ -1503,7 +1666,7 @@ extern "C" int sw_batch_tune(sw_batch* b, int trial_steps, int* choice) {
     const int P = pts[ci / 4], ppb = ppbs[ci % 4];
     if (P < maxN) continue;  // every member needs rows x N = P (equal block shapes)
     for (sw_handle* h : ex->members) {
-      h->Bp = row_block_rows(h->g.N, P);
+      h->points = P;
       h->ppb = ppb;
       ++h->version;
     }
@@ -1536,7 +1699,7 @@ extern "C" int sw_batch_tune(sw_batch* b, int trial_steps, int* choice) {
     best = 4 * pi + 3;
   }
   for (sw_handle* h : ex->members) {
-    h->Bp = row_block_rows(h->g.N, pts[best / 4]);
+    h->points = pts[best / 4];
     h->ppb = ppbs[best % 4];
     ++h->version;
   }
@@ -1573,7 +1736,7 @@ extern "C" int sw_batch_set_shape(sw_batch* b, int choice) {
   for (sw_handle* h : ex->members)
     if (pts[choice / 4] < h->g.N) return bfail(b, SW_EINVAL, "points per block below a member's N");
   for (sw_handle* h : ex->members) {
-    h->Bp = row_block_rows(h->g.N, pts[choice / 4]);
+    h->points = pts[choice / 4];
     h->ppb = ppbs[choice % 4];
     ++h->version;
   }

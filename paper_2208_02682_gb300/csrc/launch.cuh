@@ -9,66 +9,78 @@ struct sw_handle;
 
 namespace lm {
 
-// Rows per block of the row kernels: B rows of N points run with B*N/8
-// threads (one 8-element Stockham butterfly set per thread and pass).
-// `points` = B*N; 512 keeps small grids spread over many SMs.
+// Rows (row pairs in the stage kernels) per block: B of N points run with
+// B*N/8 threads (one 8-element Stockham butterfly set per thread and pass);
+// `points` = B*N.
 inline int row_block_rows(int N, int points = 512) {
-  // points = rows x N per block (the block runs points/8 threads per group)
   int B = points / N;
   if (B > N) B = N;
   if (B < 1) B = 1;
   return B;
 }
+// Row pairs per block of the stage kernels: at most N/2, but a warp's worth of
+// threads (at N = 16 the pairs then wrap around, each done twice).
+inline int row_block_pairs(int N, int points) {
+  int B = row_block_rows(N, points);
+  if (B > N / 2) B = N / 2;
+  return B * N < 256 ? 256 / N : B;
+}
+inline int row_blocks(int N, int B) { return N / 2 > B ? N / 2 / B : 1; }
 
-// Row pass: B rows per block, W groups of N/8 threads per row (see
+// Row pass: B row pairs per block, W groups of N/8 threads per pair (see
 // k_stage_row_prod); the block may hold up to row_prod_max_threads threads.
+template <typename T> bool row_prod_fused(int N, const Layout& L) {
+  // FP64 from 1024^2 the base fields take 64 KB and more per row pair and leave
+  // one block per SM: row pass alone 419 us with them, 299 us + 54 us for the
+  // planes.  FP32: 250 us against 349 us + 39 us at 2048^2.
+  return L.strategy != 2 && (sizeof(T) == 4 || N <= 512);
+}
+// Strategy 2: the gathered arrays within 96 KB per row pair.
+template <typename T> bool row_prod_gath(int N, const Layout& L) {
+  return L.strategy == 2 && (size_t)row_prod_planes(0, 1, L.has_q) * N * sizeof(cplx<T>) <= (size_t)96 * 1024;
+}
 template <typename T> size_t row_prod_smem(int N, int B, int W, const Layout& L) {
-  const size_t nur = L.strategy == 2 ? 6 : 4, nug = (size_t)row_prod_group_rows(L);
-  return (size_t)B * nur * N * sizeof(T) +
-         (size_t)B * W * (2 * row_stride<T>(N) * sizeof(cplx<T>) + nug * N * sizeof(T));
+  const size_t nu = row_prod_planes(row_prod_fused<T>(N, L), row_prod_gath<T>(N, L), L.has_q);
+  return (size_t)B * sizeof(cplx<T>) * (nu * N + (size_t)W * 2 * row_stride<T>(N));
 }
 
-// Largest W for B rows and npb product pairs per block: W > 1 needs whole
+// Largest W for B row pairs and np products per block: W > 1 needs whole
 // warps per group (N >= 256), a thread count within the block limit, at most
-// 15 named barriers (groups of N >= 512) and at most 110 KB of shared memory
-// (two blocks per SM; one resident block per SM made the wider shape slower).
-template <typename T> int row_prod_groups(int N, int B, int npb, const Layout& L) {
-  const int strategy = L.strategy;
+// 15 named barriers (groups of N >= 512) and at most 200 KB of shared memory.
+template <typename T> int row_prod_groups(int N, int B, int np, const Layout& L) {
   const int G = N / 8;
   if (G < 32) return 1;
-  int W = npb < 1 ? 1 : npb;
-  while (W > 1 && (B * W * G > row_prod_max_threads<T>() || (G >= 64 && B * W > 15) ||
-                   row_prod_smem<T>(N, B, W, L) > (size_t)110 * 1024))
-    --W;
-  // Strategy 2 transforms one base pair (xi) before the products, so the
-  // row's other groups wait at the barrier; that pays only when every pair
-  // gets a group of its own (measured slower at 1024^2 with 2 groups for 6
-  // pairs)
-  if (strategy == 2 && W < npb) W = 1;
-  return W;
+  auto fit = [&](int threads, size_t smem) {
+    int W = np < 1 ? 1 : np;
+    while (W > 1 && (B * W * G > threads || (G >= 64 && B * W > 15) || row_prod_smem<T>(N, B, W, L) > smem)) --W;
+    return W;
+  };
+  // two blocks per SM, or one of several groups where that leaves one group
+  const int W = fit(sizeof(T) == 4 ? 384 : 256, (size_t)110 * 1024);
+  return W > 1 ? W : fit(row_prod_max_threads<T>(), (size_t)200 * 1024);
 }
+
+template <typename T> constexpr int DUAL_THREADS() { return sizeof(T) == 4 ? 256 : 128; }
 
 template <typename T> cudaError_t launch_col_inv(const ColInvArgs<T>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_col_fwd(const ColFwdArgs<T>& a, cudaStream_t s);
 template <typename T, typename TO> cudaError_t launch_row_inv(const RowInvArgs<T, TO>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_row_fwd(const RowFwdArgs<T>& a, cudaStream_t s);
+// dual: the column stage with split blocks (at most DUAL_THREADS threads).
 // warp: every run's rows have N <= 256 (groups of at most one warp), so the
 // row kernels' variant without named barriers may run.  pdl: launch with
 // programmatic stream serialisation (see pdl_wait).
 template <typename T>
 cudaError_t launch_stage(int kt, const RunDesc<T>* runs, const int* start, int nruns, int blocks, int threads,
-                         size_t smem, int stage, bool warp, bool pdl, cudaStream_t s);
-// Pipelined column forward pass of the large FP32 grids (L = log2 N in
-// {10, 11}, four-column tiles): `blocks` persistent blocks over `total`
-// work items.
-cudaError_t launch_col_fwd_pipe(int L, const RunDesc<float>* runs, const int* start, int nruns, int blocks,
-                                int threads, size_t smem, int total, bool pdl, cudaStream_t s);
-// Resident blocks per SM of a pipelined column forward launch (0 on error).
-int col_fwd_pipe_occupancy(int L, int threads, size_t smem);
+                         size_t smem, int stage, bool warp, bool dual, bool pdl, cudaStream_t s);
 template <typename T>
-cudaError_t launch_spec_to_f64(const cplx<T>* y, const cplx<T>* comp, double2* out, long long ms, int fa, int fb,
+cudaError_t launch_spec_to_f64(const cplx<T>* y, const cplx<T>* comp, double2* out, const Geom& g, int fa, int fb,
                                double scale, cudaStream_t s);
-template <typename T> cudaError_t launch_spec_from_f64(const double2* in, cplx<T>* y, long long n, cudaStream_t s);
+template <typename T>
+cudaError_t launch_spec_from_f64(const double2* in, cplx<T>* y, const Geom& g, int nfields, cudaStream_t s);
+template <typename T>
+cudaError_t launch_spec_rows(const cplx<T>* in, cplx<T>* out, const Geom& g, int nfields, bool to_rows,
+                             cudaStream_t s);
 template <typename T>
 cudaError_t launch_velocity_from_vorticity(cplx<T>* y, const Geom& g, int fu, int fv, int fh, cudaStream_t s);
 cudaError_t launch_diag(const double* phys, long long np, double f0, double c2, double* part, int nblk,
@@ -109,8 +121,14 @@ template <typename T> static cudaError_t prepare_kernels_t() {
   if ((e = allow_dynamic_smem(k_col_fwd<T>, mx)) != cudaSuccess) return e;
   if ((e = allow_dynamic_smem(k_row_inv<T, T>, mx)) != cudaSuccess) return e;
   if ((e = allow_dynamic_smem(k_row_fwd<T>, mx)) != cudaSuccess) return e;
-  if ((e = allow_dynamic_smem(k_stage_col_inv<T>, mx)) != cudaSuccess) return e;
-  if ((e = allow_dynamic_smem(k_stage_col_fwd<T>, mx)) != cudaSuccess) return e;
+  if constexpr (sizeof(T) == 8)
+    if ((e = allow_dynamic_smem(k_stage_col<T, 128, false>, mx)) != cudaSuccess) return e;
+  if ((e = allow_dynamic_smem(k_stage_col<T, 256, false>, mx)) != cudaSuccess) return e;
+  if ((e = allow_dynamic_smem(k_stage_col<T, DUAL_THREADS<T>(), true>, mx)) != cudaSuccess) return e;
+  if constexpr (sizeof(T) == 4) {
+    if ((e = allow_dynamic_smem(k_stage_col<T, 512, false>, mx)) != cudaSuccess) return e;
+    if ((e = allow_dynamic_smem(k_stage_col<T, 1024, false>, mx)) != cudaSuccess) return e;
+  }
   if ((e = allow_dynamic_smem(k_stage_row_inv<T, false>, mx)) != cudaSuccess) return e;
   if ((e = allow_dynamic_smem(k_stage_row_inv<T, true>, mx)) != cudaSuccess) return e;
   if ((e = allow_dynamic_smem(k_stage_row_prod<T, false>, mx)) != cudaSuccess) return e;
@@ -146,7 +164,7 @@ template <typename T> cudaError_t launch_row_fwd(const RowFwdArgs<T>& a, cudaStr
 
 template <typename T>
 cudaError_t launch_stage(int kt, const RunDesc<T>* runs, const int* start, int nruns, int blocks, int threads,
-                         size_t smem, int stage, bool warp, bool pdl, cudaStream_t s) {
+                         size_t smem, int stage, bool warp, bool dual, bool pdl, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)blocks);
   cfg.blockDim = dim3((unsigned)threads);
@@ -158,28 +176,41 @@ cudaError_t launch_stage(int kt, const RunDesc<T>* runs, const int* start, int n
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
   switch (kt) {
-    case KT_COL_INV: return cudaLaunchKernelEx(&cfg, k_stage_col_inv<T>, runs, start, nruns, stage);
     case KT_ROW_INV:
       return warp ? cudaLaunchKernelEx(&cfg, k_stage_row_inv<T, true>, runs, start, nruns)
                   : cudaLaunchKernelEx(&cfg, k_stage_row_inv<T, false>, runs, start, nruns);
-    case KT_PHYS_Q: cfg.dynamicSmemBytes = 0; return cudaLaunchKernelEx(&cfg, k_stage_phys_q<T>, runs, start, nruns);
     case KT_ROW_PROD:
       return warp ? cudaLaunchKernelEx(&cfg, k_stage_row_prod<T, true>, runs, start, nruns, stage)
                   : cudaLaunchKernelEx(&cfg, k_stage_row_prod<T, false>, runs, start, nruns, stage);
-    case KT_COL_FWD: return cudaLaunchKernelEx(&cfg, k_stage_col_fwd<T>, runs, start, nruns);
-    default: cfg.dynamicSmemBytes = 0; return cudaLaunchKernelEx(&cfg, k_stage_update<T>, runs, start, nruns, stage);
+    default:
+      if (dual) return cudaLaunchKernelEx(&cfg, k_stage_col<T, DUAL_THREADS<T>(), true>, runs, start, nruns, stage);
+      if constexpr (sizeof(T) == 4) {
+        if (threads > 512) return cudaLaunchKernelEx(&cfg, k_stage_col<T, 1024, false>, runs, start, nruns, stage);
+        if (threads > 256) return cudaLaunchKernelEx(&cfg, k_stage_col<T, 512, false>, runs, start, nruns, stage);
+      }
+      if constexpr (sizeof(T) == 8)
+        if (threads <= 128) return cudaLaunchKernelEx(&cfg, k_stage_col<T, 128, false>, runs, start, nruns, stage);
+      return cudaLaunchKernelEx(&cfg, k_stage_col<T, 256, false>, runs, start, nruns, stage);
   }
 }
 
 template <typename T>
-cudaError_t launch_spec_to_f64(const cplx<T>* y, const cplx<T>* comp, double2* out, long long ms, int fa, int fb,
+cudaError_t launch_spec_to_f64(const cplx<T>* y, const cplx<T>* comp, double2* out, const Geom& g, int fa, int fb,
                                double scale, cudaStream_t s) {
-  k_spec_to_f64<T><<<(unsigned)((ms + 255) / 256), 256, 0, s>>>(y, comp, out, ms, fa, fb, scale);
+  k_spec_to_f64<T><<<(unsigned)((g.ms + 255) / 256), 256, 0, s>>>(y, comp, out, g.ms, g.NY, g.KXP, fa, fb, scale);
   return cudaGetLastError();
 }
 
-template <typename T> cudaError_t launch_spec_from_f64(const double2* in, cplx<T>* y, long long n, cudaStream_t s) {
-  k_spec_from_f64<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(in, y, n);
+template <typename T>
+cudaError_t launch_spec_from_f64(const double2* in, cplx<T>* y, const Geom& g, int nfields, cudaStream_t s) {
+  k_spec_from_f64<T><<<(unsigned)((g.ms * nfields + 255) / 256), 256, 0, s>>>(in, y, g, nfields);
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_spec_rows(const cplx<T>* in, cplx<T>* out, const Geom& g, int nfields, bool to_rows,
+                             cudaStream_t s) {
+  k_spec_rows<T><<<(unsigned)((g.ms * nfields + 255) / 256), 256, 0, s>>>(in, out, g, nfields, to_rows ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -195,10 +226,11 @@ cudaError_t launch_velocity_from_vorticity(cplx<T>* y, const Geom& g, int fu, in
   template cudaError_t launch_row_inv<T, T>(const RowInvArgs<T, T>&, cudaStream_t);                         \
   template cudaError_t launch_row_fwd<T>(const RowFwdArgs<T>&, cudaStream_t);                               \
   template cudaError_t launch_stage<T>(int, const RunDesc<T>*, const int*, int, int, int, size_t, int, bool,  \
-                                       bool, cudaStream_t);                                                 \
-  template cudaError_t launch_spec_to_f64<T>(const cplx<T>*, const cplx<T>*, double2*, long long, int, int,  \
+                                       bool, bool, cudaStream_t);                                                 \
+  template cudaError_t launch_spec_to_f64<T>(const cplx<T>*, const cplx<T>*, double2*, const Geom&, int, int, \
                                              double, cudaStream_t);                                         \
-  template cudaError_t launch_spec_from_f64<T>(const double2*, cplx<T>*, long long, cudaStream_t);            \
+  template cudaError_t launch_spec_from_f64<T>(const double2*, cplx<T>*, const Geom&, int, cudaStream_t);     \
+  template cudaError_t launch_spec_rows<T>(const cplx<T>*, cplx<T>*, const Geom&, int, bool, cudaStream_t);   \
   template cudaError_t launch_velocity_from_vorticity<T>(cplx<T>*, const Geom&, int, int, int, cudaStream_t);
 #endif
 

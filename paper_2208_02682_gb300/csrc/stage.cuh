@@ -8,26 +8,26 @@
 // are uniform within a launch: C*N (columns x points) and Bp*N, Bi*N (rows x
 // points) are equal for all members.
 //
-// Per stage:  col_inv -> [row_inv, phys_q: Strategy 2] -> row_prod -> col_fwd -> update
+// Per stage:  [row_inv] -> row_prod -> col_stage;
+// a replay of steps starts with one col_stage that only transforms.
 #pragma once
 #include "kernels.cuh"
 
 namespace lm {
 
-enum { KT_COL_INV = 0, KT_ROW_INV = 1, KT_PHYS_Q = 2, KT_ROW_PROD = 3, KT_COL_FWD = 4, KT_UPDATE = 5, KT_COUNT = 6 };
+enum { KT_ROW_INV = 0, KT_ROW_PROD = 1, KT_COL_STAGE = 2, KT_COUNT = 3 };
 
 template <typename T>
-struct RunDesc {
+struct alignas(16) RunDesc {
   Geom g;
   Layout L;
   StepConsts c;
   T cdt, cf0, cc2, cadvx, cadvy;  // dt, f0, c2, adv in the kernels' precision
   cplx<T>* y;     // state at t_n
-  cplx<T>* ysa;   // stage inputs of stages 1 and 3
-  cplx<T>* ysb;   // stage input of stage 2
+  cplx<T>* ysa;   // stage inputs of stages 1 and 3 (u, v, h)
+  cplx<T>* ysb;   // stage input of stage 2 (u, v, h)
   cplx<T>* acc;   // RK accumulator
   cplx<T>* comp;  // Kahan compensation (FP32 mode; null in FP64)
-  cplx<T>* ps;    // spectral products
   cplx<T>* mix;   // column-pass outputs (mixed)
   cplx<T>* pmix;  // row-pass products (mixed)
   T* phys;        // Strategy-2 gather buffer
@@ -36,9 +36,12 @@ struct RunDesc {
   long long* ctr;
   unsigned* ticket;
   int lC;         // column tile: C = 2^lC columns
-  int Bp, ppb;    // row_prod: rows per block, product pairs per block
-  int Wp;         // row_prod: groups of N/8 threads per row
-  int Bi;         // row_inv: rows per block
+  int Bp, ppb;    // row_prod: row pairs per block, products per block
+  int Wp;         // row_prod: groups of N/8 threads per row pair
+  int Bi;         // row_inv: row pairs per block
+  int fused;      // row_prod: transforms the base fields itself
+  int gath;       // row_prod: gathers all fields at x + xi at once (interleaved planes)
+  int umask[MAXP];  // row_prod: base fields each product chunk needs (bits PH_*)
   int nb[KT_COUNT];
 };
 
@@ -58,10 +61,11 @@ __device__ __forceinline__ int find_run(const int* __restrict__ start, int nruns
 template <typename T>
 __device__ __forceinline__ const RunDesc<T>& load_desc(const RunDesc<T>* __restrict__ runs, int r,
                                                        unsigned char* sbuf) {
-  static_assert(sizeof(RunDesc<T>) % sizeof(int) == 0, "descriptor size");
-  const int* src = reinterpret_cast<const int*>(runs + r);
-  int* dst = reinterpret_cast<int*>(sbuf);
-  constexpr int n = (int)(sizeof(RunDesc<T>) / sizeof(int));
+  static_assert(sizeof(RunDesc<T>) % sizeof(int4) == 0, "descriptor size");
+  const int4* src = reinterpret_cast<const int4*>(runs + r);
+  int4* dst = reinterpret_cast<int4*>(sbuf);
+  constexpr int n = (int)(sizeof(RunDesc<T>) / sizeof(int4));
+#pragma unroll 4
   for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = __ldg(src + i);
   __syncthreads();
   return *reinterpret_cast<const RunDesc<T>*>(sbuf);
@@ -76,212 +80,10 @@ __device__ __forceinline__ const cplx<T>* stage_input(const RunDesc<T>& d, int s
   return stage == 0 ? d.y : (stage == 2 ? d.ysb : d.ysa);
 }
 
-// ---------------------------------------------------------------------------
-// Column passes on group transforms: a block owns a tile of C = 2^lC
-// consecutive kx columns; thread t works on column c = t mod C and rows
-// n = j + m N/8 (j = t div C, m < 8), so the lanes of a warp read and write
-// C-wide contiguous runs of the kx-major fields straight from and to
-// registers.  Smem: C * col_buf_stride(N, C) complex.
-
-// Threads per column-pass block at most: C*N/8 is 256 up to 512^2 and in
-// FP64; FP32 tiles of 4 columns at 1024^2 and 2048^2 take 512 and 1024.
-template <typename T> constexpr int col_max_threads() { return sizeof(T) == 4 ? 1024 : 256; }
-
-// a1: column inverse pass, local block = (output field, kx tile):
-// mixed = IFFT_y(op(spectral)) with op in {id, d_x, d_y, curl}, zero-padded
-// outside |ky| <= K.
-template <typename T>
-__global__ void __launch_bounds__(col_max_threads<T>()) k_stage_col_inv(const RunDesc<T>* __restrict__ runs,
-                                                       const int* __restrict__ start, int nruns, int stage) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ unsigned red[GRedWords<T>::value];  // FP64 transforms
-  const int r = find_run(start, nruns, blockIdx.x);
-  const RunDesc<T>& d = runs[r];
-  pdl_wait();  // state written by the previous kernels: only after this
-  const int lb = blockIdx.x - start[r];
-  dispatch_L<4, 11>(d.g.log2N, [&](auto Lc) {
-    constexpr int L = decltype(Lc)::value, N = 1 << L, G = N / 8;
-    const int K = d.g.K, KXP = d.g.KXP;
-    const int lC = d.lC, C = 1 << lC;
-    const int ntile = KXP >> lC;
-    const int o = lb / ntile, tile = lb - o * ntile;
-    const int c = threadIdx.x & (C - 1), j = threadIdx.x >> lC;
-    const int kx = (tile << lC) + c;
-    const cplx<T>* src = stage_input(d, stage);
-    const int op = d.L.i_op[o];
-    const cplx<T>* s1 = src + (long long)d.L.i_src[o] * d.g.ms + kx;
-    const cplx<T>* s2 = src + (long long)(d.L.i_src2[o] < 0 ? d.L.i_src[o] : d.L.i_src2[o]) * d.g.ms + kx;
-    const bool col = kx <= K;
-    cplx<T> x[8];
-    int kyv[8];
-#pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      const int n = j + m * G;
-      kyv[m] = n <= K ? n : n - N;
-      x[m] = mk<T>(0, 0);
-      if (col && (n <= K || n >= N - K)) x[m] = s1[(kyv[m] + K) * KXP];
-    }
-    // the operator is uniform over the block
-    if (op == OP_DX) {
-#pragma unroll
-      for (int m = 0; m < 8; ++m) x[m] = cik<T>(x[m], (T)kx);
-    } else if (op == OP_DY) {
-#pragma unroll
-      for (int m = 0; m < 8; ++m) x[m] = cik<T>(x[m], (T)kyv[m]);
-    } else if (op == OP_CURL) {
-      // curl: i kx v - i ky u (s1 = u, s2 = v)
-#pragma unroll
-      for (int m = 0; m < 8; ++m) {
-        const int n = j + m * G;
-        cplx<T> b = mk<T>(0, 0);
-        if (col && (n <= K || n >= N - K)) b = s2[(kyv[m] + K) * KXP];
-        x[m] = csub<T>(cik<T>(b, (T)kx), cik<T>(x[m], (T)kyv[m]));
-      }
-    }
-    cplx<T>* b0 = reinterpret_cast<cplx<T>*>(smem_raw) + (size_t)c * col_buf_stride<T>(N, C);
-    int w = 0;
-    gfft<T, +1, L, 2>(x, b0, b0 + row_stride<T>(N), w, j, 0, d.tw, GRed{red, lC});
-    cplx<T>* dst = d.mix + (long long)o * d.g.mi + kx;
-#pragma unroll
-    for (int m = 0; m < 8; ++m) dst[(j + m * G) * KXP] = x[m];
-  });
-  pdl_release();
-}
-
-// a4 (first half): column forward pass of the products, local block =
-// (product, kx tile): spectral = FFT_y(mixed)/N on the rows |ky| <= K (zero
-// for kx > K).
-template <typename T>
-__global__ void __launch_bounds__(col_max_threads<T>()) k_stage_col_fwd(const RunDesc<T>* __restrict__ runs,
-                                                       const int* __restrict__ start, int nruns) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ unsigned red[GRedWords<T>::value];  // FP64 transforms
-  const int r = find_run(start, nruns, blockIdx.x);
-  const RunDesc<T>& d = runs[r];
-  pdl_wait();  // state written by the previous kernels: only after this
-  const int lb = blockIdx.x - start[r];
-  dispatch_L<4, 11>(d.g.log2N, [&](auto Lc) {
-    constexpr int L = decltype(Lc)::value, N = 1 << L, G = N / 8;
-    const int K = d.g.K, KXP = d.g.KXP;
-    const int lC = d.lC, C = 1 << lC;
-    const int ntile = KXP >> lC;
-    const int p = lb / ntile, tile = lb - p * ntile;
-    const int c = threadIdx.x & (C - 1), j = threadIdx.x >> lC;
-    const int kx = (tile << lC) + c;
-    const cplx<T>* src = d.pmix + (long long)p * d.g.mi + kx;
-    cplx<T> x[8];
-#pragma unroll
-    for (int m = 0; m < 8; ++m) x[m] = src[(j + m * G) * KXP];
-    cplx<T>* b0 = reinterpret_cast<cplx<T>*>(smem_raw) + (size_t)c * col_buf_stride<T>(N, C);
-    int w = 0;
-    gfft<T, -1, L, 2, -L>(x, b0, b0 + row_stride<T>(N), w, j, 0, d.tw, GRed{red, lC});
-    cplx<T>* dst = d.ps + (long long)p * d.g.ms + kx;
-#pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      const int k = j + m * G;
-      if (k <= K || k >= N - K) {
-        const int ky = k <= K ? k : k - N;
-        dst[(ky + K) * KXP] = kx <= K ? x[m] : mk<T>(0, 0);
-      }
-    }
-  });
-  pdl_release();
-}
-
-// ---------------------------------------------------------------------------
-// Column forward pass of the large grids (FP32, N = 2^L >= 1024, tiles of
-// C = 4 columns: C N/8 = 512 or 1024 threads, two or one blocks per SM).
-// With one or two blocks per SM the loads of a tile and the butterflies of
-// the previous one cannot overlap across blocks, so this pass is
-// persistent: block b takes the launch's work items b, b + gridDim.x, ...
-// (an item is the local block of k_stage_col_fwd: (product, tile) of one
-// run), and while it transforms one item, the next item's mixed tile is
-// copied into shared memory with cp.async (16-byte copies, completed by the
-// group wait before the tile is read).  The arithmetic is that of
-// k_stage_col_fwd, element for element.  (The same staging for the column
-// inverse pass, whose time is set by its 16 output writes rather than its
-// reads, measured no faster and is not used.)
-// Smem: C exchange-buffer pairs (col_buf_stride), then the staged tile of
-// N rows x C complex.
-constexpr int PIPE_C = 4;
-
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
-// Copy the mixed tile of work item `item` (N rows x 4 complex, row stride
-// KXP) into the staging buffer.
-__device__ __forceinline__ void pipe_stage(float2* st, const RunDesc<float>* __restrict__ runs,
-                                           const int* __restrict__ start, int nruns, int item) {
-  const int r = find_run(start, nruns, item);
-  const RunDesc<float>& d = runs[r];
-  const int lb = item - start[r];
-  const int ntile = d.g.KXP / PIPE_C;
-  const int p = lb / ntile, tile = lb - p * ntile;
-  const float2* src = d.pmix + (long long)p * d.g.mi + tile * PIPE_C;
-  const int rows = d.g.N, KXP = d.g.KXP;
-  for (int q = threadIdx.x; q < 2 * rows; q += blockDim.x) {
-    const int row = q >> 1, half = q & 1;
-    cp_async16(st + row * PIPE_C + half * 2, src + (long long)row * KXP + half * 2);
-  }
-}
-
-template <int L>
-__global__ void __launch_bounds__(1024, 1) k_stage_col_fwd_pipe(const RunDesc<float>* __restrict__ runs,
-                                                                const int* __restrict__ start, int nruns,
-                                                                int total) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int N = 1 << L, G = N / 8, C = PIPE_C;
-  float2* xb = reinterpret_cast<float2*>(smem_raw);
-  float2* st = xb + (size_t)C * col_buf_stride<float>(N, C);
-  const int c = threadIdx.x & (C - 1), j = threadIdx.x >> 2;
-  float2* b0 = xb + (size_t)c * col_buf_stride<float>(N, C);
-  pdl_wait();  // state written by the previous kernels: only after this
-  int item = blockIdx.x;
-  if (item < total) pipe_stage(st, runs, start, nruns, item);
-  cp_async_commit();
-  int w = 0;
-  for (; item < total; item += gridDim.x) {
-    cp_async_wait_all();
-    __syncthreads();  // the staged tile is complete and the last transform's buffers are free
-    const int r = find_run(start, nruns, item);
-    const RunDesc<float>& d = runs[r];
-    const int K = d.g.K, KXP = d.g.KXP;
-    const int lb = item - start[r];
-    const int ntile = KXP / C;
-    const int p = lb / ntile, tile = lb - p * ntile;
-    const int kx = tile * C + c;
-    float2 x[8];
-#pragma unroll
-    for (int m = 0; m < 8; ++m) x[m] = st[(j + m * G) * C + c];
-    __syncthreads();  // every thread has read the staged tile
-    if (item + gridDim.x < total) pipe_stage(st, runs, start, nruns, item + gridDim.x);
-    cp_async_commit();
-    gfft<float, -1, L, 2, -L>(x, b0, b0 + row_stride<float>(N), w, j, 0, d.tw, GRed{nullptr, 2});
-    float2* dst = d.ps + (long long)p * d.g.ms + kx;
-#pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      const int k = j + m * G;
-      if (k <= K || k >= N - K) {
-        const int ky = k <= K ? k : k - N;
-        dst[(ky + K) * KXP] = kx <= K ? x[m] : mk<float>(0, 0);
-      }
-    }
-  }
-  cp_async_wait_all();
-  pdl_release();
-}
-
-// Shared memory of a pipelined column forward launch.
-inline size_t col_fwd_pipe_smem(int N) {
-  return ((size_t)PIPE_C * col_buf_stride<float>(N, PIPE_C) + (size_t)N * PIPE_C) * sizeof(float2);
-}
-
-// a3: Strategy-2 gather buffer (physical u, v | h, zeta), local block =
-// (pair, row block of Bi rows, one row per group of N/8 threads).
+// a3: base planes (physical u, v, h, zeta and, Strategy 2, xi and, with PV
+// averaged, q = (f0 + zeta)/h, h = 1 + eta) of the runs whose row pass does not
+// form them itself.  Local block = (field, block of Bi row pairs, one pair per
+// group of N/8 threads); the field of h takes zeta and q too.
 template <typename T, bool WARP>
 __global__ void __launch_bounds__(256) k_stage_row_inv(const RunDesc<T>* __restrict__ runs,
                                                        const int* __restrict__ start, int nruns) {
@@ -290,324 +92,356 @@ __global__ void __launch_bounds__(256) k_stage_row_inv(const RunDesc<T>* __restr
   const int r = find_run(start, nruns, blockIdx.x);
   const RunDesc<T>& d = runs[r];
   pdl_wait();  // state written by the previous kernels: only after this
+  pdl_release();
   const int lb = blockIdx.x - start[r];
   auto body = [&](auto Lc) {
     constexpr int L = decltype(Lc)::value, N = 1 << L, G = N / 8;
     constexpr int SYNC = L <= 8 ? 0 : 1;
     const Geom& g = d.g;
     const int B = d.Bi;
-    const int nrb = N / B;
-    const int pair = lb / nrb, rb = lb - pair * nrb;
+    const int nrb = max(N / 2 / B, 1);
+    const int f = lb / nrb, rb = lb - f * nrb;
     const int grp = threadIdx.x / G, j = threadIdx.x - grp * G;
-    const int y = rb * B + grp;
+    const int yp = (rb * B + grp) & (N / 2 - 1);
     constexpr int rs = N + N / 8;
     cplx<T>* buf0 = reinterpret_cast<cplx<T>*>(smem_raw) + (size_t)grp * 2 * rs;
-    cplx<T>* buf1 = buf0 + rs;
-    // pairs (u, v), (h, zeta) and, Strategy 2, (xi_x, xi_y)
-    const int ia = pair == 0 ? d.L.i_u : (pair == 1 ? d.L.i_h : d.L.i_xi[0]);
-    const int ib = pair == 0 ? d.L.i_v : (pair == 1 ? d.L.i_z : d.L.i_xi[1]);
-    const int oa = pair == 0 ? PH_U : (pair == 1 ? PH_H : PH_XX);
-    const int ob = pair == 0 ? PH_V : (pair == 1 ? PH_Z : PH_XY);
-    cplx<T> x[8];
+    cplx<T> x[8], eta[8];
     int w = 0;
-    load_pair_spectrum_ct<T, L>(x, d.mix + (long long)ia * g.mi, d.mix + (long long)ib * g.mi, (long long)y * g.KXP,
-                                j, g.K);
-    gfft<T, +1, L, SYNC>(x, buf0, buf1, w, j, grp, d.tw, GRed{red, 0});
-    T* pa = d.phys + (long long)oa * g.np + (long long)y * N + j;
-    T* pb = d.phys + (long long)ob * g.np + (long long)y * N + j;
+    const bool hz = f == 2;
+#pragma unroll 1
+    for (int part = 0; part < (hz ? 2 : 1); ++part) {
+      const int src = f == 0 ? d.L.i_u : (f == 1 ? d.L.i_v : (hz ? (part ? d.L.i_z : d.L.i_h) : d.L.i_xi[f - 3]));
+      const int dst = f < 2 ? f : (hz ? (part ? PH_Z : PH_H) : f - 3 + PH_XX);
+      load_rows_ct<T, L>(x, d.mix + (long long)src * g.mi + (long long)yp * 2 * g.KXP, j, g.K);
+      gfft<T, -1, L, SYNC>(x, buf0, buf0 + rs, w, j, grp, d.tw, GRed{red, 0, 0, 0});
+      // planes [y][x]; interleaved, the four base fields as [y][x][4] and the
+      // two components of xi as [y][x][2]
+      const int es = !d.gath ? 1 : (dst < 4 ? 4 : 2);
+      T* p = d.phys + (long long)(es == 1 ? dst : (es == 4 ? 0 : PH_XX)) * g.np +
+             (es == 1 ? 0 : (es == 4 ? dst : dst - PH_XX)) + ((long long)yp * 2 * N + j) * es;
 #pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      pa[m * G] = x[m].x;
-      pb[m * G] = x[m].y;
+      for (int m = 0; m < 8; ++m) {
+        p[m * G * es] = x[m].y;
+        p[(N + m * G) * es] = x[m].x;
+      }
+      if (part == 0) {
+#pragma unroll
+        for (int m = 0; m < 8; ++m) eta[m] = x[m];
+      }
+    }
+    if (hz && d.L.has_q) {
+      T* p = d.phys + (long long)PH_Q * g.np + (long long)yp * 2 * N + j;
+#pragma unroll
+      for (int m = 0; m < 8; ++m) {
+        p[m * G] = (d.cf0 + x[m].y) / ((T)1 + eta[m].y);
+        p[N + m * G] = (d.cf0 + x[m].x) / ((T)1 + eta[m].x);
+      }
     }
   };
   if constexpr (WARP) dispatch_L<4, 8>(d.g.log2N, body);
   else dispatch_L<4, 11>(d.g.log2N, body);
-  pdl_release();
-}
-
-// q = (f0 + zeta)/h, h = 1 + eta, into the gather buffer (Strategy 2 with PV
-// averaged).
-template <typename T>
-__global__ void __launch_bounds__(256) k_stage_phys_q(const RunDesc<T>* __restrict__ runs,
-                                                      const int* __restrict__ start, int nruns) {
-  const int r = find_run(start, nruns, blockIdx.x);
-  const RunDesc<T>& d = runs[r];
-  pdl_wait();  // state written by the previous kernels: only after this
-  const long long i = (long long)(blockIdx.x - start[r]) * blockDim.x + threadIdx.x;
-  const long long np = d.g.np;
-  if (i < np) d.phys[PH_Q * np + i] = (d.cf0 + d.phys[PH_Z * np + i]) / ((T)1 + d.phys[PH_H * np + i]);
-  pdl_release();
 }
 
 // ---------------------------------------------------------------------------
-// a2: row pass with products.  Local block = (pair group, row block): Bp rows
-// and product pairs [pg*ppb, (pg+1)*ppb), with Wp groups of G = N/8 threads
-// per row.  Every transform stays in the registers of its group (gfft):
-// a row's physical values live at the thread's own positions x = j + m G,
-// where the products are formed and the forward transform of each product
-// pair starts.  First the row's base fields (u, v, h, zeta; Strategy 2: xi),
-// transformed by the row inverse pass, are read into the row's U, the loads
-// shared out over the row's groups; then the groups take the block's product
-// pairs in turn.  Wp > 1 only when a group is a whole
-// number of warps (N >= 256), so groups that do different numbers of
-// transforms never share a warp barrier.
-// Products are formed in the registers that feed the forward transform of
-// their pair: a pair holds at most one product that needs a transform or a
-// gather of its own ("heavy", placed first) unless Layout.heavy2 says
-// otherwise, so the first product overwrites its gradient pair element by
-// element and the second is formed from the base fields beside it.
-// Smem: per row U (u, v, h, zeta and, Strategy 2, xi_x, xi_y: N reals each);
-// per group two exchange buffers of row_stride(N) complex and
-// row_prod_group_rows(L) rows of N reals: Strategy 2, the first product's
-// values gathered at x + xi; with heavy2, the first product's values while
-// the second is transformed and (Strategy 2) the second product's gathered
-// values.
+// a2: row pass with products, on pairs of rows: a complex transform carries
+// row 2y as its real and row 2y + 1 as its imaginary part, so that one 16-byte
+// (FP32) access of the row-interleaved mixed layout feeds both, and products
+// are formed for the two rows at once.  (Pairing two fields of one row, as an
+// earlier form did, moved 8 bytes per access and tied products together.)
+//
+// Local block = (product chunk, block of Bp row pairs): Wp groups of G = N/8
+// threads per pair share out the chunk's ppb products, the costly ones first.
+// `fused` runs (Strategy 1, except on the largest grids): the groups first
+// transform the pair's base fields u, v, h, zeta (those the chunk needs) into
+// shared memory.  The others read base values from the planes that the row
+// inverse pass wrote; Strategy 2 gathers from them too: `gath` runs (where the
+// arrays fit) once for all products, into shared memory, from interleaved
+// planes (each product gathering for itself from separate planes took 34.7 us
+// at 512^2 with five means, this 26.7 us).  Every transform stays in the
+// registers of its group: an advection product takes the inverse transforms
+// of d_x G and d_y G and, from the same positions, the forward transform of
+// u d_x G + v d_y G; one transform instance serves both directions (the
+// inverse as a forward transform of swapped parts), which keeps the code
+// within the instruction caches.
+// Wp > 1 only when a group is a whole number of warps (N >= 256), so groups
+// that do different numbers of transforms never share a warp barrier.
+// Smem: per pair row_prod_planes() arrays of N complex (fused: the base
+// fields; gath: these, xi and the fields at x + xi); per group two
+// exchange buffers of row_stride(N) complex.
 
-// Threads per row-pass block at most (two blocks per SM: up to 85 registers
-// in FP32, 128 in FP64).
-template <typename T> constexpr int row_prod_max_threads() { return sizeof(T) == 4 ? 384 : 256; }
+// Threads per row-pass block at most: three groups at 2048^2 (FP32, 85
+// registers), 256 in FP64.
+template <typename T> constexpr int row_prod_max_threads() { return sizeof(T) == 4 ? 768 : 256; }
+
+// Arrays of a row pair in shared memory.
+__host__ __device__ __forceinline__ int row_prod_planes(int fused, int gath, int has_q) {
+  return fused ? 4 : (gath ? 10 + (has_q ? 1 : 0) : 0);
+}
 
 __device__ __forceinline__ bool product_heavy(int k) { return k == PK_ADV || k == PK_XI || k == PK_GBAR; }
 
-// Rows of N reals per group of the row pass besides its exchange buffers.
-__host__ __device__ __forceinline__ int row_prod_group_rows(const Layout& L) {
-  return (L.strategy == 2 ? 1 : 0) + (L.heavy2 ? (L.strategy == 2 ? 2 : 1) : 0);
-}
-
 template <typename T, bool WARP>
-__global__ void __launch_bounds__(row_prod_max_threads<T>(), 2) k_stage_row_prod(const RunDesc<T>* __restrict__ runs,
-                                                                                const int* __restrict__ start,
-                                                                                int nruns, int stage) {
+__global__ void __launch_bounds__(row_prod_max_threads<T>(), sizeof(T) == 4 ? 1 : 2)
+    k_stage_row_prod(const RunDesc<T>* __restrict__ runs, const int* __restrict__ start, int nruns, int stage) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned red[GRedWords<T>::value];  // FP64 transforms
   const int r = find_run(start, nruns, blockIdx.x);
   LM_STAGE_DESC(T);  // field and product lookups from shared memory
   pdl_wait();  // state written by the previous kernels: only after this
+  pdl_release();
   const int lb = blockIdx.x - start[r];
   auto body = [&](auto Lc) {
-  constexpr int L_ = decltype(Lc)::value, N = 1 << L_, G = N / 8;
-  constexpr int SYNC = L_ <= 8 ? 0 : 1;
-  const Geom& g = d.g;
-  const Layout& L = d.L;
-  const int B = d.Bp, W = d.Wp;
-  const int nrb = N / B;
-  const int pg = lb / nrb, rb = lb - pg * nrb;
-  const int gi = threadIdx.x / G, j = threadIdx.x - gi * G;
-  const int row = gi / W, wg = gi - row * W;
-  const int y = rb * B + row;
-  constexpr int rs = N + N / 8;
-  const bool s2 = L.strategy == 2;
-  const int nur = s2 ? 6 : 4, nug = row_prod_group_rows(L);
-  T* U = reinterpret_cast<T*>(smem_raw) + (size_t)row * nur * N;
-  T* XI = U + 4 * N;
-  cplx<T>* buf0 = reinterpret_cast<cplx<T>*>(reinterpret_cast<T*>(smem_raw) + (size_t)B * nur * N) +
-                  (size_t)gi * (2 * rs + (nug * N) / 2);
-  cplx<T>* buf1 = buf0 + rs;
-  T* S0 = reinterpret_cast<T*>(buf1 + rs);  // Strategy 2: first product's gathered values
-  T* P0 = S0 + (s2 ? N : 0);                // heavy2: first product's values
-  T* S1 = P0 + N;                           // heavy2, Strategy 2: second product's gathered values
-  const int np = L.np;
-  const int p0 = pg * d.ppb * 2;
-  const int p1 = min(np, p0 + d.ppb * 2);
-  const bool kin = L.model == 1;
-  const T adv_x = d.cadvx, adv_y = d.cadvy;
-  const T f0 = d.cf0;
-  const T s = stage_time<T>(d.ctr, stage, d.cdt, d.c.stepper);
-  const bool s0 = !(s > (T)0);
-  const T inv_s = s0 ? (T)0 : (T)1 / s;
-  // xi-first scheme: gbar steps with the updated xi at its time s + dt
-  const bool xf = L.scheme == SCHEME_XI_FIRST;
-  const T inv_sg = xf ? (T)1 / (s + d.cdt) : inv_s;
-  const T inv_dx = (T)N / (T)6.283185307179586476925286766559;
-  const cplx<T>* mix = d.mix;
-  // the gather buffer (written by the previous kernel) is read-only here:
-  // non-coherent loads that need not wait for this block's shared-memory stores
-  const T* __restrict__ phys = d.phys;
-  const long long npts = g.np;
-  const long long rowoff = (long long)y * g.KXP;
-  int w = 0;
-  cplx<T> x[8];
-
-  // the row's physical u, v, h, zeta (and, Strategy 2, xi_x, xi_y), written
-  // by the row inverse pass, into U (and XI = U + 4N), shared out over the
-  // row's groups
-  {
-    const int nplanes = s2 ? 6 : 4;
-#pragma unroll
-    for (int f = 0; f < 6; ++f) {
-      if (f < nplanes && f % W == wg) {
-        const T* __restrict__ src = phys + (long long)(f < 4 ? f : f + 1) * npts + (long long)y * N + j;
-        T v[8];
-#pragma unroll
-        for (int m = 0; m < 8; ++m) v[m] = __ldg(src + m * G);
-#pragma unroll
-        for (int m = 0; m < 8; ++m) U[f * N + m * G + j] = v[m];
-      }
-    }
-  }
-
-  // the gradient spectrum of a product, into the registers x; the first
-  // product of the group's first pair is loaded before the wait for the row's
-  // base fields
-  const int npair = (p1 - p0 + 1) >> 1;
-  auto load_grad = [&](int p) {
-    if (product_heavy(L.pk[p]))
-      load_pair_spectrum_ct<T, L_>(x, mix + (long long)L.pa[p] * g.mi, mix + (long long)L.pb[p] * g.mi, rowoff, j,
-                                   g.K);
-  };
-  if (wg < npair) load_grad(p0 + 2 * wg);
-  __syncthreads();
-
-  // Strategy 2: the values at x + xi (Eqs. xi_evol, barf_xi) that product p
-  // needs, by bilinear interpolation into dst (N reals)
-  auto gather = [&](int p, T* dst) {
-    const int kind = L.pk[p], pc = L.pc[p];
-    if (kind != PK_GBAR && (kind != PK_XI || kin)) return;
-    const T* __restrict__ src = phys + (long long)pc * npts;
-#pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      const int e = m * G + j;
-      dst[e] = bilinear<T>(src, e, y, XI[e], XI[N + e], inv_dx, N);
-    }
-  };
-
-  // product p at the thread's positions into the real (slot 0) or imaginary
-  // (slot 1) parts of x; a heavy product reads its gradient pair from x at
-  // the same position first, and (Strategy 2) its gathered values from sv
-  auto form = [&](int p, int slot, const T* sv) {
-    const int kind = L.pk[p], pc = L.pc[p];
-    auto put = [&](int m, T v) {
-      if (slot) x[m].y = v;
-      else x[m].x = v;
+    constexpr int L_ = decltype(Lc)::value, N = 1 << L_, G = N / 8;
+    constexpr int SYNC = L_ <= 8 ? 0 : 1;
+    constexpr int rs = N + N / 8;
+    const Geom& g = d.g;
+    const Layout& L = d.L;
+    const int B = d.Bp, W = d.Wp, ppb = d.ppb;
+    const int nrb = max(N / 2 / B, 1);
+    const int pg = lb / nrb, rb = lb - pg * nrb;
+    const int gi = threadIdx.x / G, j = threadIdx.x - gi * G;
+    const int row = gi / W, wg = gi - row * W;
+    const int yp = (rb * B + row) & (N / 2 - 1);  // row pair (2 yp, 2 yp + 1)
+    const bool fused = d.fused != 0, gath = d.gath != 0, kin = L.model == 1;
+    const int nu = row_prod_planes(d.fused, d.gath, L.has_q);
+    cplx<T>* U = reinterpret_cast<cplx<T>*>(smem_raw) + (size_t)row * nu * N + j;
+    cplx<T>* buf0 = reinterpret_cast<cplx<T>*>(smem_raw) + (size_t)B * nu * N + (size_t)gi * 2 * rs;
+    cplx<T>* buf1 = buf0 + rs;
+    const int p0 = pg * ppb, p1 = min(L.np, p0 + ppb);
+    const T adv_x = d.cadvx, adv_y = d.cadvy, f0 = d.cf0;
+    const T s = stage_time<T>(*d.ctr, stage, d.cdt, d.c.stepper);
+    const bool s0 = !(s > (T)0);
+    const T inv_s = s0 ? (T)0 : (T)1 / s;
+    // xi-first scheme: gbar steps with the updated xi at its time s + dt
+    const bool xf = L.scheme == SCHEME_XI_FIRST;
+    const T inv_sg = xf ? (T)1 / (s + d.cdt) : inv_s;
+    const T inv_dx = (T)N / (T)6.283185307179586476925286766559;
+    const cplx<T>* __restrict__ mix = d.mix + (long long)yp * 2 * g.KXP;
+    const T* __restrict__ phys = d.phys;
+    const int rowoff = yp * 2 * N + j;
+    const GRed gr = {red, 0};
+    int w = 0;
+    cplx<T> x[8], acc[8];
+    // base field f (PH_*) of both rows at the thread's position m
+    auto base = [&](int f, int m) {
+      if (fused || gath) return U[(f < 4 ? f : f - 1) * N + m * G];
+      const T* p = phys + (long long)f * g.np + rowoff + m * G;
+      return mk<T>(__ldg(p), __ldg(p + N));
     };
-    switch (kind) {
-      case PK_ZV:
+
+    if (gath) {
+      // Strategy 2: the pair's base fields and xi, and the fields at x + xi
+      // (Eqs. xi_evol, barf_xi; bilinear interpolation) into shared memory,
+      // the points shared out over the pair's threads: one 4-field access per
+      // corner serves every product
+      T* S = reinterpret_cast<T*>(U - j);
+      const T* Q = phys + (long long)PH_Q * g.np;
+      for (int e = wg * G + j; e < 2 * N; e += W * G) {
+        const int rr = e >= N ? 1 : 0, xcol = e - rr * N, y = 2 * yp + rr;
+        const int o = y * N + xcol;
+        T b[4], xi[2], f[5];
+        ld_quad(phys + 4 * (long long)o, b);
+        const cplx<T> xv = __ldg(reinterpret_cast<const cplx<T>*>(phys + (long long)PH_XX * g.np) + o);
+        xi[0] = xv.x;
+        xi[1] = xv.y;
+        const Bilin<T> bl(xcol, y, xv.x, xv.y, inv_dx, N);
 #pragma unroll
-        for (int m = 0; m < 8; ++m) put(m, U[3 * N + m * G + j] * U[N + m * G + j]);
-        break;
-      case PK_ZU:
+        for (int q = 0; q < 4; ++q) f[q] = (T)0;
+        T c[4];
+        ld_quad(phys + 4 * (long long)bl.o00, c);
 #pragma unroll
-        for (int m = 0; m < 8; ++m) put(m, U[3 * N + m * G + j] * U[m * G + j]);
-        break;
-      case PK_KE:
+        for (int q = 0; q < 4; ++q) f[q] = bl.w00 * c[q];
+        ld_quad(phys + 4 * (long long)bl.o01, c);
 #pragma unroll
-        for (int m = 0; m < 8; ++m) {
-          const T u = U[m * G + j], v = U[N + m * G + j];
-          put(m, (T)0.5 * (u * u + v * v));
+        for (int q = 0; q < 4; ++q) f[q] += bl.w01 * c[q];
+        ld_quad(phys + 4 * (long long)bl.o10, c);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) f[q] += bl.w10 * c[q];
+        ld_quad(phys + 4 * (long long)bl.o11, c);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) f[q] += bl.w11 * c[q];
+        T* dst = S + 2 * xcol + rr;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          dst[q * 2 * N] = b[q];
+          dst[(6 + q) * 2 * N] = f[q];
         }
-        break;
-      // depth h = 1 + eta; the state and the row buffers hold eta
-      case PK_HU:
-#pragma unroll
-        for (int m = 0; m < 8; ++m) {
-          const T u = U[m * G + j];
-          put(m, u + U[2 * N + m * G + j] * u);
+        dst[4 * 2 * N] = xi[0];
+        dst[5 * 2 * N] = xi[1];
+        if (L.has_q)
+          dst[10 * 2 * N] = bl.w00 * __ldg(Q + bl.o00) + bl.w01 * __ldg(Q + bl.o01) + bl.w10 * __ldg(Q + bl.o10) +
+                            bl.w11 * __ldg(Q + bl.o11);
+      }
+      __syncthreads();
+    }
+
+    // a group's transforms, one loop iteration each: the base fields of the
+    // pair (fused; group wg takes fields wg, wg + W, ...), then for each
+    // of its products the inverse transforms of two gradients (advection and
+    // Strategy-2 products) and the forward transform of the product
+    int f = fused ? wg : 4;       // next base field
+    int p = p0 + wg, sub = 0;     // next product and its part
+    bool basing = true;
+    while (true) {
+      if (basing && f >= 4) {
+        if (fused) __syncthreads();  // base fields complete
+        basing = false;
+      }
+      if (!basing && p >= p1) break;
+      const int kind = L.pk[min(p, p1 - 1)], pc = L.pc[min(p, p1 - 1)];
+      const bool heavy = product_heavy(kind);
+      const bool inv = basing || (heavy && sub < 2);
+      if (inv) {
+        if (basing && !(d.umask[pg] >> f & 1)) {
+          f += W;
+          continue;
         }
-        break;
-      case PK_HV:
+        const int src = basing ? (f == 0 ? L.i_u : (f == 1 ? L.i_v : (f == 2 ? L.i_h : L.i_z)))
+                               : (sub == 0 ? L.pa[p] : L.pb[p]);
+        load_rows_ct<T, L_>(x, mix + (long long)src * g.mi, j, g.K);
+        if (!basing && sub == 0 && kind != PK_ADV) {
+          // Strategy 2: the values at x + xi (Eqs. xi_evol, barf_xi), by
+          // bilinear interpolation, while the gradient rows arrive
+          const bool cst = kind == PK_XI && kin;
+          const T cv = pc == 0 ? adv_x : adv_y;
+          const T* __restrict__ gp = phys + (long long)pc * g.np;
 #pragma unroll
-        for (int m = 0; m < 8; ++m) {
-          const T v = U[N + m * G + j];
-          put(m, v + U[2 * N + m * G + j] * v);
+          for (int m = 0; m < 8; ++m) {
+            acc[m] = mk<T>(cv, cv);
+            if (!cst && gath) {
+              acc[m] = U[(6 + pc) * N + m * G];
+            } else if (!cst) {
+              const cplx<T> xx = base(PH_XX, m), xy = base(PH_XY, m);
+              const int e = m * G + j;
+              acc[m] = mk<T>(bilinear<T>(gp, e, 2 * yp, xx.x, xy.x, inv_dx, N),
+                             bilinear<T>(gp, e, 2 * yp + 1, xx.y, xy.y, inv_dx, N));
+            }
+          }
         }
-        break;
-      case PK_Q:
+      } else if (heavy) {
 #pragma unroll
-        for (int m = 0; m < 8; ++m) put(m, (f0 + U[3 * N + m * G + j]) / ((T)1 + U[2 * N + m * G + j]));
-        break;
-      case PK_ADV:
-        // u.grad G (Eq. gtilde-evol) or u.grad D
+        for (int m = 0; m < 8; ++m) x[m] = acc[m];
+      } else {
+        // products of the base fields alone
+        const int fa = kind == PK_ZV || kind == PK_ZU || kind == PK_Q ? PH_Z : (kind == PK_HU || kind == PK_HV ? PH_H : PH_U);
+        const int fb = kind == PK_ZU || kind == PK_HU ? PH_U : (kind == PK_Q ? PH_H : PH_V);
+        const bool ke = kind == PK_KE, hu = kind == PK_HU || kind == PK_HV;
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
-          const T ua = kin ? adv_x : U[m * G + j], va = kin ? adv_y : U[N + m * G + j];
-          put(m, ua * x[m].x + va * x[m].y);
+          const cplx<T> a = base(fa, m), b = base(fb, m);
+          if (ke) x[m] = mk<T>((T)0.5 * (a.x * a.x + b.x * b.x), (T)0.5 * (a.y * a.y + b.y * b.y));
+          else if (hu) x[m] = mk<T>(b.x + a.x * b.x, b.y + a.y * b.y);  // depth h = 1 + eta
+          else x[m] = mk<T>(a.x * b.x, a.y * b.y);
         }
-        break;
-      default: {
-        // Strategy 2, Eqs. (xi_evol), (barf_xi): w = xi/s, limit u/2 at s = 0
+        if (kind == PK_Q) {
 #pragma unroll
-        for (int m = 0; m < 8; ++m) {
-          const int e = m * G + j;
-          const T xx = XI[e], xy = XI[N + e];
-          const T ua = kin ? adv_x : U[e], va = kin ? adv_y : U[N + e];
+          for (int m = 0; m < 8; ++m) {
+            const cplx<T> z = base(PH_Z, m), h = base(PH_H, m);
+            x[m] = mk<T>((f0 + z.x) / ((T)1 + h.x), (f0 + z.y) / ((T)1 + h.y));
+          }
+        }
+      }
+      gfft<T, -1, L_, SYNC>(x, buf0, buf1, w, j, gi, d.tw, gr, inv ? 0 : -L_ - 1);
+      if (basing) {
+#pragma unroll
+        for (int m = 0; m < 8; ++m) U[f * N + m * G] = mk<T>(x[m].y, x[m].x);
+        f += W;
+      } else if (!inv) {
+        store_rows_ct<T, L_, SYNC>(x, buf0, buf1, w, d.pmix + (long long)p * g.mi + (long long)yp * 2 * g.KXP, j, gi,
+                                   g.K, g.KXP);
+        p += W;
+        sub = 0;
+      } else {
+        const bool second = sub == 1;
+        ++sub;
+        if (kind == PK_ADV) {
+          // u.grad G (Eq. gtilde-evol) or u.grad D
+          const T av = second ? adv_y : adv_x;
+#pragma unroll
+          for (int m = 0; m < 8; ++m) {
+            const cplx<T> ua = kin ? mk<T>(av, av) : base(second ? PH_V : PH_U, m);
+            const cplx<T> a = second ? acc[m] : mk<T>(0, 0);
+            acc[m] = mk<T>(fma(ua.x, x[m].y, a.x), fma(ua.y, x[m].x, a.y));
+          }
+        } else {
+          // Strategy 2, Eqs. (xi_evol), (barf_xi): w = xi/s, limit u/2 at s = 0
           const bool sz = s0 && !(xf && kind == PK_GBAR);
           const T is = kind == PK_GBAR ? inv_sg : inv_s;
-          const T wx = sz ? (T)0.5 * ua : xx * is;
-          const T wy = sz ? (T)0.5 * va : xy * is;
-          const T wgrad = wx * x[m].x + wy * x[m].y;
-          const T fi = (kind == PK_XI && kin) ? (pc == 0 ? adv_x : adv_y) : sv[e];
-          put(m, kind == PK_XI ? fi - (pc == 0 ? wx : wy) - wgrad : fi - wgrad);
-        }
-        break;
-      }
-    }
-  };
-
-  // product pairs, shared out over the row's groups
-  for (int q = wg; q < npair; q += W) {
-    const int pa = p0 + 2 * q;
-    const int npq = min(2, p1 - pa);
-    const bool h2 = npq == 2 && product_heavy(L.pk[pa + 1]);
-    if (q != wg) load_grad(pa);
-    // the next pair of this group: its gradient rows into L2 while this one
-    // runs (at 1024^2 and above the mixed fields do not stay in L2 between
-    // the column pass and the row pass)
-    if (q + W < npair) {
-      const int pn = p0 + 2 * (q + W);
-      if (product_heavy(L.pk[pn])) {
-        const char* a = reinterpret_cast<const char*>(mix + (long long)L.pa[pn] * g.mi + rowoff);
-        const char* b = reinterpret_cast<const char*>(mix + (long long)L.pb[pn] * g.mi + rowoff);
-        const int bytes = (g.K + 1) * (int)sizeof(cplx<T>);
-        for (int off = j * 128; off < bytes; off += G * 128) {
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(a + off));
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(b + off));
+          const T av = second ? adv_y : adv_x;
+          const int comp = second ? 1 : 0;
+#pragma unroll
+          for (int m = 0; m < 8; ++m) {
+            cplx<T> wv;
+            if (sz) {
+              const cplx<T> ua = kin ? mk<T>(av, av) : base(PH_U + comp, m);
+              wv = mk<T>((T)0.5 * ua.x, (T)0.5 * ua.y);
+            } else {
+              const cplx<T> xi = base(PH_XX + comp, m);
+              wv = mk<T>(xi.x * is, xi.y * is);
+            }
+            cplx<T> a = acc[m];
+            a.x -= wv.x * x[m].y;
+            a.y -= wv.y * x[m].x;
+            if (kind == PK_XI && pc == comp) {
+              a.x -= wv.x;
+              a.y -= wv.y;
+            }
+            acc[m] = a;
+          }
         }
       }
     }
-    if (s2) {
-      // both products' gathers, issued together ahead of the transforms
-      gather(pa, S0);
-      if (h2) gather(pa + 1, S1);
-    }
-    if (product_heavy(L.pk[pa])) gfft<T, +1, L_, SYNC>(x, buf0, buf1, w, j, gi, d.tw, GRed{red, 0});
-    form(pa, 0, S0);
-    if (h2) {
-      // the second product needs its own transform: park the first
-#pragma unroll
-      for (int m = 0; m < 8; ++m) P0[m * G + j] = x[m].x;
-      load_grad(pa + 1);
-      gfft<T, +1, L_, SYNC>(x, buf0, buf1, w, j, gi, d.tw, GRed{red, 0});
-      form(pa + 1, 1, S1);
-#pragma unroll
-      for (int m = 0; m < 8; ++m) x[m].x = P0[m * G + j];
-    } else if (npq == 2) {
-      form(pa + 1, 1, nullptr);
-    } else {
-#pragma unroll
-      for (int m = 0; m < 8; ++m) x[m].y = (T)0;
-    }
-    gfft<T, -1, L_, SYNC, -L_ - 1>(x, buf0, buf1, w, j, gi, d.tw, GRed{red, 0});
-    store_pair_spectrum_ct<T, L_, SYNC>(x, buf0, buf1, w, d.pmix + (long long)pa * g.mi,
-                                        npq == 2 ? d.pmix + (long long)(pa + 1) * g.mi : nullptr, rowoff, j, gi,
-                                        g.K, g.KXP);
-  }
   };
   if constexpr (WARP) dispatch_L<4, 8>(d.g.log2N, body);
   else dispatch_L<4, 11>(d.g.log2N, body);
-  pdl_release();
 }
 
 // ---------------------------------------------------------------------------
-// a4 (second half): right-hand sides and RK4 with integrating factor, one
-// thread per (evolved field, two modes); local block = (field, mode block).
-//   stage 0: a = N(y_n)      acc = E^2 a            y1 = E (y_n + dt/2 a)
-//   stage 1: b = N(y1)       acc += 2 E b           y2 = E y_n + dt/2 b
-//   stage 2: c = N(y2)       acc += 2 E c           y3 = E^2 y_n + dt E c
-//   stage 3: d = N(y3)       y_{n+1} = E^2 y_n + dt/6 (acc + d)
-// with E = exp(-nu |k|^2p dt/2) (Heun and forward Euler: see update_mode).
-// Stage inputs alternate between two buffers
-// (a thread reads other fields' stage inputs at its mode).
+// a4 and the next stage's a1 in one kernel: forward y-FFT and 2/3 mask of the
+// products, right-hand sides, the stepper's combination with the integrating
+// factor, and the inverse y-FFTs of the new stage values.  Everything between
+// the two transforms is pointwise in (ky, kx), and a forward transform leaves
+// position k of a column with the thread that feeds position k to an inverse
+// one, so the new value of a field goes from the product's transform to its
+// derivatives' transforms through registers.
+//
+// Separate kernels (forward pass, update, inverse pass) moved 96 spectral and
+// 27 mixed fields per stage of a Strategy-1 run with four means (products and
+// stage values written and read back, each once per reader); this one moves
+// 45 and 27, in one launch instead of three.
+//
+// Local block = (task, kx tile of C = 2^lC columns); thread t works on column
+// c = t mod C and rows n = j + m N/8 (j = t div C, m < 8).  A warp's accesses
+// to the spectral fields are contiguous (tile-blocked layout), those to the
+// mixed fields runs of C columns x 2 rows.  (With both layouts [row][kx], runs
+// of C columns, the kernel was bound by the number of 32-byte requests: 309 us
+// at 2048^2 with 4 columns, 608 us with 2.)  A task owns one or two evolved fields: CT_UV (u and v, with
+// the products zeta v, zeta u, |u|^2/2; their mixed fields and zeta's), CT_H,
+// CT_E2 (the two-dimensional Euler vorticity and its slaved velocity), CT_KIN
+// (the kinematic model's u, v, h), CT_G (a mean field and its Eulerian
+// accumulator), CT_P (a displacement component).  Only u, v and h are read by
+// other tasks (linear terms, f_hat), so only their stage values go to memory;
+// they alternate between two buffers, because the other tasks of the launch
+// read the previous ones.  stage = -1 only transforms: the mixed fields of the
+// state y, before the first step of a replay; with STAGE_FINAL set the mixed
+// fields are left out, after its last.
+//   RK4   stage 0: a = N(y_n)      acc = E^2 a            y1 = E (y_n + dt/2 a)
+//         stage 1: b = N(y1)       acc += 2 E b           y2 = E y_n + dt/2 b
+//         stage 2: c = N(y2)       acc += 2 E c           y3 = E^2 y_n + dt E c
+//         stage 3: d = N(y3)       y_{n+1} = E^2 y_n + dt/6 (acc + d)
+//   Heun  stage 0: acc = E^2 a, y1 = E^2 (y_n + dt a);  stage 1: y_{n+1} =
+//         E^2 y_n + dt/2 (acc + b)
+//   Euler stage 0: acc = dt E^2 a;  stage 1 (no products): y_{n+1} = E^2 y_n
+//         + acc (two launches: the first reads other fields' y_n)
+// with E = exp(-nu |k|^2p dt/2).
+// The code is kept small (one transform instance for both directions, the
+// inverse as a forward transform of swapped parts; the update in a rolled
+// loop): a block runs each instruction only a few times, and with the
+// transforms and updates of every task unrolled the kernel waited for
+// instruction fetches (2048^2: 528 us).
+// Smem: C exchange-buffer pairs (col_buf_stride) per half, then 6 complex per
+// thread of a half (its parked values: the positions m = 3, 4 of a column, n in
+// [3N/8, 5N/8), lie outside the 2/3 box).
 __device__ __forceinline__ float kahan_add_rn(float sum, float add, float& comp) {
   const float yk = __fsub_rn(add, comp);
   const float t = __fadd_rn(sum, yk);
@@ -621,216 +455,534 @@ __device__ __forceinline__ double kahan_add_rn(double sum, double add, double& c
   return t;
 }
 
-// Two-dimensional Euler model: the velocity of the vorticity zeta in buffer b
-// at mode m, through the streamfunction (lap psi = zeta, u = -d_y psi,
+// Two-dimensional Euler model: the velocity of the vorticity zeta at mode m of
+// buffer b, through the streamfunction (lap psi = zeta, u = -d_y psi,
 // v = d_x psi): u_hat = i ky zeta_hat/|k|^2, v_hat = -i kx zeta_hat/|k|^2, zero
 // at k = 0; written beside zeta.
 template <typename T>
-__device__ __forceinline__ void slave_velocity(cplx<T>* b, const Layout& L, long long ms, long long m, T kxf, T kyf) {
-  const cplx<T> z = b[L.f_h * ms + m];
+__device__ __forceinline__ void slave_velocity(cplx<T>* b, const Layout& L, int ms, int m, T kxf, T kyf, cplx<T> z) {
   const T k2 = kxf * kxf + kyf * kyf;
   const T inv = k2 > (T)0 ? (T)1 / k2 : (T)0;
-  b[L.f_u * ms + m] = mk<T>(-kyf * z.y * inv, kyf * z.x * inv);
-  b[L.f_v * ms + m] = mk<T>(kxf * z.y * inv, -kxf * z.x * inv);
+  gst(b + L.f_u * ms + m, mk<T>(-kyf * z.y * inv, kyf * z.x * inv));
+  gst(b + L.f_v * ms + m, mk<T>(kxf * z.y * inv, -kxf * z.x * inv));
 }
 
-// y_{n+1} = E^2 y_n + inc at element o of field f, with the factor E^2 given
-// as the unevaluated sum e2h + e2l (the part e2l y_n joins the increment);
-// compensated in FP32 for the fields marked so.
+// y_{n+1} = E^2 y_n + inc, with the factor E^2 given as the unevaluated sum
+// e2h + e2l (the part e2l y_n joins the increment); compensated if `kahan`
+// (cc: the compensation term, replaced).
 template <typename T>
-__device__ __forceinline__ void commit_mode(const RunDesc<T>& d, int f, long long o, T e2h, T e2l, cplx<T> inc) {
-  const cplx<T> yn = d.y[o];
+__device__ __forceinline__ cplx<T> commit_mode(bool kahan, T e2h, T e2l, cplx<T> yn, cplx<T>& cc, cplx<T> inc) {
   inc.x = fma(yn.x, e2l, inc.x);
   inc.y = fma(yn.y, e2l, inc.y);
-  if (d.comp && d.L.fkahan[f]) {
-    cplx<T> cc = d.comp[o];
+  if (kahan) {
     cc.x *= e2h;
     cc.y *= e2h;
-    cplx<T> out;
-    out.x = kahan_add_rn(yn.x * e2h, inc.x, cc.x);
-    out.y = kahan_add_rn(yn.y * e2h, inc.y, cc.y);
-    d.y[o] = out;
-    d.comp[o] = cc;
-  } else {
-    d.y[o] = mk<T>(fma(yn.x, e2h, inc.x), fma(yn.y, e2h, inc.y));
+    return mk<T>(kahan_add_rn(yn.x * e2h, inc.x, cc.x), kahan_add_rn(yn.y * e2h, inc.y, cc.y));
   }
+  return mk<T>(fma(yn.x, e2h, inc.x), fma(yn.y, e2h, inc.y));
 }
 
-// Right-hand side and RK4 update of evolved field f at mode m = kyi*KXP + kx
-// (kx <= K); prod(p) returns the spectral product p at this mode.
-template <typename T, typename PF>
-__device__ __forceinline__ void update_mode(const RunDesc<T>& d, int stage, T sd, bool even, int f, int m,
-                                            int kx, int kyi, PF prod) {
-  const Geom& g = d.g;
-  const Layout& L = d.L;
-  const int st = d.c.stepper;
-  const int msi = (int)g.ms;
-  const int role = L.frole[f], slot = L.fslot[f];
-  // two-dimensional Euler model: u and v follow zeta (written with it)
-  const bool e2 = L.model == 2;
-  if (e2 && (role == R_U || role == R_V)) return;
-  const int cls = L.fclass[f];
-  const T E = cls == IF_NONE ? (T)1 : d.ef[3 * cls * msi + m];
-  // E^2 = e2h + e2l for the commit of y_{n+1} (read where it is committed)
-  auto e2h = [&]() { return cls == IF_NONE ? (T)1 : d.ef[(3 * cls + 1) * msi + m]; };
-  auto e2l = [&]() { return cls == IF_NONE ? (T)0 : d.ef[(3 * cls + 2) * msi + m]; };
-  const int o = f * msi + m;
-  const T kxf = (T)kx, kyf = (T)(kyi - g.K);
-  // xi-first scheme (Strategy 2, forward Euler): xi steps by 2 dt on even
-  // steps, gbar on odd ones (integrating factor over 2 dt: E^4)
-  const bool x1 = L.scheme == SCHEME_XI_FIRST && (role == R_P || role == R_G);
-  const bool active = !x1 || ((role == R_P) == even);
-  if (!active) return;
-  if (st == 2 && stage == 1) {
-    // forward Euler, second pass: y_{n+1} = E^2 y_n + dt E^2 a, the increment
-    // from the first pass (a separate pass: the first reads other fields' y_n)
-    const T h2 = e2h(), l2 = e2l();
-    if (x1) {
-      // E^4 = (h2 + l2)^2 to the same precision (exact product of h2 by fma)
-      const T e4h = h2 * h2;
-      const T e4l = fma(h2, h2, -e4h) + (T)2 * h2 * l2;
-      commit_mode<T>(d, f, o, e4h, e4l, d.acc[o]);
-    } else {
-      commit_mode<T>(d, f, o, h2, l2, d.acc[o]);
-    }
-    if (e2 && role == R_H) slave_velocity<T>(d.y, L, g.ms, m, kxf, kyf);
-    return;
-  }
+// Integer as a T; FP64 by integer instructions (a conversion is an FP64-pipe
+// instruction), |k| < 2^20.
+__device__ __forceinline__ float to_real(int k, float) { return (float)k; }
+__device__ __forceinline__ double to_real(int k, double) {
+  const unsigned a = (unsigned)abs(k);
+  const int lz = __clz((int)a);
+  const unsigned hi = ((a << lz) >> 11) + ((unsigned)(1022 + 31 - lz) << 20);
+  return __hiloint2double(a ? (int)(hi | ((unsigned)k & 0x80000000u)) : 0, 0);
+}
+
+// The kinematic model's u, v and h when nothing is averaged (no products, so
+// no transforms): pointwise, KIN_MODES modes per block.
+constexpr int KIN_MODES = 512;
+template <typename T>
+__device__ __forceinline__ void kinematic_update(const RunDesc<T>& d, int stage, int lb) {
+  const int st = d.c.stepper, ms = (int)d.g.ms, NY = d.g.NY;
+  constexpr int CS = spec_tile<T>();
+  const bool last = stage == stage_count(st) - 1;
   const T dt = d.cdt;
   const cplx<T>* yin = stage_input(d, stage);
-  cplx<T> rhs;
-  if (role <= R_H) {
-    // shallow-water right-hand side, Eq. (sw_eqs_dimless)
-    if (e2) {
-      // vorticity of the two-dimensional Euler flow: d_t zeta = -div(u zeta)
-      rhs = csub<T>(mk<T>(0, 0), cadd<T>(cik<T>(prod(L.p_zu), kxf), cik<T>(prod(L.p_zv), kyf)));
-    } else if (L.model == 0) {
-      if (role == R_H) {
-        rhs = csub<T>(mk<T>(0, 0), cadd<T>(cik<T>(prod(L.p_hu), kxf), cik<T>(prod(L.p_hv), kyf)));
+  cplx<T>* yout = last ? d.y : (stage == 1 ? d.ysb : d.ysa);
+  for (int m = lb * KIN_MODES + threadIdx.x; m < min(ms, (lb + 1) * KIN_MODES); m += blockDim.x) {
+    const int tile = m / (NY * CS), e = m - tile * NY * CS;
+    const int kx = tile * CS + e % CS, ky = e / CS - d.g.K;
+    if (kx > d.g.K) continue;
+    const T kc = (T)kx * d.cadvx + (T)ky * d.cadvy;
+    for (int f = 0; f < 3; ++f) {
+      const int o = f * ms + m, cls = d.L.fclass[f];
+      const T* ef = d.ef + 3 * cls * ms + m;
+      const T e1 = cls == IF_NONE ? (T)1 : ef[0], ee = e1 * e1;
+      const cplx<T> rr = cik<T>(yin[o], -kc), yn = d.y[o];
+      if (last) {
+        const T ci = st == 0 ? dt / (T)6 : (st == 1 ? dt / (T)2 : (T)1);
+        const cplx<T> inc = st == 2 ? d.acc[o] : cscale<T>(cadd<T>(d.acc[o], rr), ci);
+        cplx<T> cc = mk<T>(0, 0);
+        d.y[o] = commit_mode<T>(false, cls == IF_NONE ? (T)1 : ef[ms], cls == IF_NONE ? (T)0 : ef[2 * ms], yn, cc, inc);
+      } else if (st == 2) {
+        d.acc[o] = cscale<T>(rr, dt * ee);
       } else {
-        const cplx<T> hh = yin[L.f_h * msi + m];
-        const cplx<T> Bq = cadd<T>(cscale<T>(hh, d.cc2), prod(L.p_ke));
-        if (role == R_U)
-          rhs = csub<T>(cadd<T>(cscale<T>(yin[L.f_v * msi + m], d.cf0), prod(L.p_zv)), cik<T>(Bq, kxf));
-        else
-          rhs = csub<T>(csub<T>(cscale<T>(yin[L.f_u * msi + m], -d.cf0), prod(L.p_zu)), cik<T>(Bq, kyf));
+        const T cr = stage == 0 ? ee : (T)2 * e1;
+        const T ca = st == 1 || stage == 2 ? ee : e1;
+        const T cb = st == 1 ? dt * ee : (stage == 0 ? (T)0.5 * dt * e1 : (stage == 1 ? (T)0.5 * dt : dt * e1));
+        const cplx<T> ac = stage == 0 ? mk<T>(0, 0) : d.acc[o];
+        d.acc[o] = mk<T>(fma(cr, rr.x, ac.x), fma(cr, rr.y, ac.y));
+        yout[o] = mk<T>(fma(ca, yn.x, cb * rr.x), fma(ca, yn.y, cb * rr.y));
       }
-    } else {
-      const T kc = kxf * d.cadvx + kyf * d.cadvy;
-      rhs = cik<T>(yin[f * msi + m], -kc);
-    }
-  } else if (role == R_P) {
-    const cplx<T> pp = prod(L.p_p[slot]);
-    if (L.strategy == 1) {
-      // d_t D = s u - u.grad D
-      cplx<T> ua;
-      if (L.model == 1) {
-        const bool k0 = (kx == 0 && kyi == g.K);
-        ua = mk<T>(k0 ? (slot == 0 ? d.cadvx : d.cadvy) : (T)0, 0);
-      } else {
-        ua = yin[(slot == 0 ? L.f_u : L.f_v) * msi + m];
-      }
-      rhs = csub<T>(cscale<T>(ua, (T)sd), pp);
-    } else {
-      rhs = pp;  // xi: the product holds u(x+xi) - w - w.grad xi
-    }
-  } else {
-    // f_hat of the averaged scalar at this stage
-    const int sc = L.lmf[slot];
-    cplx<T> fh;
-    if (sc == LMF_ZETA)
-      fh = e2 ? yin[L.f_h * msi + m]  // the evolved vorticity (its mean included)
-              : csub<T>(cik<T>(yin[L.f_v * msi + m], kxf), cik<T>(yin[L.f_u * msi + m], kyf));
-    else if (sc == LMF_H) fh = yin[L.f_h * msi + m];
-    else if (sc == LMF_U) fh = yin[L.f_u * msi + m];
-    else if (sc == LMF_V) fh = yin[L.f_v * msi + m];
-    else fh = prod(L.p_q);
-    if (role == R_E) {
-      rhs = fh;  // Eq. (ave)
-    } else {
-      const cplx<T> pg = prod(L.p_g[slot]);
-      // S1: f - u.grad g (Eq. gtilde-evol); S2: f(x+xi) - w.grad g
-      rhs = L.strategy == 1 ? csub<T>(fh, pg) : pg;
     }
   }
-  const cplx<T> yn = d.y[o];
-  cplx<T>* yout = stage == 1 ? d.ysb : d.ysa;
-  const bool last = stage == stage_count(st) - 1;
-  if (st == 2) {
-    // forward Euler, first pass: the increment dt E^2 a (xi-first mean
-    // fields: 2 dt E^4 a)
-    d.acc[o] = cscale<T>(rhs, x1 ? (T)2 * dt * (E * E) * (E * E) : dt * E * E);
-  } else if (!last && st != 0) {
-    // Heun, stage 0: acc = E^2 a, y1 = E^2 (y_n + dt a)
-    d.acc[o] = cscale<T>(rhs, E * E);
-    yout[o] = cscale<T>(cadd<T>(yn, cscale<T>(rhs, dt)), E * E);
-  } else if (stage == 0 && !last) {
-    d.acc[o] = cscale<T>(rhs, E * E);
-    yout[o] = cscale<T>(cadd<T>(yn, cscale<T>(rhs, (T)0.5 * dt)), E);
-  } else if (stage == 1 && !last) {
-    d.acc[o] = cadd<T>(d.acc[o], cscale<T>(rhs, (T)2 * E));
-    yout[o] = cadd<T>(cscale<T>(yn, E), cscale<T>(rhs, (T)0.5 * dt));
-  } else if (stage == 2) {
-    d.acc[o] = cadd<T>(d.acc[o], cscale<T>(rhs, (T)2 * E));
-    yout[o] = cadd<T>(cscale<T>(yn, E * E), cscale<T>(rhs, dt * E));
-  } else {
-    // final stage: y_{n+1} = E^2 y_n + inc, with inc = dt/6 (acc + d) (RK4)
-    // or dt/2 (acc + b) (Heun); its inputs are the stage buffers, not y
-    commit_mode<T>(d, f, o, e2h(), e2l(), cscale<T>(cadd<T>(d.acc[o], rhs), st == 0 ? dt / (T)6 : dt / (T)2));
-  }
-  if (e2 && role == R_H && st != 2) slave_velocity<T>(last ? d.y : yout, L, g.ms, m, kxf, kyf);
 }
 
-// Modes per block of the update kernel: 512 (two per thread: the grid of a
-// 256^2 Strategy-1 + Strategy-2 batch then fits in one wave of blocks, with
-// six resident blocks per SM in FP32, i.e. at most 40 registers) up to
-// 512^2; 2048 (eight per thread) from 1024^2, where the larger blocks
-// amortise their set-up (7% faster at 2048^2, twice slower at 256^2).
-constexpr int UPD_MODES = 512;
-__host__ __device__ __forceinline__ int update_modes(int N) { return N >= 1024 ? 2048 : UPD_MODES; }
-template <typename T> constexpr int update_min_blocks() { return sizeof(T) == 4 ? 6 : 4; }
+template <typename T> __device__ __forceinline__ cplx<T> cswap(cplx<T> a) { return mk<T>(a.y, a.x); }
 
-template <typename T>
-__global__ void __launch_bounds__(256, update_min_blocks<T>()) k_stage_update(const RunDesc<T>* __restrict__ runs,
-                                                      const int* __restrict__ start, int nruns, int stage) {
+// Column-stage kernels by the largest block: FP64 128 threads (grids up to
+// 512^2: few warps per SM, so many registers and three modes in flight; 64^2
+// 42 -> 38 us, 256^2 56 -> 50 us) and 256; FP32 256 (to 512^2), 512 (1024^2) and
+// 1024 (2048^2).
+// DUAL: a task's steps are shared out over two halves of a block, each with
+// its own exchange buffers and barrier (block barriers where a value passes
+// between them): while a launch has about one block per SM its time is the
+// longest task's chain, which this cuts from 6 transforms and 2 updates to 3
+// and 1 (CT_UV) and from 3 and 1 to 2 and 1 (CT_G).  Step of one Strategy-1
+// run, whole blocks -> halves: 64^2 FP64 0.240 -> 0.188 ms, 256^2 FP32 0.078 ->
+// 0.071 ms; at 512^2, more than a block per SM, no difference.
+constexpr int STAGE_FINAL = 256;
+template <typename T, int MAXT, bool DUAL> struct ColShape {
+  static constexpr bool f32 = sizeof(T) == 4;
+  static constexpr int LO = f32 ? (MAXT <= 256 ? 4 : (MAXT <= 512 ? 10 : 11)) : (MAXT <= 128 ? 4 : 10);
+  static constexpr int HI = DUAL ? 8 : f32 ? (MAXT <= 256 ? 9 : LO) : (MAXT <= 128 ? 9 : 11);
+  static constexpr int NB = f32 ? 2 : (MAXT <= 128 ? 3 : 1);  // modes whose loads are issued together
+  static constexpr int BLOCKS = MAXT <= 512 ? 2 : 1;
+};
+template <typename T, int MAXT, bool DUAL>
+__global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, DUAL>::BLOCKS) k_stage_col(const RunDesc<T>* __restrict__ runs,
+                                                                              const int* __restrict__ start,
+                                                                              int nruns, int stage_arg) {
+  const bool final_step = stage_arg >= 0 && (stage_arg & STAGE_FINAL);
+  const int stage = stage_arg < 0 ? stage_arg : stage_arg & ~STAGE_FINAL;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ unsigned red[GRedWords<T>::value];  // FP64 transforms
   const int r = find_run(start, nruns, blockIdx.x);
-  LM_STAGE_DESC(T);  // many field lookups per thread: read from shared memory
+  LM_STAGE_DESC(T);  // field and product lookups from shared memory
   pdl_wait();  // state written by the previous kernels: only after this
-  const Geom& g = d.g;
-  const Layout& L = d.L;
+  pdl_release();
   const int lb = blockIdx.x - start[r];
-  const int upm = update_modes(g.N);
-  const int mblocks = (int)((g.ms + upm - 1) / upm);
-  const int f = lb / mblocks;
-  const long long m0 = (long long)(lb - f * mblocks) * upm + threadIdx.x;
-  const T sd = stage_time<T>(d.ctr, stage, d.cdt, d.c.stepper);
-  const bool even = L.scheme == SCHEME_XI_FIRST ? ((*d.ctr & 1LL) == 0) : true;
-  auto modes = [&](auto Uc) {
-    constexpr int NU = decltype(Uc)::value;
-    // element offsets of a run fit in 32 bits (16 fields x 933,465 modes at
-    // 2048^2); the mode's (ky, kx) advance by 256 modes per step without a
-    // division each
-    const int msi = (int)g.ms, KXP = g.KXP;
-    int mi = (int)m0;
-    int kyi = mi / KXP, kx = mi - kyi * KXP;
-    const int dq = 256 / KXP, dr = 256 - dq * KXP;
+  if (d.L.np == 0) {  // no transforms
+    if (stage >= 0) kinematic_update<T>(d, stage, lb);
+  }
+  else dispatch_L<ColShape<T, MAXT, DUAL>::LO, ColShape<T, MAXT, DUAL>::HI>(d.g.log2N, [&](auto Lc) {
+    constexpr int L = decltype(Lc)::value, N = 1 << L, G = N / 8;
+    constexpr int NB = ColShape<T, MAXT, DUAL>::NB;
+    const Layout& Y = d.L;
+    const int K = d.g.K, KXP = d.g.KXP, ms = (int)d.g.ms;
+    const int lC = d.lC, C = 1 << lC;
+    const int ntile = KXP >> lC;
+    const int task = lb / ntile, tile = lb - task * ntile;
+    const ColTask& ct = Y.ct[task];
+    const int kind = ct.kind, slot = ct.slot;
+    constexpr int SYNC = DUAL ? 3 : 2;
+    const int ps = DUAL ? blockDim.x >> 1 : blockDim.x;  // threads per half
+    const int lane = DUAL && threadIdx.x >= ps ? 1 : 0, tid = threadIdx.x - lane * ps;
+    const int c = tid & (C - 1), j = tid >> lC;
+    const int st = d.c.stepper;
+    const bool begin = stage < 0;
+    const bool last = stage == stage_count(st) - 1;  // commits y_{n+1}
+    const bool euler0 = st == 2 && stage == 0;       // forward Euler's first pass
+    const bool commit = st == 2 && stage == 1;       // and its second: no products
+    const long long nstep = *d.ctr;
+    auto sd = [&]() { return stage_time<T>(nstep, stage, d.cdt, st); };
+    const int kx = (tile << lC) + c;
+    const T kxf = to_real(kx, (T)0);
+    const bool col = kx <= K;
+    const bool e2 = Y.model == 2, kin = Y.model == 1;
+    const int xs = C * col_buf_stride<T>(N, C);  // exchange buffers of a half
+    cplx<T>* b0 = reinterpret_cast<cplx<T>*>(smem_raw) + lane * xs + c * col_buf_stride<T>(N, C);
+    cplx<T>* park = reinterpret_cast<cplx<T>*>(smem_raw) + (DUAL ? 2 : 1) * xs + tid;
+    const GRed gr = {red + lane * (GRED_WORDS / 4), lC, tid, ps};
+    int w = 0;
+    cplx<T> x[8];
+    // the column's first mode, the row stride of its modes, and its elements
+    // of a mixed field (row n = j + m G at mx + m * mG)
+    constexpr int CS = spec_tile<T>();
+    const int m00 = (kx / CS) * (d.g.NY * CS) + kx % CS;
+    const int mx = (j >> 1) * 2 * KXP + 2 * kx + (j & 1), mG = G * KXP;
+    // wavenumber of the thread's position s = 0..5 (m = s or s + 2), and
+    // whether it lies in the box
+    auto kyof = [&](int s) { return j + s * G - (s >= 3 ? 6 * G : 0); };
+    auto inband = [&](int s) { return col && kyof(s) <= K && kyof(s) >= -K; };
+    const cplx<T>* yin = stage_input(d, stage);
+    cplx<T>* yout = last || begin ? d.y : (stage == 1 ? d.ysb : d.ysa);
+    auto store_park = [&]() {
 #pragma unroll
-    for (int u = 0; u < NU; ++u) {
-      if (mi < msi && kx <= g.K) {
-        const int mm = mi;
-        update_mode<T>(d, stage, sd, even, f, mm, kx, kyi, [&](int p) { return d.ps[p * msi + mm]; });
+      for (int i = 0; i < 3; ++i) {
+        park[i * ps] = x[i];
+        park[(3 + i) * ps] = x[5 + i];
       }
-      mi += 256;
-      kx += dr;
-      kyi += dq;
-      if (kx >= KXP) {
-        kx -= KXP;
-        ++kyi;
+    };
+
+    // The task's update of field f (and, fe >= 0, of the Eulerian accumulator
+    // fe) at the thread's modes: x, the transformed product (times 1/N), is
+    // replaced by the new values.  fa, fb: stage inputs read with it (-1:
+    // none).  Loads are unconditional over the thread's positions, from
+    // clamped addresses (a load under a per-lane condition waits where the
+    // lanes rejoin), and issued together for NB modes.  Before the commit the
+    // combinations of all steppers and stages are acc' = [acc +] cr rhs,
+    // y' = ca y_n + cb rhs.
+    auto update = [&](int f, int fe, int fa, int fb) {
+      const int role = Y.frole[f];
+      const int cls = Y.fclass[f];
+      const bool damped = cls != IF_NONE;
+      const T* ef = d.ef + (damped ? 3 * cls * ms : 0);
+      // xi-first scheme (Strategy 2, forward Euler): xi steps by 2 dt on even
+      // steps, gbar on odd ones (integrating factor over 2 dt: E^4)
+      const bool x1 = Y.scheme == SCHEME_XI_FIRST && (role == R_P || role == R_G);
+      const bool act = !x1 || ((role == R_P) == ((nstep & 1) == 0));
+      const bool add = st == 0 && stage > 0;
+      const bool kah = d.comp && Y.fkahan[f];
+      const bool keep = role <= R_H && !euler0;  // stage values that other tasks read
+      cplx<T>* const yf = d.y + f * ms;
+      cplx<T>* const af = d.acc + f * ms;
+      cplx<T>* const ye = d.y + max(fe, 0) * ms;
+      cplx<T>* const ae = d.acc + max(fe, 0) * ms;
+      const cplx<T>* const qa = yin + max(fa, 0) * ms;
+      const cplx<T>* const qb = yin + max(fb, 0) * ms;
+      const T dt = d.cdt;
+      const cplx<T> z = mk<T>(0, 0);
+      // right-hand sides rr of the NB modes from s0 on (wavenumbers ky) from
+      // the transformed products tv and the stage inputs pa, pb; fh: the
+      // averaged scalar's f_hat (CT_G).  Branches are taken once for the NB
+      // modes, whose arithmetic then overlaps.
+      auto rhs = [&](int s0, const T* ky, const cplx<T>* tv, const cplx<T>* pa, const cplx<T>* pb, cplx<T>* rr,
+                     cplx<T>* fh) {
+        if (kind == CT_G) {
+          // S1: f - u.grad g (Eq. gtilde-evol), S2: f(x+xi) - w.grad g
+          const bool s1 = Y.strategy == 1;
+          if (fb >= 0) {
+#pragma unroll
+            for (int i = 0; i < NB; ++i) fh[i] = csub<T>(cik<T>(pa[i], kxf), cik<T>(pb[i], ky[i]));
+          } else {
+            const bool pk = fa < 0;
+#pragma unroll
+            for (int i = 0; i < NB; ++i) fh[i] = pk ? park[(s0 + i) * ps] : pa[i];
+          }
+#pragma unroll
+          for (int i = 0; i < NB; ++i) rr[i] = s1 ? csub<T>(fh[i], tv[i]) : tv[i];
+        } else if (kind == CT_P) {
+          // S1: d_t D = s u - u.grad D; S2: the product holds u(x+xi) - w - w.grad xi
+          const bool s1 = Y.strategy == 1;
+          const T sv = sd(), av = slot == 0 ? d.cadvx : d.cadvy;
+#pragma unroll
+          for (int i = 0; i < NB; ++i) {
+            const cplx<T> u = kin ? mk<T>(kx == 0 && kyof(s0 + i) == 0 ? av : (T)0, 0) : pa[i];
+            rr[i] = s1 ? csub<T>(cscale<T>(u, sv), tv[i]) : tv[i];
+          }
+        } else if (kind == CT_UV) {
+          // shallow-water momentum, Eq. (sw_eqs_dimless); pa: h, pb: v or u,
+          // parked |u|^2/2: u_t = f0 v + (zeta v) - d_x B, v_t = -(f0 u + (zeta u)) - d_y B
+          const bool iu = role == R_U;
+          const T sg = iu ? (T)1 : (T)-1, f0 = d.cf0, c2 = d.cc2;
+#pragma unroll
+          for (int i = 0; i < NB; ++i) {
+            const cplx<T> pk = park[(s0 + i) * ps];
+            const cplx<T> Bq = mk<T>(fma(pa[i].x, c2, pk.x), fma(pa[i].y, c2, pk.y));
+            const cplx<T> lin = mk<T>(fma(pb[i].x, f0, tv[i].x), fma(pb[i].y, f0, tv[i].y));
+            const T k = iu ? kxf : ky[i];
+            rr[i] = mk<T>(fma(Bq.y, k, sg * lin.x), fma(Bq.x, -k, sg * lin.y));
+          }
+        } else if (kind == CT_KIN) {
+#pragma unroll
+          for (int i = 0; i < NB; ++i) rr[i] = cik<T>(pa[i], -(kxf * d.cadvx + ky[i] * d.cadvy));
+        } else {
+          // -div(h u), or the two-dimensional Euler vorticity's -div(u zeta);
+          // the x component parked
+#pragma unroll
+          for (int i = 0; i < NB; ++i)
+            rr[i] = csub<T>(z, cadd<T>(cik<T>(park[(s0 + i) * ps], kxf), cik<T>(tv[i], ky[i])));
+        }
+      };
+      // NB modes at a time; t rotates
+      cplx<T> t[6] = {x[0], x[1], x[2], x[5], x[6], x[7]};
+      if (!last) {
+#pragma unroll 1
+        for (int s0 = 0; s0 < 6; s0 += NB) {
+          cplx<T> yn[NB], ac[NB], pa[NB], pb[NB], ea[NB], nv[NB];
+          T E[NB];
+          int ml[NB];
+#pragma unroll
+          for (int i = 0; i < NB; ++i) {
+            ml[i] = (min(max(kyof(s0 + i), -K), K) + K) * CS + m00;
+            yn[i] = yf[ml[i]];
+            ac[i] = pa[i] = pb[i] = ea[i] = z;
+            E[i] = (T)1;
+          }
+          if (damped) {
+#pragma unroll
+            for (int i = 0; i < NB; ++i) E[i] = ef[ml[i]];
+          }
+          if (fa >= 0) {
+#pragma unroll
+            for (int i = 0; i < NB; ++i) pa[i] = qa[ml[i]];
+          }
+          if (fb >= 0) {
+#pragma unroll
+            for (int i = 0; i < NB; ++i) pb[i] = qb[ml[i]];
+          }
+          if (add) {
+#pragma unroll
+            for (int i = 0; i < NB; ++i) ac[i] = af[ml[i]];
+            if (fe >= 0) {
+#pragma unroll
+              for (int i = 0; i < NB; ++i) ea[i] = ae[ml[i]];
+            }
+          }
+          T ky[NB];
+          bool in[NB];
+          cplx<T> rr[NB], fh[NB];
+#pragma unroll
+          for (int i = 0; i < NB; ++i) {
+            ky[i] = to_real(kyof(s0 + i), (T)0);
+            in[i] = inband(s0 + i);
+            fh[i] = z;
+          }
+          rhs(s0, ky, t, pa, pb, rr, fh);
+          // coefficients: RK4, Heun (E^2, E^2, dt E^2) and forward Euler (acc
+          // alone, dt E^2; xi-first means 2 dt E^4)
+          const T hdt = (T)0.5 * dt;
+#pragma unroll
+          for (int i = 0; i < NB; ++i) {
+            const T e1 = E[i], ee = e1 * e1;
+            T cr = stage == 0 ? ee : (T)2 * e1;
+            T ca = stage == 2 ? ee : e1;
+            T cb = stage == 0 ? hdt * e1 : (stage == 1 ? hdt : dt * e1);
+            if (st != 0) {
+              cr = ca = ee;
+              cb = dt * ee;
+              if (st == 2) cr = x1 ? (T)2 * dt * ee * ee : dt * ee;
+            }
+            nv[i] = mk<T>(fma(ca, yn[i].x, cb * rr[i].x), fma(ca, yn[i].y, cb * rr[i].y));
+            ac[i] = mk<T>(fma(cr, rr[i].x, ac[i].x), fma(cr, rr[i].y, ac[i].y));
+            if (in[i] && act) gst(af + ml[i], ac[i]);
+            nv[i] = in[i] ? nv[i] : z;
+          }
+          if (fe >= 0) {
+            // Eq. (ave), undamped
+            const T ce = st == 0 ? (stage == 0 ? (T)1 : (T)2) : (st == 1 ? (T)1 : dt);
+#pragma unroll
+            for (int i = 0; i < NB; ++i)
+              if (in[i]) gst(ae + ml[i], mk<T>(fma(ce, fh[i].x, ea[i].x), fma(ce, fh[i].y, ea[i].y)));
+          }
+          if (keep) {
+#pragma unroll
+            for (int i = 0; i < NB; ++i)
+              if (in[i]) gst(yout + f * ms + ml[i], nv[i]);
+            if (kind == CT_E2) {
+#pragma unroll
+              for (int i = 0; i < NB; ++i)
+                if (in[i]) slave_velocity<T>(yout, Y, ms, ml[i], kxf, ky[i], nv[i]);
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < 6; ++i) t[i] = i < 6 - NB ? t[(i + NB) % 6] : nv[i < 6 - NB ? 0 : i - (6 - NB)];
+        }
+      } else {
+        // final stage: y_{n+1} = E^2 y_n + inc, with inc = dt/6 (acc + d) (RK4),
+        // dt/2 (acc + b) (Heun) or forward Euler's increment acc
+        const T ci = st == 0 ? dt / (T)6 : (st == 1 ? dt / (T)2 : (T)1);
+#pragma unroll 1
+        for (int s0 = 0; s0 < 6; s0 += NB) {
+          cplx<T> yn[NB], ac[NB], cc[NB], pa[NB], pb[NB], en[NB], ea[NB], ec[NB], nv[NB];
+          T eh[NB], el[NB];
+          int ml[NB];
+#pragma unroll
+          for (int i = 0; i < NB; ++i) {
+            ml[i] = (min(max(kyof(s0 + i), -K), K) + K) * CS + m00;
+            yn[i] = yf[ml[i]];
+            ac[i] = af[ml[i]];
+            cc[i] = pa[i] = pb[i] = en[i] = ea[i] = ec[i] = z;
+            eh[i] = (T)1;
+            el[i] = (T)0;
+          }
+          if (damped) {
+#pragma unroll
+            for (int i = 0; i < NB; ++i) {
+              eh[i] = ef[ms + ml[i]];
+              el[i] = ef[2 * ms + ml[i]];
+            }
+          }
+          if (fa >= 0) {
+#pragma unroll
+            for (int i = 0; i < NB; ++i) pa[i] = qa[ml[i]];
+          }
+          if (fb >= 0) {
+#pragma unroll
+            for (int i = 0; i < NB; ++i) pb[i] = qb[ml[i]];
+          }
+          if (kah) {
+#pragma unroll
+            for (int i = 0; i < NB; ++i) cc[i] = d.comp[f * ms + ml[i]];
+          }
+          if (fe >= 0) {
+#pragma unroll
+            for (int i = 0; i < NB; ++i) {
+              en[i] = ye[ml[i]];
+              ea[i] = ae[ml[i]];
+            }
+            if (d.comp) {
+#pragma unroll
+              for (int i = 0; i < NB; ++i) ec[i] = d.comp[fe * ms + ml[i]];
+            }
+          }
+          T ky[NB];
+          bool in[NB];
+          cplx<T> rr[NB], fh[NB];
+#pragma unroll
+          for (int i = 0; i < NB; ++i) {
+            ky[i] = to_real(kyof(s0 + i), (T)0);
+            in[i] = inband(s0 + i);
+            rr[i] = fh[i] = z;
+          }
+          if (!commit) rhs(s0, ky, t, pa, pb, rr, fh);
+          if (x1) {
+            // E^4 = (eh + el)^2 to the same precision (exact product of eh by fma)
+#pragma unroll
+            for (int i = 0; i < NB; ++i) {
+              const T h2 = eh[i] * eh[i];
+              el[i] = fma(eh[i], eh[i], -h2) + (T)2 * eh[i] * el[i];
+              eh[i] = h2;
+            }
+          }
+          cplx<T>* const cf = d.comp + f * ms;
+#pragma unroll
+          for (int i = 0; i < NB; ++i) {
+            nv[i] = commit_mode<T>(kah, eh[i], el[i], yn[i], cc[i], cscale<T>(cadd<T>(ac[i], rr[i]), ci));
+            if (!act) nv[i] = yn[i];
+            if (in[i] && act) {
+              gst(yf + ml[i], nv[i]);
+              if (kah) gst(cf + ml[i], cc[i]);
+            }
+            nv[i] = in[i] ? nv[i] : z;
+          }
+          if (fe >= 0) {
+            const bool ke = d.comp != nullptr;
+            cplx<T>* const cfe = d.comp + fe * ms;
+#pragma unroll
+            for (int i = 0; i < NB; ++i) {
+              const cplx<T> v = commit_mode<T>(ke, (T)1, (T)0, en[i], ec[i], cscale<T>(cadd<T>(ea[i], fh[i]), ci));
+              if (in[i]) {
+                gst(ye + ml[i], v);
+                if (ke) gst(cfe + ml[i], ec[i]);
+              }
+            }
+          }
+          if (kind == CT_E2) {
+#pragma unroll
+            for (int i = 0; i < NB; ++i)
+              if (in[i]) slave_velocity<T>(yout, Y, ms, ml[i], kxf, ky[i], nv[i]);
+          }
+#pragma unroll
+          for (int i = 0; i < 6; ++i) t[i] = i < 6 - NB ? t[(i + NB) % 6] : nv[i < 6 - NB ? 0 : i - (6 - NB)];
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        x[i] = t[i];
+        x[5 + i] = t[3 + i];
+      }
+    };
+    auto load_park = [&]() {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        x[i] = park[i * ps];
+        x[5 + i] = park[(3 + i) * ps];
+      }
+    };
+    // field f of the stage's output at the thread's positions (u, v, h only:
+    // written by this thread, or the state)
+    auto load_out = [&](int f) {
+      const cplx<T>* y = yout + f * ms + m00;
+#pragma unroll
+      for (int s = 0; s < 6; ++s) {
+        const cplx<T> v = gld(y + (min(max(kyof(s), -K), K) + K) * CS);
+        x[s < 3 ? s : s + 2] = inband(s) ? v : mk<T>(0, 0);
+      }
+    };
+
+    // The task's steps: transforms of its products (a forward transform and
+    // what becomes of it) and of its mixed fields IFFT_y(op(value)), op in
+    // {id, d_x, d_y, curl}, as a forward transform of swapped parts.  None of
+    // the latter after forward Euler's first pass, or a replay's last step;
+    // only these when beginning.
+    const bool outs = !euler0 && !final_step;
+    for (int q = 0; q < ct.n; ++q) {
+      const int p = ct.prod[q], act = ct.act[q], op = ct.op[q];
+      const bool fwd = op < 0;
+      if (DUAL && ct.bar[q]) __syncthreads();
+      if ((fwd ? begin : !outs) || (DUAL && ct.half[q] != lane)) continue;
+      if (fwd) {
+        if (p >= 0 && !commit) {
+          const cplx<T>* src = d.pmix + (long long)p * d.g.mi + mx;
+#pragma unroll
+          for (int m = 0; m < 8; ++m) x[m] = src[m * mG];
+        }
+      } else {
+        // the value: in x after an update, or the parked one, or (when
+        // beginning, and for the fields of CT_UV, CT_E2 and CT_KIN) in memory
+        if (begin || act == CA_MEM) {
+          if (op == OP_CURL) {
+            // i kx v - i ky u
+            cplx<T> u[6];
+            load_out(Y.f_u);
+#pragma unroll
+            for (int s = 0; s < 6; ++s) u[s] = x[s < 3 ? s : s + 2];
+            load_out(Y.f_v);
+#pragma unroll
+            for (int s = 0; s < 6; ++s)
+              x[s < 3 ? s : s + 2] = csub<T>(cik<T>(x[s < 3 ? s : s + 2], kxf), cik<T>(u[s], to_real(kyof(s), (T)0)));
+          } else {
+            load_out(ct.fld[q]);
+          }
+        } else if (act == CA_PARKED) {
+          load_park();
+        }
+#pragma unroll
+        for (int s = 0; s < 6; ++s) {
+          cplx<T> v = x[s < 3 ? s : s + 2];
+          if (op == OP_DX) v = cik<T>(v, kxf);
+          else if (op == OP_DY) v = cik<T>(v, to_real(kyof(s), (T)0));
+          x[s < 3 ? s : s + 2] = cswap<T>(v);
+        }
+        x[3] = x[4] = mk<T>(0, 0);
+      }
+      if (!(fwd && (p < 0 || commit)))
+        gfft<T, -1, L, SYNC>(x, b0, b0 + row_stride<T>(N), w, j, lane, d.tw, gr, fwd ? -L : 0);
+      if (fwd) {
+        if (act != CA_PARK && act != CA_KEEP) {
+          int fe = -1, fa = -1, fb = -1;
+          const int fu = ct.fld[q];
+          if (kind == CT_UV) {
+            fa = Y.f_h;
+            fb = act == CA_U ? Y.f_v : Y.f_u;
+          } else if (kind == CT_KIN) {
+            fa = fu;
+          } else if (kind == CT_P) {
+            if (Y.strategy == 1 && !kin) fa = slot == 0 ? Y.f_u : Y.f_v;
+          } else if (kind == CT_G) {
+            const int sc = Y.lmf[slot];
+            fe = Y.f_e[slot];
+            if ((Y.strategy == 1 || fe >= 0) && sc != LMF_Q) {
+              fa = sc == LMF_ZETA ? (e2 ? Y.f_h : Y.f_v) : (sc == LMF_H ? Y.f_h : (sc == LMF_U ? Y.f_u : Y.f_v));
+              if (sc == LMF_ZETA && !e2) fb = Y.f_u;
+            }
+          }
+          update(fu, fe, fa, fb);
+        }
+        if (act == CA_PARK || act == CA_UPD_PARK) store_park();
+      } else {
+        cplx<T>* dst = d.mix + (long long)p * d.g.mi + mx;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) gst(dst + m * mG, cswap<T>(x[m]));
       }
     }
-  };
-  if (upm == UPD_MODES) modes(IntC<UPD_MODES / 256>());
-  else modes(IntC<2048 / 256>());
+  });
   if (stage == stage_count(d.c.stepper) - 1) {
     // the run's last block to finish advances its step counter (every block
     // of the run has read it above, before taking its ticket)
@@ -838,14 +990,13 @@ __global__ void __launch_bounds__(256, update_min_blocks<T>()) k_stage_update(co
     if (threadIdx.x == 0) {
       __threadfence();
       const unsigned t = atomicAdd(d.ticket, 1u);
-      if (t == (unsigned)d.nb[KT_UPDATE] - 1u) {
+      if (t == (unsigned)d.nb[KT_COL_STAGE] - 1u) {
         *d.ticket = 0u;
         *d.ctr = *d.ctr + 1;
         __threadfence();
       }
     }
   }
-  pdl_release();
 }
 
 }  // namespace lm
