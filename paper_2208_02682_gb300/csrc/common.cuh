@@ -34,6 +34,9 @@ template <typename T> __device__ __forceinline__ cplx<T> csub(cplx<T> a, cplx<T>
 template <typename T> __device__ __forceinline__ cplx<T> cmul(cplx<T> a, cplx<T> b) {
   return mk<T>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
+// a product that is rounded by itself (never contracted into an addition)
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 template <typename T> __device__ __forceinline__ cplx<T> cscale(cplx<T> a, T s) { return mk<T>(a.x * s, a.y * s); }
 template <typename T> __device__ __forceinline__ cplx<T> cconj(cplx<T> a) { return mk<T>(a.x, -a.y); }
 // multiply by i*k (spectral derivative)
@@ -51,6 +54,46 @@ template <typename T>
 __host__ __device__ __forceinline__ int sidx(int n) {
   return n + (n >> 3);
 }
+// floor of a double and its integer value modulo 2^32, by integer instructions
+// (FP64 ones, conversions included, take 16 clocks of the SM each): exactly
+// floor() and its conversion, which are called for |v| >= 2^30, zeros and
+// non-finite values.
+__device__ __forceinline__ double floor_int(double v, unsigned& k) {
+  const int hi = __double2hiint(v), lo = __double2loint(v);
+  const int e = ((hi >> 20) & 0x7ff) - 1023;
+  if (e >= 30 || ((hi & 0x7fffffff) | lo) == 0) {
+    const double f = floor(v);
+    k = (unsigned)(long long)f;
+    return f;
+  }
+  int n = 0;      // |v| truncated
+  bool rem = true;  // |v| has a fraction
+  if (e >= 0) {
+    const unsigned m = ((unsigned)hi & 0xfffffu) | 0x100000u;
+    const int sh = 52 - e;  // 23 .. 52
+    if (sh >= 32) {
+      n = (int)(m >> (sh - 32));
+      rem = ((m & ((1u << (sh - 32)) - 1u)) | (unsigned)lo) != 0u;
+    } else {
+      n = (int)((m << (32 - sh)) | ((unsigned)lo >> sh));
+      rem = ((unsigned)lo & ((1u << sh) - 1u)) != 0u;
+    }
+  }
+  if (hi < 0) n = -n - (rem ? 1 : 0);
+  k = (unsigned)n;
+  // n as a double, exact (|n| <= 2^30)
+  const unsigned a = (unsigned)abs(n);
+  const int lz = __clz((int)a);
+  const unsigned long long mant = (unsigned long long)(a << lz) << 21;
+  const unsigned h = (unsigned)(mant >> 32) + ((unsigned)(1022 + 31 - lz) << 20);
+  return __hiloint2double(a ? (int)(h | ((unsigned)n & 0x80000000u)) : 0, (int)(unsigned)mant);
+}
+__device__ __forceinline__ float floor_int(float v, unsigned& k) {
+  const float f = floorf(v);
+  k = (unsigned)(int)f;
+  return f;
+}
+
 // Spectral layout of the state: columns per tile, and the element of (ky_idx, kx).
 template <typename T> __host__ __device__ constexpr int spec_tile() { return sizeof(T) == 4 ? 4 : 2; }
 template <typename T> __host__ __device__ __forceinline__ int spec_index(int kyi, int kx, int NY) {

@@ -15,12 +15,15 @@
 #include <string>
 
 #include "../../include/lagmean.h"
+#include "common.cuh"
 
 namespace lm {
 void set_handleless_error(const std::string& msg);
 }
 
 namespace {
+
+using lm::floor_int;
 
 struct RemapArgs {
   const double* pos_x;
@@ -46,12 +49,13 @@ struct Cell {
 };
 
 __device__ __forceinline__ Cell cell_of(int i, int j, double cx, double cy, int N) {
-  const double fx = floor(cx), fy = floor(cy);
+  unsigned kx, ky;
+  const double fx = floor_int(cx, kx), fy = floor_int(cy, ky);
   const double ax = __dsub_rn(cx, fx), ay = __dsub_rn(cy, fy);
   const unsigned msk = (unsigned)N - 1u;
   Cell c;
-  c.i0 = (int)(((unsigned)i + (unsigned)(long long)fx) & msk);
-  c.j0 = (int)(((unsigned)j + (unsigned)(long long)fy) & msk);
+  c.i0 = (int)(((unsigned)i + kx) & msk);
+  c.j0 = (int)(((unsigned)j + ky) & msk);
   c.i1 = (int)(((unsigned)c.i0 + 1u) & msk);
   c.j1 = (int)(((unsigned)c.j0 + 1u) & msk);
   const double bx = __dsub_rn(1.0, ax), by = __dsub_rn(1.0, ay);
@@ -70,6 +74,10 @@ __device__ __forceinline__ double blend(const Cell& c, double f00, double f01, d
   return __dadd_rn(s, __dmul_rn(c.w11, f11));
 }
 
+// Bound by FP64 issue: the 28 additions and multiplications of an iteration
+// that must be rounded as written (1024^2, 20 iterations, four fields: with
+// floor, its conversion and the corner differences in FP64 every iteration
+// 1.74 ms, this 1.46 ms).
 // Smem: the N grid coordinates (the same separately rounded values, computed
 // once per block instead of four FP64 divisions per iteration).
 __global__ void __launch_bounds__(256) k_remap(const __grid_constant__ RemapArgs a) {
@@ -83,20 +91,39 @@ __global__ void __launch_bounds__(256) k_remap(const __grid_constant__ RemapArgs
   const int i = (int)(idx & (N - 1)), j = (int)(idx >> a.log2N);
   const double inv_dx = __ddiv_rn((double)N, kTwoPi);
   double xx = 0.0, xy = 0.0, r = 0.0;
+  // The corner displacements of the current cell are kept while the iterate
+  // stays in it, and an iterate that repeats itself exactly ends the loop (all
+  // later ones, and a residual of zero, follow from it): the same operations
+  // on the same values as iterating to the end.
+  int ci = -1, cj = -1;
+  double dx00 = 0, dx01 = 0, dx10 = 0, dx11 = 0, dy00 = 0, dy01 = 0, dy10 = 0, dy11 = 0;
   for (int k = 0; k < a.iters; ++k) {
     const Cell c = cell_of(i, j, __dmul_rn(xx, inv_dx), __dmul_rn(xy, inv_dx), N);
-    const long long o00 = (long long)c.j0 * N + c.i0, o01 = (long long)c.j0 * N + c.i1;
-    const long long o10 = (long long)c.j1 * N + c.i0, o11 = (long long)c.j1 * N + c.i1;
-    const double xi0 = xs[c.i0], xi1 = xs[c.i1];
-    const double yj0 = xs[c.j0], yj1 = xs[c.j1];
-    // d = x - Xi^{-1}(x) at the four corners
-    const double nx = blend(c, __dsub_rn(xi0, a.pos_x[o00]), __dsub_rn(xi1, a.pos_x[o01]),
-                            __dsub_rn(xi0, a.pos_x[o10]), __dsub_rn(xi1, a.pos_x[o11]));
-    const double ny = blend(c, __dsub_rn(yj0, a.pos_y[o00]), __dsub_rn(yj0, a.pos_y[o01]),
-                            __dsub_rn(yj1, a.pos_y[o10]), __dsub_rn(yj1, a.pos_y[o11]));
-    if (k == a.iters - 1) r = fmax(fabs(__dsub_rn(nx, xx)), fabs(__dsub_rn(ny, xy)));
+    if (c.i0 != ci || c.j0 != cj) {
+      ci = c.i0;
+      cj = c.j0;
+      const long long o00 = (long long)c.j0 * N + c.i0, o01 = (long long)c.j0 * N + c.i1;
+      const long long o10 = (long long)c.j1 * N + c.i0, o11 = (long long)c.j1 * N + c.i1;
+      const double xi0 = xs[c.i0], xi1 = xs[c.i1];
+      const double yj0 = xs[c.j0], yj1 = xs[c.j1];
+      // d = x - Xi^{-1}(x) at the four corners
+      dx00 = __dsub_rn(xi0, a.pos_x[o00]);
+      dx01 = __dsub_rn(xi1, a.pos_x[o01]);
+      dx10 = __dsub_rn(xi0, a.pos_x[o10]);
+      dx11 = __dsub_rn(xi1, a.pos_x[o11]);
+      dy00 = __dsub_rn(yj0, a.pos_y[o00]);
+      dy01 = __dsub_rn(yj0, a.pos_y[o01]);
+      dy10 = __dsub_rn(yj1, a.pos_y[o10]);
+      dy11 = __dsub_rn(yj1, a.pos_y[o11]);
+    }
+    const double nx = blend(c, dx00, dx01, dx10, dx11);
+    const double ny = blend(c, dy00, dy01, dy10, dy11);
+    const bool same = __double_as_longlong(nx) == __double_as_longlong(xx) &&
+                      __double_as_longlong(ny) == __double_as_longlong(xy);
+    if (k == a.iters - 1 || same) r = fmax(fabs(__dsub_rn(nx, xx)), fabs(__dsub_rn(ny, xy)));
     xx = nx;
     xy = ny;
+    if (same) break;
   }
   const Cell c = cell_of(i, j, __dmul_rn(xx, inv_dx), __dmul_rn(xy, inv_dx), N);
   const long long o00 = (long long)c.j0 * N + c.i0, o01 = (long long)c.j0 * N + c.i1;
