@@ -381,12 +381,13 @@ template <typename T> struct Bilin {
   unsigned o00, o01, o10, o11;
   T w00, w01, w10, w11;
   __device__ __forceinline__ Bilin(int i, int j, T xi_x, T xi_y, T inv_dx, int N) {
-    const T dxc = xi_x * inv_dx, dyc = xi_y * inv_dx;
-    const T fx = floor(dxc), fy = floor(dyc);
+    const T dxc = mul_rn(xi_x, inv_dx), dyc = mul_rn(xi_y, inv_dx);
+    unsigned kx, ky;
+    const T fx = floor_int(dxc, kx), fy = floor_int(dyc, ky);
     const T ax = dxc - fx, ay = dyc - fy;
     const unsigned msk = (unsigned)N - 1u;
-    const unsigned i0 = ((unsigned)i + (unsigned)(int)fx) & msk;
-    const unsigned j0 = ((unsigned)j + (unsigned)(int)fy) & msk;
+    const unsigned i0 = ((unsigned)i + kx) & msk;
+    const unsigned j0 = ((unsigned)j + ky) & msk;
     const unsigned i1 = (i0 + 1u) & msk, j1 = (j0 + 1u) & msk;
     o00 = j0 * N + i0;
     o01 = j0 * N + i1;
@@ -401,7 +402,7 @@ template <typename T> struct Bilin {
 template <typename T>
 __device__ __forceinline__ T bilinear(const T* __restrict__ f, int i, int j, T xi_x, T xi_y, T inv_dx, int N) {
   const Bilin<T> b(i, j, xi_x, xi_y, inv_dx, N);
-  return b.w00 * __ldg(f + b.o00) + b.w01 * __ldg(f + b.o01) + b.w10 * __ldg(f + b.o10) + b.w11 * __ldg(f + b.o11);
+  return fma(b.w11, __ldg(f + b.o11), fma(b.w10, __ldg(f + b.o10), fma(b.w01, __ldg(f + b.o01), mul_rn(b.w00, __ldg(f + b.o00)))));
 }
 __device__ __forceinline__ void ld_quad(const float* p, float* v) {
   const float4 q = __ldg(reinterpret_cast<const float4*>(p));
@@ -438,39 +439,161 @@ __global__ void k_velocity_from_vorticity(cplx<T>* __restrict__ y, Geom g, int f
 }
 
 // ---------------------------------------------------------------------------
-// Spectral FP64 copy of selected fields, value = (y - comp) * scale.
-template <typename T>
-__global__ void k_spec_to_f64(const cplx<T>* __restrict__ y, const cplx<T>* __restrict__ comp,
-                              double2* __restrict__ out, long long ms, int NY, int KXP, int f0_idx, int f1_idx,
-                              double scale) {
-  const long long m = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= ms) return;
-  const int o = spec_index<T>((int)m / KXP, (int)m % KXP, NY);
-  const int idx[2] = {f0_idx, f1_idx};
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    if (idx[q] < 0) continue;
-    const cplx<T> v = y[idx[q] * ms + o];
-    double re = (double)v.x, im = (double)v.y;
-    if (comp) {
-      const cplx<T> c = comp[idx[q] * ms + o];
-      re -= (double)c.x;
-      im -= (double)c.y;
-    }
-    out[q * ms + m] = make_double2(re * scale, im * scale);
-  }
+// FP64 transforms around the stepping (initial conditions, results), on the
+// fixed-point group transforms.  A launch takes up to four fields: a column
+// pass between the state (tile-blocked, in T) and FP64 mixed fields
+// (interleaved row pairs), and a row pass between these and FP64 physical
+// planes.  (As one FP64-butterfly launch each for a conversion, a column and a
+// row pass per pair of fields, u, v, h and zeta took nine launches and XXOUT.)
+constexpr int IO_MAX = 4;
+// Columns per block: as the column stage in FP64.
+__host__ __device__ __forceinline__ int io_log2C(int N) {
+  int l = 0;
+  while ((N << l) < 256 || ((N << l) < 2 * N && N < 2048)) ++l;
+  return l;
 }
 
-// Add delta to the real part of one spectral coefficient (mean depth).
-__global__ void k_add_real(double2* p, double delta);
+template <typename T> struct OutArgs {
+  const cplx<T>* y;
+  const cplx<T>* comp;  // compensation terms to subtract (null: none)
+  double2* mix;
+  double* phys;
+  const TwFx* tw;
+  Geom g;
+  int n;
+  int field[IO_MAX], field2[IO_MAX];  // field2 >= 0: i kx field2 - i ky field
+  int slot[IO_MAX];                   // plane of phys
+  // value = scale*val + ax*x + ay*y + cst
+  double scale[IO_MAX], ax[IO_MAX], ay[IO_MAX], cst[IO_MAX];
+};
 
-// FP64 spectral -> T spectral (initial condition).
+// Local block = (field, kx tile).
 template <typename T>
-__global__ void k_spec_from_f64(const double2* __restrict__ in, cplx<T>* __restrict__ y, Geom g, int nfields) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= g.ms * nfields) return;
-  const int f = (int)(i / g.ms), m = (int)(i - f * g.ms);
-  y[f * g.ms + spec_index<T>(m / g.KXP, m % g.KXP, g.NY)] = mk<T>((T)in[i].x, (T)in[i].y);
+__global__ void __launch_bounds__(256) k_out_col(const __grid_constant__ OutArgs<T> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ unsigned red[GRED_WORDS];
+  dispatch_L<4, 11>(a.g.log2N, [&](auto Lc) {
+    constexpr int L = decltype(Lc)::value, N = 1 << L, G = N / 8, CS = spec_tile<T>();
+    const int lC = io_log2C(N), C = 1 << lC;
+    const int i = blockIdx.y, c = threadIdx.x & (C - 1), j = threadIdx.x >> lC;
+    const int kx = (blockIdx.x << lC) + c, K = a.g.K, KXP = a.g.KXP, ms = (int)a.g.ms;
+    const int m00 = (kx / CS) * (a.g.NY * CS) + kx % CS;
+    double2 x[8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+      const int n = j + m * G, ky = n <= K ? n : n - N;
+      x[m] = make_double2(0.0, 0.0);
+      if (kx <= K && ky >= -K) {
+        const int o = (ky + K) * CS + m00;
+        auto val = [&](int f) {
+          const cplx<T> v = a.y[f * ms + o];
+          double2 r = make_double2((double)v.x, (double)v.y);
+          if (a.comp) {
+            const cplx<T> q = a.comp[f * ms + o];
+            r.x -= (double)q.x;
+            r.y -= (double)q.y;
+          }
+          return r;
+        };
+        x[m] = val(a.field[i]);
+        if (a.field2[i] >= 0)
+          x[m] = csub<double>(cik<double>(val(a.field2[i]), (double)kx), cik<double>(x[m], (double)ky));
+      }
+    }
+    double2* b0 = reinterpret_cast<double2*>(smem_raw) + (size_t)c * col_buf_stride<double>(N, C);
+    int w = 0;
+    gfft<double, +1, L, 2>(x, b0, b0 + row_stride<double>(N), w, j, 0, a.tw, GRed{red, lC, (int)threadIdx.x, (int)blockDim.x});
+    double2* dst = a.mix + (long long)i * a.g.mi + (j >> 1) * 2 * KXP + 2 * kx + (j & 1);
+#pragma unroll
+    for (int m = 0; m < 8; ++m) dst[m * G * KXP] = x[m];
+  });
+}
+
+// Local block = (field, block of row pairs, one per group of N/8 threads).
+template <typename T>
+__global__ void __launch_bounds__(256) k_out_row(const __grid_constant__ OutArgs<T> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ unsigned red[GRED_WORDS];
+  dispatch_L<4, 11>(a.g.log2N, [&](auto Lc) {
+    constexpr int L = decltype(Lc)::value, N = 1 << L, G = N / 8, SYNC = L <= 8 ? 0 : 1;
+    constexpr int rs = N + N / 8;
+    const int i = blockIdx.y, gi = threadIdx.x / G, j = threadIdx.x - gi * G;
+    const int yp = (blockIdx.x * (blockDim.x / G) + gi) & (N / 2 - 1);
+    double2* buf0 = reinterpret_cast<double2*>(smem_raw) + (size_t)gi * 2 * rs;
+    double2 x[8];
+    int w = 0;
+    load_rows_ct<double, L>(x, a.mix + (long long)i * a.g.mi + (long long)yp * 2 * a.g.KXP, j, a.g.K);
+    gfft<double, -1, L, SYNC>(x, buf0, buf0 + rs, w, j, gi, a.tw, GRed{red, 0, 0, 0});
+    const double dxg = 6.283185307179586476925286766559 / (double)N;
+    const double s = a.scale[i], ax = a.ax[i], ay = a.ay[i], cst = a.cst[i];
+    double* p = a.phys + (long long)a.slot[i] * a.g.np + (long long)yp * 2 * N + j;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+      const double xg = ax * ((j + m * G) * dxg);
+      p[m * G] = s * x[m].y + xg + ay * ((2 * yp) * dxg) + cst;
+      p[N + m * G] = s * x[m].x + xg + ay * ((2 * yp + 1) * dxg) + cst;
+    }
+  });
+}
+
+template <typename T> struct InArgs {
+  const double* phys;
+  double2* mix;
+  cplx<T>* y;
+  const TwFx* tw;
+  Geom g;
+  int n;
+  int slot[IO_MAX], field[IO_MAX];
+  double mean[IO_MAX];  // added to the k = 0 coefficient
+};
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_in_row(const __grid_constant__ InArgs<T> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ unsigned red[GRED_WORDS];
+  dispatch_L<4, 11>(a.g.log2N, [&](auto Lc) {
+    constexpr int L = decltype(Lc)::value, N = 1 << L, G = N / 8, SYNC = L <= 8 ? 0 : 1;
+    constexpr int rs = N + N / 8;
+    const int i = blockIdx.y, gi = threadIdx.x / G, j = threadIdx.x - gi * G;
+    const int yp = (blockIdx.x * (blockDim.x / G) + gi) & (N / 2 - 1);
+    double2* buf0 = reinterpret_cast<double2*>(smem_raw) + (size_t)gi * 2 * rs;
+    const double* p = a.phys + (long long)a.slot[i] * a.g.np + (long long)yp * 2 * N + j;
+    double2 x[8];
+    int w = 0;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) x[m] = make_double2(p[m * G], p[N + m * G]);
+    gfft<double, -1, L, SYNC>(x, buf0, buf0 + rs, w, j, gi, a.tw, GRed{red, 0, 0, 0}, -L - 1);
+    store_rows_ct<double, L, SYNC>(x, buf0, buf0 + rs, w, a.mix + (long long)i * a.g.mi + (long long)yp * 2 * a.g.KXP,
+                                   j, gi, a.g.K, a.g.KXP);
+  });
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_in_col(const __grid_constant__ InArgs<T> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ unsigned red[GRED_WORDS];
+  dispatch_L<4, 11>(a.g.log2N, [&](auto Lc) {
+    constexpr int L = decltype(Lc)::value, N = 1 << L, G = N / 8, CS = spec_tile<T>();
+    const int lC = io_log2C(N), C = 1 << lC;
+    const int i = blockIdx.y, c = threadIdx.x & (C - 1), j = threadIdx.x >> lC;
+    const int kx = (blockIdx.x << lC) + c, K = a.g.K, KXP = a.g.KXP;
+    const double2* src = a.mix + (long long)i * a.g.mi + (j >> 1) * 2 * KXP + 2 * kx + (j & 1);
+    double2 x[8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) x[m] = src[m * G * KXP];
+    double2* b0 = reinterpret_cast<double2*>(smem_raw) + (size_t)c * col_buf_stride<double>(N, C);
+    int w = 0;
+    gfft<double, -1, L, 2>(x, b0, b0 + row_stride<double>(N), w, j, 0, a.tw, GRed{red, lC, (int)threadIdx.x, (int)blockDim.x},
+                           -L);
+    cplx<T>* dst = a.y + (long long)a.field[i] * a.g.ms + (kx / CS) * (a.g.NY * CS) + kx % CS;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+      const int n = j + m * G, ky = n <= K ? n : n - N;
+      if (ky < -K) continue;
+      if (n == 0 && kx == 0) x[m].x += a.mean[i];
+      dst[(ky + K) * CS] = kx <= K ? mk<T>((T)x[m].x, (T)x[m].y) : mk<T>((T)0, (T)0);
+    }
+  });
 }
 
 // Copy of nf spectral fields between the tile-blocked layout and rows

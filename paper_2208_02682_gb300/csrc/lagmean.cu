@@ -43,7 +43,8 @@ struct sw_handle {
   size_t arena_bytes = 0;
   void *y = nullptr, *ys = nullptr, *ys2 = nullptr, *acc = nullptr, *comp = nullptr;
   void *mix = nullptr, *pmix = nullptr, *phys = nullptr, *ef = nullptr, *tw = nullptr;
-  double2 *tw64 = nullptr, *spec64 = nullptr, *mix64 = nullptr;
+  TwFx* tw64 = nullptr;
+  double2 *spec64 = nullptr, *mix64 = nullptr;
   double *out64 = nullptr, *part = nullptr, *dres = nullptr;
   long long* ctr = nullptr;
   unsigned* ticket = nullptr;
@@ -56,8 +57,8 @@ struct sw_handle {
   Layout L{};
   // launch shapes: column tiles of at most 2^lC columns; row_prod `points`
   // per block (row pairs x N) and ppb products per block (0: automatic, see
-  // batch_build_t); the FP64 row transforms take Bi rows per block
-  int lC = 2, points = 256, ppb = 0, Bi = 1;
+  // batch_build_t)
+  int lC = 2, points = 256, ppb = 0;
   uint64_t version = 1;  // bumped whenever L or the launch shapes change
   BatchExec* self = nullptr;  // batch of one used by sw_step / lmean_step
   int64_t launches = 0;  // kernels launched since creation
@@ -455,7 +456,7 @@ static void fill_desc(sw_handle* h, RunDesc<T>& d, int points, int ppb, int lC, 
                         : k == PK_HV ? e | v : k == PK_Q ? z | e : (k == PK_ADV && L.model != 1) ? u | v : 0;
   }
   d.fused = row_prod_fused<T>(g.N, L) ? 1 : 0;
-  d.gath = row_prod_gath<T>(g.N, L) ? 1 : 0;
+  d.gath = row_prod_gath<T>(g.N, L) && d.ppb >= L.np ? 1 : 0;
   d.nb[KT_ROW_INV] = L.np > 0 && !d.fused ? (L.strategy == 2 ? 5 : 3) * row_blocks(g.N, d.Bi) : 0;
   d.nb[KT_ROW_PROD] = row_blocks(g.N, d.Bp) * chunks;
   d.nb[KT_COL_STAGE] = L.np > 0 ? ntile * d.L.nct : (int)((g.ms + KIN_MODES - 1) / KIN_MODES);
@@ -570,7 +571,7 @@ static int batch_build_t(BatchExec* b) {
     const size_t csm = ((size_t)col_buf_stride<T>(N, 1 << lC) << lC) * cs;
     const int thr[KT_COUNT] = {d.Bi * N / 8, d.Bp * W * N / 8, halves * cthr};
     const size_t sm[KT_COUNT] = {(size_t)2 * d.Bi * row_stride<T>(N) * cs,
-                                 row_prod_smem<T>(N, d.Bp, W, h->L), halves * csm + (size_t)6 * cthr * cs};
+                                 row_prod_smem<T>(N, d.Bp, W, h->L, d.gath != 0), halves * csm + (size_t)6 * cthr * cs};
     const KBytes kb = kernel_bytes(h, h->L);
     if (h->L.np > 0) b->start_bytes += kb.col_inv;
     const double by[KT_COUNT] = {kb.row_inv, kb.row_prod, 0.0};
@@ -777,105 +778,64 @@ struct OutSpec {
   double scale, ax, ay;
   int slot;   // output slot in out64
   double cst; // constant added (1 for the depth h = 1 + eta)
+  int field2 = -1;  // >= 0: the curl i kx field2 - i ky field
 };
 
-static int spectral_pair_to_phys(sw_handle* h, const OutSpec& a, const OutSpec* b) {
-  const Geom& g = h->g;
-  cudaStream_t s = h->stream;
-  // FP64 spectral copies (scale applied in the row pass epilogue)
-  if (h->fp32)
-    CK(h, launch_spec_to_f64<float>((const cplx<float>*)h->y, (const cplx<float>*)h->comp, h->spec64, g,
-                                    a.field, b ? b->field : -1, 1.0, s));
-  else
-    CK(h, launch_spec_to_f64<double>((const cplx<double>*)h->y, nullptr, h->spec64, g, a.field,
-                                     b ? b->field : -1, 1.0, s));
-  ColInvArgs<double> ci;
-  ci.src = h->spec64;
-  ci.dst = h->mix64;
-  ci.tw = h->tw64;
-  ci.g = g;
-  ci.nout = b ? 2 : 1;
-  for (int i = 0; i < 2; ++i) {
-    ci.src_idx[i] = i;
-    ci.src2_idx[i] = -1;
-    ci.op[i] = OP_ID;
-    ci.dst_idx[i] = i;
+template <typename T>
+static int phys_outputs_t(sw_handle* h, const OutSpec* os, int n) {
+  for (int i = 0; i < n; i += IO_MAX) {
+    OutArgs<T> a;
+    std::memset(&a, 0, sizeof(a));
+    a.y = (const cplx<T>*)h->y;
+    a.comp = h->fp32 ? (const cplx<T>*)h->comp : nullptr;
+    a.mix = h->mix64;
+    a.phys = h->out64;
+    a.tw = h->tw64;
+    a.g = h->g;
+    a.n = n - i < IO_MAX ? n - i : IO_MAX;
+    for (int q = 0; q < a.n; ++q) {
+      const OutSpec& o = os[i + q];
+      a.field[q] = o.field;
+      a.field2[q] = o.field2;
+      a.slot[q] = o.slot;
+      a.scale[q] = o.scale;
+      a.ax[q] = o.ax;
+      a.ay[q] = o.ay;
+      a.cst[q] = o.cst;
+    }
+    CK(h, launch_out<T>(a, h->stream));
+    h->launches += 2;
   }
-  CK(h, launch_col_inv<double>(ci, s));
-  RowInvArgs<double, double> ri;
-  std::memset(&ri, 0, sizeof(ri));
-  ri.src = h->mix64;
-  ri.dst = h->out64;
-  ri.dst_stride = g.np;
-  ri.tw = h->tw64;
-  ri.g = g;
-  ri.B = h->Bi;
-  ri.npairs = 1;
-  ri.a_idx[0] = 0;
-  ri.b_idx[0] = b ? 1 : -1;
-  ri.oa[0] = a.slot;
-  ri.ob[0] = b ? b->slot : -1;
-  ri.sa[0] = a.scale;
-  ri.axa[0] = a.ax;
-  ri.aya[0] = a.ay;
-  ri.ca[0] = a.cst;
-  if (b) {
-    ri.sb[0] = b->scale;
-    ri.axb[0] = b->ax;
-    ri.ayb[0] = b->ay;
-    ri.cb[0] = b->cst;
-  }
-  CK(h, launch_row_inv<double, double>(ri, s));
-  h->launches += 3;
   return SW_OK;
 }
-
 static int phys_outputs(sw_handle* h, const OutSpec* os, int n) {
-  for (int i = 0; i < n; i += 2) {
-    int rc = spectral_pair_to_phys(h, os[i], i + 1 < n ? &os[i + 1] : nullptr);
-    if (rc) return rc;
-  }
-  return SW_OK;
+  return h->fp32 ? phys_outputs_t<float>(h, os, n) : phys_outputs_t<double>(h, os, n);
 }
 
 // Load a physical FP64 initial condition (already in out64[0..2]) into the
 // dynamics fields of the state.
-static int load_ic_from_out64(sw_handle* h) {
-  const Geom& g = h->g;
-  cudaStream_t s = h->stream;
-  RowFwdArgs<double> rf;
-  std::memset(&rf, 0, sizeof(rf));
-  rf.src = h->out64;
-  rf.dst = h->mix64;
-  rf.tw = h->tw64;
-  rf.g = g;
-  rf.B = h->Bi;
-  rf.npairs = 2;
-  rf.a_idx[0] = 0; rf.b_idx[0] = 1; rf.oa[0] = 0; rf.ob[0] = 1;
-  rf.a_idx[1] = 2; rf.b_idx[1] = -1; rf.oa[1] = 2; rf.ob[1] = -1;
-  CK(h, launch_row_fwd<double>(rf, s));
-  ColFwdArgs<double> cf;
-  cf.src = h->mix64;
-  cf.dst = h->spec64;
-  cf.tw = h->tw64;
-  cf.g = g;
-  cf.nout = 3;
-  for (int i = 0; i < 3; ++i) cf.src_idx[i] = cf.dst_idx[i] = i;
-  CK(h, launch_col_fwd<double>(cf, s));
+template <typename T>
+static int load_ic_t(sw_handle* h) {
+  InArgs<T> a;
+  std::memset(&a, 0, sizeof(a));
+  a.phys = h->out64;
+  a.mix = h->mix64;
+  a.y = (cplx<T>*)h->y;
+  a.tw = h->tw64;
+  a.g = h->g;
+  a.n = 3;
+  for (int i = 0; i < 3; ++i) a.slot[i] = a.field[i] = i;
   // the state holds the depth perturbation eta = h - 1 (mean depth 1 removed
   // from the k = 0 mode), which keeps its relative precision in FP32; the
   // two-dimensional Euler model holds the vorticity there and derives u, v
   const bool e2 = h->p.model == SW_MODEL_EULER2D;
-  if (!e2) CK(h, launch_add_real(h->spec64 + 2 * g.ms + (long long)g.K * g.KXP, -1.0, s));
-  if (h->fp32) CK(h, launch_spec_from_f64<float>(h->spec64, (cplx<float>*)h->y, g, 3, s));
-  else CK(h, launch_spec_from_f64<double>(h->spec64, (cplx<double>*)h->y, g, 3, s));
-  if (e2) {
-    if (h->fp32) CK(h, launch_velocity_from_vorticity<float>((cplx<float>*)h->y, g, h->L.f_u, h->L.f_v, h->L.f_h, s));
-    else CK(h, launch_velocity_from_vorticity<double>((cplx<double>*)h->y, g, h->L.f_u, h->L.f_v, h->L.f_h, s));
-  }
-  h->launches += e2 ? 5 : 4;
+  if (!e2) a.mean[2] = -1.0;
+  CK(h, launch_in<T>(a, h->stream));
+  if (e2) CK(h, launch_velocity_from_vorticity<T>((cplx<T>*)h->y, h->g, h->L.f_u, h->L.f_v, h->L.f_h, h->stream));
+  h->launches += e2 ? 3 : 2;
   return SW_OK;
 }
+static int load_ic_from_out64(sw_handle* h) { return h->fp32 ? load_ic_t<float>(h) : load_ic_t<double>(h); }
 
 static int copy_in_uvh(sw_handle* h, const double* uvh, int on_device) {
   const size_t bytes = (size_t)3 * h->g.np * sizeof(double);
@@ -948,7 +908,7 @@ static ArenaPlan plan_arena(const Geom& g, size_t tsz) {
       MAXF * g.ms * cs,                                                        // comp
       MAXI * g.mi * cs, MAXP * g.mi * cs,                                      // mix, pmix
       NPH * g.np * tsz, 6 * g.ms * tsz, g.N * cs,                              // phys, ef, tw
-      g.N * sizeof(double2), 4 * g.ms * sizeof(double2),                       // tw64, spec64
+      g.N * sizeof(TwFx), g.ms * sizeof(double2),                              // tw64, spec64
       4 * g.mi * sizeof(double2), 12 * g.np * sizeof(double),                  // mix64, out64
       2 * DIAG_BLOCKS * sizeof(double), 4 * sizeof(double),                    // part, dres
       sizeof(long long), sizeof(unsigned)};                                    // ctr, ticket
@@ -972,7 +932,7 @@ extern "C" int64_t sw_state_bytes(const sw_params* p) {
 }
 
 template <typename T>
-static void host_tables(const sw_params& p, const Geom& g, void* ef_host, void* tw_host, double2* tw64_host) {
+static void host_tables(const sw_params& p, const Geom& g, void* ef_host, void* tw_host, TwFx* tw64_host) {
   T* ef = (T*)ef_host;
   static_assert(sizeof(twid<T>) == sizeof(cplx<T>), "twiddle table size");
   // per class (dynamics, mean fields): E = exp(-nu |k|^2p dt/2) for the
@@ -1001,13 +961,14 @@ static void host_tables(const sw_params& p, const Geom& g, void* ef_host, void* 
           }
         }
   if (classes == 1) std::memcpy(ef + 3 * g.ms, ef, 3 * g.ms * sizeof(T));
-  std::vector<double> re(g.N, 1.0), im(g.N, 0.0);
-  fft_twiddle_table(g.log2N, re.data(), im.data());
-  for (int t = 0; t < g.N; ++t) {
-    tw64_host[t] = make_double2(re[t], im[t]);
-    if (sizeof(T) == 4) ((float2*)tw_host)[t] = make_float2((float)re[t], (float)im[t]);
+  fft_twiddle_table_fx(g.log2N, tw64_host);
+  if (sizeof(T) == 8) {
+    std::memcpy(tw_host, tw64_host, g.N * sizeof(TwFx));
+  } else {
+    std::vector<double> re(g.N, 1.0), im(g.N, 0.0);
+    fft_twiddle_table(g.log2N, re.data(), im.data());
+    for (int t = 0; t < g.N; ++t) ((float2*)tw_host)[t] = make_float2((float)re[t], (float)im[t]);
   }
-  if (sizeof(T) == 8) fft_twiddle_table_fx(g.log2N, (TwFx*)tw_host);
 }
 
 extern "C" int sw_create(const sw_params* p, const double* ic_uvh, int ic_on_device, void* stream,
@@ -1036,7 +997,6 @@ extern "C" int sw_create(const sw_params* p, const double* ic_uvh, int ic_on_dev
   plan_geometry(p->N, h->tsz, g, h->lC);
   const size_t cs = 2 * h->tsz;  // complex T
   h->diag_blocks = DIAG_BLOCKS;
-  h->Bi = row_block_rows(g.N);
   h->ppb = 0;  // automatic (batch_build_t)
   const ArenaPlan A = plan_arena(g, h->tsz);
   const size_t o_y = A.o[0], o_ys = A.o[1], o_ys2 = A.o[2], o_acc = A.o[3], o_comp = A.o[4];
@@ -1054,26 +1014,26 @@ extern "C" int sw_create(const sw_params* p, const double* ic_uvh, int ic_on_dev
   char* base = (char*)h->arena;
   h->y = base + o_y; h->ys = base + o_ys; h->ys2 = base + o_ys2; h->acc = base + o_acc; h->comp = base + o_comp;
   h->mix = base + o_mix; h->pmix = base + o_pmix; h->phys = base + o_phys; h->ef = base + o_ef;
-  h->tw = base + o_tw; h->tw64 = (double2*)(base + o_tw64); h->spec64 = (double2*)(base + o_spec64);
+  h->tw = base + o_tw; h->tw64 = (TwFx*)(base + o_tw64); h->spec64 = (double2*)(base + o_spec64);
   h->mix64 = (double2*)(base + o_mix64); h->out64 = (double*)(base + o_out64);
   h->part = (double*)(base + o_part); h->dres = (double*)(base + o_dres);
   h->ctr = (long long*)(base + o_ctr); h->ticket = (unsigned*)(base + o_ticket);
   // tables
   const size_t ef_bytes = 6 * g.ms * h->tsz, tw_bytes = g.N * cs;
-  char* hbuf = (char*)std::malloc(ef_bytes + tw_bytes + g.N * sizeof(double2));
+  char* hbuf = (char*)std::malloc(ef_bytes + tw_bytes + g.N * sizeof(TwFx));
   if (!hbuf) {
     cudaFree(h->arena);
     delete h;
     return fail(nullptr, SW_ENOMEM, "host allocation failed");
   }
-  if (h->fp32) host_tables<float>(*p, g, hbuf, hbuf + ef_bytes, (double2*)(hbuf + ef_bytes + tw_bytes));
-  else host_tables<double>(*p, g, hbuf, hbuf + ef_bytes, (double2*)(hbuf + ef_bytes + tw_bytes));
+  if (h->fp32) host_tables<float>(*p, g, hbuf, hbuf + ef_bytes, (TwFx*)(hbuf + ef_bytes + tw_bytes));
+  else host_tables<double>(*p, g, hbuf, hbuf + ef_bytes, (TwFx*)(hbuf + ef_bytes + tw_bytes));
   rc = SW_OK;
   do {
     if ((e = cudaMemsetAsync(h->arena, 0, h->arena_bytes, h->stream)) != cudaSuccess) break;
     if ((e = cudaMemcpyAsync(h->ef, hbuf, ef_bytes, cudaMemcpyHostToDevice, h->stream)) != cudaSuccess) break;
     if ((e = cudaMemcpyAsync(h->tw, hbuf + ef_bytes, tw_bytes, cudaMemcpyHostToDevice, h->stream)) != cudaSuccess) break;
-    if ((e = cudaMemcpyAsync(h->tw64, hbuf + ef_bytes + tw_bytes, g.N * sizeof(double2), cudaMemcpyHostToDevice,
+    if ((e = cudaMemcpyAsync(h->tw64, hbuf + ef_bytes + tw_bytes, g.N * sizeof(TwFx), cudaMemcpyHostToDevice,
                              h->stream)) != cudaSuccess) break;
     if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) break;
   } while (0);
@@ -1267,51 +1227,12 @@ extern "C" int sw_set_fields(sw_handle* h, const double* uvh, int on_device) {
 // (zeta by a spectral curl in FP64), on the handle's stream.
 static int phys_uvhz(sw_handle* h) {
   const bool e2 = h->p.model == SW_MODEL_EULER2D;
-  OutSpec os[3] = {{h->L.f_u, 1.0, 0, 0, 0, 0.0}, {h->L.f_v, 1.0, 0, 0, 1, 0.0},
-                   {h->L.f_h, 1.0, 0, 0, 2, e2 ? 0.0 : 1.0}};
-  int rc = phys_outputs(h, os, 3);
-  if (rc) return rc;
-  if (e2) {
-    // the evolved vorticity (with its mean) in both the h and the zeta slot
-    CK(h, cudaMemcpyAsync(h->out64 + 3 * h->g.np, h->out64 + 2 * h->g.np, (size_t)h->g.np * sizeof(double),
-                          cudaMemcpyDeviceToDevice, h->stream));
-    return SW_OK;
-  }
-  // zeta = i kx v - i ky u from FP64 copies of u, v
-  const Geom& g = h->g;
-  if (h->fp32)
-    CK(h, launch_spec_to_f64<float>((const cplx<float>*)h->y, nullptr, h->spec64, g, h->L.f_u, h->L.f_v, 1.0,
-                                    h->stream));
-  else
-    CK(h, launch_spec_to_f64<double>((const cplx<double>*)h->y, nullptr, h->spec64, g, h->L.f_u, h->L.f_v, 1.0,
-                                     h->stream));
-  ColInvArgs<double> ci;
-  ci.src = h->spec64;
-  ci.dst = h->mix64;
-  ci.tw = h->tw64;
-  ci.g = g;
-  ci.nout = 1;
-  ci.src_idx[0] = 0;
-  ci.src2_idx[0] = 1;
-  ci.op[0] = OP_CURL;
-  ci.dst_idx[0] = 0;
-  CK(h, launch_col_inv<double>(ci, h->stream));
-  RowInvArgs<double, double> ri;
-  std::memset(&ri, 0, sizeof(ri));
-  ri.src = h->mix64;
-  ri.dst = h->out64;
-  ri.dst_stride = g.np;
-  ri.tw = h->tw64;
-  ri.g = g;
-  ri.B = h->Bi;
-  ri.npairs = 1;
-  ri.a_idx[0] = 0;
-  ri.b_idx[0] = -1;
-  ri.oa[0] = 3;
-  ri.ob[0] = -1;
-  ri.sa[0] = 1.0;
-  CK(h, launch_row_inv<double, double>(ri, h->stream));
-  return SW_OK;
+  // (the dynamics fields carry no compensation term: it stays zero)
+  OutSpec os[4] = {{h->L.f_u, 1.0, 0, 0, 0, 0.0}, {h->L.f_v, 1.0, 0, 0, 1, 0.0},
+                   {h->L.f_h, 1.0, 0, 0, 2, e2 ? 0.0 : 1.0}, {h->L.f_u, 1.0, 0, 0, 3, 0.0, h->L.f_v}};
+  // the evolved vorticity (with its mean) in both the h and the zeta slot
+  if (e2) os[3] = OutSpec{h->L.f_h, 1.0, 0, 0, 3, 0.0};
+  return phys_outputs(h, os, 4);
 }
 
 namespace lm {
@@ -1469,27 +1390,18 @@ extern "C" int sw_spectrum(sw_handle* h, const double* field, int on_device, dou
   // into staging slot 1
   CK(h, cudaMemcpyAsync(h->out64, field, (size_t)g.np * sizeof(double),
                         on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
-  RowFwdArgs<double> rf;
-  std::memset(&rf, 0, sizeof(rf));
-  rf.src = h->out64;
-  rf.dst = h->mix64;
-  rf.tw = h->tw64;
-  rf.g = g;
-  rf.B = h->Bi;
-  rf.npairs = 1;
-  rf.a_idx[0] = 0; rf.b_idx[0] = -1; rf.oa[0] = 0; rf.ob[0] = -1;
-  CK(h, launch_row_fwd<double>(rf, s));
-  ColFwdArgs<double> cf;
-  cf.src = h->mix64;
-  cf.dst = h->spec64;
-  cf.tw = h->tw64;
-  cf.g = g;
-  cf.nout = 1;
-  cf.src_idx[0] = cf.dst_idx[0] = 0;
-  CK(h, launch_col_fwd<double>(cf, s));
+  InArgs<double> ia;
+  std::memset(&ia, 0, sizeof(ia));
+  ia.phys = h->out64;
+  ia.mix = h->mix64;
+  ia.y = h->spec64;
+  ia.tw = h->tw64;
+  ia.g = g;
+  ia.n = 1;
+  CK(h, launch_in<double>(ia, s));
   double* acc = h->out64 + g.np;
   CK(h, cudaMemsetAsync(acc, 0, (size_t)ns * sizeof(double), s));
-  CK(h, launch_spectrum_shells(h->spec64, g.K, g.KXP, acc, s));
+  CK(h, launch_spectrum_shells(h->spec64, g, acc, s));
   h->launches += 3;
   std::vector<double> tmp(ns);
   CK(h, cudaMemcpyAsync(tmp.data(), acc, (size_t)ns * sizeof(double), cudaMemcpyDeviceToHost, s));

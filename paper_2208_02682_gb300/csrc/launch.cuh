@@ -39,8 +39,8 @@ template <typename T> bool row_prod_fused(int N, const Layout& L) {
 template <typename T> bool row_prod_gath(int N, const Layout& L) {
   return L.strategy == 2 && (size_t)row_prod_planes(0, 1, L.has_q) * N * sizeof(cplx<T>) <= (size_t)96 * 1024;
 }
-template <typename T> size_t row_prod_smem(int N, int B, int W, const Layout& L) {
-  const size_t nu = row_prod_planes(row_prod_fused<T>(N, L), row_prod_gath<T>(N, L), L.has_q);
+template <typename T> size_t row_prod_smem(int N, int B, int W, const Layout& L, bool all_products = true) {
+  const size_t nu = row_prod_planes(row_prod_fused<T>(N, L), all_products && row_prod_gath<T>(N, L), L.has_q);
   return (size_t)B * sizeof(cplx<T>) * (nu * N + (size_t)W * 2 * row_stride<T>(N));
 }
 
@@ -73,11 +73,9 @@ template <typename T> cudaError_t launch_row_fwd(const RowFwdArgs<T>& a, cudaStr
 template <typename T>
 cudaError_t launch_stage(int kt, const RunDesc<T>* runs, const int* start, int nruns, int blocks, int threads,
                          size_t smem, int stage, bool warp, bool dual, bool pdl, cudaStream_t s);
-template <typename T>
-cudaError_t launch_spec_to_f64(const cplx<T>* y, const cplx<T>* comp, double2* out, const Geom& g, int fa, int fb,
-                               double scale, cudaStream_t s);
-template <typename T>
-cudaError_t launch_spec_from_f64(const double2* in, cplx<T>* y, const Geom& g, int nfields, cudaStream_t s);
+// FP64 transforms between the state and physical planes (see k_out_col).
+template <typename T> cudaError_t launch_out(const OutArgs<T>& a, cudaStream_t s);
+template <typename T> cudaError_t launch_in(const InArgs<T>& a, cudaStream_t s);
 template <typename T>
 cudaError_t launch_spec_rows(const cplx<T>* in, cplx<T>* out, const Geom& g, int nfields, bool to_rows,
                              cudaStream_t s);
@@ -85,8 +83,7 @@ template <typename T>
 cudaError_t launch_velocity_from_vorticity(cplx<T>* y, const Geom& g, int fu, int fv, int fh, cudaStream_t s);
 cudaError_t launch_diag(const double* phys, long long np, double f0, double c2, double* part, int nblk,
                         double* out, cudaStream_t s);
-cudaError_t launch_add_real(double2* p, double delta, cudaStream_t s);
-cudaError_t launch_spectrum_shells(const double2* F, int K, int KXP, double* acc, cudaStream_t s);
+cudaError_t launch_spectrum_shells(const double2* F, const Geom& g, double* acc, cudaStream_t s);
 
 // Handle hooks for other translation units (defined in lagmean.cu).
 struct HandleInfo {
@@ -117,10 +114,16 @@ template <typename T> static cudaError_t prepare_kernels_t() {
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&mx, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
-  if ((e = allow_dynamic_smem(k_col_inv<T>, mx)) != cudaSuccess) return e;
-  if ((e = allow_dynamic_smem(k_col_fwd<T>, mx)) != cudaSuccess) return e;
-  if ((e = allow_dynamic_smem(k_row_inv<T, T>, mx)) != cudaSuccess) return e;
-  if ((e = allow_dynamic_smem(k_row_fwd<T>, mx)) != cudaSuccess) return e;
+  if constexpr (sizeof(T) == 8) {
+    if ((e = allow_dynamic_smem(k_col_inv<T>, mx)) != cudaSuccess) return e;
+    if ((e = allow_dynamic_smem(k_col_fwd<T>, mx)) != cudaSuccess) return e;
+    if ((e = allow_dynamic_smem(k_row_inv<T, T>, mx)) != cudaSuccess) return e;
+    if ((e = allow_dynamic_smem(k_row_fwd<T>, mx)) != cudaSuccess) return e;
+  }
+  if ((e = allow_dynamic_smem(k_out_col<T>, mx)) != cudaSuccess) return e;
+  if ((e = allow_dynamic_smem(k_out_row<T>, mx)) != cudaSuccess) return e;
+  if ((e = allow_dynamic_smem(k_in_row<T>, mx)) != cudaSuccess) return e;
+  if ((e = allow_dynamic_smem(k_in_col<T>, mx)) != cudaSuccess) return e;
   if constexpr (sizeof(T) == 8)
     if ((e = allow_dynamic_smem(k_stage_col<T, 128, false>, mx)) != cudaSuccess) return e;
   if ((e = allow_dynamic_smem(k_stage_col<T, 256, false>, mx)) != cudaSuccess) return e;
@@ -194,16 +197,30 @@ cudaError_t launch_stage(int kt, const RunDesc<T>* runs, const int* start, int n
   }
 }
 
-template <typename T>
-cudaError_t launch_spec_to_f64(const cplx<T>* y, const cplx<T>* comp, double2* out, const Geom& g, int fa, int fb,
-                               double scale, cudaStream_t s) {
-  k_spec_to_f64<T><<<(unsigned)((g.ms + 255) / 256), 256, 0, s>>>(y, comp, out, g.ms, g.NY, g.KXP, fa, fb, scale);
+struct IoShape {
+  dim3 cols, rows;
+  int cthr, rthr;
+  size_t csm, rsm;
+  IoShape(const Geom& g, int n) {
+    const int lC = io_log2C(g.N), B = row_block_pairs(g.N, 512);
+    cols = dim3((unsigned)(g.KXP >> lC), (unsigned)n);
+    rows = dim3((unsigned)row_blocks(g.N, B), (unsigned)n);
+    cthr = (g.N << lC) / 8;
+    rthr = B * g.N / 8;
+    csm = ((size_t)col_buf_stride<double>(g.N, 1 << lC) << lC) * sizeof(double2);
+    rsm = (size_t)B * 2 * row_stride<double>(g.N) * sizeof(double2);
+  }
+};
+template <typename T> cudaError_t launch_out(const OutArgs<T>& a, cudaStream_t s) {
+  const IoShape q(a.g, a.n);
+  k_out_col<T><<<q.cols, q.cthr, q.csm, s>>>(a);
+  k_out_row<T><<<q.rows, q.rthr, q.rsm, s>>>(a);
   return cudaGetLastError();
 }
-
-template <typename T>
-cudaError_t launch_spec_from_f64(const double2* in, cplx<T>* y, const Geom& g, int nfields, cudaStream_t s) {
-  k_spec_from_f64<T><<<(unsigned)((g.ms * nfields + 255) / 256), 256, 0, s>>>(in, y, g, nfields);
+template <typename T> cudaError_t launch_in(const InArgs<T>& a, cudaStream_t s) {
+  const IoShape q(a.g, a.n);
+  k_in_row<T><<<q.rows, q.rthr, q.rsm, s>>>(a);
+  k_in_col<T><<<q.cols, q.cthr, q.csm, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -221,17 +238,18 @@ cudaError_t launch_velocity_from_vorticity(cplx<T>* y, const Geom& g, int fu, in
 }
 
 #define LM_INSTANTIATE_ALL(T)                                                                               \
-  template cudaError_t launch_col_inv<T>(const ColInvArgs<T>&, cudaStream_t);                               \
-  template cudaError_t launch_col_fwd<T>(const ColFwdArgs<T>&, cudaStream_t);                               \
-  template cudaError_t launch_row_inv<T, T>(const RowInvArgs<T, T>&, cudaStream_t);                         \
-  template cudaError_t launch_row_fwd<T>(const RowFwdArgs<T>&, cudaStream_t);                               \
   template cudaError_t launch_stage<T>(int, const RunDesc<T>*, const int*, int, int, int, size_t, int, bool,  \
-                                       bool, bool, cudaStream_t);                                                 \
-  template cudaError_t launch_spec_to_f64<T>(const cplx<T>*, const cplx<T>*, double2*, const Geom&, int, int, \
-                                             double, cudaStream_t);                                         \
-  template cudaError_t launch_spec_from_f64<T>(const double2*, cplx<T>*, const Geom&, int, cudaStream_t);     \
+                                       bool, bool, cudaStream_t);                                           \
+  template cudaError_t launch_out<T>(const OutArgs<T>&, cudaStream_t);                                       \
+  template cudaError_t launch_in<T>(const InArgs<T>&, cudaStream_t);                                         \
   template cudaError_t launch_spec_rows<T>(const cplx<T>*, cplx<T>*, const Geom&, int, bool, cudaStream_t);   \
   template cudaError_t launch_velocity_from_vorticity<T>(cplx<T>*, const Geom&, int, int, int, cudaStream_t);
+// the generic FP64 transforms (csrc/project_static.cu)
+#define LM_INSTANTIATE_GENERIC                                                                              \
+  template cudaError_t launch_col_inv<double>(const ColInvArgs<double>&, cudaStream_t);                      \
+  template cudaError_t launch_col_fwd<double>(const ColFwdArgs<double>&, cudaStream_t);                      \
+  template cudaError_t launch_row_inv<double, double>(const RowInvArgs<double, double>&, cudaStream_t);      \
+  template cudaError_t launch_row_fwd<double>(const RowFwdArgs<double>&, cudaStream_t);
 #endif
 
 }  // namespace lm

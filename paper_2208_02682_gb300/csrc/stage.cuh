@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(256) k_stage_row_inv(const RunDesc<T>* __restr
 // transform the pair's base fields u, v, h, zeta (those the chunk needs) into
 // shared memory.  The others read base values from the planes that the row
 // inverse pass wrote; Strategy 2 gathers from them too: `gath` runs (where the
-// arrays fit) once for all products, into shared memory, from interleaved
+// arrays fit and a block takes all products) once for all products, into shared memory, from interleaved
 // planes (each product gathering for itself from separate planes took 34.7 us
 // at 512^2 with five means, this 26.7 us).  Every transform stays in the
 // registers of its group: an advection product takes the inverse transforms
@@ -239,27 +239,25 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), sizeof(T) == 4 ? 1 
       for (int e = wg * G + j; e < 2 * N; e += W * G) {
         const int rr = e >= N ? 1 : 0, xcol = e - rr * N, y = 2 * yp + rr;
         const int o = y * N + xcol;
-        T b[4], xi[2], f[5];
+        T b[4], xi[2], f[4];
         ld_quad(phys + 4 * (long long)o, b);
         const cplx<T> xv = __ldg(reinterpret_cast<const cplx<T>*>(phys + (long long)PH_XX * g.np) + o);
         xi[0] = xv.x;
         xi[1] = xv.y;
         const Bilin<T> bl(xcol, y, xv.x, xv.y, inv_dx, N);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) f[q] = (T)0;
         T c[4];
         ld_quad(phys + 4 * (long long)bl.o00, c);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) f[q] = bl.w00 * c[q];
+        for (int q = 0; q < 4; ++q) f[q] = mul_rn(bl.w00, c[q]);
         ld_quad(phys + 4 * (long long)bl.o01, c);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) f[q] += bl.w01 * c[q];
+        for (int q = 0; q < 4; ++q) f[q] = fma(bl.w01, c[q], f[q]);
         ld_quad(phys + 4 * (long long)bl.o10, c);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) f[q] += bl.w10 * c[q];
+        for (int q = 0; q < 4; ++q) f[q] = fma(bl.w10, c[q], f[q]);
         ld_quad(phys + 4 * (long long)bl.o11, c);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) f[q] += bl.w11 * c[q];
+        for (int q = 0; q < 4; ++q) f[q] = fma(bl.w11, c[q], f[q]);
         T* dst = S + 2 * xcol + rr;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -269,8 +267,8 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), sizeof(T) == 4 ? 1 
         dst[4 * 2 * N] = xi[0];
         dst[5 * 2 * N] = xi[1];
         if (L.has_q)
-          dst[10 * 2 * N] = bl.w00 * __ldg(Q + bl.o00) + bl.w01 * __ldg(Q + bl.o01) + bl.w10 * __ldg(Q + bl.o10) +
-                            bl.w11 * __ldg(Q + bl.o11);
+          dst[10 * 2 * N] = fma(bl.w11, __ldg(Q + bl.o11), fma(bl.w10, __ldg(Q + bl.o10),
+                                fma(bl.w01, __ldg(Q + bl.o01), mul_rn(bl.w00, __ldg(Q + bl.o00)))));
       }
       __syncthreads();
     }
