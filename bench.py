@@ -648,20 +648,15 @@ def measure_served(lm, n_jobs=24, rate=50.0, sizes=(128, 256, 512, 1024, 2048), 
 # keyed by (kernel, N).  Valid only while the stage-kernel sources are those
 # of the captures (their hash below); otherwise `traffic` is reported null.
 TRAFFIC_CAPTURES = {
-    # bench workload (256^2, S1 + S2 batch): warm L2 as in the timed run, mean of
-    # five captured launches (each covering both runs) halved
-    ("row_prod", 256): 150_963,
-    # FP32 Strategy 1 (zeta, h, u, v, positions, Eulerian), one launch, cold caches
-    ("row_prod", 1024): 52_500_000, ("col_inv", 1024): 17_800_000, ("col_fwd", 1024): 31_000_000,
-    ("update", 1024): 55_600_000, ("row_inv", 1024): 11_400_000,
-    ("row_prod", 2048): 291_800_000, ("col_inv", 2048): 193_200_000, ("col_fwd", 2048): 168_000_000,
-    ("update", 2048): 387_200_000, ("row_inv", 2048): 58_000_000,
+    # FP32 Strategy 1 (zeta, h, u, v, positions, Eulerian), one launch, cold
+    # caches (column stage: an early stage of a step)
+    ("row_prod", 2048): 264_500_000, ("col_stage", 2048): 528_400_000,
 }
-TRAFFIC_SOURCES_SHA256 = "fa76517f9aaad40a3c3e75365a13ecdd0fdd7afdae7108cebdd0f27f98c4b8f6"
+TRAFFIC_SOURCES_SHA256 = "b8dc5b24545ba38d69bc2c4496d162b795b733e78e26b8a43aba5963d9011e65"
 
 
 # the sources that define the stage kernels and their launch shapes
-STAGE_SOURCES = ("common.cuh", "fft.cuh", "kernels.cuh", "stage.cuh", "launch.cuh", "kernels_f32.cu", "lagmean.cu")
+STAGE_SOURCES = ("common.cuh", "fft.cuh", "fft64.cuh", "kernels.cuh", "stage.cuh", "launch.cuh", "kernels_f32.cu", "lagmean.cu")
 
 
 def kernel_sources_sha256():

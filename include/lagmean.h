@@ -290,15 +290,15 @@ int sw_batch_create(sw_handle* const* handles, int n, sw_batch** out);
 int sw_batch_step(sw_batch* b, int64_t nsteps);
 
 /* Autotuner: times the row-pass launch shapes (points per block 256, 512,
- * 1024 or 2048, as long as every member fits; product pairs per block 1, 2, 3
- * or all; choice = 4 * points index + pairs index) on trial_steps >= 1
+ * 1024 or 2048, as long as every member fits; products per block 1, 2, 3
+ * or all; choice = 4 * points index + products index) on trial_steps >= 1
  * replayed steps each (after as many untimed ones), keeps the fastest for all members and returns its
  * index in *choice (may be NULL).  The members' states are saved before the trials and
  * restored after them (temporary device copies).  Synchronises. */
 int sw_batch_tune(sw_batch* b, int trial_steps, int* choice);
 
 /* Set the row-pass launch shape that sw_batch_tune would pick as `choice`
- * (4 * points index + pairs index, as above) without timing anything: for
+ * (4 * points index + products index, as above) without timing anything: for
  * callers that replay a shape tuned earlier, and for tests that must cover
  * every shape.  The members' arithmetic and results do not depend on it.
  * SW_EINVAL if choice is outside 0..15 or its points per block are fewer

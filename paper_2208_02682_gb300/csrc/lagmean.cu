@@ -587,6 +587,8 @@ static int batch_build_t(BatchExec* b) {
       for (int st = 0; st < 4; ++st) b->bytes[k][st] += (k == KT_COL_STAGE ? kb.col_stage[st] : by[k]);
     }
   }
+  // kinematic dynamics alone: pointwise blocks of any size
+  if (n > 0 && b->start_bytes == 0.0) b->threads[KT_COL_STAGE] = 128;
   const size_t desc_bytes = (sizeof(RunDesc<T>) * n + 255) & ~(size_t)255;
   const size_t need = desc_bytes + sizeof(int) * b->start.size();
   if (need > b->table_bytes) {
