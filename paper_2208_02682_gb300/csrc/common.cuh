@@ -100,15 +100,58 @@ template <typename T> __host__ __device__ __forceinline__ int spec_index(int kyi
   constexpr int S = sizeof(T) == 4 ? 4 : 2;
   return (kx / S) * (NY * S) + kyi * S + kx % S;
 }
+
+// Global loads and stores of memory that the kernels of a step hand to one
+// another.  A stage kernel is resident while the previous one still writes (see
+// pdl_wait), so nothing that a kernel of the step writes may be read through the
+// read-only path (__ldg, or loads that the compiler may take for such): that
+// path is for data no kernel writes while this one lives (run descriptors,
+// tables).  The compiler keeps these accesses in order with one another and
+// with pdl_wait, and does not treat them as touching other memory: after a
+// plain store through a pointer it would reload every run-descriptor field it
+// uses (kept in shared memory), a chain of waits per store.  Values handed from
+// one thread of a block to another through them need a __syncthreads between
+// the store and the load (the split column blocks' u, v and h).
+__device__ __forceinline__ void gst(float2* p, float2 v) {
+  asm volatile("st.global.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(v.x), "f"(v.y));
+}
+__device__ __forceinline__ void gst(double2* p, double2 v) {
+  asm volatile("st.global.v2.f64 [%0], {%1, %2};" ::"l"(p), "d"(v.x), "d"(v.y));
+}
+__device__ __forceinline__ float gld(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double gld(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float2 gld(const float2* p) {
+  float2 v;
+  asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double2 gld(const double2* p) {
+  double2 v;
+  asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 gld(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
 // The two rows of a pair at one kx of a mixed field.
 __device__ __forceinline__ void ld_pair(const float2* p, float2& a, float2& b) {
-  const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+  const float4 v = gld(reinterpret_cast<const float4*>(p));
   a = make_float2(v.x, v.y);
   b = make_float2(v.z, v.w);
 }
 __device__ __forceinline__ void ld_pair(const double2* p, double2& a, double2& b) {
-  a = __ldg(p);
-  b = __ldg(p + 1);
+  a = gld(p);
+  b = gld(p + 1);
 }
 __device__ __forceinline__ void st_pair(float2* p, float2 a, float2 b) {
   *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
@@ -233,27 +276,6 @@ struct StepConsts {
   int stepper;  // SW_STEP_* (0 RK4, 1 Heun, 2 forward Euler)
   int pad;
 };
-
-// Global store and load of a complex value that the compiler keeps in order
-// with one another but does not treat as touching other memory: after a plain
-// store through a pointer it would reload every run-descriptor field it uses
-// (kept in shared memory), a chain of waits per store.
-__device__ __forceinline__ void gst(float2* p, float2 v) {
-  asm volatile("st.global.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(v.x), "f"(v.y));
-}
-__device__ __forceinline__ void gst(double2* p, double2 v) {
-  asm volatile("st.global.v2.f64 [%0], {%1, %2};" ::"l"(p), "d"(v.x), "d"(v.y));
-}
-__device__ __forceinline__ float2 gld(const float2* p) {
-  float2 v;
-  asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
-  return v;
-}
-__device__ __forceinline__ double2 gld(const double2* p) {
-  double2 v;
-  asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
-  return v;
-}
 
 // Programmatic dependent launch (PTX griddepcontrol).  The stage kernels of
 // a step are launched with programmatic stream serialisation, so a kernel's

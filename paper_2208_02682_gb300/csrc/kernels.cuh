@@ -201,7 +201,7 @@ __device__ void row_pair_forward_store(cplx<T>* buf, cplx<T>* __restrict__ da,
 // transform does.  Parts are swapped: the inverse transform runs as a forward
 // one, and leaves row A in the imaginary and row B in the real part.
 template <typename T, int L>
-__device__ __forceinline__ void load_rows_ct(cplx<T> (&x)[8], const cplx<T>* __restrict__ r, int j, int K) {
+__device__ __forceinline__ void load_rows_ct(cplx<T> (&x)[8], const cplx<T>* r, int j, int K) {
   constexpr int N = 1 << L, G = N / 8;
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
@@ -400,19 +400,19 @@ template <typename T> struct Bilin {
   }
 };
 template <typename T>
-__device__ __forceinline__ T bilinear(const T* __restrict__ f, int i, int j, T xi_x, T xi_y, T inv_dx, int N) {
+__device__ __forceinline__ T bilinear(const T* f, int i, int j, T xi_x, T xi_y, T inv_dx, int N) {
   const Bilin<T> b(i, j, xi_x, xi_y, inv_dx, N);
-  return fma(b.w11, __ldg(f + b.o11), fma(b.w10, __ldg(f + b.o10), fma(b.w01, __ldg(f + b.o01), mul_rn(b.w00, __ldg(f + b.o00)))));
+  return fma(b.w11, gld(f + b.o11), fma(b.w10, gld(f + b.o10), fma(b.w01, gld(f + b.o01), mul_rn(b.w00, gld(f + b.o00)))));
 }
 __device__ __forceinline__ void ld_quad(const float* p, float* v) {
-  const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+  const float4 q = gld(reinterpret_cast<const float4*>(p));
   v[0] = q.x;
   v[1] = q.y;
   v[2] = q.z;
   v[3] = q.w;
 }
 __device__ __forceinline__ void ld_quad(const double* p, double* v) {
-  const double2 a = __ldg(reinterpret_cast<const double2*>(p)), b = __ldg(reinterpret_cast<const double2*>(p) + 1);
+  const double2 a = gld(reinterpret_cast<const double2*>(p)), b = gld(reinterpret_cast<const double2*>(p) + 1);
   v[0] = a.x;
   v[1] = a.y;
   v[2] = b.x;

@@ -216,8 +216,8 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), sizeof(T) == 4 ? 1 
     const bool xf = L.scheme == SCHEME_XI_FIRST;
     const T inv_sg = xf ? (T)1 / (s + d.cdt) : inv_s;
     const T inv_dx = (T)N / (T)6.283185307179586476925286766559;
-    const cplx<T>* __restrict__ mix = d.mix + (long long)yp * 2 * g.KXP;
-    const T* __restrict__ phys = d.phys;
+    const cplx<T>* mix = d.mix + (long long)yp * 2 * g.KXP;
+    const T* phys = d.phys;
     const int rowoff = yp * 2 * N + j;
     const GRed gr = {red, 0};
     int w = 0;
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), sizeof(T) == 4 ? 1 
     auto base = [&](int f, int m) {
       if (fused || gath) return U[(f < 4 ? f : f - 1) * N + m * G];
       const T* p = phys + (long long)f * g.np + rowoff + m * G;
-      return mk<T>(__ldg(p), __ldg(p + N));
+      return mk<T>(gld(p), gld(p + N));
     };
 
     if (gath) {
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), sizeof(T) == 4 ? 1 
         const int o = y * N + xcol;
         T b[4], xi[2], f[4];
         ld_quad(phys + 4 * (long long)o, b);
-        const cplx<T> xv = __ldg(reinterpret_cast<const cplx<T>*>(phys + (long long)PH_XX * g.np) + o);
+        const cplx<T> xv = gld(reinterpret_cast<const cplx<T>*>(phys + (long long)PH_XX * g.np) + o);
         xi[0] = xv.x;
         xi[1] = xv.y;
         const Bilin<T> bl(xcol, y, xv.x, xv.y, inv_dx, N);
@@ -267,8 +267,8 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), sizeof(T) == 4 ? 1 
         dst[4 * 2 * N] = xi[0];
         dst[5 * 2 * N] = xi[1];
         if (L.has_q)
-          dst[10 * 2 * N] = fma(bl.w11, __ldg(Q + bl.o11), fma(bl.w10, __ldg(Q + bl.o10),
-                                fma(bl.w01, __ldg(Q + bl.o01), mul_rn(bl.w00, __ldg(Q + bl.o00)))));
+          dst[10 * 2 * N] = fma(bl.w11, gld(Q + bl.o11), fma(bl.w10, gld(Q + bl.o10),
+                                fma(bl.w01, gld(Q + bl.o01), mul_rn(bl.w00, gld(Q + bl.o00)))));
       }
       __syncthreads();
     }
@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), sizeof(T) == 4 ? 1 
           // bilinear interpolation, while the gradient rows arrive
           const bool cst = kind == PK_XI && kin;
           const T cv = pc == 0 ? adv_x : adv_y;
-          const T* __restrict__ gp = phys + (long long)pc * g.np;
+          const T* gp = phys + (long long)pc * g.np;
 #pragma unroll
           for (int m = 0; m < 8; ++m) {
             acc[m] = mk<T>(cv, cv);
