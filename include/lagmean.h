@@ -242,7 +242,8 @@ int sw_time(sw_handle* h, double* t);
 #define SW_K_ROW_INV 1  /* row pass: mixed -> physical base fields (u, v, h, zeta, xi) */
 #define SW_K_ROW_PROD 2 /* row pass: inverse x-FFT, products, forward x-FFT        */
 #define SW_K_COL_FWD 3  /* not reported (part of SW_K_COL_STAGE)                    */
-#define SW_K_UPDATE 4   /* not reported (part of SW_K_COL_STAGE)                    */
+#define SW_K_UPDATE 4   /* right-hand sides and update of runs without transforms   */
+                        /* (kinematic dynamics; else part of SW_K_COL_STAGE)        */
 #define SW_K_PHYS_Q 5   /* potential vorticity in the gather buffer (Strategy 2)    */
 #define SW_K_COL_STAGE 6 /* column pass: forward y-FFT and 2/3 mask, right-hand     */
                          /* sides and integrating-factor update, inverse y-FFT of   */

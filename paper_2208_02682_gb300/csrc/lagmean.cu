@@ -372,7 +372,7 @@ static const int GRAPH_STEPS = 8;
 static const long long ROW_WARPS = 1216;
 // column-stage blocks up to which blocks are split in two halves
 static const long long DUAL_BLOCKS = 456;
-static const int SW_K_OF_KT[KT_COUNT] = {SW_K_ROW_INV, SW_K_ROW_PROD, SW_K_COL_STAGE};
+static const int SW_K_OF_KT[KT_COUNT] = {SW_K_ROW_INV, SW_K_ROW_PROD, SW_K_COL_STAGE, SW_K_UPDATE};
 
 struct BatchExec {
   std::vector<sw_handle*> members;
@@ -459,7 +459,8 @@ static void fill_desc(sw_handle* h, RunDesc<T>& d, int points, int ppb, int lC, 
   d.gath = row_prod_gath<T>(g.N, L) && d.ppb >= L.np ? 1 : 0;
   d.nb[KT_ROW_INV] = L.np > 0 && !d.fused ? (L.strategy == 2 ? 5 : 3) * row_blocks(g.N, d.Bi) : 0;
   d.nb[KT_ROW_PROD] = row_blocks(g.N, d.Bp) * chunks;
-  d.nb[KT_COL_STAGE] = L.np > 0 ? ntile * d.L.nct : (int)((g.ms + KIN_MODES - 1) / KIN_MODES);
+  d.nb[KT_COL_STAGE] = L.np > 0 ? ntile * d.L.nct : 0;
+  d.nb[KT_KIN] = L.np > 0 ? 0 : (int)((g.ms + kin_modes(g.N) - 1) / kin_modes(g.N));
 }
 
 // Build (or rebuild) the descriptor table of a batch from its members.
@@ -569,26 +570,20 @@ static int batch_build_t(BatchExec* b) {
     const int halves = b->dual ? 2 : 1;
     const int cthr = (N << lC) / 8;
     const size_t csm = ((size_t)col_buf_stride<T>(N, 1 << lC) << lC) * cs;
-    const int thr[KT_COUNT] = {d.Bi * N / 8, d.Bp * W * N / 8, halves * cthr};
+    const int thr[KT_COUNT] = {d.Bi * N / 8, d.Bp * W * N / 8, halves * cthr, 256};
     const size_t sm[KT_COUNT] = {(size_t)2 * d.Bi * row_stride<T>(N) * cs,
-                                 row_prod_smem<T>(N, d.Bp, W, h->L, d.gath != 0), halves * csm + (size_t)6 * cthr * cs};
+                                 row_prod_smem<T>(N, d.Bp, W, h->L, d.gath != 0), halves * csm + (size_t)6 * cthr * cs, 0};
     const KBytes kb = kernel_bytes(h, h->L);
     if (h->L.np > 0) b->start_bytes += kb.col_inv;
-    const double by[KT_COUNT] = {kb.row_inv, kb.row_prod, 0.0};
+    const double by[KT_COUNT] = {kb.row_inv, kb.row_prod, 0.0, 0.0};
     for (int k = 0; k < KT_COUNT; ++k) {
       b->start[(size_t)k * (n + 1) + r + 1] = b->start[(size_t)k * (n + 1) + r] + d.nb[k];
       if (d.nb[k] == 0) continue;
-      if (h->L.np == 0) {
-        b->threads[k] = std::max(b->threads[k], 32);
-      } else {
-        b->threads[k] = thr[k];
-      }
+      b->threads[k] = thr[k];
       if (sm[k] > b->smem[k]) b->smem[k] = sm[k];
-      for (int st = 0; st < 4; ++st) b->bytes[k][st] += (k == KT_COL_STAGE ? kb.col_stage[st] : by[k]);
+      for (int st = 0; st < 4; ++st) b->bytes[k][st] += (k >= KT_COL_STAGE ? kb.col_stage[st] : by[k]);
     }
   }
-  // kinematic dynamics alone: pointwise blocks of any size
-  if (n > 0 && b->start_bytes == 0.0) b->threads[KT_COL_STAGE] = 128;
   const size_t desc_bytes = (sizeof(RunDesc<T>) * n + 255) & ~(size_t)255;
   const size_t need = desc_bytes + sizeof(int) * b->start.size();
   if (need > b->table_bytes) {
@@ -668,12 +663,12 @@ static cudaError_t enqueue_batch_start(BatchExec* b, cudaStream_t s, Prof* pf, i
 // state for the next one (not after the final step of a replay).
 template <typename T>
 static cudaError_t enqueue_batch_step(BatchExec* b, bool final_step, cudaStream_t s, Prof* pf, int64_t* nlaunch) {
-  static const int order[] = {KT_ROW_INV, KT_ROW_PROD, KT_COL_STAGE};
+  static const int order[] = {KT_ROW_INV, KT_ROW_PROD, KT_COL_STAGE, KT_KIN};
   for (int stage = 0; stage < b->nstages; ++stage) {
     // forward Euler's second pass only commits
     const bool commit_only = b->stepper == SW_STEP_EULER && stage == 1;
     for (int k : order) {
-      if (commit_only && k != KT_COL_STAGE) continue;
+      if (commit_only && k != KT_COL_STAGE && k != KT_KIN) continue;
       const bool fin = final_step && k == KT_COL_STAGE && stage == b->nstages - 1;
       const cudaError_t e = enqueue_kernel<T>(b, k, stage, fin, pf == nullptr, s, pf, nlaunch);
       if (e != cudaSuccess) return e;

@@ -185,6 +185,8 @@ cudaError_t launch_stage(int kt, const RunDesc<T>* runs, const int* start, int n
     case KT_ROW_PROD:
       return warp ? cudaLaunchKernelEx(&cfg, k_stage_row_prod<T, true>, runs, start, nruns, stage)
                   : cudaLaunchKernelEx(&cfg, k_stage_row_prod<T, false>, runs, start, nruns, stage);
+    case KT_KIN:
+      return cudaLaunchKernelEx(&cfg, k_stage_kin<T>, runs, start, nruns, stage);
     default:
       if (dual) return cudaLaunchKernelEx(&cfg, k_stage_col<T, DUAL_THREADS<T>(), true>, runs, start, nruns, stage);
       if constexpr (sizeof(T) == 4) {

@@ -8,14 +8,14 @@
 // are uniform within a launch: C*N (columns x points) and Bp*N, Bi*N (rows x
 // points) are equal for all members.
 //
-// Per stage:  [row_inv] -> row_prod -> col_stage;
-// a replay of steps starts with one col_stage that only transforms.
+// Per stage:  [row_inv] -> row_prod -> col_stage [-> kin, for runs without
+// transforms]; a replay of steps starts with one col_stage that only transforms.
 #pragma once
 #include "kernels.cuh"
 
 namespace lm {
 
-enum { KT_ROW_INV = 0, KT_ROW_PROD = 1, KT_COL_STAGE = 2, KT_COUNT = 3 };
+enum { KT_ROW_INV = 0, KT_ROW_PROD = 1, KT_COL_STAGE = 2, KT_KIN = 3, KT_COUNT = 4 };
 
 template <typename T>
 struct alignas(16) RunDesc {
@@ -490,42 +490,17 @@ __device__ __forceinline__ double to_real(int k, double) {
   return __hiloint2double(a ? (int)(hi | ((unsigned)k & 0x80000000u)) : 0, 0);
 }
 
-// The kinematic model's u, v and h when nothing is averaged (no products, so
-// no transforms): pointwise, KIN_MODES modes per block.
-constexpr int KIN_MODES = 512;
-template <typename T>
-__device__ __forceinline__ void kinematic_update(const RunDesc<T>& d, int stage, int lb) {
-  const int st = d.c.stepper, ms = (int)d.g.ms, NY = d.g.NY;
-  constexpr int CS = spec_tile<T>();
-  const bool last = stage == stage_count(st) - 1;
-  const T dt = d.cdt;
-  const cplx<T>* yin = stage_input(d, stage);
-  cplx<T>* yout = last ? d.y : (stage == 1 ? d.ysb : d.ysa);
-  for (int m = lb * KIN_MODES + threadIdx.x; m < min(ms, (lb + 1) * KIN_MODES); m += blockDim.x) {
-    const int tile = m / (NY * CS), e = m - tile * NY * CS;
-    const int kx = tile * CS + e % CS, ky = e / CS - d.g.K;
-    if (kx > d.g.K) continue;
-    const T kc = (T)kx * d.cadvx + (T)ky * d.cadvy;
-    for (int f = 0; f < 3; ++f) {
-      const int o = f * ms + m, cls = d.L.fclass[f];
-      const T* ef = d.ef + 3 * cls * ms + m;
-      const T e1 = cls == IF_NONE ? (T)1 : ef[0], ee = e1 * e1;
-      const cplx<T> rr = cik<T>(yin[o], -kc), yn = d.y[o];
-      if (last) {
-        const T ci = st == 0 ? dt / (T)6 : (st == 1 ? dt / (T)2 : (T)1);
-        const cplx<T> inc = st == 2 ? d.acc[o] : cscale<T>(cadd<T>(d.acc[o], rr), ci);
-        cplx<T> cc = mk<T>(0, 0);
-        d.y[o] = commit_mode<T>(false, cls == IF_NONE ? (T)1 : ef[ms], cls == IF_NONE ? (T)0 : ef[2 * ms], yn, cc, inc);
-      } else if (st == 2) {
-        d.acc[o] = cscale<T>(rr, dt * ee);
-      } else {
-        const T cr = stage == 0 ? ee : (T)2 * e1;
-        const T ca = st == 1 || stage == 2 ? ee : e1;
-        const T cb = st == 1 ? dt * ee : (stage == 0 ? (T)0.5 * dt * e1 : (stage == 1 ? (T)0.5 * dt : dt * e1));
-        const cplx<T> ac = stage == 0 ? mk<T>(0, 0) : d.acc[o];
-        d.acc[o] = mk<T>(fma(cr, rr.x, ac.x), fma(cr, rr.y, ac.y));
-        yout[o] = mk<T>(fma(ca, yn.x, cb * rr.x), fma(ca, yn.y, cb * rr.y));
-      }
+// The run's last block to finish its step advances the step counter (every block
+// of the run has read it before taking its ticket).
+template <typename T> __device__ __forceinline__ void finish_step(const RunDesc<T>& d, int kt) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned t = atomicAdd(d.ticket, 1u);
+    if (t == (unsigned)d.nb[kt] - 1u) {
+      *d.ticket = 0u;
+      *d.ctr = *d.ctr + 1;
+      __threadfence();
     }
   }
 }
@@ -564,10 +539,7 @@ __global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, DUAL>::BLOCKS) k_stage
   pdl_wait();  // state written by the previous kernels: only after this
   pdl_release();
   const int lb = blockIdx.x - start[r];
-  if (d.L.np == 0) {  // no transforms
-    if (stage >= 0) kinematic_update<T>(d, stage, lb);
-  }
-  else dispatch_L<ColShape<T, MAXT, DUAL>::LO, ColShape<T, MAXT, DUAL>::HI>(d.g.log2N, [&](auto Lc) {
+  dispatch_L<ColShape<T, MAXT, DUAL>::LO, ColShape<T, MAXT, DUAL>::HI>(d.g.log2N, [&](auto Lc) {
     constexpr int L = decltype(Lc)::value, N = 1 << L, G = N / 8;
     constexpr int NB = ColShape<T, MAXT, DUAL>::NB;
     const Layout& Y = d.L;
@@ -981,20 +953,103 @@ __global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, DUAL>::BLOCKS) k_stage
       }
     }
   });
-  if (stage == stage_count(d.c.stepper) - 1) {
-    // the run's last block to finish advances its step counter (every block
-    // of the run has read it above, before taking its ticket)
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      __threadfence();
-      const unsigned t = atomicAdd(d.ticket, 1u);
-      if (t == (unsigned)d.nb[KT_COL_STAGE] - 1u) {
-        *d.ticket = 0u;
-        *d.ctr = *d.ctr + 1;
-        __threadfence();
+  if (stage == stage_count(d.c.stepper) - 1) finish_step(d, KT_COL_STAGE);
+}
+
+// ---------------------------------------------------------------------------
+// The kinematic model's u, v and h when nothing is averaged: no products, so no
+// transforms, one pointwise pass per stage.  Bound by FP64 issue or memory (large
+// grids) or by the launch (small ones): a thread takes the three fields of a mode
+// (one wavenumber and one set of coefficients for them, their loads issued
+// together), one mode up to 512^2 (short chains, many blocks), two above; no
+// shared memory and at most 80 registers.  A step, as blocks of the column stage
+// (255 registers in FP64, its exchange buffers allocated) -> this: @@
+__host__ __device__ __forceinline__ int kin_modes(int N) { return N >= 1024 ? 512 : 256; }
+template <typename T>
+__global__ void __launch_bounds__(256, 3) k_stage_kin(const RunDesc<T>* __restrict__ runs,
+                                                      const int* __restrict__ start, int nruns, int stage) {
+  const int r = find_run(start, nruns, blockIdx.x);
+  const RunDesc<T>& d = runs[r];
+  const int st = d.c.stepper, ms = (int)d.g.ms, NY = d.g.NY, K = d.g.K, per = kin_modes(d.g.N);
+  constexpr int CS = spec_tile<T>();
+  const bool last = stage == stage_count(st) - 1;
+  const int m0 = (blockIdx.x - start[r]) * per, m1 = min(ms, m0 + per);
+  // u and v are of class IF_DYN; h too, or undamped
+  const bool hdamped = d.L.fclass[2] != IF_NONE;
+  const T* const ef = d.ef;
+  const T dt = d.cdt, ax = d.cadvx, ay = d.cadvy;
+  const cplx<T>* const yin = stage_input(d, stage);
+  cplx<T>* const yout = stage == 1 ? d.ysb : d.ysa;
+  cplx<T>* const y = d.y;
+  cplx<T>* const acc = d.acc;
+  // acc' = [acc +] cr rhs, y' = ca y_n + cb rhs (see k_stage_col)
+  struct Coef { T cr, ca, cb; };
+  const T hdt = (T)0.5 * dt;
+  auto coef = [&](T e1) {
+    Coef c;
+    if (st != 0) {
+      c.cr = c.ca = e1 * e1;
+      c.cb = dt * c.ca;
+    } else if (stage == 0) {
+      c.cr = e1 * e1;
+      c.ca = e1;
+      c.cb = hdt * e1;
+    } else {
+      c.cr = (T)2 * e1;
+      c.ca = stage == 1 ? e1 : e1 * e1;
+      c.cb = stage == 1 ? hdt : dt * e1;
+    }
+    return c;
+  };
+  const T ci = st == 0 ? dt / (T)6 : dt / (T)2;
+  const bool radd = !last || st != 2;              // the stage adds a right-hand side
+  const bool racc = last || (st == 0 && stage > 0);  // acc is read
+  pdl_wait();  // state written by the previous kernels: only after this
+  pdl_release();
+  for (int m = m0 + threadIdx.x; m < m1; m += blockDim.x) {
+    const int tile = m / (NY * CS), e = m - tile * NY * CS;
+    const int kx = tile * CS + e % CS, ky = e / CS - K;
+    if (kx > K) continue;
+    cplx<T> yn[3], rr[3], ac[3];
+    T e1[2] = {(T)1, (T)0};  // E, or E^2 as hi + lo at the commit
+    if (last) {
+      e1[0] = ef[ms + m];
+      e1[1] = ef[2 * ms + m];
+    } else {
+      e1[0] = ef[m];
+    }
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+      yn[f] = y[f * ms + m];
+      rr[f] = ac[f] = mk<T>(0, 0);
+      if (radd) rr[f] = yin[f * ms + m];
+      if (racc) ac[f] = acc[f * ms + m];
+    }
+    const T kc = to_real(kx, (T)0) * ax + to_real(ky, (T)0) * ay;
+    if (last) {
+#pragma unroll
+      for (int f = 0; f < 3; ++f) {
+        const bool dm = f < 2 || hdamped;
+        const cplx<T> inc = st == 2 ? ac[f] : cscale<T>(cadd<T>(ac[f], cik<T>(rr[f], -kc)), ci);
+        cplx<T> cc = mk<T>(0, 0);
+        y[f * ms + m] = commit_mode<T>(false, dm ? e1[0] : (T)1, dm ? e1[1] : (T)0, yn[f], cc, inc);
+      }
+    } else {
+      const Coef c0 = coef(e1[0]), ch = hdamped ? c0 : coef((T)1);
+#pragma unroll
+      for (int f = 0; f < 3; ++f) {
+        const Coef c = f < 2 ? c0 : ch;
+        const cplx<T> q = cik<T>(rr[f], -kc);
+        if (st == 2) {
+          acc[f * ms + m] = cscale<T>(q, c.cb);
+        } else {
+          acc[f * ms + m] = mk<T>(fma(c.cr, q.x, ac[f].x), fma(c.cr, q.y, ac[f].y));
+          yout[f * ms + m] = mk<T>(fma(c.ca, yn[f].x, c.cb * q.x), fma(c.ca, yn[f].y, c.cb * q.y));
+        }
       }
     }
   }
+  if (last) finish_step(d, KT_KIN);
 }
 
 }  // namespace lm
