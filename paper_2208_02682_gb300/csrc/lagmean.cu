@@ -1296,6 +1296,20 @@ struct BlobHeader {
   int64_t done, steps_total;
 };
 
+// The state's nf fields and compensation terms from (to_rows) or to rows
+// [ky + K][kx], as blobs hold them, in the mixed fields' buffer, which the next
+// replay fills anew (2 x 16 spectral fields of 2K + 1 < 2N/3 rows fit in its 24
+// fields of N rows).
+static_assert(2 * MAXF * 2 <= 3 * MAXI, "blob staging");
+static int spec_rows(sw_handle* h, int nf, bool to_rows) {
+  if (h->fp32)
+    CK(h, launch_spec_rows<float>((float2*)h->y, (float2*)h->comp, (float2*)h->mix, h->g, nf, to_rows, h->stream));
+  else
+    CK(h, launch_spec_rows<double>((double2*)h->y, (double2*)h->comp, (double2*)h->mix, h->g, nf, to_rows, h->stream));
+  h->launches += 1;
+  return SW_OK;
+}
+
 static size_t blob_size(sw_handle* h, int nf) {
   return sizeof(BlobHeader) + (size_t)2 * nf * h->g.ms * 2 * h->tsz;
 }
@@ -1325,16 +1339,8 @@ extern "C" int sw_get_state(sw_handle* h, void* blob, size_t* size) {
   hd.done = h->done;
   hd.steps_total = h->steps_total;
   std::memcpy(blob, &hd, sizeof(hd));
-  const size_t fb = (size_t)nf * h->g.ms * 2 * h->tsz;
-  char* dst = (char*)blob + sizeof(hd);
-  // blobs hold rows [ky + K][kx] (through the mixed fields' buffer, which the
-  // next replay fills anew)
-  for (int k = 0; k < 2; ++k) {
-    const void* src = k == 0 ? h->y : h->comp;
-    if (h->fp32) CK(h, launch_spec_rows<float>((const float2*)src, (float2*)h->mix, h->g, nf, true, h->stream));
-    else CK(h, launch_spec_rows<double>((const double2*)src, (double2*)h->mix, h->g, nf, true, h->stream));
-    CK(h, cudaMemcpyAsync(dst + k * fb, h->mix, fb, cudaMemcpyDeviceToHost, h->stream));
-  }
+  if (const int rc = spec_rows(h, nf, true)) return rc;
+  CK(h, cudaMemcpyAsync((char*)blob + sizeof(hd), h->mix, need - sizeof(hd), cudaMemcpyDeviceToHost, h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
   *size = need;
   return SW_OK;
@@ -1354,14 +1360,9 @@ extern "C" int sw_set_state(sw_handle* h, const void* blob, size_t size) {
   Layout L = hd.lm_open ? build_layout(h->p, hd.lp.strategy, hd.lp.fields, hd.lp.eulerian, hd.lp.scheme)
                         : build_layout(h->p, 0, 0, 0);
   if (L.nf != hd.nf || size < blob_size(h, hd.nf)) return fail(h, SW_EINVAL, "blob size mismatch");
-  const size_t fb = (size_t)hd.nf * h->g.ms * 2 * h->tsz;
-  const char* src = (const char*)blob + sizeof(hd);
-  for (int k = 0; k < 2; ++k) {
-    void* dst = k == 0 ? h->y : h->comp;
-    CK(h, cudaMemcpyAsync(h->mix, src + k * fb, fb, cudaMemcpyHostToDevice, h->stream));
-    if (h->fp32) CK(h, launch_spec_rows<float>((const float2*)h->mix, (float2*)dst, h->g, hd.nf, false, h->stream));
-    else CK(h, launch_spec_rows<double>((const double2*)h->mix, (double2*)dst, h->g, hd.nf, false, h->stream));
-  }
+  CK(h, cudaMemcpyAsync(h->mix, (const char*)blob + sizeof(hd), blob_size(h, hd.nf) - sizeof(hd),
+                        cudaMemcpyHostToDevice, h->stream));
+  if (const int rc = spec_rows(h, hd.nf, false)) return rc;
   long long ctr = hd.done;
   CK(h, cudaMemcpyAsync(h->ctr, &ctr, sizeof(ctr), cudaMemcpyHostToDevice, h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
