@@ -1266,7 +1266,7 @@ extern "C" int sw_diag(sw_handle* h, double out[3]) {
   if (rc) return rc;
   const Geom& g = h->g;
   CK(h, launch_diag(h->out64, g.np, h->p.f0, h->p.c2, h->part, h->diag_blocks, h->dres, h->stream));
-  h->launches += 5;
+  h->launches += 2;  // (phys_uvhz counts its own)
   double res[4] = {0, 0, 0, 0};
   CK(h, cudaMemcpyAsync(res, h->dres, 3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   // mass: the k = 0 coefficient of h (row ky = 0, column kx = 0)
