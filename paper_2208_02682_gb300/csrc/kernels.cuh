@@ -599,11 +599,13 @@ __global__ void __launch_bounds__(256) k_in_col(const __grid_constant__ InArgs<T
 
 // Copy of nf fields of the state (t0) and of their compensation terms (t1)
 // between the tile-blocked layout and rows [ky + K][kx] (checkpoint blobs: the
-// fields of t0, then those of t1); to_rows: rows get the copy.
+// fields of t0, then those of t1); to_rows: rows get the copy, else the step
+// counter ctr is set to `done` too.
 template <typename T>
 __global__ void k_spec_rows(cplx<T>* __restrict__ t0, cplx<T>* __restrict__ t1, cplx<T>* __restrict__ rows, Geom g,
-                            int nf, int to_rows) {
+                            int nf, int to_rows, long long* ctr, long long done) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0 && !to_rows) *ctr = done;
   if (i >= g.ms * 2 * nf) return;
   const int f = (int)(i / g.ms), m = (int)(i - f * g.ms);
   cplx<T>* t = (f < nf ? t0 + f * g.ms : t1 + (f - nf) * g.ms) + spec_index<T>(m / g.KXP, m % g.KXP, g.NY);

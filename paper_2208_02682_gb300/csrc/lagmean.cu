@@ -1298,14 +1298,16 @@ struct BlobHeader {
 
 // The state's nf fields and compensation terms from (to_rows) or to rows
 // [ky + K][kx], as blobs hold them, in the mixed fields' buffer, which the next
-// replay fills anew (2 x 16 spectral fields of 2K + 1 < 2N/3 rows fit in its 24
-// fields of N rows).
+// replay fills anew; from rows, the step counter too.  (2 x 16 spectral fields
+// of 2K + 1 < 2N/3 rows fit in its 24 fields of N rows.)
 static_assert(2 * MAXF * 2 <= 3 * MAXI, "blob staging");
-static int spec_rows(sw_handle* h, int nf, bool to_rows) {
+static int spec_rows(sw_handle* h, int nf, bool to_rows, long long done = 0) {
   if (h->fp32)
-    CK(h, launch_spec_rows<float>((float2*)h->y, (float2*)h->comp, (float2*)h->mix, h->g, nf, to_rows, h->stream));
+    CK(h, launch_spec_rows<float>((float2*)h->y, (float2*)h->comp, (float2*)h->mix, h->g, nf, to_rows, h->ctr, done,
+                                  h->stream));
   else
-    CK(h, launch_spec_rows<double>((double2*)h->y, (double2*)h->comp, (double2*)h->mix, h->g, nf, to_rows, h->stream));
+    CK(h, launch_spec_rows<double>((double2*)h->y, (double2*)h->comp, (double2*)h->mix, h->g, nf, to_rows, h->ctr, done,
+                                   h->stream));
   h->launches += 1;
   return SW_OK;
 }
@@ -1362,9 +1364,7 @@ extern "C" int sw_set_state(sw_handle* h, const void* blob, size_t size) {
   if (L.nf != hd.nf || size < blob_size(h, hd.nf)) return fail(h, SW_EINVAL, "blob size mismatch");
   CK(h, cudaMemcpyAsync(h->mix, (const char*)blob + sizeof(hd), blob_size(h, hd.nf) - sizeof(hd),
                         cudaMemcpyHostToDevice, h->stream));
-  if (const int rc = spec_rows(h, hd.nf, false)) return rc;
-  long long ctr = hd.done;
-  CK(h, cudaMemcpyAsync(h->ctr, &ctr, sizeof(ctr), cudaMemcpyHostToDevice, h->stream));
+  if (const int rc = spec_rows(h, hd.nf, false, hd.done)) return rc;
   CK(h, cudaStreamSynchronize(h->stream));
   set_layout(h, L);
   h->lm_open = hd.lm_open != 0;

@@ -78,7 +78,7 @@ template <typename T> cudaError_t launch_out(const OutArgs<T>& a, cudaStream_t s
 template <typename T> cudaError_t launch_in(const InArgs<T>& a, cudaStream_t s);
 template <typename T>
 cudaError_t launch_spec_rows(cplx<T>* t0, cplx<T>* t1, cplx<T>* rows, const Geom& g, int nf, bool to_rows,
-                             cudaStream_t s);
+                             long long* ctr, long long done, cudaStream_t s);
 template <typename T>
 cudaError_t launch_velocity_from_vorticity(cplx<T>* y, const Geom& g, int fu, int fv, int fh, cudaStream_t s);
 cudaError_t launch_diag(const double* phys, long long np, double f0, double c2, double* part, int nblk,
@@ -228,8 +228,8 @@ template <typename T> cudaError_t launch_in(const InArgs<T>& a, cudaStream_t s) 
 
 template <typename T>
 cudaError_t launch_spec_rows(cplx<T>* t0, cplx<T>* t1, cplx<T>* rows, const Geom& g, int nf, bool to_rows,
-                             cudaStream_t s) {
-  k_spec_rows<T><<<(unsigned)((g.ms * 2 * nf + 255) / 256), 256, 0, s>>>(t0, t1, rows, g, nf, to_rows ? 1 : 0);
+                             long long* ctr, long long done, cudaStream_t s) {
+  k_spec_rows<T><<<(unsigned)((g.ms * 2 * nf + 255) / 256), 256, 0, s>>>(t0, t1, rows, g, nf, to_rows ? 1 : 0, ctr, done);
   return cudaGetLastError();
 }
 
@@ -244,7 +244,8 @@ cudaError_t launch_velocity_from_vorticity(cplx<T>* y, const Geom& g, int fu, in
                                        bool, bool, cudaStream_t);                                           \
   template cudaError_t launch_out<T>(const OutArgs<T>&, cudaStream_t);                                       \
   template cudaError_t launch_in<T>(const InArgs<T>&, cudaStream_t);                                         \
-  template cudaError_t launch_spec_rows<T>(cplx<T>*, cplx<T>*, cplx<T>*, const Geom&, int, bool, cudaStream_t); \
+  template cudaError_t launch_spec_rows<T>(cplx<T>*, cplx<T>*, cplx<T>*, const Geom&, int, bool, long long*, long long,   \
+                                           cudaStream_t);                                                    \
   template cudaError_t launch_velocity_from_vorticity<T>(cplx<T>*, const Geom&, int, int, int, cudaStream_t);
 // the generic FP64 transforms (csrc/project_static.cu)
 #define LM_INSTANTIATE_GENERIC                                                                              \
