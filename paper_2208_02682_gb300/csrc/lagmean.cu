@@ -368,8 +368,9 @@ struct Prof {
 // Batch executor: the device table of run descriptors, per-kernel block
 // prefix sums and the captured step graphs for a set of handles.
 static const int GRAPH_STEPS = 8;
+static const long long SMS = 152;  // of a GB300
 // warps in the row pass below which its products are split over blocks
-static const long long ROW_WARPS = 1216;
+static const long long ROW_WARPS = 8 * SMS;
 // column-stage blocks up to which blocks are split in two halves
 static const long long DUAL_BLOCKS = 456;
 static const int SW_K_OF_KT[KT_COUNT] = {SW_K_ROW_INV, SW_K_ROW_PROD, SW_K_COL_STAGE, SW_K_UPDATE};
@@ -446,7 +447,7 @@ static void fill_desc(sw_handle* h, RunDesc<T>& d, int points, int ppb, int lC, 
   d.Bp = row_block_pairs(g.N, points);
   d.ppb = ppb < L.np || L.np == 0 ? ppb : L.np;
   d.Wp = 1;
-  d.Bi = row_block_pairs(g.N, points > 512 ? points : 512);
+  d.Bi = row_inv_pairs(g.N, points);
   const int ntile = g.KXP >> lC;
   const int chunks = L.np > 0 ? (L.np + d.ppb - 1) / d.ppb : 0;
   for (int q = 0; q < L.np; ++q) {
@@ -540,6 +541,18 @@ static int batch_build_t(BatchExec* b) {
   // fewer warps than ROW_WARPS (about 8 per SM): the products are split over
   // blocks, each transforming the base fields its products need
   const int chunks = warps > 0 ? (int)std::min<long long>(MAXP, (ROW_WARPS + warps - 1) / warps) : 1;
+  auto products = [&](const sw_handle* h) {
+    return h->ppb != 0 ? h->ppb : std::max(1, (h->L.np + chunks - 1) / chunks);
+  };
+  bool team = warps > 0;
+  long long team_blocks = 0;
+  for (int r = 0; r < n; ++r) {
+    const sw_handle* h = b->members[r];
+    if (h->L.np == 0) continue;
+    team = team && row_team<T>(h->g.N, points, products(h));
+    team_blocks += (long long)row_blocks(h->g.N, row_block_pairs(h->g.N, points)) * h->L.np;
+  }
+  team = team && team_blocks <= SMS * row_team_blocks<T>();
   // column tiles: the narrowest that still move whole 32-byte sectors (4 FP32
   // or 2 FP64 columns of the largest grid, 1 at 2048^2 in FP64), at least a
   // warp per block; the same points per block for every member.  Narrow tiles
@@ -563,16 +576,18 @@ static int batch_build_t(BatchExec* b) {
     // automatic pairs per block: all of them when the row's groups share
     // them out or the grid has rows enough to fill the GPU (N >= 1024), else
     // one (the row's pairs spread over blocks)
-    fill_desc<T>(h, descs[r], points, h->ppb != 0 ? h->ppb : std::max(1, (h->L.np + chunks - 1) / chunks), lC, b->dual);
-    descs[r].Wp = W;
+    fill_desc<T>(h, descs[r], points, products(h), lC, b->dual);
+    descs[r].Wp = team ? 4 : W;
+    descs[r].team = team ? 1 : 0;
     const RunDesc<T>& d = descs[r];
     const int N = h->g.N;
     const int halves = b->dual ? 2 : 1;
     const int cthr = (N << lC) / 8;
     const size_t csm = ((size_t)col_buf_stride<T>(N, 1 << lC) << lC) * cs;
-    const int thr[KT_COUNT] = {d.Bi * N / 8, d.Bp * W * N / 8, halves * cthr, 256};
-    const size_t sm[KT_COUNT] = {(size_t)2 * d.Bi * row_stride<T>(N) * cs,
-                                 row_prod_smem<T>(N, d.Bp, W, h->L, d.gath != 0), halves * csm + (size_t)6 * cthr * cs, 0};
+    const int sets = team ? 4 : 1;
+    const int thr[KT_COUNT] = {sets * d.Bi * N / 8, d.Bp * d.Wp * N / 8, halves * cthr, 256};
+    const size_t sm[KT_COUNT] = {(size_t)sets * 2 * d.Bi * row_stride<T>(N) * cs,
+                                 row_prod_smem<T>(N, d.Bp, d.Wp, h->L, d.gath != 0), halves * csm + (size_t)6 * cthr * cs, 0};
     const KBytes kb = kernel_bytes(h, h->L);
     if (h->L.np > 0) b->start_bytes += kb.col_inv;
     const double by[KT_COUNT] = {kb.row_inv, kb.row_prod, 0.0, 0.0};

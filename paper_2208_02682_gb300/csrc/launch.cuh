@@ -44,7 +44,7 @@ template <typename T> size_t row_prod_smem(int N, int B, int W, const Layout& L,
   return (size_t)B * sizeof(cplx<T>) * (nu * N + (size_t)W * 2 * row_stride<T>(N));
 }
 
-// Largest W for B row pairs and np products per block: W > 1 needs whole
+// Largest W for B row pairs and np products per block (other than a team): W > 1 needs whole
 // warps per group (N >= 256), a thread count within the block limit, at most
 // 15 named barriers (groups of N >= 512) and at most 200 KB of shared memory.
 template <typename T> int row_prod_groups(int N, int B, int np, const Layout& L) {
@@ -58,6 +58,23 @@ template <typename T> int row_prod_groups(int N, int B, int np, const Layout& L)
   // two blocks per SM, or one of several groups where that leaves one group
   const int W = fit(sizeof(T) == 4 ? 384 : 256, (size_t)110 * 1024);
   return W > 1 ? W : fit(row_prod_max_threads<T>(), (size_t)200 * 1024);
+}
+
+// Row pairs per block of the row inverse pass.
+inline int row_inv_pairs(int N, int points) { return row_block_pairs(N, points > 512 ? points : 512); }
+
+// Row passes by teams of four sets of groups per row pair (see
+// k_stage_row_prod): one product per block, groups within a warp, few enough row
+// pairs for the block, and all blocks resident at once, row_team_blocks() per SM (by
+// registers), since a team's blocks hold four times the warps.  A step, without -> with
+// teams: FP64 16^2 Strategy 2 239 -> 173 us, 64^2 Strategy 1 168 -> 141, four 64^2 runs 191 ->
+// 157; FP32 64^2 Strategy 1 54 -> 45.  Beyond: 16 64^2 runs' dynamics in FP64 (640 blocks)
+// 166 against 180, 32 in FP32 (1280) 68 against 76.
+template <typename T> constexpr int row_team_blocks() { return sizeof(T) == 4 ? 6 : 4; }
+template <typename T> bool row_team(int N, int points, int ppb) {
+  const int G = N / 8;
+  return G < 32 && ppb == 1 && 4 * row_block_pairs(N, points) * G <= row_prod_max_threads<T>() &&
+         4 * row_inv_pairs(N, points) * G <= 256;
 }
 
 template <typename T> constexpr int DUAL_THREADS() { return sizeof(T) == 4 ? 256 : 128; }

@@ -38,6 +38,7 @@ struct alignas(16) RunDesc {
   int lC;         // column tile: C = 2^lC columns
   int Bp, ppb;    // row_prod: row pairs per block, products per block
   int Wp;         // row_prod: groups of N/8 threads per row pair
+  int team;       // row_inv, row_prod: a team of four sets of groups per row pair
   int Bi;         // row_inv: row pairs per block
   int fused;      // row_prod: transforms the base fields itself
   int gath;       // row_prod: gathers all fields at x + xi at once (interleaved planes)
@@ -102,14 +103,16 @@ __global__ void __launch_bounds__(256) k_stage_row_inv(const RunDesc<T>* __restr
     const int nrb = max(N / 2 / B, 1);
     const int f = lb / nrb, rb = lb - f * nrb;
     const int grp = threadIdx.x / G, j = threadIdx.x - grp * G;
-    const int yp = (rb * B + grp) & (N / 2 - 1);
+    const bool team = G < 32 && d.team != 0;
+    const int set = team ? grp / B : 0, row = grp - set * B;
+    const int yp = (rb * B + row) & (N / 2 - 1);
     constexpr int rs = N + N / 8;
     cplx<T>* buf0 = reinterpret_cast<cplx<T>*>(smem_raw) + (size_t)grp * 2 * rs;
     cplx<T> x[8], eta[8];
     int w = 0;
     const bool hz = f == 2;
 #pragma unroll 1
-    for (int part = 0; part < (hz ? 2 : 1); ++part) {
+    for (int part = set; part < (hz ? (set ? 2 : (team ? 1 : 2)) : 1); ++part) {
       const int src = f == 0 ? d.L.i_u : (f == 1 ? d.L.i_v : (hz ? (part ? d.L.i_z : d.L.i_h) : d.L.i_xi[f - 3]));
       const int dst = f < 2 ? f : (hz ? (part ? PH_Z : PH_H) : f - 3 + PH_XX);
       load_rows_ct<T, L>(x, d.mix + (long long)src * g.mi + (long long)yp * 2 * g.KXP, j, g.K);
@@ -129,7 +132,24 @@ __global__ void __launch_bounds__(256) k_stage_row_inv(const RunDesc<T>* __restr
         for (int m = 0; m < 8; ++m) eta[m] = x[m];
       }
     }
-    if (hz && d.L.has_q) {
+    if (team && hz && d.L.has_q) {
+      // eta and zeta to the four sets, two of the eight positions each
+      cplx<T>* E = reinterpret_cast<cplx<T>*>(smem_raw) + (size_t)(2 * B + row) * 2 * rs + j;
+      cplx<T>* Z = E + (size_t)B * 2 * rs;
+      if (set < 2) {
+#pragma unroll
+        for (int m = 0; m < 8; ++m) (set ? Z : E)[m * G] = x[m];
+      }
+      __syncthreads();
+      T* p = d.phys + (long long)PH_Q * g.np + (long long)yp * 2 * N + j;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int m = 2 * set + i;
+        const cplx<T> z = Z[m * G], e = E[m * G];
+        p[m * G] = (d.cf0 + z.y) / ((T)1 + e.y);
+        p[N + m * G] = (d.cf0 + z.x) / ((T)1 + e.x);
+      }
+    } else if (hz && d.L.has_q) {
       T* p = d.phys + (long long)PH_Q * g.np + (long long)yp * 2 * N + j;
 #pragma unroll
       for (int m = 0; m < 8; ++m) {
@@ -163,8 +183,15 @@ __global__ void __launch_bounds__(256) k_stage_row_inv(const RunDesc<T>* __restr
 // u d_x G + v d_y G; one transform instance serves both directions (the
 // inverse as a forward transform of swapped parts), which keeps the code
 // within the instruction caches.
-// Wp > 1 only when a group is a whole number of warps (N >= 256), so groups
-// that do different numbers of transforms never share a warp barrier.
+// Groups that do different numbers of transforms never share a warp barrier:
+// Wp > 1 only when a group is a whole number of warps (N >= 256), or for a `team`.
+// Team: while a small grid (N <= 128) leaves most of the GPU idle a launch is as long
+// as one block's chain of dependent transforms and of the pointwise work of a lone
+// warp (in FP64 64 clocks an instruction), so a block takes one product with four
+// sets of groups, a warp or more each: the base fields side by side, then set 0 d_x and
+// the forward transform, set 1 d_y, sets 2 and 3 (Strategy 2) the gather of a row each.
+// An advection product's chain is three transforms instead of five, a Strategy-2
+// product's two instead of three and the gather (16^2 FP64 alone: 34 -> 17.5 us).
 // Smem: per pair row_prod_planes() arrays of N complex (fused: the base
 // fields; gath: these, xi and the fields at x + xi); per group two
 // exchange buffers of row_stride(N) complex.
@@ -200,7 +227,13 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), sizeof(T) == 4 ? 1 
     const int nrb = max(N / 2 / B, 1);
     const int pg = lb / nrb, rb = lb - pg * nrb;
     const int gi = threadIdx.x / G, j = threadIdx.x - gi * G;
-    const int row = gi / W, wg = gi - row * W;
+    // sets of groups: whole warps each for a team, neighbours otherwise
+    const bool team = G < 32 && d.team != 0;
+    int row = gi / W, wg = gi - row * W;
+    if (team) {
+      wg = gi / B;
+      row = gi - wg * B;
+    }
     const int yp = (rb * B + row) & (N / 2 - 1);  // row pair (2 yp, 2 yp + 1)
     const bool fused = d.fused != 0, gath = d.gath != 0, kin = L.model == 1;
     const int nu = row_prod_planes(d.fused, d.gath, L.has_q);
@@ -276,9 +309,15 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), sizeof(T) == 4 ? 1 
     // a group's transforms, one loop iteration each: the base fields of the
     // pair (fused; group wg takes fields wg, wg + W, ...), then for each
     // of its products the inverse transforms of two gradients (advection and
-    // Strategy-2 products) and the forward transform of the product
+    // Strategy-2 products) and the forward transform of the product.  A team
+    // shares its one product: set 0 takes d_x and the forward transform, set 1 d_y,
+    // and, Strategy 2, sets 2 and 3 the values at x + xi of the two rows; set 0
+    // gets theirs through the exchange buffers of sets 2 and 3.
+    const bool shared = team && product_heavy(L.pk[p0]);
+    cplx<T>* const XY = buf0 + (size_t)(2 - wg) * B * 2 * rs + j;  // set 1's transform
+    cplx<T>* const XA = buf0 + (size_t)(3 - wg) * B * 2 * rs + j;  // values at x + xi
     int f = fused ? wg : 4;       // next base field
-    int p = p0 + wg, sub = 0;     // next product and its part
+    int p = shared ? p0 : p0 + wg, sub = shared ? wg : 0;  // next product and its part
     bool basing = true;
     while (true) {
       if (basing && f >= 4) {
@@ -288,6 +327,19 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), sizeof(T) == 4 ? 1 
       if (!basing && p >= p1) break;
       const int kind = L.pk[min(p, p1 - 1)], pc = L.pc[min(p, p1 - 1)];
       const bool heavy = product_heavy(kind);
+      if (shared && !basing && sub >= 2 && wg >= 2) {
+        if (kind == PK_GBAR || (kind == PK_XI && !kin)) {
+          const int rr = wg - 2;
+          const T* gp = phys + (long long)pc * g.np;
+          const T* xp = phys + (long long)PH_XX * g.np + rowoff + rr * N;
+          T* dst = reinterpret_cast<T*>(XA) + rr;
+#pragma unroll
+          for (int m = 0; m < 8; ++m)
+            dst[2 * m * G] = bilinear<T>(gp, m * G + j, 2 * yp + rr, gld(xp + m * G), gld(xp + g.np + m * G), inv_dx, N);
+        }
+        __syncthreads();
+        break;
+      }
       const bool inv = basing || (heavy && sub < 2);
       if (inv) {
         if (basing && !(d.umask[pg] >> f & 1)) {
@@ -297,7 +349,7 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), sizeof(T) == 4 ? 1 
         const int src = basing ? (f == 0 ? L.i_u : (f == 1 ? L.i_v : (f == 2 ? L.i_h : L.i_z)))
                                : (sub == 0 ? L.pa[p] : L.pb[p]);
         load_rows_ct<T, L_>(x, mix + (long long)src * g.mi, j, g.K);
-        if (!basing && sub == 0 && kind != PK_ADV) {
+        if (!basing && sub == 0 && kind != PK_ADV && !shared) {
           // Strategy 2: the values at x + xi (Eqs. xi_evol, barf_xi), by
           // bilinear interpolation, while the gradient rows arrive
           const bool cst = kind == PK_XI && kin;
@@ -350,8 +402,28 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), sizeof(T) == 4 ? 1 
         p += W;
         sub = 0;
       } else {
-        const bool second = sub == 1;
-        ++sub;
+        if (shared) {
+          if (wg == 1) {
+#pragma unroll
+            for (int m = 0; m < 8; ++m) XY[m * G] = x[m];
+          }
+          __syncthreads();
+          if (wg == 1) break;
+          if (kind != PK_ADV) {
+            const T cv = pc == 0 ? adv_x : adv_y;
+#pragma unroll
+            for (int m = 0; m < 8; ++m) acc[m] = kind == PK_XI && kin ? mk<T>(cv, cv) : XA[m * G];
+          }
+        }
+        const int from = sub;
+        sub = shared ? 2 : sub + 1;
+#pragma unroll 1
+        for (int part = from; part < sub; ++part) {
+        const bool second = part == 1;
+        if (shared && second) {
+#pragma unroll
+          for (int m = 0; m < 8; ++m) x[m] = XY[m * G];
+        }
         if (kind == PK_ADV) {
           // u.grad G (Eq. gtilde-evol) or u.grad D
           const T av = second ? adv_y : adv_x;
@@ -386,6 +458,7 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), sizeof(T) == 4 ? 1 
             }
             acc[m] = a;
           }
+        }
         }
       }
     }
