@@ -217,8 +217,8 @@ enum { CT_UV = 0, CT_E2 = 1, CT_KIN = 2, CT_H = 3, CT_G = 4, CT_P = 5, MAXCT = 1
 // CA_UPD; CA_UPD_PARK: the new value is parked too); with op = OP_* the inverse
 // transform of op(value) into mixed field `prod`, the value being what the
 // update before left (CA_X), the parked one (CA_PARKED) or that of field `fld`
-// in memory (CA_MEM).  half: which half of the block takes the step when the
-// block is split; bar: a block barrier comes before it then.
+// in memory (CA_MEM).  part: which part of the block takes the step when the
+// block is split in halves or quarters; bar: a block barrier comes before it then.
 enum {
   CA_PARK = 0, CA_U = 1, CA_V = 2, CA_UPD = 3, CA_UPD_PARK = 4, CA_X = 5, CA_PARKED = 6, CA_MEM = 7, CA_KEEP = 8,
   MAXCS = 8
@@ -229,7 +229,7 @@ enum {
 struct ColTask {
   signed char kind, slot;  // CT_*; mean-field slot or component
   signed char n;
-  signed char prod[MAXCS], act[MAXCS], op[MAXCS], fld[MAXCS], half[MAXCS], bar[MAXCS];
+  signed char prod[MAXCS], act[MAXCS], op[MAXCS], fld[MAXCS], part[MAXCS], bar[MAXCS];
 };
 // role of an evolved field in the right-hand side
 enum { R_U = 0, R_V = 1, R_H = 2, R_G = 3, R_P = 4, R_E = 5 };

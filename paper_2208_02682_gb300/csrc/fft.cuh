@@ -199,19 +199,22 @@ __device__ __forceinline__ void dft_r(cplx<T>* v) {
 // table holds w^0 = 1 there; the product is exact).
 // SYNC: 0 the warp (G <= 32: several groups per warp execute the same
 // instructions), 1 named barrier grp + 1 over the group's G threads, 2 the
-// block (groups whose threads interleave, column tiles), 3 half grp of the
-// block (the same, two sets of them).  A named barrier
+// block (groups whose threads interleave, column tiles), 3 and 4 half or
+// quarter grp of the block (the same, two or four sets of them).  A named barrier
 // with a run-time id reserves all 16 of a block's barriers, which limits the
 // blocks resident on an SM, so kernels whose groups all fit in a warp are
 // compiled without it.
 
 template <int SYNC, int G>
 __device__ __forceinline__ void gsync(int grp) {
-  if (SYNC == 2) __syncthreads();
-  else if (SYNC == 3) {
-    if (grp == 0) asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x >> 1) : "memory");
-    else asm volatile("bar.sync 2, %0;" ::"r"(blockDim.x >> 1) : "memory");
-  } else if (SYNC == 1) asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(G) : "memory");
+  if constexpr (SYNC == 2) __syncthreads();
+  else if constexpr (SYNC >= 3) {
+    const unsigned n = blockDim.x >> (SYNC - 2);
+    if (grp == 0) asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory");
+    else if (SYNC == 3 || grp == 1) asm volatile("bar.sync 2, %0;" ::"r"(n) : "memory");
+    else if (grp == 2) asm volatile("bar.sync 3, %0;" ::"r"(n) : "memory");
+    else asm volatile("bar.sync 4, %0;" ::"r"(n) : "memory");
+  } else if constexpr (SYNC == 1) asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(G) : "memory");
   else __syncwarp();
 }
 
@@ -336,7 +339,7 @@ template <typename V, int SIGN> __device__ __forceinline__ void gpass_first(V (&
 
 // Reduction scratch of a block's transforms (FP64 only): the groups' warps
 // leave their maxima in the first half and their sums in the second.  For
-// column tiles (SYNC 2 and 3) lC: log2 of the interleaved columns, tid and n:
+// column tiles (SYNC 2 to 4) lC: log2 of the interleaved columns, tid and n:
 // the thread's index in and the threads of its set of transforms.
 constexpr int GRED_WORDS = 512;
 struct GRed {

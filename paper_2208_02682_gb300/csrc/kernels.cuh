@@ -223,11 +223,12 @@ __device__ __forceinline__ void load_rows_ct(cplx<T> (&x)[8], const cplx<T>* r, 
 }
 
 // Spectrum Z of p + i q (the two rows), times 1/(2 N), held at the thread's
-// positions -> kx in [0, KXP) halves of p and q (times 1/N), interleaved at r.
-// One exchange through the free buffer.
+// positions -> kx in [0, K] halves of p and q (times 1/N), interleaved at r.
+// One exchange through the free buffer.  (The padding columns kx > K are left as
+// they are: a column pass transforms them and drops the result.)
 template <typename T, int L, int SYNC>
 __device__ __forceinline__ void store_rows_ct(const cplx<T> (&x)[8], cplx<T>* buf0, cplx<T>* buf1, int& w,
-                                              cplx<T>* __restrict__ r, int j, int grp, int K, int KXP) {
+                                              cplx<T>* __restrict__ r, int j, int grp, int K) {
   constexpr int N = 1 << L, G = N / 8;
   cplx<T>* b = w ? buf1 : buf0;
   if constexpr (G % 8 == 0) {
@@ -240,24 +241,18 @@ __device__ __forceinline__ void store_rows_ct(const cplx<T> (&x)[8], cplx<T>* bu
     for (int m = 0; m < 8; ++m) b[sidx<T>(j + m * G)] = x[m];
   }
   gsync<SYNC, G>(grp);
-  // KXP <= 3 G: K + 1 <= N/3, rounded up to a multiple of the column tile
+  // K < 3 G
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     const int k = j + i * G;
-    if (k < KXP) {
-      cplx<T> P = mk<T>(0, 0), Q = mk<T>(0, 0);
-      if (k <= K) {
-        const cplx<T> z1 = b[k + (k >> 3)];
-        const int k2 = (N - k) & (N - 1);
-        const cplx<T> z2 = b[k2 + (k2 >> 3)];
-        // P = Z(k) + conj Z(N-k), Q = (Z(k) - conj Z(N-k))/i
-        P = mk<T>(z1.x + z2.x, z1.y - z2.y);
-        Q = mk<T>(z1.y + z2.y, z2.x - z1.x);
-      }
-      st_pair(r + 2 * k, P, Q);
+    if (k <= K) {
+      const cplx<T> z1 = b[k + (k >> 3)];
+      const int k2 = (N - k) & (N - 1);
+      const cplx<T> z2 = b[k2 + (k2 >> 3)];
+      // P = Z(k) + conj Z(N-k), Q = (Z(k) - conj Z(N-k))/i
+      st_pair(r + 2 * k, mk<T>(z1.x + z2.x, z1.y - z2.y), mk<T>(z1.y + z2.y, z2.x - z1.x));
     }
   }
-  for (int k = j + 3 * G; k < KXP; k += G) st_pair(r + 2 * k, mk<T>(0, 0), mk<T>(0, 0));
   w ^= 1;
 }
 
@@ -565,7 +560,7 @@ __global__ void __launch_bounds__(256) k_in_row(const __grid_constant__ InArgs<T
     for (int m = 0; m < 8; ++m) x[m] = make_double2(p[m * G], p[N + m * G]);
     gfft<double, -1, L, SYNC>(x, buf0, buf0 + rs, w, j, gi, a.tw, GRed{red, 0, 0, 0}, -L - 1);
     store_rows_ct<double, L, SYNC>(x, buf0, buf0 + rs, w, a.mix + (long long)i * a.g.mi + (long long)yp * 2 * a.g.KXP,
-                                   j, gi, a.g.K, a.g.KXP);
+                                   j, gi, a.g.K);
   });
 }
 

@@ -216,29 +216,38 @@ static Layout build_layout(const sw_params& p, int strategy, int fields, int eul
 }
 
 // Tasks of the column-stage kernel (the longest first) for whole blocks or
-// for blocks split in two halves.
-static void build_tasks(Layout& L, bool dual) {
+// for blocks split in `parts` = 2 or 4 parts.
+static void build_tasks(Layout& L, int parts) {
   std::memset(L.ct, 0, sizeof(L.ct));
   L.nct = 0;
+  const bool split = parts > 1, quad = parts == 4;
   ColTask* t = nullptr;
   auto task = [&](int kind, int slot) {
     t = &L.ct[L.nct++];
     t->kind = (signed char)kind;
     t->slot = (signed char)slot;
   };
-  auto step = [&](int prod, int act, int op, int fld, int half = 0, int bar = 0) {
+  auto step = [&](int prod, int act, int op, int fld, int part = 0, int bar = 0) {
     const int i = t->n++;
     t->prod[i] = (signed char)prod;
     t->act[i] = (signed char)act;
     t->op[i] = (signed char)op;
     t->fld[i] = (signed char)fld;
-    t->half[i] = (signed char)half;
+    t->part[i] = (signed char)part;
     t->bar[i] = (signed char)bar;
   };
   if (L.model == SW_MODEL_SW) {
     task(CT_UV, 0);
     step(L.p_ke, CA_PARK, -1, -1);
-    if (dual) {
+    if (quad) {
+      step(L.p_zv, CA_KEEP, -1, -1, 1);
+      step(L.p_zu, CA_KEEP, -1, -1, 2);
+      step(-1, CA_U, -1, L.f_u, 1, 1);
+      step(-1, CA_V, -1, L.f_v, 2);
+      step(L.i_z, CA_MEM, OP_CURL, L.f_u, 0, 1);
+      step(L.i_u, CA_X, OP_ID, L.f_u, 1);
+      step(L.i_v, CA_X, OP_ID, L.f_v, 2);
+    } else if (split) {
       step(L.p_zu, CA_KEEP, -1, -1, 1);
       step(L.p_zv, CA_U, -1, L.f_u, 0, 1);
       step(-1, CA_V, -1, L.f_v, 1);
@@ -255,17 +264,17 @@ static void build_tasks(Layout& L, bool dual) {
   } else if (L.model == SW_MODEL_EULER2D) {
     task(CT_E2, 0);
     step(L.p_zu, CA_PARK, -1, -1);
-    if (dual) step(L.p_zv, CA_KEEP, -1, -1, 1);
-    step(dual ? -1 : L.p_zv, CA_UPD, -1, L.f_h, 1, 1);
+    if (split) step(L.p_zv, CA_KEEP, -1, -1, 1);
+    step(split ? -1 : L.p_zv, CA_UPD, -1, L.f_h, 1, 1);
     step(L.i_h, CA_X, OP_ID, L.f_h, 1, 1);
     step(L.i_u, CA_MEM, OP_ID, L.f_u);
-    step(L.i_v, CA_MEM, OP_ID, L.f_v);
+    step(L.i_v, CA_MEM, OP_ID, L.f_v, quad ? 2 : 0);
   } else {
     task(CT_KIN, 0);
-    for (int f = 0; f < 3; ++f) step(-1, CA_UPD, -1, f);
-    step(L.i_h, CA_MEM, OP_ID, L.f_h, 0, 1);
-    step(L.i_z, CA_MEM, OP_CURL, L.f_u, 0);
-    step(L.i_u, CA_MEM, OP_ID, L.f_u, 1);
+    for (int f = 0; f < 3; ++f) step(-1, CA_UPD, -1, f, quad ? f : 0);
+    step(L.i_h, CA_MEM, OP_ID, L.f_h, quad ? 2 : 0, 1);
+    step(L.i_z, CA_MEM, OP_CURL, L.f_u, quad ? 3 : 0);
+    step(L.i_u, CA_MEM, OP_ID, L.f_u, quad ? 0 : 1);
     step(L.i_v, CA_MEM, OP_ID, L.f_v, 1);
   }
   if (L.has_pos)
@@ -275,7 +284,7 @@ static void build_tasks(Layout& L, bool dual) {
       step(q, CA_UPD_PARK, -1, L.f_p[c]);
       if (L.strategy == 2) {
         step(L.i_xi[c], CA_X, OP_ID, L.f_p[c], 0, 1);
-        step(L.pa[q], CA_PARKED, OP_DX, L.f_p[c], 0);
+        step(L.pa[q], CA_PARKED, OP_DX, L.f_p[c], quad ? 2 : 0);
       } else {
         step(L.pa[q], CA_X, OP_DX, L.f_p[c], 0, 1);
       }
@@ -284,16 +293,18 @@ static void build_tasks(Layout& L, bool dual) {
   for (int j = 0; j < L.nlm; ++j) {
     const int q = L.p_g[j];
     task(CT_G, j);
-    if (L.lmf[j] == LMF_Q) step(L.p_q, CA_PARK, -1, -1);
-    step(q, CA_UPD_PARK, -1, L.f_g[j]);
+    const bool apart = quad && L.lmf[j] == LMF_Q;  // q's transform beside the product's
+    if (L.lmf[j] == LMF_Q) step(L.p_q, CA_PARK, -1, -1, apart ? 1 : 0);
+    if (apart) step(q, CA_KEEP, -1, -1);
+    step(apart ? -1 : q, CA_UPD_PARK, -1, L.f_g[j], 0, apart ? 1 : 0);
     step(L.pa[q], CA_X, OP_DX, L.f_g[j], 0, 1);
     step(L.pb[q], CA_PARKED, OP_DY, L.f_g[j], 1);
   }
   if (L.model == SW_MODEL_SW) {
     task(CT_H, 0);
     step(L.p_hu, CA_PARK, -1, -1);
-    if (dual) step(L.p_hv, CA_KEEP, -1, -1, 1);
-    step(dual ? -1 : L.p_hv, CA_UPD, -1, L.f_h, 1, 1);
+    if (split) step(L.p_hv, CA_KEEP, -1, -1, 1);
+    step(split ? -1 : L.p_hv, CA_UPD, -1, L.f_h, 1, 1);
     step(L.i_h, CA_X, OP_ID, L.f_h, 1);
   }
 }
@@ -371,8 +382,14 @@ static const int GRAPH_STEPS = 8;
 static const long long SMS = 152;  // of a GB300
 // warps in the row pass below which its products are split over blocks
 static const long long ROW_WARPS = 8 * SMS;
-// column-stage blocks up to which blocks are split in two halves
-static const long long DUAL_BLOCKS = 456;
+// Column-stage blocks up to which blocks are split in quarters (the two blocks
+// an SM holds; a step of one Strategy-1 run, halves -> quarters: FP64 64^2 157 -> 141
+// us, 128^2 190 -> 172, 16^2 dynamics 136 -> 123; FP32 128^2 64 -> 61) and in halves
+// (beyond one wave: half of 456 blocks still end sooner than the whole ones: FP64 two
+// 128^2 runs, 384 blocks, whole 297 -> 226 us, 256^2 Strategy 2, 352 blocks, 451 -> 427;
+// FP32 256^2 both strategies, 352 blocks, 122 -> 117).
+static const long long QUAD_BLOCKS = 2 * SMS;
+static const long long DUAL_BLOCKS = 3 * SMS;
 static const int SW_K_OF_KT[KT_COUNT] = {SW_K_ROW_INV, SW_K_ROW_PROD, SW_K_COL_STAGE, SW_K_UPDATE};
 
 struct BatchExec {
@@ -397,7 +414,7 @@ struct BatchExec {
   bool built = false;
   int nstages = 4;  // stage passes per step of the members' (common) stepper
   int stepper = SW_STEP_RK4;
-  bool dual = false;  // split column-stage blocks
+  int parts = 1;  // parts that column-stage blocks are split into
   bool warp = false;  // every member's N <= 256: row kernels without named barriers
   std::string err;
 };
@@ -418,12 +435,12 @@ static void batch_free(BatchExec* b) {
 }
 
 template <typename T>
-static void fill_desc(sw_handle* h, RunDesc<T>& d, int points, int ppb, int lC, bool dual) {
+static void fill_desc(sw_handle* h, RunDesc<T>& d, int points, int ppb, int lC, int parts) {
   std::memset(&d, 0, sizeof(d));
   const Geom& g = h->g;
   d.g = g;
   d.L = h->L;
-  build_tasks(d.L, dual);
+  build_tasks(d.L, parts);
   d.c = StepConsts{h->p.dt, h->p.f0, h->p.c2, h->p.adv_x, h->p.adv_y, h->p.stepper, 0};
   d.cdt = (T)h->p.dt;
   d.cf0 = (T)h->p.f0;
@@ -562,13 +579,14 @@ static int batch_build_t(BatchExec* b) {
   for (int r = 0; r < n; ++r)
     if (b->members[r]->L.np > 0) P = std::max(P, b->members[r]->g.N * (sizeof(T) == 4 ? 4 : 2));
   if (sizeof(T) == 8) P = std::min(P, 2048);
-  // split column blocks (see ColShape) while they all fit on the GPU at once
+  // split column blocks (see ColShape)
   long long col_blocks = 0;
   for (int r = 0; r < n; ++r) {
     const Layout& L = b->members[r]->L;
     if (L.np > 0) col_blocks += (long long)b->members[r]->g.KXP * b->members[r]->g.N / P * (L.nlm + (L.has_pos ? 2 : 0) + 2);
   }
-  b->dual = P / 4 <= DUAL_THREADS<T>() && col_blocks <= DUAL_BLOCKS;
+  b->parts = P / 2 <= SPLIT_THREADS<T>() && col_blocks <= QUAD_BLOCKS ? 4
+             : P / 4 <= SPLIT_THREADS<T>() && col_blocks <= DUAL_BLOCKS ? 2 : 1;
   for (int r = 0; r < n; ++r) {
     sw_handle* h = b->members[r];
     int lC = 0;
@@ -576,18 +594,17 @@ static int batch_build_t(BatchExec* b) {
     // automatic pairs per block: all of them when the row's groups share
     // them out or the grid has rows enough to fill the GPU (N >= 1024), else
     // one (the row's pairs spread over blocks)
-    fill_desc<T>(h, descs[r], points, products(h), lC, b->dual);
+    fill_desc<T>(h, descs[r], points, products(h), lC, b->parts);
     descs[r].Wp = team ? 4 : W;
     descs[r].team = team ? 1 : 0;
     const RunDesc<T>& d = descs[r];
     const int N = h->g.N;
-    const int halves = b->dual ? 2 : 1;
     const int cthr = (N << lC) / 8;
     const size_t csm = ((size_t)col_buf_stride<T>(N, 1 << lC) << lC) * cs;
     const int sets = team ? 4 : 1;
-    const int thr[KT_COUNT] = {sets * d.Bi * N / 8, d.Bp * d.Wp * N / 8, halves * cthr, 256};
+    const int thr[KT_COUNT] = {sets * d.Bi * N / 8, d.Bp * d.Wp * N / 8, b->parts * cthr, 256};
     const size_t sm[KT_COUNT] = {(size_t)sets * 2 * d.Bi * row_stride<T>(N) * cs,
-                                 row_prod_smem<T>(N, d.Bp, d.Wp, h->L, d.gath != 0), halves * csm + (size_t)6 * cthr * cs, 0};
+                                 row_prod_smem<T>(N, d.Bp, d.Wp, h->L, d.gath != 0), b->parts * csm + (size_t)6 * cthr * cs, 0};
     const KBytes kb = kernel_bytes(h, h->L);
     if (h->L.np > 0) b->start_bytes += kb.col_inv;
     const double by[KT_COUNT] = {kb.row_inv, kb.row_prod, 0.0, 0.0};
@@ -662,7 +679,7 @@ static cudaError_t enqueue_kernel(BatchExec* b, int k, int stage, bool fin, bool
   if (total == 0) return cudaSuccess;
   LAUNCH(stage < 0 ? SW_K_COL_INV : SW_K_OF_KT[k], stage < 0 ? b->start_bytes : b->bytes[k][stage],
          launch_stage<T>(k, (const RunDesc<T>*)b->d_table, b->d_start + (size_t)k * (n + 1), n, total, b->threads[k],
-                         b->smem[k], fin ? stage | STAGE_FINAL : stage, b->warp, b->dual, pdl, s));
+                         b->smem[k], fin ? stage | STAGE_FINAL : stage, b->warp, b->parts, pdl, s));
   return cudaSuccess;
 }
 

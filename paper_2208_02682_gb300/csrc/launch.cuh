@@ -77,19 +77,20 @@ template <typename T> bool row_team(int N, int points, int ppb) {
          4 * row_inv_pairs(N, points) * G <= 256;
 }
 
-template <typename T> constexpr int DUAL_THREADS() { return sizeof(T) == 4 ? 256 : 128; }
+template <typename T> constexpr int SPLIT_THREADS() { return sizeof(T) == 4 ? 256 : 128; }
 
 template <typename T> cudaError_t launch_col_inv(const ColInvArgs<T>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_col_fwd(const ColFwdArgs<T>& a, cudaStream_t s);
 template <typename T, typename TO> cudaError_t launch_row_inv(const RowInvArgs<T, TO>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_row_fwd(const RowFwdArgs<T>& a, cudaStream_t s);
-// dual: the column stage with split blocks (at most DUAL_THREADS threads).
+// parts: into how many the column stage's blocks are split (2 and 4: at most
+// SPLIT_THREADS threads).
 // warp: every run's rows have N <= 256 (groups of at most one warp), so the
 // row kernels' variant without named barriers may run.  pdl: launch with
 // programmatic stream serialisation (see pdl_wait).
 template <typename T>
 cudaError_t launch_stage(int kt, const RunDesc<T>* runs, const int* start, int nruns, int blocks, int threads,
-                         size_t smem, int stage, bool warp, bool dual, bool pdl, cudaStream_t s);
+                         size_t smem, int stage, bool warp, int parts, bool pdl, cudaStream_t s);
 // FP64 transforms between the state and physical planes (see k_out_col).
 template <typename T> cudaError_t launch_out(const OutArgs<T>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_in(const InArgs<T>& a, cudaStream_t s);
@@ -142,12 +143,13 @@ template <typename T> static cudaError_t prepare_kernels_t() {
   if ((e = allow_dynamic_smem(k_in_row<T>, mx)) != cudaSuccess) return e;
   if ((e = allow_dynamic_smem(k_in_col<T>, mx)) != cudaSuccess) return e;
   if constexpr (sizeof(T) == 8)
-    if ((e = allow_dynamic_smem(k_stage_col<T, 128, false>, mx)) != cudaSuccess) return e;
-  if ((e = allow_dynamic_smem(k_stage_col<T, 256, false>, mx)) != cudaSuccess) return e;
-  if ((e = allow_dynamic_smem(k_stage_col<T, DUAL_THREADS<T>(), true>, mx)) != cudaSuccess) return e;
+    if ((e = allow_dynamic_smem(k_stage_col<T, 128, 1>, mx)) != cudaSuccess) return e;
+  if ((e = allow_dynamic_smem(k_stage_col<T, 256, 1>, mx)) != cudaSuccess) return e;
+  if ((e = allow_dynamic_smem(k_stage_col<T, SPLIT_THREADS<T>(), 2>, mx)) != cudaSuccess) return e;
+  if ((e = allow_dynamic_smem(k_stage_col<T, SPLIT_THREADS<T>(), 4>, mx)) != cudaSuccess) return e;
   if constexpr (sizeof(T) == 4) {
-    if ((e = allow_dynamic_smem(k_stage_col<T, 512, false>, mx)) != cudaSuccess) return e;
-    if ((e = allow_dynamic_smem(k_stage_col<T, 1024, false>, mx)) != cudaSuccess) return e;
+    if ((e = allow_dynamic_smem(k_stage_col<T, 512, 1>, mx)) != cudaSuccess) return e;
+    if ((e = allow_dynamic_smem(k_stage_col<T, 1024, 1>, mx)) != cudaSuccess) return e;
   }
   if ((e = allow_dynamic_smem(k_stage_row_inv<T, false>, mx)) != cudaSuccess) return e;
   if ((e = allow_dynamic_smem(k_stage_row_inv<T, true>, mx)) != cudaSuccess) return e;
@@ -184,7 +186,7 @@ template <typename T> cudaError_t launch_row_fwd(const RowFwdArgs<T>& a, cudaStr
 
 template <typename T>
 cudaError_t launch_stage(int kt, const RunDesc<T>* runs, const int* start, int nruns, int blocks, int threads,
-                         size_t smem, int stage, bool warp, bool dual, bool pdl, cudaStream_t s) {
+                         size_t smem, int stage, bool warp, int parts, bool pdl, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)blocks);
   cfg.blockDim = dim3((unsigned)threads);
@@ -205,14 +207,15 @@ cudaError_t launch_stage(int kt, const RunDesc<T>* runs, const int* start, int n
     case KT_KIN:
       return cudaLaunchKernelEx(&cfg, k_stage_kin<T>, runs, start, nruns, stage);
     default:
-      if (dual) return cudaLaunchKernelEx(&cfg, k_stage_col<T, DUAL_THREADS<T>(), true>, runs, start, nruns, stage);
+      if (parts == 4) return cudaLaunchKernelEx(&cfg, k_stage_col<T, SPLIT_THREADS<T>(), 4>, runs, start, nruns, stage);
+      if (parts == 2) return cudaLaunchKernelEx(&cfg, k_stage_col<T, SPLIT_THREADS<T>(), 2>, runs, start, nruns, stage);
       if constexpr (sizeof(T) == 4) {
-        if (threads > 512) return cudaLaunchKernelEx(&cfg, k_stage_col<T, 1024, false>, runs, start, nruns, stage);
-        if (threads > 256) return cudaLaunchKernelEx(&cfg, k_stage_col<T, 512, false>, runs, start, nruns, stage);
+        if (threads > 512) return cudaLaunchKernelEx(&cfg, k_stage_col<T, 1024, 1>, runs, start, nruns, stage);
+        if (threads > 256) return cudaLaunchKernelEx(&cfg, k_stage_col<T, 512, 1>, runs, start, nruns, stage);
       }
       if constexpr (sizeof(T) == 8)
-        if (threads <= 128) return cudaLaunchKernelEx(&cfg, k_stage_col<T, 128, false>, runs, start, nruns, stage);
-      return cudaLaunchKernelEx(&cfg, k_stage_col<T, 256, false>, runs, start, nruns, stage);
+        if (threads <= 128) return cudaLaunchKernelEx(&cfg, k_stage_col<T, 128, 1>, runs, start, nruns, stage);
+      return cudaLaunchKernelEx(&cfg, k_stage_col<T, 256, 1>, runs, start, nruns, stage);
   }
 }
 
@@ -258,7 +261,7 @@ cudaError_t launch_velocity_from_vorticity(cplx<T>* y, const Geom& g, int fu, in
 
 #define LM_INSTANTIATE_ALL(T)                                                                               \
   template cudaError_t launch_stage<T>(int, const RunDesc<T>*, const int*, int, int, int, size_t, int, bool,  \
-                                       bool, bool, cudaStream_t);                                           \
+                                       int, bool, cudaStream_t);                                            \
   template cudaError_t launch_out<T>(const OutArgs<T>&, cudaStream_t);                                       \
   template cudaError_t launch_in<T>(const InArgs<T>&, cudaStream_t);                                         \
   template cudaError_t launch_spec_rows<T>(cplx<T>*, cplx<T>*, cplx<T>*, const Geom&, int, bool, long long*, long long,   \

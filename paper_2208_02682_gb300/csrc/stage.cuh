@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), sizeof(T) == 4 ? 1 
         f += W;
       } else if (!inv) {
         store_rows_ct<T, L_, SYNC>(x, buf0, buf1, w, d.pmix + (long long)p * g.mi + (long long)yp * 2 * g.KXP, j, gi,
-                                   g.K, g.KXP);
+                                   g.K);
         p += W;
         sub = 0;
       } else {
@@ -510,8 +510,8 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), sizeof(T) == 4 ? 1 
 // loop): a block runs each instruction only a few times, and with the
 // transforms and updates of every task unrolled the kernel waited for
 // instruction fetches (2048^2: 528 us).
-// Smem: C exchange-buffer pairs (col_buf_stride) per half, then 6 complex per
-// thread of a half (its parked values: the positions m = 3, 4 of a column, n in
+// Smem: C exchange-buffer pairs (col_buf_stride) per part, then 6 complex per
+// thread of a part (its parked values: the positions m = 3, 4 of a column, n in
 // [3N/8, 5N/8), lie outside the 2/3 box).
 __device__ __forceinline__ float kahan_add_rn(float sum, float add, float& comp) {
   const float yk = __fsub_rn(add, comp);
@@ -584,23 +584,25 @@ template <typename T> __device__ __forceinline__ cplx<T> cswap(cplx<T> a) { retu
 // 512^2: few warps per SM, so many registers and three modes in flight; 64^2
 // 42 -> 38 us, 256^2 56 -> 50 us) and 256; FP32 256 (to 512^2), 512 (1024^2) and
 // 1024 (2048^2).
-// DUAL: a task's steps are shared out over two halves of a block, each with
-// its own exchange buffers and barrier (block barriers where a value passes
+// PARTS: a task's steps are shared out over two or four parts of a block, each
+// with its own exchange buffers and barrier (block barriers where a value passes
 // between them): while a launch has about one block per SM its time is the
-// longest task's chain, which this cuts from 6 transforms and 2 updates to 3
-// and 1 (CT_UV) and from 3 and 1 to 2 and 1 (CT_G).  Step of one Strategy-1
-// run, whole blocks -> halves: 64^2 FP64 0.240 -> 0.188 ms, 256^2 FP32 0.078 ->
-// 0.071 ms; at 512^2, more than a block per SM, no difference.
+// longest task's chain, which halves cut from 6 transforms and 2 updates to 3
+// and 1 (CT_UV) and from 3 and 1 to 2 and 1 (CT_G), and quarters (N <= 128) to 2 and 1 for
+// every task.  Step of one Strategy-1 run, whole blocks -> halves: 64^2 FP64 0.240 ->
+// 0.188 ms, 256^2 FP32 0.078 -> 0.071 ms; at 512^2, more than a block per SM, no
+// difference; quarters: see QUAD_BLOCKS.  (Quarters at 256^2 in FP32, 512 threads
+// and one block per SM, lose: the kernel alone 8.1 -> 9.6 us.)
 constexpr int STAGE_FINAL = 256;
-template <typename T, int MAXT, bool DUAL> struct ColShape {
+template <typename T, int MAXT, int PARTS> struct ColShape {
   static constexpr bool f32 = sizeof(T) == 4;
   static constexpr int LO = f32 ? (MAXT <= 256 ? 4 : (MAXT <= 512 ? 10 : 11)) : (MAXT <= 128 ? 4 : 10);
-  static constexpr int HI = DUAL ? 8 : f32 ? (MAXT <= 256 ? 9 : LO) : (MAXT <= 128 ? 9 : 11);
+  static constexpr int HI = PARTS == 4 ? 7 : PARTS == 2 ? 8 : f32 ? (MAXT <= 256 ? 9 : LO) : (MAXT <= 128 ? 9 : 11);
   static constexpr int NB = f32 ? 2 : (MAXT <= 128 ? 3 : 1);  // modes whose loads are issued together
   static constexpr int BLOCKS = MAXT <= 512 ? 2 : 1;
 };
-template <typename T, int MAXT, bool DUAL>
-__global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, DUAL>::BLOCKS) k_stage_col(const RunDesc<T>* __restrict__ runs,
+template <typename T, int MAXT, int PARTS>
+__global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, PARTS>::BLOCKS) k_stage_col(const RunDesc<T>* __restrict__ runs,
                                                                               const int* __restrict__ start,
                                                                               int nruns, int stage_arg) {
   const bool final_step = stage_arg >= 0 && (stage_arg & STAGE_FINAL);
@@ -612,9 +614,9 @@ __global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, DUAL>::BLOCKS) k_stage
   pdl_wait();  // state written by the previous kernels: only after this
   pdl_release();
   const int lb = blockIdx.x - start[r];
-  dispatch_L<ColShape<T, MAXT, DUAL>::LO, ColShape<T, MAXT, DUAL>::HI>(d.g.log2N, [&](auto Lc) {
+  dispatch_L<ColShape<T, MAXT, PARTS>::LO, ColShape<T, MAXT, PARTS>::HI>(d.g.log2N, [&](auto Lc) {
     constexpr int L = decltype(Lc)::value, N = 1 << L, G = N / 8;
-    constexpr int NB = ColShape<T, MAXT, DUAL>::NB;
+    constexpr int NB = ColShape<T, MAXT, PARTS>::NB;
     const Layout& Y = d.L;
     const int K = d.g.K, KXP = d.g.KXP, ms = (int)d.g.ms;
     const int lC = d.lC, C = 1 << lC;
@@ -622,9 +624,9 @@ __global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, DUAL>::BLOCKS) k_stage
     const int task = lb / ntile, tile = lb - task * ntile;
     const ColTask& ct = Y.ct[task];
     const int kind = ct.kind, slot = ct.slot;
-    constexpr int SYNC = DUAL ? 3 : 2;
-    const int ps = DUAL ? blockDim.x >> 1 : blockDim.x;  // threads per half
-    const int lane = DUAL && threadIdx.x >= ps ? 1 : 0, tid = threadIdx.x - lane * ps;
+    constexpr int SYNC = PARTS == 4 ? 4 : PARTS == 2 ? 3 : 2;
+    const int ps = blockDim.x / PARTS;  // threads per part
+    const int part = PARTS > 1 ? threadIdx.x / ps : 0, tid = threadIdx.x - part * ps;
     const int c = tid & (C - 1), j = tid >> lC;
     const int st = d.c.stepper;
     const bool begin = stage < 0;
@@ -637,10 +639,10 @@ __global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, DUAL>::BLOCKS) k_stage
     const T kxf = to_real(kx, (T)0);
     const bool col = kx <= K;
     const bool e2 = Y.model == 2, kin = Y.model == 1;
-    const int xs = C * col_buf_stride<T>(N, C);  // exchange buffers of a half
-    cplx<T>* b0 = reinterpret_cast<cplx<T>*>(smem_raw) + lane * xs + c * col_buf_stride<T>(N, C);
-    cplx<T>* park = reinterpret_cast<cplx<T>*>(smem_raw) + (DUAL ? 2 : 1) * xs + tid;
-    const GRed gr = {red + lane * (GRED_WORDS / 4), lC, tid, ps};
+    const int xs = C * col_buf_stride<T>(N, C);  // exchange buffers of a part
+    cplx<T>* b0 = reinterpret_cast<cplx<T>*>(smem_raw) + part * xs + c * col_buf_stride<T>(N, C);
+    cplx<T>* park = reinterpret_cast<cplx<T>*>(smem_raw) + PARTS * xs + tid;
+    const GRed gr = {red + part * (GRED_WORDS / 2 / PARTS), lC, tid, ps};
     int w = 0;
     cplx<T> x[8];
     // the column's first mode, the row stride of its modes, and its elements
@@ -958,8 +960,8 @@ __global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, DUAL>::BLOCKS) k_stage
     for (int q = 0; q < ct.n; ++q) {
       const int p = ct.prod[q], act = ct.act[q], op = ct.op[q];
       const bool fwd = op < 0;
-      if (DUAL && ct.bar[q]) __syncthreads();
-      if ((fwd ? begin : !outs) || (DUAL && ct.half[q] != lane)) continue;
+      if (PARTS > 1 && ct.bar[q]) __syncthreads();
+      if ((fwd ? begin : !outs) || (PARTS > 1 && ct.part[q] != part)) continue;
       if (fwd) {
         if (p >= 0 && !commit) {
           const cplx<T>* src = d.pmix + (long long)p * d.g.mi + mx;
@@ -996,7 +998,7 @@ __global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, DUAL>::BLOCKS) k_stage
         x[3] = x[4] = mk<T>(0, 0);
       }
       if (!(fwd && (p < 0 || commit)))
-        gfft<T, -1, L, SYNC>(x, b0, b0 + row_stride<T>(N), w, j, lane, d.tw, gr, fwd ? -L : 0);
+        gfft<T, -1, L, SYNC>(x, b0, b0 + row_stride<T>(N), w, j, part, d.tw, gr, fwd ? -L : 0);
       if (fwd) {
         if (act != CA_PARK && act != CA_KEEP) {
           int fe = -1, fa = -1, fb = -1;
