@@ -435,7 +435,7 @@ static void batch_free(BatchExec* b) {
 }
 
 template <typename T>
-static void fill_desc(sw_handle* h, RunDesc<T>& d, int points, int ppb, int lC, int parts) {
+static void fill_desc(sw_handle* h, RunDesc<T>& d, int points, int ppb, int lC, int parts, bool team) {
   std::memset(&d, 0, sizeof(d));
   const Geom& g = h->g;
   d.g = g;
@@ -475,7 +475,12 @@ static void fill_desc(sw_handle* h, RunDesc<T>& d, int points, int ppb, int lC, 
   }
   d.fused = row_prod_fused<T>(g.N, L) ? 1 : 0;
   d.gath = row_prod_gath<T>(g.N, L) && d.ppb >= L.np ? 1 : 0;
-  d.nb[KT_ROW_INV] = L.np > 0 && !d.fused ? (L.strategy == 2 ? 5 : 3) * row_blocks(g.N, d.Bi) : 0;
+  d.team = team ? 1 : 0;
+  // (a launch below a wave of blocks is as long as its longest block: 256^2
+  // 103 -> 101 us a step; above, fewer blocks of more work: 2048^2 67 us against 74)
+  d.hzsep = !team && !L.has_q && g.N <= 256 ? 1 : 0;
+  d.nb[KT_ROW_INV] =
+      L.np > 0 && !d.fused ? ((L.strategy == 2 ? 5 : 3) + d.hzsep) * row_blocks(g.N, d.Bi) : 0;
   d.nb[KT_ROW_PROD] = row_blocks(g.N, d.Bp) * chunks;
   d.nb[KT_COL_STAGE] = L.np > 0 ? ntile * d.L.nct : 0;
   d.nb[KT_KIN] = L.np > 0 ? 0 : (int)((g.ms + kin_modes(g.N) - 1) / kin_modes(g.N));
@@ -541,8 +546,14 @@ static int batch_build_t(BatchExec* b) {
     if (!half) break;
     points /= 2;
   }
+  long long row_blks = 0;
+  for (int r = 0; r < n; ++r) {
+    const int N = b->members[r]->g.N;
+    if (b->members[r]->L.np > 0) row_blks += row_blocks(N, row_block_pairs(N, points));
+  }
   auto groups = [&](const sw_handle* h, int npb) {
-    return row_prod_groups<T>(h->g.N, row_block_pairs(h->g.N, points), npb < h->L.np ? npb : h->L.np, h->L);
+    return row_prod_groups<T>(h->g.N, row_block_pairs(h->g.N, points), npb < h->L.np ? npb : h->L.np, h->L,
+                              row_blks <= SMS);
   };
   int W = 1 << 20;
   long long warps = 0;
@@ -555,9 +566,14 @@ static int batch_build_t(BatchExec* b) {
     const sw_handle* h = b->members[r];
     if (h->L.np > 0) warps += std::max<long long>(1, (long long)W * (h->g.N / 2) * (h->g.N / 8) / 32);
   }
-  // fewer warps than ROW_WARPS (about 8 per SM): the products are split over
-  // blocks, each transforming the base fields its products need
-  const int chunks = warps > 0 ? (int)std::min<long long>(MAXP, (ROW_WARPS + warps - 1) / warps) : 1;
+  // fewer warps than ROW_WARPS (8 per SM): the products are split over
+  // blocks, each transforming the base fields its products need.  Not where
+  // several groups per row pair share them, in FP32: a split gives up the shared
+  // base fields and gather (256^2, split -> not: dynamics 63 -> 51 us a step, Strategy
+  // 2 of one field 104 -> 98; FP64, bound by issue, the other way round: Strategy 1 of
+  // four 302 against 328)
+  const int chunks =
+      warps == 0 || (W > 1 && sizeof(T) == 4) ? 1 : (int)std::min<long long>(MAXP, (ROW_WARPS + warps - 1) / warps);
   auto products = [&](const sw_handle* h) {
     return h->ppb != 0 ? h->ppb : std::max(1, (h->L.np + chunks - 1) / chunks);
   };
@@ -591,12 +607,8 @@ static int batch_build_t(BatchExec* b) {
     sw_handle* h = b->members[r];
     int lC = 0;
     while ((h->g.N << lC) < P && lC < h->lC) ++lC;
-    // automatic pairs per block: all of them when the row's groups share
-    // them out or the grid has rows enough to fill the GPU (N >= 1024), else
-    // one (the row's pairs spread over blocks)
-    fill_desc<T>(h, descs[r], points, products(h), lC, b->parts);
+    fill_desc<T>(h, descs[r], points, products(h), lC, b->parts, team);
     descs[r].Wp = team ? 4 : W;
-    descs[r].team = team ? 1 : 0;
     const RunDesc<T>& d = descs[r];
     const int N = h->g.N;
     const int cthr = (N << lC) / 8;
@@ -604,7 +616,8 @@ static int batch_build_t(BatchExec* b) {
     const int sets = team ? 4 : 1;
     const int thr[KT_COUNT] = {sets * d.Bi * N / 8, d.Bp * d.Wp * N / 8, b->parts * cthr, 256};
     const size_t sm[KT_COUNT] = {(size_t)sets * 2 * d.Bi * row_stride<T>(N) * cs,
-                                 row_prod_smem<T>(N, d.Bp, d.Wp, h->L, d.gath != 0), b->parts * csm + (size_t)6 * cthr * cs, 0};
+                                 row_prod_smem<T>(N, d.Bp, d.Wp, h->L, d.gath != 0),
+                                 b->parts * csm + (size_t)6 * cthr * cs, 0};
     const KBytes kb = kernel_bytes(h, h->L);
     if (h->L.np > 0) b->start_bytes += kb.col_inv;
     const double by[KT_COUNT] = {kb.row_inv, kb.row_prod, 0.0, 0.0};

@@ -47,7 +47,7 @@ template <typename T> size_t row_prod_smem(int N, int B, int W, const Layout& L,
 // Largest W for B row pairs and np products per block (other than a team): W > 1 needs whole
 // warps per group (N >= 256), a thread count within the block limit, at most
 // 15 named barriers (groups of N >= 512) and at most 200 KB of shared memory.
-template <typename T> int row_prod_groups(int N, int B, int np, const Layout& L) {
+template <typename T> int row_prod_groups(int N, int B, int np, const Layout& L, bool alone) {
   const int G = N / 8;
   if (G < 32) return 1;
   auto fit = [&](int threads, size_t smem) {
@@ -55,9 +55,11 @@ template <typename T> int row_prod_groups(int N, int B, int np, const Layout& L)
     while (W > 1 && (B * W * G > threads || (G >= 64 && B * W > 15) || row_prod_smem<T>(N, B, W, L) > smem)) --W;
     return W;
   };
-  // two blocks per SM, or one of several groups where that leaves one group
+  // two blocks per SM, or one of several groups where that leaves one group or,
+  // FP32, the launch has no second block for an SM anyway (`alone`; 256^2, Strategy 2
+  // with PV, 13 products: 12 -> 13 groups, a step 115 -> 107 us)
   const int W = fit(sizeof(T) == 4 ? 384 : 256, (size_t)110 * 1024);
-  return W > 1 ? W : fit(row_prod_max_threads<T>(), (size_t)200 * 1024);
+  return W > 1 && !(alone && sizeof(T) == 4) ? W : fit(row_prod_max_threads<T>(), (size_t)200 * 1024);
 }
 
 // Row pairs per block of the row inverse pass.

@@ -39,6 +39,7 @@ struct alignas(16) RunDesc {
   int Bp, ppb;    // row_prod: row pairs per block, products per block
   int Wp;         // row_prod: groups of N/8 threads per row pair
   int team;       // row_inv, row_prod: a team of four sets of groups per row pair
+  int hzsep;      // row_inv: zeta in blocks of its own
   int Bi;         // row_inv: row pairs per block
   int fused;      // row_prod: transforms the base fields itself
   int gath;       // row_prod: gathers all fields at x + xi at once (interleaved planes)
@@ -84,7 +85,7 @@ __device__ __forceinline__ const cplx<T>* stage_input(const RunDesc<T>& d, int s
 // a3: base planes (physical u, v, h, zeta and, Strategy 2, xi and, with PV
 // averaged, q = (f0 + zeta)/h, h = 1 + eta) of the runs whose row pass does not
 // form them itself.  Local block = (field, block of Bi row pairs, one pair per
-// group of N/8 threads); the field of h takes zeta and q too.
+// group of N/8 threads).
 template <typename T, bool WARP>
 __global__ void __launch_bounds__(256) k_stage_row_inv(const RunDesc<T>* __restrict__ runs,
                                                        const int* __restrict__ start, int nruns) {
@@ -110,11 +111,13 @@ __global__ void __launch_bounds__(256) k_stage_row_inv(const RunDesc<T>* __restr
     cplx<T>* buf0 = reinterpret_cast<cplx<T>*>(smem_raw) + (size_t)grp * 2 * rs;
     cplx<T> x[8], eta[8];
     int w = 0;
-    const bool hz = f == 2;
+    // the field of h takes zeta too, unless zeta has blocks of its own (the last)
+    const bool hz = f == 2 && !d.hzsep, zl = f == (d.L.strategy == 2 ? 5 : 3);
 #pragma unroll 1
     for (int part = set; part < (hz ? (set ? 2 : (team ? 1 : 2)) : 1); ++part) {
-      const int src = f == 0 ? d.L.i_u : (f == 1 ? d.L.i_v : (hz ? (part ? d.L.i_z : d.L.i_h) : d.L.i_xi[f - 3]));
-      const int dst = f < 2 ? f : (hz ? (part ? PH_Z : PH_H) : f - 3 + PH_XX);
+      const bool z = zl || (hz && part);
+      const int src = z ? d.L.i_z : (f == 0 ? d.L.i_u : (f == 1 ? d.L.i_v : (f == 2 ? d.L.i_h : d.L.i_xi[f - 3])));
+      const int dst = z ? PH_Z : (f <= PH_H ? f : f - 3 + PH_XX);
       load_rows_ct<T, L>(x, d.mix + (long long)src * g.mi + (long long)yp * 2 * g.KXP, j, g.K);
       gfft<T, -1, L, SYNC>(x, buf0, buf0 + rs, w, j, grp, d.tw, GRed{red, 0, 0, 0});
       // planes [y][x]; interleaved, the four base fields as [y][x][4] and the
