@@ -447,6 +447,7 @@ static void fill_desc(sw_handle* h, RunDesc<T>& d, int points, int ppb, int lC, 
   d.cc2 = (T)h->p.c2;
   d.cadvx = (T)h->p.adv_x;
   d.cadvy = (T)h->p.adv_y;
+  d.cci = h->p.stepper == SW_STEP_RK4 ? d.cdt / (T)6 : (h->p.stepper == SW_STEP_HEUN ? d.cdt / (T)2 : (T)1);
   d.y = (cplx<T>*)h->y;
   d.ysa = (cplx<T>*)h->ys;
   d.ysb = (cplx<T>*)h->ys2;

@@ -23,6 +23,7 @@ struct alignas(16) RunDesc {
   Layout L;
   StepConsts c;
   T cdt, cf0, cc2, cadvx, cadvy;  // dt, f0, c2, adv in the kernels' precision
+  T cci;          // weight of the summed right-hand sides in the commit: dt/6, dt/2 or 1 (by stepper)
   cplx<T>* y;     // state at t_n
   cplx<T>* ysa;   // stage inputs of stages 1 and 3 (u, v, h)
   cplx<T>* ysb;   // stage input of stage 2 (u, v, h)
@@ -174,12 +175,12 @@ __global__ void __launch_bounds__(256) k_stage_row_inv(const RunDesc<T>* __restr
 //
 // Local block = (product chunk, block of Bp row pairs): Wp groups of G = N/8
 // threads per pair share out the chunk's ppb products, the costly ones first.
-// `fused` runs (Strategy 1, except on the largest grids): the groups first
+// `fused` runs (Strategy 1, except in FP64 from 1024^2): the groups first
 // transform the pair's base fields u, v, h, zeta (those the chunk needs) into
 // shared memory.  The others read base values from the planes that the row
 // inverse pass wrote; Strategy 2 gathers from them too: `gath` runs (where the
-// arrays fit and a block takes all products) once for all products, into shared memory, from interleaved
-// planes (each product gathering for itself from separate planes took 34.7 us
+// arrays fit and a block takes all products) once for all products, into shared
+// memory, from interleaved planes (each product gathering for itself from separate planes took 34.7 us
 // at 512^2 with five means, this 26.7 us).  Every transform stays in the
 // registers of its group: an advection product takes the inverse transforms
 // of d_x G and d_y G and, from the same positions, the forward transform of
@@ -245,12 +246,18 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), sizeof(T) == 4 ? 1 
     cplx<T>* buf1 = buf0 + rs;
     const int p0 = pg * ppb, p1 = min(L.np, p0 + ppb);
     const T adv_x = d.cadvx, adv_y = d.cadvy, f0 = d.cf0;
-    const T s = stage_time<T>(*d.ctr, stage, d.cdt, d.c.stepper);
-    const bool s0 = !(s > (T)0);
-    const T inv_s = s0 ? (T)0 : (T)1 / s;
-    // xi-first scheme: gbar steps with the updated xi at its time s + dt
+    // Strategy 2: the interval time s (the others skip its conversions and
+    // divisions in FP64, where they are slow)
     const bool xf = L.scheme == SCHEME_XI_FIRST;
-    const T inv_sg = xf ? (T)1 / (s + d.cdt) : inv_s;
+    bool s0 = true;
+    T inv_s = (T)0, inv_sg = (T)0;
+    if (sizeof(T) == 4 || L.strategy == 2) {
+      const T s = stage_time<T>(*d.ctr, stage, d.cdt, d.c.stepper);
+      s0 = !(s > (T)0);
+      if (!s0) inv_s = (T)1 / s;
+      // xi-first scheme: gbar steps with the updated xi at its time s + dt
+      inv_sg = xf ? (T)1 / (s + d.cdt) : inv_s;
+    }
     const T inv_dx = (T)N / (T)6.283185307179586476925286766559;
     const cplx<T>* mix = d.mix + (long long)yp * 2 * g.KXP;
     const T* phys = d.phys;
@@ -556,6 +563,12 @@ __device__ __forceinline__ cplx<T> commit_mode(bool kahan, T e2h, T e2l, cplx<T>
   return mk<T>(fma(yn.x, e2h, inc.x), fma(yn.y, e2h, inc.y));
 }
 
+// v or -v, by an integer instruction in FP64.
+__device__ __forceinline__ float neg_if(bool n, float v) { return n ? -v : v; }
+__device__ __forceinline__ double neg_if(bool n, double v) {
+  return __hiloint2double(__double2hiint(v) ^ (n ? (int)0x80000000 : 0), __double2loint(v));
+}
+
 // Integer as a T; FP64 by integer instructions (a conversion is an FP64-pipe
 // instruction), |k| < 2^20.
 __device__ __forceinline__ float to_real(int k, float) { return (float)k; }
@@ -571,12 +584,13 @@ __device__ __forceinline__ double to_real(int k, double) {
 template <typename T> __device__ __forceinline__ void finish_step(const RunDesc<T>& d, int kt) {
   __syncthreads();
   if (threadIdx.x == 0) {
+    const long long n = *d.ctr;
     __threadfence();
     const unsigned t = atomicAdd(d.ticket, 1u);
     if (t == (unsigned)d.nb[kt] - 1u) {
+      // (visible to the next kernels: they wait for the end of this one)
       *d.ticket = 0u;
-      *d.ctr = *d.ctr + 1;
-      __threadfence();
+      *d.ctr = n + 1;
     }
   }
 }
@@ -685,7 +699,7 @@ __global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, PARTS>::BLOCKS) k_stag
       const bool x1 = Y.scheme == SCHEME_XI_FIRST && (role == R_P || role == R_G);
       const bool act = !x1 || ((role == R_P) == ((nstep & 1) == 0));
       const bool add = st == 0 && stage > 0;
-      const bool kah = d.comp && Y.fkahan[f];
+      const bool kah = sizeof(T) == 4 && d.comp && Y.fkahan[f];  // (FP64 runs have no compensation)
       const bool keep = role <= R_H && !euler0;  // stage values that other tasks read
       cplx<T>* const yf = d.y + f * ms;
       cplx<T>* const af = d.acc + f * ms;
@@ -734,7 +748,9 @@ __global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, PARTS>::BLOCKS) k_stag
             const cplx<T> Bq = mk<T>(fma(pa[i].x, c2, pk.x), fma(pa[i].y, c2, pk.y));
             const cplx<T> lin = mk<T>(fma(pb[i].x, f0, tv[i].x), fma(pb[i].y, f0, tv[i].y));
             const T k = iu ? kxf : ky[i];
-            rr[i] = mk<T>(fma(Bq.y, k, sg * lin.x), fma(Bq.x, -k, sg * lin.y));
+            // (FP64: the sign by an integer instruction)
+            const T lx = sizeof(T) == 8 ? neg_if(!iu, lin.x) : sg * lin.x, ly = sizeof(T) == 8 ? neg_if(!iu, lin.y) : sg * lin.y;
+            rr[i] = mk<T>(fma(Bq.y, k, lx), fma(Bq.x, -k, ly));
           }
         } else if (kind == CT_KIN) {
 #pragma unroll
@@ -800,11 +816,23 @@ __global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, PARTS>::BLOCKS) k_stag
             const T e1 = E[i], ee = e1 * e1;
             T cr = stage == 0 ? ee : (T)2 * e1;
             T ca = stage == 2 ? ee : e1;
-            T cb = stage == 0 ? hdt * e1 : (stage == 1 ? hdt : dt * e1);
-            if (st != 0) {
-              cr = ca = ee;
-              cb = dt * ee;
-              if (st == 2) cr = x1 ? (T)2 * dt * ee * ee : dt * ee;
+            T cb;
+            if (sizeof(T) == 8) {
+              // few FP64 operations: both sides of a choice between products are
+              // evaluated, so the choice is between their factors
+              cb = (st == 0 && stage < 2 ? hdt : dt) * (st != 0 ? ee : (stage == 1 ? (T)1 : e1));
+              if (st != 0) ca = ee;
+              if (st == 2) {
+                asm volatile("");  // a branch
+                cr = x1 ? (T)2 * dt * ee * ee : dt * ee;
+              }
+            } else {
+              cb = stage == 0 ? hdt * e1 : (stage == 1 ? hdt : dt * e1);
+              if (st != 0) {
+                cr = ca = ee;
+                cb = dt * ee;
+                if (st == 2) cr = x1 ? (T)2 * dt * ee * ee : dt * ee;
+              }
             }
             nv[i] = mk<T>(fma(ca, yn[i].x, cb * rr[i].x), fma(ca, yn[i].y, cb * rr[i].y));
             ac[i] = mk<T>(fma(cr, rr[i].x, ac[i].x), fma(cr, rr[i].y, ac[i].y));
@@ -834,7 +862,7 @@ __global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, PARTS>::BLOCKS) k_stag
       } else {
         // final stage: y_{n+1} = E^2 y_n + inc, with inc = dt/6 (acc + d) (RK4),
         // dt/2 (acc + b) (Heun) or forward Euler's increment acc
-        const T ci = st == 0 ? dt / (T)6 : (st == 1 ? dt / (T)2 : (T)1);
+        const T ci = sizeof(T) == 8 ? d.cci : (st == 0 ? dt / (T)6 : (st == 1 ? dt / (T)2 : (T)1));
 #pragma unroll 1
         for (int s0 = 0; s0 < 6; s0 += NB) {
           cplx<T> yn[NB], ac[NB], cc[NB], pa[NB], pb[NB], en[NB], ea[NB], ec[NB], nv[NB];
@@ -874,7 +902,7 @@ __global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, PARTS>::BLOCKS) k_stag
               en[i] = ye[ml[i]];
               ea[i] = ae[ml[i]];
             }
-            if (d.comp) {
+            if (sizeof(T) == 4 && d.comp) {
 #pragma unroll
               for (int i = 0; i < NB; ++i) ec[i] = d.comp[fe * ms + ml[i]];
             }
@@ -890,6 +918,7 @@ __global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, PARTS>::BLOCKS) k_stag
           }
           if (!commit) rhs(s0, ky, t, pa, pb, rr, fh);
           if (x1) {
+            if (sizeof(T) == 8) asm volatile("");  // a branch
             // E^4 = (eh + el)^2 to the same precision (exact product of eh by fma)
 #pragma unroll
             for (int i = 0; i < NB; ++i) {
@@ -910,7 +939,7 @@ __global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, PARTS>::BLOCKS) k_stag
             nv[i] = in[i] ? nv[i] : z;
           }
           if (fe >= 0) {
-            const bool ke = d.comp != nullptr;
+            const bool ke = sizeof(T) == 4 && d.comp != nullptr;
             cplx<T>* const cfe = d.comp + fe * ms;
 #pragma unroll
             for (int i = 0; i < NB; ++i) {
@@ -1079,7 +1108,7 @@ __global__ void __launch_bounds__(256, 3) k_stage_kin(const RunDesc<T>* __restri
     }
     return c;
   };
-  const T ci = st == 0 ? dt / (T)6 : dt / (T)2;
+  const T ci = d.cci;
   const bool radd = !last || st != 2;              // the stage adds a right-hand side
   const bool racc = last || (st == 0 && stage > 0);  // acc is read
   pdl_wait();  // state written by the previous kernels: only after this
