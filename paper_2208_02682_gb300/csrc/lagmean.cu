@@ -1408,8 +1408,13 @@ extern "C" int sw_set_state(sw_handle* h, const void* blob, size_t size) {
   Layout L = hd.lm_open ? build_layout(h->p, hd.lp.strategy, hd.lp.fields, hd.lp.eulerian, hd.lp.scheme)
                         : build_layout(h->p, 0, 0, 0);
   if (L.nf != hd.nf || size < blob_size(h, hd.nf)) return fail(h, SW_EINVAL, "blob size mismatch");
-  CK(h, cudaMemcpyAsync(h->mix, (const char*)blob + sizeof(hd), blob_size(h, hd.nf) - sizeof(hd),
-                        cudaMemcpyHostToDevice, h->stream));
+  // (in halves of at most 64 KB where that lets the copies go with the commands)
+  const size_t bytes = blob_size(h, hd.nf) - sizeof(hd), half = bytes / 2;
+  const size_t first = bytes > (64 << 10) && half <= (64 << 10) ? half : bytes;
+  const char* src = (const char*)blob + sizeof(hd);
+  CK(h, cudaMemcpyAsync(h->mix, src, first, cudaMemcpyHostToDevice, h->stream));
+  if (first < bytes)
+    CK(h, cudaMemcpyAsync((char*)h->mix + first, src + first, bytes - first, cudaMemcpyHostToDevice, h->stream));
   if (const int rc = spec_rows(h, hd.nf, false, hd.done)) return rc;
   CK(h, cudaStreamSynchronize(h->stream));
   set_layout(h, L);
