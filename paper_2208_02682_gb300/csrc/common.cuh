@@ -13,8 +13,8 @@
 // The mixed layout interleaves pairs of rows: the row pass, which transforms
 // two rows as one complex sequence, reads and writes both with one 16- or
 // 32-byte access per lane, and the column pass moves runs of 2 rows x C
-// columns.  (The FP64 transforms around the stepping use plain rows [ky][kx]
-// and [y][kx] in buffers of their own.)
+// columns.  (The transforms around the stepping use the same layouts, their
+// mixed fields in FP64.)
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -38,7 +38,6 @@ template <typename T> __device__ __forceinline__ cplx<T> cmul(cplx<T> a, cplx<T>
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 template <typename T> __device__ __forceinline__ cplx<T> cscale(cplx<T> a, T s) { return mk<T>(a.x * s, a.y * s); }
-template <typename T> __device__ __forceinline__ cplx<T> cconj(cplx<T> a) { return mk<T>(a.x, -a.y); }
 // multiply by i*k (spectral derivative)
 template <typename T> __device__ __forceinline__ cplx<T> cik(cplx<T> a, T k) { return mk<T>(-a.y * k, a.x * k); }
 
@@ -252,7 +251,6 @@ struct Layout {
   int fclass[MAXF];  // IF_* class of each evolved field
   int fkahan[MAXF];  // compensated final update (FP32 mode) for this field
   int frole[MAXF];   // R_* role
-  int fslot[MAXF];   // LM slot (R_G, R_E) or component (R_P)
   // column pass: output i = op(src[i] (, src2[i]))
   int i_src[MAXI], i_src2[MAXI], i_op[MAXI];
   int i_u, i_v, i_h, i_z;      // dynamics intermediates

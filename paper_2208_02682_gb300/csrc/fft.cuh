@@ -62,52 +62,18 @@ __device__ __forceinline__ void dft8(cplx<T>* v) {
 }
 
 // Twiddles w^{r k}, 1 <= r < R, w = exp(sigma 2 pi i / (Ns R)), of one
-// butterfly.  FP64 loads all R - 1 from the table (FP64 multiplies are the
-// scarce resource).  FP32 evaluates w^k, w^2k, w^4k and forms the others as
-// products (at most two multiplications deep): from the table rows r = 1, 2,
-// 4, or, with TWC, from sincospif of 2 e / (Ns R) (exact in FP32) for e = k,
-// 2k, 4k.  The generic column kernels compute them; the stage kernels load
-// the table (their loads stay in L1; at 1024^2-2048^2 the column passes ran
-// 10-15% faster with the table than with sincospif).
-template <typename T, int SIGN, int R, bool TWC>
+// butterfly, all from the table (FP64 multiplies are the scarce resource).
+template <typename T, int SIGN, int R>
 __device__ __forceinline__ void butterfly_twiddles(cplx<T>* w, int k, int lNs, const cplx<T>* __restrict__ tw) {
-  constexpr int LR = R == 8 ? 3 : (R == 4 ? 2 : 1);
   const cplx<T>* t = tw + (k - 1);
-  if (sizeof(T) == 4) {
-    auto ev = [&](int r) {
-      cplx<T> c;
-      if (TWC) {
-        float sn, cs;
-        sincospif(ldexpf((float)(r * k), 1 - lNs - LR), &sn, &cs);
-        c.x = (T)cs;
-        c.y = (T)(-sn);
-      } else {
-        c = __ldg(t + (r << lNs));
-      }
-      if (SIGN > 0) c.y = -c.y;
-      return c;
-    };
-    w[1] = ev(1);
-    if (R >= 4) {
-      w[2] = ev(2);
-      w[3] = cmul<T>(w[1], w[2]);
-    }
-    if (R == 8) {
-      w[4] = ev(4);
-      w[5] = cmul<T>(w[4], w[1]);
-      w[6] = cmul<T>(w[4], w[2]);
-      w[7] = cmul<T>(w[4], w[3]);
-    }
-  } else {
 #pragma unroll
-    for (int r = 1; r < R; ++r) {
-      w[r] = __ldg(t + (r << lNs));
-      if (SIGN > 0) w[r].y = -w[r].y;
-    }
+  for (int r = 1; r < R; ++r) {
+    w[r] = __ldg(t + (r << lNs));
+    if (SIGN > 0) w[r].y = -w[r].y;
   }
 }
 
-template <typename T, int SIGN, int LR, bool TWC>
+template <typename T, int SIGN, int LR>
 __device__ __forceinline__ void stockham_pass(cplx<T>* buf, int log2N, int lNs, int bstride,
                                               const cplx<T>* __restrict__ tw) {
   constexpr int R = 1 << LR;
@@ -131,7 +97,7 @@ __device__ __forceinline__ void stockham_pass(cplx<T>* buf, int log2N, int lNs, 
     for (int r = 0; r < R; ++r) v[u * R + r] = src[sidx<T>(j + r * NR)];
     if (k > 0) {
       cplx<T> w[R];
-      butterfly_twiddles<T, SIGN, R, TWC>(w, k, lNs, tw);
+      butterfly_twiddles<T, SIGN, R>(w, k, lNs, tw);
 #pragma unroll
       for (int r = 1; r < R; ++r) v[u * R + r] = cmul<T>(v[u * R + r], w[r]);
     }
@@ -157,19 +123,19 @@ __device__ __forceinline__ void stockham_pass(cplx<T>* buf, int log2N, int lNs, 
 
 // Block-wide FFT of `batch` transforms of length 2^log2N; requires
 // blockDim.x * 8 == batch * 2^log2N and log2N >= 1.  Callers synchronise
-// before (data in place); the function ends with a barrier.  TWC: computed
-// FP32 twiddles (see twiddle()).
-template <typename T, int SIGN, bool TWC = false>
+// before (data in place); the function ends with a barrier.  (FP64, for
+// csrc/project_static.cu; the other transforms are group transforms.)
+template <typename T, int SIGN>
 __device__ void block_fft(cplx<T>* buf, int log2N, int bstride, const cplx<T>* __restrict__ tw) {
   int lNs = 0;
   int rem = log2N;
   while (rem >= 3) {
-    stockham_pass<T, SIGN, 3, TWC>(buf, log2N, lNs, bstride, tw);
+    stockham_pass<T, SIGN, 3>(buf, log2N, lNs, bstride, tw);
     lNs += 3;
     rem -= 3;
   }
-  if (rem == 2) stockham_pass<T, SIGN, 2, TWC>(buf, log2N, lNs, bstride, tw);
-  if (rem == 1) stockham_pass<T, SIGN, 1, TWC>(buf, log2N, lNs, bstride, tw);
+  if (rem == 2) stockham_pass<T, SIGN, 2>(buf, log2N, lNs, bstride, tw);
+  if (rem == 1) stockham_pass<T, SIGN, 1>(buf, log2N, lNs, bstride, tw);
 }
 
 template <typename T, int SIGN, int R>
@@ -219,7 +185,9 @@ __device__ __forceinline__ void gsync(int grp) {
 }
 
 // Twiddles w^{r k}, 1 <= r < R, of a butterfly of the pass with stride
-// Ns = 2^LNS (see butterfly_twiddles).
+// Ns = 2^LNS: the table's for r = 1, 2, 4, the others as products (at most two
+// multiplications deep).  (At 1024^2-2048^2 the column passes ran 10-15% faster
+// with the table than with sincospif.)
 template <int SIGN, int R, int LNS>
 __device__ __forceinline__ void twiddles_ct(float2* w, int k, const float2* __restrict__ tw) {
   const float2* t = tw + (k - 1);

@@ -1,15 +1,16 @@
-// kernels.cuh -- GB300 kernels of one RK stage and of the transforms around it.
+// kernels.cuh -- what the stage kernels (stage.cuh) are built from, and the
+// transforms around the stepping.
 //
-// One RK4 stage of the coupled shallow-water + Lagrangian-mean system is
-//   col_inv   spectral state -> mixed fields   (derivatives, inverse y-FFT)
-//   row_prod  mixed fields -> products          (inverse x-FFT, physical-space
-//             products of the shallow-water equations and of the
-//             Lagrangian-mean PDEs, forward x-FFT)
-//   col_fwd   products -> spectral products     (forward y-FFT, 2/3 mask)
-//   update    right-hand sides and the RK4 integrating-factor combination
-// (Strategy 2 adds row_inv into a physical gather buffer before row_prod.)
-// The dealiased pseudospectral method is the one the paper uses for both the
-// dynamics and the mean equations (Sec. 4.1, 4.2).
+// One RK stage of the coupled shallow-water + Lagrangian-mean system is
+//   row_prod   mixed fields -> products       (inverse x-FFT, physical-space
+//              products of the shallow-water equations and of the
+//              Lagrangian-mean PDEs, forward x-FFT)
+//   col_stage  products -> next mixed fields  (forward y-FFT and 2/3 mask,
+//              right-hand sides and the integrating-factor combination,
+//              derivatives and inverse y-FFT)
+// (Strategy 2, and FP64 from 1024^2, add row_inv into physical planes before
+// row_prod.)  The dealiased pseudospectral method is the one the paper uses for
+// both the dynamics and the mean equations (Sec. 4.1, 4.2).
 #pragma once
 #include "common.cuh"
 #include "fft.cuh"
@@ -21,36 +22,24 @@ namespace lm {
 // of C, KXP a multiple of C), C*N/8 threads, smem C*col_stride(N, C) complex.  The
 // tile's global accesses are C-wide contiguous runs along kx.
 
-// inverse: d = IFFT_y(op(s1[, s2])), op in {id, d_x, d_y, curl}, zero-padded
-// outside |ky| <= K.
+// inverse: d = IFFT_y(s), zero-padded outside |ky| <= K.
 template <typename T>
-__device__ void col_inverse_tile(cplx<T>* buf, const cplx<T>* __restrict__ s1, const cplx<T>* __restrict__ s2,
-                                 int op, cplx<T>* __restrict__ d, const Geom& g, int lC, int kx0,
-                                 const cplx<T>* __restrict__ tw) {
+__device__ void col_inverse_tile(cplx<T>* buf, const cplx<T>* __restrict__ s, cplx<T>* __restrict__ d, const Geom& g,
+                                 int lC, int kx0, const cplx<T>* __restrict__ tw) {
   const int N = g.N, K = g.K, KXP = g.KXP;
   const int C = 1 << lC, bst = col_stride<T>(N, C);
   const int nthr = blockDim.x, tid = threadIdx.x;
-  // every element written once: op(S) at n = ky mod N for |ky| <= K, else 0
+  // every element written once: s at n = ky mod N for |ky| <= K, else 0
   for (int e = tid; e < N * C; e += nthr) {
     const int n = e >> lC, c = e & (C - 1);
     const int kx = kx0 + c;
     const int ky = n <= K ? n : n - N;
     cplx<T> v = mk<T>(0, 0);
-    if (kx <= K && (n <= K || n >= N - K)) {
-      const long long m = (long long)(ky + K) * KXP + kx;
-      cplx<T> x = s1[m];
-      if (op == OP_ID) v = x;
-      else if (op == OP_DX) v = cik<T>(x, (T)kx);
-      else if (op == OP_DY) v = cik<T>(x, (T)ky);
-      else {  // curl: i kx v - i ky u, s1 = u, s2 = v
-        cplx<T> y = s2[m];
-        v = csub<T>(cik<T>(y, (T)kx), cik<T>(x, (T)ky));
-      }
-    }
+    if (kx <= K && (n <= K || n >= N - K)) v = s[(long long)(ky + K) * KXP + kx];
     buf[c * bst + sidx<T>(n)] = v;
   }
   __syncthreads();
-  block_fft<T, +1, true>(buf, g.log2N, bst, tw);
+  block_fft<T, +1>(buf, g.log2N, bst, tw);
   for (int e = tid; e < N * C; e += nthr) {
     const int n = e >> lC, c = e & (C - 1);
     d[(long long)n * KXP + kx0 + c] = buf[c * bst + sidx<T>(n)];
@@ -69,7 +58,7 @@ __device__ void col_forward_tile(cplx<T>* buf, const cplx<T>* __restrict__ s, cp
     buf[c * bst + sidx<T>(n)] = s[(long long)n * KXP + kx0 + c];
   }
   __syncthreads();
-  block_fft<T, -1, true>(buf, g.log2N, bst, tw);
+  block_fft<T, -1>(buf, g.log2N, bst, tw);
   const T inv = (T)1 / (T)N;
   for (int e = tid; e < g.NY * C; e += nthr) {
     const int kyi = e >> lC, c = e & (C - 1);
@@ -81,64 +70,43 @@ __device__ void col_forward_tile(cplx<T>* buf, const cplx<T>* __restrict__ s, cp
   }
 }
 
-// Generic column passes over explicit field lists (initial condition, output
-// transforms): grid (KXP/4, nout), 4 columns per block.
+// Column passes of one field: grid KXP/4, 4 columns per block.
 template <typename T>
-struct ColInvArgs {
-  const cplx<T>* src;  // spectral fields, stride ms
-  cplx<T>* dst;        // mixed fields, stride mi
+struct ColArgs {
+  const cplx<T>* src;  // inverse: spectral; forward: mixed
+  cplx<T>* dst;
   const cplx<T>* tw;
   Geom g;
-  int nout;
-  int src_idx[MAXI], src2_idx[MAXI], op[MAXI], dst_idx[MAXI];
 };
 
 template <typename T>
-__global__ void __launch_bounds__(1024) k_col_inv(const __grid_constant__ ColInvArgs<T> a) {
+__global__ void __launch_bounds__(1024) k_col_inv(const __grid_constant__ ColArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int o = blockIdx.y;
-  const cplx<T>* s1 = a.src + (long long)a.src_idx[o] * a.g.ms;
-  const cplx<T>* s2 = a.src + (long long)(a.src2_idx[o] < 0 ? a.src_idx[o] : a.src2_idx[o]) * a.g.ms;
-  col_inverse_tile<T>(reinterpret_cast<cplx<T>*>(smem_raw), s1, s2, a.op[o], a.dst + (long long)a.dst_idx[o] * a.g.mi,
-                      a.g, 2, blockIdx.x * 4, a.tw);
+  col_inverse_tile<T>(reinterpret_cast<cplx<T>*>(smem_raw), a.src, a.dst, a.g, 2, blockIdx.x * 4, a.tw);
 }
 
 template <typename T>
-struct ColFwdArgs {
-  const cplx<T>* src;  // mixed, stride mi
-  cplx<T>* dst;        // spectral, stride ms
-  const cplx<T>* tw;
-  Geom g;
-  int nout;
-  int src_idx[MAXP + 8], dst_idx[MAXP + 8];
-};
-
-template <typename T>
-__global__ void __launch_bounds__(1024) k_col_fwd(const __grid_constant__ ColFwdArgs<T> a) {
+__global__ void __launch_bounds__(1024) k_col_fwd(const __grid_constant__ ColArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int o = blockIdx.y;
-  col_forward_tile<T>(reinterpret_cast<cplx<T>*>(smem_raw), a.src + (long long)a.src_idx[o] * a.g.mi,
-                      a.dst + (long long)a.dst_idx[o] * a.g.ms, a.g, 2, blockIdx.x * 4, a.tw);
+  col_forward_tile<T>(reinterpret_cast<cplx<T>*>(smem_raw), a.src, a.dst, a.g, 2, blockIdx.x * 4, a.tw);
 }
 
 // ---------------------------------------------------------------------------
 // Row helpers.  A block owns B consecutive rows; its FFT buffer holds B
 // transforms of length N at stride row_stride(N).
 
-// Fill buf with the Hermitian-paired spectrum Z = A + iB of two real rows
-// whose kx >= 0 halves are mixed fields a and b (b < 0: zero), then inverse
-// FFT: afterwards buf[row][x] = a(x) + i b(x).  The kx = 0 imaginary parts
-// are dropped, as a real inverse transform does.
+// Fill buf with the Hermitian spectrum of real rows whose kx >= 0 halves are the
+// mixed field m, then inverse FFT: afterwards the real part of buf[row][x] is the
+// row.  The kx = 0 imaginary part is dropped, as a real inverse transform does.
 template <typename T>
-__device__ void row_pair_inverse(cplx<T>* buf, const cplx<T>* __restrict__ ma,
-                                 const cplx<T>* __restrict__ mb, int row0, int B,
-                                 const Geom& g, const cplx<T>* __restrict__ tw) {
+__device__ void row_inverse(cplx<T>* buf, const cplx<T>* __restrict__ m, int row0, int B, const Geom& g,
+                            const cplx<T>* __restrict__ tw) {
   const int N = g.N, K = g.K, KXP = g.KXP;
   const int bst = row_stride<T>(N);
   const int nthr = blockDim.x, tid = threadIdx.x;
-  // Z(k) = A + iB and Z(N-k) = conj(A) + i conj(B) for k <= K (each input
-  // read once); the band K < n < N-K is zeroed.  The two writes never touch
-  // the same element, so no barrier separates them.
+  // Z(k) = A and Z(N-k) = conj(A) for k <= K (each input read once); the band
+  // K < n < N-K is zeroed.  The two writes never touch the same element, so no
+  // barrier separates them.
   const int nz = N - 2 * K - 1;
   for (int e = tid; e < B * nz; e += nthr) {
     const int r = e / nz, n = K + 1 + (e - r * nz);
@@ -146,27 +114,24 @@ __device__ void row_pair_inverse(cplx<T>* buf, const cplx<T>* __restrict__ ma,
   }
   for (int e = tid; e < B * (K + 1); e += nthr) {
     const int r = e / (K + 1), k = e - r * (K + 1);
-    const long long off = (long long)(row0 + r) * KXP + k;
-    const cplx<T> A = ma[off];
-    const cplx<T> Bv = mb ? mb[off] : mk<T>(0, 0);
+    const cplx<T> A = m[(long long)(row0 + r) * KXP + k];
     cplx<T>* z = buf + r * bst;
     if (k == 0) {
-      z[0] = mk<T>(A.x, Bv.x);
+      z[0] = mk<T>(A.x, 0);
     } else {
-      z[sidx<T>(k)] = mk<T>(A.x - Bv.y, A.y + Bv.x);
-      z[sidx<T>(N - k)] = mk<T>(A.x + Bv.y, -A.y + Bv.x);
+      z[sidx<T>(k)] = A;
+      z[sidx<T>(N - k)] = mk<T>(A.x, -A.y);
     }
   }
   __syncthreads();
   block_fft<T, +1>(buf, g.log2N, bst, tw);
 }
 
-// Forward FFT of buf (rows holding p(x) + i q(x)) and scatter of the kx in
-// [0, KXP) halves of p and q, scaled by 1/N, into mixed fields da and db.
+// Forward FFT of buf (real rows) and store of the kx in [0, KXP) half, scaled by
+// 1/N, into the mixed field d.
 template <typename T>
-__device__ void row_pair_forward_store(cplx<T>* buf, cplx<T>* __restrict__ da,
-                                       cplx<T>* __restrict__ db, int row0, int B,
-                                       const Geom& g, const cplx<T>* __restrict__ tw) {
+__device__ void row_forward_store(cplx<T>* buf, cplx<T>* __restrict__ d, int row0, int B, const Geom& g,
+                                  const cplx<T>* __restrict__ tw) {
   const int N = g.N, K = g.K, KXP = g.KXP;
   const int bst = row_stride<T>(N);
   const int nthr = blockDim.x, tid = threadIdx.x;
@@ -176,19 +141,14 @@ __device__ void row_pair_forward_store(cplx<T>* buf, cplx<T>* __restrict__ da,
   for (int e = tid; e < B * KXP; e += nthr) {
     const int r = e / KXP, k = e - r * KXP;
     const cplx<T>* z = buf + r * bst;
-    cplx<T> P = mk<T>(0, 0), Q = mk<T>(0, 0);
+    cplx<T> P = mk<T>(0, 0);
     if (k <= K) {
-      cplx<T> z1 = z[sidx<T>(k)];
-      cplx<T> z2 = z[sidx<T>((N - k) & (N - 1))];
-      // P = (Z(k) + conj Z(N-k))/2, Q = (Z(k) - conj Z(N-k))/(2i)
+      // (Z(k) + conj Z(N-k))/2
+      const cplx<T> z1 = z[sidx<T>(k)], z2 = z[sidx<T>((N - k) & (N - 1))];
       P = mk<T>((z1.x + z2.x) * h, (z1.y - z2.y) * h);
-      Q = mk<T>((z1.y + z2.y) * h, (z2.x - z1.x) * h);
     }
-    const long long off = (long long)(row0 + r) * KXP + k;
-    da[off] = P;
-    if (db) db[off] = Q;
+    d[(long long)(row0 + r) * KXP + k] = P;
   }
-  __syncthreads();
 }
 
 // Group-owned row transforms (one row per group of G = N/8 threads, N = 2^L
@@ -268,87 +228,41 @@ __device__ __forceinline__ void dispatch_L(int L, F&& f) {
 }
 
 // ---------------------------------------------------------------------------
-// Row pass, inverse: physical outputs from pairs of mixed fields, with an
-// affine epilogue out = scale*val + ax*x + ay*y + c (mean positions; the
-// depth h = 1 + eta from the stored perturbation eta).
-template <typename T, typename TO>
-struct RowInvArgs {
-  const cplx<T>* src;  // mixed, stride mi
-  TO* dst;             // physical, stride dst_stride
-  long long dst_stride;
+// Row passes of one field between mixed rows and FP64 physical rows, B rows per
+// block.
+template <typename T, typename S, typename D>
+struct RowArgs {
+  const S* src;
+  D* dst;
   const cplx<T>* tw;
   Geom g;
   int B;
-  int npairs;
-  int a_idx[8], b_idx[8];  // source mixed fields (b: -1 for none)
-  int oa[8], ob[8];        // output field indices (-1: skip)
-  double sa[8], sb[8];     // scales
-  double axa[8], aya[8], axb[8], ayb[8];
-  double ca[8], cb[8];  // constant offsets
 };
+template <typename T> using RowInvArgs = RowArgs<T, cplx<T>, double>;
+template <typename T> using RowFwdArgs = RowArgs<T, double, cplx<T>>;
 
-template <typename T, typename TO>
-__global__ void __launch_bounds__(256) k_row_inv(const __grid_constant__ RowInvArgs<T, TO> a) {
+template <typename T>
+__global__ void __launch_bounds__(256) k_row_inv(const __grid_constant__ RowInvArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
-  const Geom& g = a.g;
-  const int N = g.N, B = a.B;
-  const int row0 = blockIdx.x * B;
-  const int nthr = blockDim.x, tid = threadIdx.x;
-  const double dxg = 6.283185307179586476925286766559 / (double)N;
-  for (int p = 0; p < a.npairs; ++p) {
-    const cplx<T>* ma = a.src + (long long)a.a_idx[p] * g.mi;
-    const cplx<T>* mb = a.b_idx[p] >= 0 ? a.src + (long long)a.b_idx[p] * g.mi : nullptr;
-    row_pair_inverse<T>(buf, ma, mb, row0, B, g, a.tw);
-    for (int e = tid; e < B * N; e += nthr) {
-      const int r = e / N, x = e - r * N;
-      const int y = row0 + r;
-      const cplx<T> v = buf[r * row_stride<T>(N) + sidx<T>(x)];
-      const long long off = (long long)y * N + x;
-      if (a.oa[p] >= 0)
-        a.dst[a.oa[p] * a.dst_stride + off] =
-            (TO)(a.sa[p] * (double)v.x + a.axa[p] * (x * dxg) + a.aya[p] * (y * dxg) + a.ca[p]);
-      if (a.ob[p] >= 0)
-        a.dst[a.ob[p] * a.dst_stride + off] =
-            (TO)(a.sb[p] * (double)v.y + a.axb[p] * (x * dxg) + a.ayb[p] * (y * dxg) + a.cb[p]);
-    }
-    __syncthreads();
+  const int N = a.g.N, B = a.B, row0 = blockIdx.x * B;
+  row_inverse<T>(buf, a.src, row0, B, a.g, a.tw);
+  for (int e = threadIdx.x; e < B * N; e += blockDim.x) {
+    const int r = e / N, x = e - r * N;
+    a.dst[(long long)(row0 + r) * N + x] = (double)buf[r * row_stride<T>(N) + sidx<T>(x)].x;
   }
 }
-
-// ---------------------------------------------------------------------------
-// Row pass, forward: mixed outputs from pairs of FP64 physical fields.
-template <typename T>
-struct RowFwdArgs {
-  const double* src;  // physical, stride np
-  cplx<T>* dst;       // mixed, stride mi
-  const cplx<T>* tw;
-  Geom g;
-  int B;
-  int npairs;
-  int a_idx[4], b_idx[4], oa[4], ob[4];
-};
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_row_fwd(const __grid_constant__ RowFwdArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
-  const Geom& g = a.g;
-  const int N = g.N, B = a.B;
-  const int row0 = blockIdx.x * B;
-  const int nthr = blockDim.x, tid = threadIdx.x;
-  for (int p = 0; p < a.npairs; ++p) {
-    const double* pa = a.src + (long long)a.a_idx[p] * g.np;
-    const double* pb = a.b_idx[p] >= 0 ? a.src + (long long)a.b_idx[p] * g.np : nullptr;
-    for (int e = tid; e < B * N; e += nthr) {
-      const int r = e / N, x = e - r * N;
-      const long long off = (long long)(row0 + r) * N + x;
-      buf[r * row_stride<T>(N) + sidx<T>(x)] = mk<T>((T)pa[off], pb ? (T)pb[off] : (T)0);
-    }
-    row_pair_forward_store<T>(buf, a.dst + (long long)a.oa[p] * g.mi,
-                              a.ob[p] >= 0 ? a.dst + (long long)a.ob[p] * g.mi : nullptr,
-                              row0, B, g, a.tw);
+  const int N = a.g.N, B = a.B, row0 = blockIdx.x * B;
+  for (int e = threadIdx.x; e < B * N; e += blockDim.x) {
+    const int r = e / N, x = e - r * N;
+    buf[r * row_stride<T>(N) + sidx<T>(x)] = mk<T>((T)a.src[(long long)(row0 + r) * N + x], (T)0);
   }
+  row_forward_store<T>(buf, a.dst, row0, B, a.g, a.tw);
 }
 
 // ---------------------------------------------------------------------------

@@ -101,7 +101,6 @@ static Layout build_layout(const sw_params& p, int strategy, int fields, int eul
     L.fclass[f] = (f == 2 && p.visc == SW_VISC_LAPLACE) ? IF_NONE : IF_DYN;
     L.fkahan[f] = 0;
     L.frole[f] = R_U + f;
-    L.fslot[f] = 0;
   }
   if (strategy > 0) {
     const int bits[NLMF] = {LM_ZETA, LM_H, LM_U, LM_V, LM_Q};
@@ -110,18 +109,17 @@ static Layout build_layout(const sw_params& p, int strategy, int fields, int eul
     L.has_q = (fields & LM_Q) ? 1 : 0;
     L.has_pos = (strategy == 2 || (fields & LM_POS)) ? 1 : 0;
     L.eulerian = eulerian ? 1 : 0;
-    auto addf = [&](int cls, int role, int slot) {
+    auto addf = [&](int cls, int role) {
       L.fclass[nf] = cls;
       L.fkahan[nf] = 1;
       L.frole[nf] = role;
-      L.fslot[nf] = slot;
       return nf++;
     };
-    for (int j = 0; j < L.nlm; ++j) L.f_g[j] = addf(IF_LM, R_G, j);
+    for (int j = 0; j < L.nlm; ++j) L.f_g[j] = addf(IF_LM, R_G);
     if (L.has_pos)
-      for (int c = 0; c < 2; ++c) L.f_p[c] = addf(IF_LM, R_P, c);
+      for (int c = 0; c < 2; ++c) L.f_p[c] = addf(IF_LM, R_P);
     if (L.eulerian)
-      for (int j = 0; j < L.nlm; ++j) L.f_e[j] = addf(IF_NONE, R_E, j);
+      for (int j = 0; j < L.nlm; ++j) L.f_e[j] = addf(IF_NONE, R_E);
   }
   L.nf = nf;
   // column-pass outputs

@@ -81,9 +81,10 @@ template <typename T> bool row_team(int N, int points, int ppb) {
 
 template <typename T> constexpr int SPLIT_THREADS() { return sizeof(T) == 4 ? 256 : 128; }
 
-template <typename T> cudaError_t launch_col_inv(const ColInvArgs<T>& a, cudaStream_t s);
-template <typename T> cudaError_t launch_col_fwd(const ColFwdArgs<T>& a, cudaStream_t s);
-template <typename T, typename TO> cudaError_t launch_row_inv(const RowInvArgs<T, TO>& a, cudaStream_t s);
+// one field at a time, without device memory of their own (csrc/project_static.cu)
+template <typename T> cudaError_t launch_col_inv(const ColArgs<T>& a, cudaStream_t s);
+template <typename T> cudaError_t launch_col_fwd(const ColArgs<T>& a, cudaStream_t s);
+template <typename T> cudaError_t launch_row_inv(const RowInvArgs<T>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_row_fwd(const RowFwdArgs<T>& a, cudaStream_t s);
 // parts: into how many the column stage's blocks are split (2 and 4: at most
 // SPLIT_THREADS threads).
@@ -137,7 +138,7 @@ template <typename T> static cudaError_t prepare_kernels_t() {
   if constexpr (sizeof(T) == 8) {
     if ((e = allow_dynamic_smem(k_col_inv<T>, mx)) != cudaSuccess) return e;
     if ((e = allow_dynamic_smem(k_col_fwd<T>, mx)) != cudaSuccess) return e;
-    if ((e = allow_dynamic_smem(k_row_inv<T, T>, mx)) != cudaSuccess) return e;
+    if ((e = allow_dynamic_smem(k_row_inv<T>, mx)) != cudaSuccess) return e;
     if ((e = allow_dynamic_smem(k_row_fwd<T>, mx)) != cudaSuccess) return e;
   }
   if ((e = allow_dynamic_smem(k_out_col<T>, mx)) != cudaSuccess) return e;
@@ -160,23 +161,21 @@ template <typename T> static cudaError_t prepare_kernels_t() {
   return cudaSuccess;
 }
 
-template <typename T> cudaError_t launch_col_inv(const ColInvArgs<T>& a, cudaStream_t s) {
+template <typename T> cudaError_t launch_col_inv(const ColArgs<T>& a, cudaStream_t s) {
   const size_t sm = (size_t)4 * col_stride<T>(a.g.N, 4) * sizeof(cplx<T>);
-  dim3 grid(a.g.KXP / 4, a.nout);
-  k_col_inv<T><<<grid, a.g.N / 2, sm, s>>>(a);
+  k_col_inv<T><<<a.g.KXP / 4, a.g.N / 2, sm, s>>>(a);
   return cudaGetLastError();
 }
 
-template <typename T> cudaError_t launch_col_fwd(const ColFwdArgs<T>& a, cudaStream_t s) {
+template <typename T> cudaError_t launch_col_fwd(const ColArgs<T>& a, cudaStream_t s) {
   const size_t sm = (size_t)4 * col_stride<T>(a.g.N, 4) * sizeof(cplx<T>);
-  dim3 grid(a.g.KXP / 4, a.nout);
-  k_col_fwd<T><<<grid, a.g.N / 2, sm, s>>>(a);
+  k_col_fwd<T><<<a.g.KXP / 4, a.g.N / 2, sm, s>>>(a);
   return cudaGetLastError();
 }
 
-template <typename T, typename TO> cudaError_t launch_row_inv(const RowInvArgs<T, TO>& a, cudaStream_t s) {
+template <typename T> cudaError_t launch_row_inv(const RowInvArgs<T>& a, cudaStream_t s) {
   const size_t sm = (size_t)a.B * row_stride<T>(a.g.N) * sizeof(cplx<T>);
-  k_row_inv<T, TO><<<a.g.N / a.B, a.B * a.g.N / 8, sm, s>>>(a);
+  k_row_inv<T><<<a.g.N / a.B, a.B * a.g.N / 8, sm, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -271,9 +270,9 @@ cudaError_t launch_velocity_from_vorticity(cplx<T>* y, const Geom& g, int fu, in
   template cudaError_t launch_velocity_from_vorticity<T>(cplx<T>*, const Geom&, int, int, int, cudaStream_t);
 // the generic FP64 transforms (csrc/project_static.cu)
 #define LM_INSTANTIATE_GENERIC                                                                              \
-  template cudaError_t launch_col_inv<double>(const ColInvArgs<double>&, cudaStream_t);                      \
-  template cudaError_t launch_col_fwd<double>(const ColFwdArgs<double>&, cudaStream_t);                      \
-  template cudaError_t launch_row_inv<double, double>(const RowInvArgs<double, double>&, cudaStream_t);      \
+  template cudaError_t launch_col_inv<double>(const ColArgs<double>&, cudaStream_t);                         \
+  template cudaError_t launch_col_fwd<double>(const ColArgs<double>&, cudaStream_t);                         \
+  template cudaError_t launch_row_inv<double>(const RowInvArgs<double>&, cudaStream_t);                      \
   template cudaError_t launch_row_fwd<double>(const RowFwdArgs<double>&, cudaStream_t);
 #endif
 

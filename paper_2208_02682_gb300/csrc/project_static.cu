@@ -1,9 +1,9 @@
 // project_static.cu -- sw_project_static: projection of one physical field
 // onto the 2/3-dealiased spectral box with no device allocation.
 //
-// Same kernels as the initial-condition and output transforms of a handle
-// (FP64 row forward pass, column forward pass with the 2/3 mask, column
-// inverse pass, row inverse pass); the mixed and spectral intermediates and
+// FP64 block transforms of one field (row forward pass, column forward pass with
+// the 2/3 mask, column inverse pass, row inverse pass), which take every pointer as
+// an argument; the mixed and spectral intermediates and
 // the twiddle table live in the file-scope array below instead of memory
 // obtained from cudaMalloc.
 #include <cuda_runtime.h>
@@ -123,59 +123,10 @@ extern "C" int sw_project_static(const double* in, double* out, int N, void* str
   k_static_twiddles<<<(N + 255) / 256, 256, 0, s>>>(tw, N, g.log2N);
   cudaError_t e = cudaGetLastError();
   const int B = row_block_rows(N);
-  if (e == cudaSuccess) {
-    RowFwdArgs<double> rf = {};
-    rf.src = in;
-    rf.dst = mixed;
-    rf.tw = tw;
-    rf.g = g;
-    rf.B = B;
-    rf.npairs = 1;
-    rf.a_idx[0] = 0;
-    rf.b_idx[0] = -1;
-    rf.oa[0] = 0;
-    rf.ob[0] = -1;
-    e = launch_row_fwd<double>(rf, s);
-  }
-  if (e == cudaSuccess) {
-    ColFwdArgs<double> cf;
-    cf.src = mixed;
-    cf.dst = spec;
-    cf.tw = tw;
-    cf.g = g;
-    cf.nout = 1;
-    cf.src_idx[0] = cf.dst_idx[0] = 0;
-    e = launch_col_fwd<double>(cf, s);
-  }
-  if (e == cudaSuccess) {
-    ColInvArgs<double> ci;
-    ci.src = spec;
-    ci.dst = mixed;
-    ci.tw = tw;
-    ci.g = g;
-    ci.nout = 1;
-    ci.src_idx[0] = 0;
-    ci.src2_idx[0] = -1;
-    ci.op[0] = OP_ID;
-    ci.dst_idx[0] = 0;
-    e = launch_col_inv<double>(ci, s);
-  }
-  if (e == cudaSuccess) {
-    RowInvArgs<double, double> ri = {};
-    ri.src = mixed;
-    ri.dst = out;
-    ri.dst_stride = g.np;
-    ri.tw = tw;
-    ri.g = g;
-    ri.B = B;
-    ri.npairs = 1;
-    ri.a_idx[0] = 0;
-    ri.b_idx[0] = -1;
-    ri.oa[0] = 0;
-    ri.ob[0] = -1;
-    ri.sa[0] = 1.0;
-    e = launch_row_inv<double, double>(ri, s);
-  }
+  if (e == cudaSuccess) e = launch_row_fwd<double>({in, mixed, tw, g, B}, s);
+  if (e == cudaSuccess) e = launch_col_fwd<double>({mixed, spec, tw, g}, s);
+  if (e == cudaSuccess) e = launch_col_inv<double>({spec, mixed, tw, g}, s);
+  if (e == cudaSuccess) e = launch_row_inv<double>({mixed, out, tw, g, B}, s);
   if (e != cudaSuccess) {
     set_handleless_error(std::string("sw_project_static: launch: ") + cudaGetErrorString(e));
     return SW_ECUDA;
