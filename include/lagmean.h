@@ -244,7 +244,7 @@ int sw_time(sw_handle* h, double* t);
 #define SW_K_COL_FWD 3  /* not reported (part of SW_K_COL_STAGE)                    */
 #define SW_K_UPDATE 4   /* right-hand sides and update of runs without transforms   */
                         /* (kinematic dynamics; else part of SW_K_COL_STAGE)        */
-#define SW_K_PHYS_Q 5   /* potential vorticity in the gather buffer (Strategy 2)    */
+#define SW_K_PHYS_Q 5   /* not reported (part of SW_K_ROW_INV)                      */
 #define SW_K_COL_STAGE 6 /* column pass: forward y-FFT and 2/3 mask, right-hand     */
                          /* sides and integrating-factor update, inverse y-FFT of   */
                          /* the next stage (SW_K_COL_INV: the first stage only)     */

@@ -286,7 +286,7 @@ extern "C" int sw_sl_create(sw_handle* h, const sl_params* p, sl_interval** out)
       return rc;
     }
     SLArgs a = sl_args(s, phys);
-    a.f1 = s->f[s->cur];  // f at tau is read by the first step
+    a.f1 = s->f[s->cur];  // dt f/2 at tau is read by the first step
     k_sl_init<<<(unsigned)((np + 255) / 256), 256, 0, st>>>(a);
     e = cudaGetLastError();
   }

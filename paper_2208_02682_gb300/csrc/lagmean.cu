@@ -907,22 +907,17 @@ static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 static const int DIAG_BLOCKS = 1024;
 
-// Grid geometry: cutoff K, column tiles of C = 2048/N columns (at most 32:
-// C*N is the same for all grids up to 512, so they can share batched
-// launches; in FP32 at least 4, so that the lanes of a warp move 32-byte runs
-// of a row: one-column tiles at 2048^2 used a quarter of every 32-byte
-// sector of their strided accesses) and the padded column count KXP (a
-// multiple of C and of 4).  FP64 keeps C*N = 2048 (256 threads per column
-// block): its column passes are bound by FP64 arithmetic, and four FP64
-// columns of 2048 points would not fit in shared memory.
+// Grid geometry: cutoff K, the most columns 2^lC a column tile may have (2048/N, at
+// most 32, so that grids of 64 to 512 can have tiles of equal points in a batch;
+// in FP32 at least 4, which move whole 32-byte sectors; four FP64 columns of 2048
+// points would not fit in shared memory; a launch's own tiles: batch_build_t) and the
+// padded column count KXP (a multiple of 2^lC and of 4).
 static void plan_geometry(int N, size_t tsz, Geom& g, int& lC) {
   g.N = N;
   g.log2N = 0;
   while ((1 << g.log2N) < g.N) ++g.log2N;
   g.K = (g.N - 1) / 3;
   g.KX = g.K + 1;
-  // C = 2048/N columns (at most 32): every column block holds 2048
-  // elements (256 threads); KXP stays a multiple of 4 for the generic passes
   lC = 0;
   while ((1 << lC) * g.N < 2048 && lC < 5) ++lC;
   if (tsz == 4 && lC < 2) lC = 2;
@@ -1652,7 +1647,7 @@ extern "C" int sw_batch_tune(sw_batch* b, int trial_steps, int* choice) {
     }
   }
   if (rc == SW_OK && e != cudaSuccess) rc = bfail(b, SW_ECUDA, std::string("tuning trial: ") + cudaGetErrorString(e));
-  if (best < 0) {  // no trial ran: the default shape (512 points or one row, all pairs)
+  if (best < 0) {  // no trial ran: a shape every member fits (512 points or one row pair, all products)
     int pi = 1;
     while (pi < 3 && pts[pi] < maxN) ++pi;
     best = 4 * pi + 3;

@@ -74,7 +74,7 @@ __device__ __forceinline__ double blend(const Cell& c, double f00, double f01, d
   return __dadd_rn(s, __dmul_rn(c.w11, f11));
 }
 
-// Bound by FP64 issue: the 28 additions and multiplications of an iteration
+// Bound by FP64 issue: the 24 additions and multiplications of an iteration
 // that must be rounded as written (1024^2, 20 iterations, four fields: with
 // floor, its conversion and the corner differences in FP64 every iteration
 // 1.74 ms, this 1.46 ms).

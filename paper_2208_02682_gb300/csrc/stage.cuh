@@ -86,7 +86,8 @@ __device__ __forceinline__ const cplx<T>* stage_input(const RunDesc<T>& d, int s
 // a3: base planes (physical u, v, h, zeta and, Strategy 2, xi and, with PV
 // averaged, q = (f0 + zeta)/h, h = 1 + eta) of the runs whose row pass does not
 // form them itself.  Local block = (field, block of Bi row pairs, one pair per
-// group of N/8 threads).
+// group of N/8 threads); a team's block has four sets of groups, of which h, zeta and q
+// use more than one (16^2 FP64: 12.3 -> 10.5 us, with q 18.4 -> 12.4).
 template <typename T, bool WARP>
 __global__ void __launch_bounds__(256) k_stage_row_inv(const RunDesc<T>* __restrict__ runs,
                                                        const int* __restrict__ start, int nruns) {
@@ -180,8 +181,8 @@ __global__ void __launch_bounds__(256) k_stage_row_inv(const RunDesc<T>* __restr
 // shared memory.  The others read base values from the planes that the row
 // inverse pass wrote; Strategy 2 gathers from them too: `gath` runs (where the
 // arrays fit and a block takes all products) once for all products, into shared
-// memory, from interleaved planes (each product gathering for itself from separate planes took 34.7 us
-// at 512^2 with five means, this 26.7 us).  Every transform stays in the
+// memory, from interleaved planes (each product gathering for itself from
+// separate planes took 34.7 us at 512^2 with five means, this 26.7 us).  Every transform stays in the
 // registers of its group: an advection product takes the inverse transforms
 // of d_x G and d_y G and, from the same positions, the forward transform of
 // u d_x G + v d_y G; one transform instance serves both directions (the
@@ -598,9 +599,10 @@ template <typename T> __device__ __forceinline__ void finish_step(const RunDesc<
 template <typename T> __device__ __forceinline__ cplx<T> cswap(cplx<T> a) { return mk<T>(a.y, a.x); }
 
 // Column-stage kernels by the largest block: FP64 128 threads (grids up to
-// 512^2: few warps per SM, so many registers and three modes in flight; 64^2
-// 42 -> 38 us, 256^2 56 -> 50 us) and 256; FP32 256 (to 512^2), 512 (1024^2) and
-// 1024 (2048^2).
+// 512^2: few warps per SM, so many registers and three modes in flight, which spill 250
+// to 410 bytes at 255 registers; two spill none: a Strategy-1 step 143.1 against 141.9 us
+// at 64^2, but 295.7 against 300.5 at 256^2 and 610 against 647 at 512^2) and 256;
+// FP32 256 (to 512^2), 512 (1024^2) and 1024 (2048^2).
 // PARTS: a task's steps are shared out over two or four parts of a block, each
 // with its own exchange buffers and barrier (block barriers where a value passes
 // between them): while a launch has about one block per SM its time is the
