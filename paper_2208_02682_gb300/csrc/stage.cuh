@@ -836,7 +836,11 @@ __global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, PARTS>::BLOCKS) k_stag
                 if (st == 2) cr = x1 ? (T)2 * dt * ee * ee : dt * ee;
               }
             }
-            nv[i] = mk<T>(fma(ca, yn[i].x, cb * rr[i].x), fma(ca, yn[i].y, cb * rr[i].y));
+            nv[i] = z;
+            if (sizeof(T) == 4 || st != 2) {  // (forward Euler's first pass has no stage value)
+              if (sizeof(T) == 8) asm volatile("");
+              nv[i] = mk<T>(fma(ca, yn[i].x, cb * rr[i].x), fma(ca, yn[i].y, cb * rr[i].y));
+            }
             ac[i] = mk<T>(fma(cr, rr[i].x, ac[i].x), fma(cr, rr[i].y, ac[i].y));
             if (in[i] && act) gst(af + ml[i], ac[i]);
             nv[i] = in[i] ? nv[i] : z;
@@ -932,7 +936,12 @@ __global__ void __launch_bounds__(MAXT, ColShape<T, MAXT, PARTS>::BLOCKS) k_stag
           cplx<T>* const cf = d.comp + f * ms;
 #pragma unroll
           for (int i = 0; i < NB; ++i) {
-            nv[i] = commit_mode<T>(kah, eh[i], el[i], yn[i], cc[i], cscale<T>(cadd<T>(ac[i], rr[i]), ci));
+            cplx<T> inc = ac[i];
+            if (sizeof(T) == 4 || !commit) {  // (forward Euler commits acc itself)
+              if (sizeof(T) == 8) asm volatile("");
+              inc = cscale<T>(cadd<T>(ac[i], rr[i]), ci);
+            }
+            nv[i] = commit_mode<T>(kah, eh[i], el[i], yn[i], cc[i], inc);
             if (!act) nv[i] = yn[i];
             if (in[i] && act) {
               gst(yf + ml[i], nv[i]);
