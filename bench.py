@@ -656,7 +656,7 @@ TRAFFIC_CAPTURES = {
     # caches (column stage: an early stage of a step)
     ("row_prod", 2048): 264_500_000, ("col_stage", 2048): 521_600_000,
 }
-TRAFFIC_SOURCES_SHA256 = "34d0d78091ef4021232649ef8cbc51e7bf35c44eb2af4b0b4bfcfa6bddb832bf"
+TRAFFIC_SOURCES_SHA256 = "6ca1bface21eb141f784fcc68af8575dfddd6267ddad8ecd963e25e6da563f33"
 
 
 # the sources that define the stage kernels and their launch shapes

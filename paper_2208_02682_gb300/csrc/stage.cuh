@@ -430,46 +430,46 @@ __global__ void __launch_bounds__(row_prod_max_threads<T>(), sizeof(T) == 4 ? 1 
         sub = shared ? 2 : sub + 1;
 #pragma unroll 1
         for (int part = from; part < sub; ++part) {
-        const bool second = part == 1;
-        if (shared && second) {
+          const bool second = part == 1;
+          if (shared && second) {
 #pragma unroll
-          for (int m = 0; m < 8; ++m) x[m] = XY[m * G];
-        }
-        if (kind == PK_ADV) {
-          // u.grad G (Eq. gtilde-evol) or u.grad D
-          const T av = second ? adv_y : adv_x;
-#pragma unroll
-          for (int m = 0; m < 8; ++m) {
-            const cplx<T> ua = kin ? mk<T>(av, av) : base(second ? PH_V : PH_U, m);
-            const cplx<T> a = second ? acc[m] : mk<T>(0, 0);
-            acc[m] = mk<T>(fma(ua.x, x[m].y, a.x), fma(ua.y, x[m].x, a.y));
+            for (int m = 0; m < 8; ++m) x[m] = XY[m * G];
           }
-        } else {
-          // Strategy 2, Eqs. (xi_evol), (barf_xi): w = xi/s, limit u/2 at s = 0
-          const bool sz = s0 && !(xf && kind == PK_GBAR);
-          const T is = kind == PK_GBAR ? inv_sg : inv_s;
-          const T av = second ? adv_y : adv_x;
-          const int comp = second ? 1 : 0;
+          if (kind == PK_ADV) {
+            // u.grad G (Eq. gtilde-evol) or u.grad D
+            const T av = second ? adv_y : adv_x;
 #pragma unroll
-          for (int m = 0; m < 8; ++m) {
-            cplx<T> wv;
-            if (sz) {
-              const cplx<T> ua = kin ? mk<T>(av, av) : base(PH_U + comp, m);
-              wv = mk<T>((T)0.5 * ua.x, (T)0.5 * ua.y);
-            } else {
-              const cplx<T> xi = base(PH_XX + comp, m);
-              wv = mk<T>(xi.x * is, xi.y * is);
+            for (int m = 0; m < 8; ++m) {
+              const cplx<T> ua = kin ? mk<T>(av, av) : base(second ? PH_V : PH_U, m);
+              const cplx<T> a = second ? acc[m] : mk<T>(0, 0);
+              acc[m] = mk<T>(fma(ua.x, x[m].y, a.x), fma(ua.y, x[m].x, a.y));
             }
-            cplx<T> a = acc[m];
-            a.x -= wv.x * x[m].y;
-            a.y -= wv.y * x[m].x;
-            if (kind == PK_XI && pc == comp) {
-              a.x -= wv.x;
-              a.y -= wv.y;
+          } else {
+            // Strategy 2, Eqs. (xi_evol), (barf_xi): w = xi/s, limit u/2 at s = 0
+            const bool sz = s0 && !(xf && kind == PK_GBAR);
+            const T is = kind == PK_GBAR ? inv_sg : inv_s;
+            const T av = second ? adv_y : adv_x;
+            const int comp = second ? 1 : 0;
+#pragma unroll
+            for (int m = 0; m < 8; ++m) {
+              cplx<T> wv;
+              if (sz) {
+                const cplx<T> ua = kin ? mk<T>(av, av) : base(PH_U + comp, m);
+                wv = mk<T>((T)0.5 * ua.x, (T)0.5 * ua.y);
+              } else {
+                const cplx<T> xi = base(PH_XX + comp, m);
+                wv = mk<T>(xi.x * is, xi.y * is);
+              }
+              cplx<T> a = acc[m];
+              a.x -= wv.x * x[m].y;
+              a.y -= wv.y * x[m].x;
+              if (kind == PK_XI && pc == comp) {
+                a.x -= wv.x;
+                a.y -= wv.y;
+              }
+              acc[m] = a;
             }
-            acc[m] = a;
           }
-        }
         }
       }
     }
